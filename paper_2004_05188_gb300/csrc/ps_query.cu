@@ -35,6 +35,7 @@
 #include <vector>
 
 #include "ps_internal.cuh"
+#include "ps_sweep.cuh"
 
 namespace ps {
 
@@ -71,7 +72,6 @@ struct QueryArgs {
   int fallback;           // 1: only the centrals marked in need[] (the full-radius kNN pass)
   uint32_t* next_front;   // work counters of the front (heavy) and back (light) items
   uint32_t* next_light;
-  const uint32_t* pfx;    // symmetric RDF pass: central prefix over the neighbour records
   int vertex;             // near kNN pass on the vertex-centred central list (see vertex_run)
   // bin lookup table (lut_shift = 0: none): cell c covers the float32 bit patterns
   // [(lut_base + c) << lut_shift, (lut_base + c + 1) << lut_shift), at most one interior edge each
@@ -932,214 +932,205 @@ __global__ void __launch_bounds__(256) k_query_cta(const QueryArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// symmetric RDF pass: every unordered pair of neighbour records once
-//
-// The RDF counts ordered pairs (i central, j neighbour, j != i).  When the centrals are
-// neighbour records, an unordered pair {i, j} contributes c_i + c_j (c = 1 for a central
-// record), and d2_ij == d2_ji bit for bit (x_j - x_i == -(x_i - x_j) in IEEE arithmetic), so
-// each pair is tested once, from the lower of its two cells: the half of the stencil with
-// (dz > 0) or (dz == 0 and dy > 0) or (dz == dy == 0 and dx > 0), plus the pairs i < j inside
-// the cell.  A warp takes 32 cells at a time, and for each non-empty cell tests the half
-// stencil's records (the lanes, 32 per load) against the cell's records (staged in shared
-// memory, read by all lanes at once, two at a time with packed float32 math); the hits (d2,
-// weight) are compacted into a warp list and binned into the warp's 32-bit shared row by all
-// lanes.  The flags come from the central prefix pfx over the records (c_j = pfx[j+1] - pfx[j]).
+// symmetric RDF pass: every unordered pair of neighbour records once (sweep_pairs)
 // ---------------------------------------------------------------------------
+constexpr float kMagic = 12582912.0f;           // 1.5 * 2^23: x + kMagic holds floor(x) in its low bits
+constexpr uint32_t kMagicBits = 0x4B400000u;
+constexpr float kBinBias = 1.0f / 2097152.0f;   // 2^-21
 
-// half-stencil run r of cell c: the x-runs of the rows with dz > 0 (all dy) and of the rows
-// dz == 0, dy > 0 (each over its width, see row_width); the row dz == dy == 0 from cx + 1 on.
-// (2s+1)s + s + 1 runs.
-__device__ __forceinline__ void sym_run(const QueryArgs& a, const Geo& ng, uint32_t c, uint32_t r, uint32_t& src,
-                                        uint32_t& len) {
-  const int s = a.stencil, W = 2 * s + 1;
-  const uint32_t cx = c % ng.dims[0], cy = (c / ng.dims[0]) % ng.dims[1], cz = c / (ng.dims[0] * ng.dims[1]);
-  src = 0;
-  len = 0;
-  int dy, dz;
-  if ((int)r < W * s) {
-    dz = 1 + (int)r / W;
-    dy = (int)r % W - s;
-  } else if ((int)r < W * s + s) {
-    dz = 0;
-    dy = 1 + ((int)r - W * s);
-  } else if ((int)r == W * s + s) {
-    // own row, the cells after c: cx + 1 .. cx + s
-    const uint32_t xhi = cx + s < ng.dims[0] ? cx + s : ng.dims[0] - 1;
-    if (cx + 1 <= xhi) {
-      const uint32_t row = (cz * ng.dims[1] + cy) * ng.dims[0];
-      src = a.nstart[row + cx + 1];
-      len = a.nstart[row + xhi + 1] - src;
-    }
-    return;
-  } else {
-    return;
-  }
-  row_run(a, ng, cx, (int)cy + dy, (int)cz + dz, row_width(a, dy, dz), src, len);
+__device__ __forceinline__ float sqrt_fast(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f2_fma_down(unsigned long long a, unsigned long long b,
+                                                          unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ void red_shared_inc(uint32_t addr) {
+  asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr));
+}
+__device__ __forceinline__ void red_shared(uint32_t addr, uint32_t v) {
+  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v));
 }
 
-constexpr uint32_t kSymGroup = 64;  // records of a cell staged at a time by the symmetric pass
+// Bins of the direct form (r0 = 0).  With s = sqrt.approx(d2) and inv = (1 +- 2^-21) / dr, the true
+// quotient sqrt(d2) / dr lies between s * inv- and s * inv+ (the root is good to 2^-23, inv to 2^-24,
+// the edge table to 2^-25 of the distance).  The bin is floor(s * inv+), or the one below where the two floors
+// differ (2 in 10^4 pairs at 200 bins): those compare d2 with that edge.  Pairs out of range are
+// clamped into the unused bin n_bins, so that every lane increments and no instruction is
+// predicated: the compiler branches around a predicated shared-memory increment.  Measured on the
+// pair loop alone (cycles per 32 tests and scheduler): 23 with a predicated increment and the excess over
+// the edge computed, 17 in this form, of which 14.5 are the distance, root and floor; no table load per pair, so
+// the shared-memory pipe is left to the increments (increments by one merge in a bin).
+struct FastBins {
+  const float* sE;
+  unsigned long long hi2, lo2, magic2;
+  float s_far;
+  __device__ void init(const QueryArgs& a, const float* edges) {
+    sE = edges;
+    const float hi = (float)((1.0 + (double)kBinBias) / a.dr), lo = (float)((1.0 - (double)kBinBias) / a.dr);
+    hi2 = f2_pack(hi, hi);
+    lo2 = f2_pack(lo, lo);
+    magic2 = f2_pack(kMagic, kMagic);
+    s_far = (float)(((double)a.n_bins + 0.5) * a.dr);
+  }
+  // counts two pairs in the row at shared address `base` (bin b at base + 4 (kMagicBits + b));
+  // returns 0 unless one of them may lie under the edge of its bin
+  __device__ __forceinline__ uint32_t count2(unsigned long long d2, uint32_t base) const {
+    float da, db, ma, mb, la, lb;
+    f2_unpack(d2, da, db);
+    const unsigned long long s2 = f2_pack(fminf(sqrt_fast(da), s_far), fminf(sqrt_fast(db), s_far));
+    f2_unpack(f2_fma_down(s2, hi2, magic2), ma, mb);
+    f2_unpack(f2_fma_down(s2, lo2, magic2), la, lb);
+    red_shared_inc(__float_as_uint(ma) * 4u + base);
+    red_shared_inc(__float_as_uint(mb) * 4u + base);
+    return (__float_as_uint(ma) ^ __float_as_uint(la)) | (__float_as_uint(mb) ^ __float_as_uint(lb));
+  }
+  // a counted pair that may lie under the edge of its bin: moved to the bin below if it does
+  __device__ __forceinline__ void settle(float d2, uint32_t base) const {
+    float m, x;
+    f2_unpack(f2_fma_down(f2_pack(fminf(sqrt_fast(d2), s_far), 0.f), hi2, magic2), m, x);
+    const uint32_t addr = __float_as_uint(m) * 4u + base;
+    if (d2 < sE[__float_as_uint(m) - kMagicBits]) {
+      red_shared(addr, ~0u);
+      red_shared_inc(addr - 4u);
+    }
+  }
+  __device__ __forceinline__ void settle2(unsigned long long d2, uint32_t base) const {
+    float da, db;
+    f2_unpack(d2, da, db);
+    settle(da, base);
+    settle(db, base);
+  }
+};
 
-__global__ void __launch_bounds__(256, 4) k_rdf_sym(const QueryArgs a) {
+// Bound by instruction issue and the shared-memory pipe (ncu, 2e5 cylinder: 77 % of the issue slots,
+// two bank cycles per increment).  FAST (r0 = 0, at most kPrivBins bins; the host's rule in run_query):
+// two 32-bit rows per warp, for pairs of weight 1 and 2, and one increment per test by every
+// lane.  With the candidates cut down to those near the staged records two of five tests hit, and a
+// warp list of the hits (ballots, counts, a store and a load each) costs more than the idle lanes.
+// Measured, all-all, one box (ms): 1e8-ion needle 192.8 -> 76.7, 8e6-ion needle 14.95 -> 5.85,
+// 2e5 cylinder 0.504 -> 0.232 (before: full half stencils, warp list of hits, bin table).
+// Otherwise (r0 > 0 or more bins): the general bins of Hist, a branch per hit.
+template <bool FAST>
+__global__ void __launch_bounds__(256, 4) k_rdf_sym(const QueryArgs a, const __grid_constant__ SweepArgs sw) {
   griddep_wait();
   griddep_launch();
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ float4 s_grp[8][kSymGroup];          // per warp: the cell's records as interleaved pairs
-  __shared__ uint32_t s_hits[8][32 * kHalf + 32];  // per warp: the hits of 8 record pairs + a trash row: the
-                                                  // bits of d2, the sign bit set for weight 2
-  __shared__ uint32_t s_rsrc[8][kMaxRuns], s_rpre[8][kMaxRuns + 1];
-  Hist<true> H;
-  H.init(a, smem, 0, true);
+  __shared__ SweepBuf s_sweep[8];
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint32_t lt = (1u << lane) - 1u;
-  uint64_t wcount = 0;  // increments of this warp's private row since its last flush (uniform)
-  const Geo ng = *a.ngeo;
-  const uint32_t n_cells = ng.n_cells;
-  const int s = a.stencil, n_runs = (2 * s + 1) * s + s + 1;
-  uint64_t my_binned = 0;
-  uint32_t my_below = 0;
-  float* gf = reinterpret_cast<float*>(s_grp[w]);
-  uint32_t* wlist = s_hits[w];
-  uint32_t* rsrc = s_rsrc[w];
-  uint32_t* rpre = s_rpre[w];
-  const float E_max = H.Emax;
-
-  // cells per take: a share of the cells left (at most 32, at least 1), so that the warps finish
-  // together -- a take of 32 cells is a large part of a warp's work on a small grid
-  const uint32_t n_warps = gridDim.x * (blockDim.x >> 5);
-  for (;;) {
-    uint32_t base = 0, take = 0;
-    if (lane == 0) {
-      const uint32_t cur = *reinterpret_cast<volatile uint32_t*>(&a.cgeo->sym_next);
-      const uint32_t left = cur < n_cells ? n_cells - cur : 0u;
-      take = min(32u, max(1u, left / (8 * n_warps)));
-      base = atomicAdd(&a.cgeo->sym_next, take);
+  SweepBuf& buf = s_sweep[w];
+  uint64_t wcount = 0;  // bound on the increments of this warp's rows since their last flush (uniform)
+  if constexpr (FAST) {
+    const uint32_t nb = a.n_bins, stride = nb + 1;  // bin n_bins: out of range
+    float* sE = reinterpret_cast<float*>(smem);
+    uint32_t* rows = reinterpret_cast<uint32_t*>(sE + stride);  // [8][2][stride]
+    for (uint32_t b = threadIdx.x; b <= nb; b += blockDim.x) {
+      const double e = __dadd_rn(a.r0, __dmul_rn((double)b, a.dr));
+      sE[b] = __double2float_rn(__dmul_rn(e, e));
     }
-    base = __shfl_sync(0xffffffffu, base, 0);
-    take = __shfl_sync(0xffffffffu, take, 0);
-    if (base >= n_cells) break;
-    uint32_t s0 = 0, s1 = 0;
-    if (lane < take && base + lane < n_cells) s0 = a.nstart[base + lane], s1 = a.nstart[base + lane + 1];
-    uint32_t todo = __ballot_sync(0xffffffffu, s1 > s0);
-    while (todo) {
-      const int src_lane = __ffs(todo) - 1;
-      todo &= todo - 1u;
-      const uint32_t c = base + (uint32_t)src_lane;
-      const uint32_t a0 = __shfl_sync(0xffffffffu, s0, src_lane), a1 = __shfl_sync(0xffffffffu, s1, src_lane);
-      // run table of the half stencil
-      const uint32_t n_cand = run_table(lane, n_runs, rsrc, rpre,
-                                        [&](uint32_t r, uint32_t& src, uint32_t& len) { sym_run(a, ng, c, r, src, len); });
-
-      // pairs inside the cell: record i (a lane) with j in (i, a1), each lane on its own (a small
-      // share of the pairs)
-      for (uint32_t i0 = a0; i0 < a1; i0 += 32) {
-        const uint32_t i = i0 + lane;
-        uint32_t inc = 0;
-        if (i < a1) {
-          const float4 p = __ldg(a.nrec + i);
-          const uint32_t ci = __ldg(a.pfx + i + 1) - __ldg(a.pfx + i);
-          const bool big = a1 - a0 > (1u << 20);  // per-lane increments stay far below the row's 2^32
-          for (uint32_t j = i + 1; j < a1; ++j) {
-            const float4 q = __ldg(a.nrec + j);
-            const float d2 = dist2(p.x, p.y, p.z, q.x, q.y, q.z);
-            const uint32_t wt = ci + (__ldg(a.pfx + j + 1) - __ldg(a.pfx + j));
-            if (d2 < E_max && wt) {
-              if (big) {
-                H.pair_global(a, d2, wt, my_binned, my_below);
-              } else {
-                H.pair_w(d2, wt, my_below);
-                inc += wt;
-              }
-            }
-          }
-        }
-        wcount += __reduce_add_sync(0xffffffffu, inc);
-        if (wcount >= (1ull << 31)) {
-          H.flush_warp(a);
-          wcount = 0;
+    for (uint32_t b = threadIdx.x; b < 16 * stride; b += blockDim.x) rows[b] = 0;
+    __syncthreads();
+    FastBins fb;
+    fb.init(a, sE);
+    uint32_t* row1 = rows + 2 * w * stride;
+    const uint32_t a1 = smem_u32(row1), base1 = a1 - 4u * kMagicBits, base2 = base1 + 4u * stride;
+    const unsigned long long one2 = f2_pack(sw.one, sw.one);
+    sweep_pairs<false>(sw, buf, [&](uint32_t n_pr, uint32_t, uint32_t nc, bool) __attribute__((always_inline)) {
+      const float4 far = make_float4(INFINITY, INFINITY, INFINITY, __uint_as_float(kCandSingle));
+      const float4 c0 = lane < nc ? buf.cand[lane] : far, c1 = lane + 32 < nc ? buf.cand[lane + 32] : far;
+      const uint32_t k0 = __float_as_uint(c0.w), k1 = __float_as_uint(c1.w);
+      const uint32_t b0 = k0 == kCandBoth ? base2 : base1, b1 = k1 == kCandBoth ? base2 : base1;
+      const unsigned long long x0 = f2_pack(c0.x, c0.x), y0 = f2_pack(c0.y, c0.y), z0 = f2_pack(c0.z, c0.z);
+      const unsigned long long x1 = f2_pack(c1.x, c1.x), y1 = f2_pack(c1.y, c1.y), z1 = f2_pack(c1.z, c1.z);
+      const ulonglong2* rxy = reinterpret_cast<const ulonglong2*>(buf.rxy);
+      const ulonglong2* rz = reinterpret_cast<const ulonglong2*>(buf.rz);
+#pragma unroll 1
+      for (uint32_t k = 0; k < n_pr; k += 2) {  // 4 records against the lane's 2 candidates
+        const ulonglong2 xy = rxy[k], xy2 = rxy[k + 1], zz = rz[k >> 1];
+        const unsigned long long d0 = dist2_x2_fma(xy.x, xy.y, zz.x, x0, y0, z0, one2);
+        const unsigned long long d1 = dist2_x2_fma(xy.x, xy.y, zz.x, x1, y1, z1, one2);
+        const unsigned long long d2 = dist2_x2_fma(xy2.x, xy2.y, zz.y, x0, y0, z0, one2);
+        const unsigned long long d3 = dist2_x2_fma(xy2.x, xy2.y, zz.y, x1, y1, z1, one2);
+        const uint32_t x = fb.count2(d0, b0) | fb.count2(d1, b1) | fb.count2(d2, b0) | fb.count2(d3, b1);
+        if (__any_sync(0xffffffffu, x != 0u)) {
+          fb.settle2(d0, b0);
+          fb.settle2(d1, b1);
+          fb.settle2(d2, b0);
+          fb.settle2(d3, b1);
         }
       }
-      if (n_cand == 0) continue;
-
-      // the half stencil: the candidates are the lanes (32 per coalesced load, each in registers),
-      // the cell's records are staged in shared memory (up to kSymGroup at a time, as interleaved
-      // pairs xa xb ya yb za zb ea eb) and read by every lane at once, two per packed test; a
-      // record's e (and a candidate's) is E[nb] for a central and -1 otherwise, the range of a
-      // pair max(e_rec, e_cand), weight 2 (sign bit) when both are central.  The lanes stay busy
-      // whatever the cell's record count.
-      for (uint32_t g0 = a0; g0 < a1; g0 += kSymGroup) {
-        const uint32_t m = min(kSymGroup, a1 - g0), n_pr = (m + 1) >> 1;
+      // the staged records met themselves once each, at d2 = 0
+      const uint32_t self = __popc(__ballot_sync(0xffffffffu, k0 == kCandSelf)) +
+                            __popc(__ballot_sync(0xffffffffu, k1 == kCandSelf));
+      if (self && lane == 0) red_shared(a1, 0u - self);
+      wcount += 2u * kSweepTile * n_pr;
+      if (wcount >= (1ull << 31)) {
         __syncwarp();
+        unsigned long long tot = 0;
+        for (uint32_t b = lane; b < nb; b += 32) {
+          const unsigned long long v = row1[b] + 2ull * row1[stride + b];
+          if (v) atomicAdd((unsigned long long*)&a.rdf[b], v);
+          tot += v;
+          row1[b] = row1[stride + b] = 0;
+        }
+        if (tot) atomicAdd((unsigned long long*)&a.meta[PS_META_N_PAIRS], tot);
+        __syncwarp();
+        wcount = 0;
+      }
+    });
+    __syncthreads();
+    unsigned long long tot = 0;
+    for (uint32_t b = threadIdx.x; b < nb; b += blockDim.x) {
+      unsigned long long sum = 0;
+      for (uint32_t r = 0; r < 8; ++r) sum += rows[2 * r * stride + b] + 2ull * rows[(2 * r + 1) * stride + b];
+      if (sum) atomicAdd((unsigned long long*)&a.rdf[b], sum);
+      tot += sum;
+    }
 #pragma unroll
-        for (uint32_t h = 0; h < kSymGroup; h += 32) {
-          const uint32_t r = h + lane;
-          if (r < 2 * n_pr) {
-            float4 q = make_float4(INFINITY, INFINITY, INFINITY, -1.f);  // the pad of an odd group never hits
-            if (r < m) {
-              q = __ldg(a.nrec + g0 + r);
-              q.w = __ldg(a.pfx + g0 + r + 1) > __ldg(a.pfx + g0 + r) ? E_max : -1.f;
-            }
-            float* d = gf + (r >> 1) * 8 + (r & 1);
-            d[0] = q.x, d[2] = q.y, d[4] = q.z, d[6] = q.w;
-          }
-        }
-        __syncwarp();
-        int rr = 0;
-        auto fetch = [&](uint32_t pos) -> float4 {
-          if (pos >= n_cand) return make_float4(INFINITY, INFINITY, INFINITY, -1.f);
-          while (pos >= rpre[rr + 1]) ++rr;
-          const uint32_t j = rsrc[rr] + (pos - rpre[rr]);
-          float4 q = __ldg(a.nrec + j);
-          q.w = __ldg(a.pfx + j + 1) > __ldg(a.pfx + j) ? E_max : -1.f;
-          return q;
-        };
-        float4 nxt = fetch(lane);
-        for (uint32_t b = 0; b < n_cand; b += 32) {
-          const float4 q = nxt;
-          nxt = fetch(b + 32 + lane);
-          const unsigned long long qx = f2_pack(q.x, q.x), qy = f2_pack(q.y, q.y), qz = f2_pack(q.z, q.z);
-          const float eq = q.w;
-          const uint32_t w2q = eq > 0.f ? 0x80000000u : 0u;
-          for (uint32_t k0 = 0; k0 < n_pr; k0 += 8) {
-            const uint32_t k1 = min(n_pr, k0 + 8);
-            uint32_t nh = 0;  // hits in the warp list (uniform)
-#pragma unroll 4
-            for (uint32_t k = k0; k < k1; ++k) {
-              const ulonglong2 xy = reinterpret_cast<const ulonglong2*>(gf)[2 * k];
-              const ulonglong2 zw = reinterpret_cast<const ulonglong2*>(gf)[2 * k + 1];
-              float d2a, d2b;
-              dist2_x2(xy.x, xy.y, zw.x, qx, qy, qz, d2a, d2b);
-              float ea, eb;
-              f2_unpack(zw.y, ea, eb);
-              const bool ha = d2a < fmaxf(eq, ea);
-              const bool hb = d2b < fmaxf(eq, eb);
-              const uint32_t va = __float_as_uint(d2a) | (~__float_as_uint(ea) & w2q);
-              const uint32_t vb = __float_as_uint(d2b) | (~__float_as_uint(eb) & w2q);
-              // every lane stores (no branch): a hit at its compacted slot, a miss in the trash row
-              const uint32_t ba = __ballot_sync(0xffffffffu, ha);
-              wlist[ha ? nh + __popc(ba & lt) : 32 * kHalf + lane] = va;
-              nh += __popc(ba);
-              const uint32_t bb = __ballot_sync(0xffffffffu, hb);
-              wlist[hb ? nh + __popc(bb & lt) : 32 * kHalf + lane] = vb;
-              nh += __popc(bb);
-            }
-            __syncwarp();
-            for (uint32_t h = lane; h < nh; h += 32) {
-              const uint32_t v = wlist[h];
-              H.pair_w(__uint_as_float(v & 0x7FFFFFFFu), 1u + (v >> 31), my_below);
-            }
-            __syncwarp();
-            wcount += 2ull * nh;
-            if (wcount >= (1ull << 31)) {
-              H.flush_warp(a);
-              wcount = 0;
-            }
-          }
+    for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    if (lane == 0 && tot) atomicAdd((unsigned long long*)&a.meta[PS_META_N_PAIRS], tot);
+  } else {
+    Hist<true> H{};
+    H.init(a, smem, 0, true);
+    const float Emax = H.Emax;
+    uint32_t my_below = 0;
+    sweep_pairs<true>(sw, buf, [&](uint32_t, uint32_t m, uint32_t nc, bool) __attribute__((always_inline)) {
+      const float* rxy = reinterpret_cast<const float*>(buf.rxy);
+      const float* rz = reinterpret_cast<const float*>(buf.rz);
+      for (uint32_t h = lane; h < nc; h += 32) {
+        const float4 q = buf.cand[h];
+        const uint32_t j = buf.cidx[h], wt = __float_as_uint(q.w) == kCandBoth ? 2u : 1u;
+        for (uint32_t k = 0; k < m; ++k) {
+          const float* p = rxy + (k >> 1) * 4 + (k & 1u);
+          const float d2 = dist2(p[0], p[2], rz[k], q.x, q.y, q.z);
+          if (d2 < Emax && buf.ridx[k] != j) H.pair_w(d2, wt, my_below);
         }
       }
-    }
+      __syncwarp();
+      wcount += 2u * kSweepTile * m;
+      if (wcount >= (1ull << 31)) {
+        H.flush_warp(a);
+        wcount = 0;
+      }
+    });
+    H.flush(a);
+    add_pair_counters(a, 0, my_below);
   }
-  H.flush(a);
-  add_pair_counters(a, my_binned, my_below);
+}
+
+template <bool FAST>
+static int launch_rdf_sym(const ps_grid* g, const QueryArgs& qa, const SweepArgs& sw, uint32_t smem, cudaStream_t s) {
+  auto k = k_rdf_sym<FAST>;
+  PS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int per_sm = 0;
+  PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem));
+  if (per_sm < 1) return fail(PS_ERR_UNSUPPORTED, "symmetric RDF kernel does not fit on an SM");
+  PS_LAUNCH(PS_KID_RDF_SYM, s, PS_CUDA(launch_pdl(k, g->num_sms * per_sm, 256, smem, s, qa, sw)));
+  return PS_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -1462,13 +1453,16 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
     }
     QueryArgs qs = qa;
     qs.n_k = 0;
-    qs.pfx = reinterpret_cast<const uint32_t*>(g->cr);  // written by the central-list compaction
-    const uint32_t smem_sym = smem_layout(bins.n_bins, 0, true, 0, true, qa.lut_n).total;
-    PS_CUDA(cudaFuncSetAttribute(k_rdf_sym, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_sym));
-    int per_sm = 0;
-    PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rdf_sym, 256, smem_sym));
-    if (per_sm < 1) return fail(PS_ERR_UNSUPPORTED, "symmetric RDF kernel does not fit on an SM");
-    PS_LAUNCH(PS_KID_RDF_SYM, s, PS_CUDA(launch_pdl(k_rdf_sym, g->num_sms * per_sm, 256, smem_sym, s, qs)));
+    SweepArgs sw = sweep_args(g, &g->ctr.geo->sym_next);
+    memcpy(sw.row_w, qa.row_w, sizeof(sw.row_w));
+    const double stop = (double)bins.n_bins * bins.dr;
+    sw.range = (float)((bins.r0 + stop) * (bins.r0 + stop));
+    // direct bins: r0 = 0, the two rows of a warp at most 4 KB, and edges and ranges far from the
+    // limits of float32 (the approximate root flushes subnormals)
+    const bool fast = bins.r0 == 0.0 && bins.n_bins <= kPrivBins && bins.dr > 1e-15 && stop < 1e15;
+    rc = fast ? launch_rdf_sym<true>(g, qs, sw, (bins.n_bins + 1) * 4 * 17, s)
+              : launch_rdf_sym<false>(g, qs, sw, smem_layout(bins.n_bins, 0, true, 0, true, qa.lut_n).total, s);
+    if (rc) return rc;
   } else if (n_k > 0 || rdf) {
     rc = rdf ? dispatch_k<true>(g, qa, smem_cta, smem_warp, s) : dispatch_k<false>(g, qa, smem_cta, smem_warp, s);
     if (rc) return rc;

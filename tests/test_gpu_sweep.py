@@ -1,0 +1,49 @@
+"""GPU parity of the sweep over unordered pairs (the RDF of the query in passes) against the oracle,
+at the sizes where it can go wrong: blocks of 1 .. 200 records (partly filled tiles, several staged
+groups), central and other records mixed in a block, the direct bins at their limit (512 bins) and
+the general ones beside it (513 bins, r0 > 0), pairs exactly on the edges, coincident ions, and
+clouds of few cells whose candidates are split into parts."""
+import numpy as np
+import pytest
+
+from test_gpu_exact import assert_same, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def ps():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_2004_05188_gb300 as ps
+
+    return ps
+
+
+@pytest.mark.parametrize("n,L,cs", [(2, 0.5, 0.5), (63, 1.0, 0.5), (64, 1.0, 0.75), (65, 1.0, 0.5), (700, 2.0, 0.75),
+                                    (3000, 12.0, 1 / 3), (9000, 9.0, 0.4), (5000, 40.0, 0.5)])
+@pytest.mark.parametrize("bins", [(0.0, 0.005, 300), (0.0, 1.5 / 512, 512), (0.0, 1.5 / 513, 513), (0.4, 0.1, 11),
+                                  (0.0, 1.5, 1)])
+def test_rdf_over_unordered_pairs(ps, orc, spec, n, L, cs, bins):
+    xyz, t, d = spec.cube(300 + n, n, L, (0.5, 0.5))
+    half = float(np.median(d))  # about half of the ions central
+    for ctr, nbr, dmin in (("all", "all", -1.0), ("all", "all", half), ([1], "all", 0.0)):
+        g = run_gpu(ps, xyz, t, d, ctr, nbr, dmin, bins, [], cell_scale=cs, split=True)
+        r = orc.spatstat(xyz, t, d, ctr, nbr, dmin, *bins, [])
+        assert_same(g, r, [])
+
+
+def test_lattice_edges_and_coincident_ions(ps, orc, spec):
+    xyz, t, d = spec.simple_cubic(14, 0.25, 0.125)  # every distance on or near an edge
+    xyz = np.concatenate([xyz, xyz[:100], xyz[:7]])
+    t, d = np.zeros(xyz.shape[0], np.uint8), np.concatenate([d, d[:100], d[:7]])
+    for bins in ((0.0, 0.01, 150), (0.0, 0.25, 6), (0.25, 0.25, 5)):
+        for dmin in (0.0, 0.6):
+            g = run_gpu(ps, xyz, t, d, "all", "all", dmin, bins, [], cell_scale=0.5, split=True)
+            r = orc.spatstat(xyz, t, d, "all", "all", dmin, *bins, [])
+            assert_same(g, r, [])
