@@ -854,10 +854,10 @@ int build_neighbour_grid(ps_grid* g, const uint64_t nbr_mask[4], float r_cut, cu
 }
 
 int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsrf_min, cudaStream_t s,
-                       ZeroOut z, bool split, bool vertex) {
+                       ZeroOut z, bool split, bool vertex, bool items) {
   Mask m;
-  bool subset = !g->pack_type;
-  for (int w = 0; w < 4; ++w) m.w[w] = ctr_mask[w], subset = subset && (ctr_mask[w] & ~g->nbr_mask[w]) == 0;
+  for (int w = 0; w < 4; ++w) m.w[w] = ctr_mask[w];
+  const bool subset = centrals_in_neighbours(g, ctr_mask);
   if (subset && vertex) {
     // the central prefix over the neighbour records, then the centrals sorted by the
     // vertex-centred grid (ranks in the dense-cell list, unused without dense cells)
@@ -886,7 +886,8 @@ int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4]
               PS_CUDA(launch_pdl(k_central_subset, grid_blocks(g, 1), kScanThreads, 0, s, g->nbr.rec, g->nbr.geo,
                                  g->ctr.geo, g->type, dsrf, m, dsrf_min, g->ctr.rec, pfx, g->scan_state, g->scan_ctr, z,
                                  (uint32_t*)nullptr)));
-    PS_LAUNCH(PS_KID_SCAN, s,
+    if (items)
+      PS_LAUNCH(PS_KID_SCAN, s,
               PS_CUDA(launch_pdl(k_central_items, grid_blocks(g, 4), kThreads, 0, s, g->nbr.start, pfx, g->ctr.geo,
                                  g->ctr.start, g->ctr.work, g->ctr.witem, g->dense_min, g->item_cap, g->stencil, split,
                                  split ? g->nbr_witem : nullptr)));

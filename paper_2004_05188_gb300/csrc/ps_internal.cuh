@@ -212,8 +212,16 @@ struct ZeroOut {
 // split: size the warp items of dense cells for lanes_per_central (the exact query's staged path);
 // vertex: centrals among the neighbour records sorted by the vertex-centred grid (the query in
 // passes on cells smaller than r_cut), the central prefix in g->cr
+// items: false leaves out the central list's cell starts and work items where the centrals are
+// neighbour records (the sweep over unordered pairs needs the records' prefix only)
 int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsrf_min, cudaStream_t s,
-                       ZeroOut z = ZeroOut(), bool split = false, bool vertex = false);
+                       ZeroOut z = ZeroOut(), bool split = false, bool vertex = false, bool items = true);
+// the centrals are neighbour records of the last build
+inline bool centrals_in_neighbours(const ps_grid* g, const uint64_t ctr_mask[4]) {
+  bool subset = !g->pack_type;
+  for (int w = 0; w < 4; ++w) subset = subset && (ctr_mask[w] & ~g->nbr_mask[w]) == 0;
+  return subset;
+}
 int soft_forward(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsrf_min, float sigma, float scale,
                  ps_bins bins, float* d_h, cudaStream_t s);
 int run_sdm(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsrf_min, ps_sdm_spec spec,

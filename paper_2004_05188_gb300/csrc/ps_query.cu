@@ -934,8 +934,6 @@ __global__ void __launch_bounds__(256) k_query_cta(const QueryArgs a) {
 // ---------------------------------------------------------------------------
 // symmetric RDF pass: every unordered pair of neighbour records once (sweep_pairs)
 // ---------------------------------------------------------------------------
-constexpr float kMagic = 12582912.0f;           // 1.5 * 2^23: x + kMagic holds floor(x) in its low bits
-constexpr uint32_t kMagicBits = 0x4B400000u;
 constexpr float kBinBias = 1.0f / 2097152.0f;   // 2^-21
 
 __device__ __forceinline__ float sqrt_fast(float x) {
@@ -1333,26 +1331,6 @@ static void choose_lut(ps_bins bins, QueryArgs& qa) {
   }
 }
 
-// Row widths of a stencil of s cells for cells of edge h >= r_cut * cs * (1 + 2^-10) (plus the
-// grid's rounding margin extent * 2^-20, which covers the float32 rounding of the cell index).
-// Two points whose cells are |d| >= 2 apart along an axis are more than (|d| - 1) r_cut cs apart
-// along it, so cell offset (dx, dy, dz) can hold a pair within r_cut only if
-// sum_i max(0, |d_i| - 1)^2 (cs (1 + 2^-10))^2 < 1; the test keeps a further 2^-20 margin.
-// Stencils of three cells (cs < 1/2) lose the 4 far corner cells of each octant; two-cell stencils
-// lose corners or rows only for cs above ~0.58.
-static void row_widths(int s, double cs, int8_t* w) {
-  const int W = 2 * s + 1;
-  const double f = cs * (1.0 + 1.0 / 1024.0), lim = (1.0 + 1.0 / 1048576.0) * (1.0 + 1.0 / 1048576.0);
-  auto m2 = [](int d) { const int m = d < 0 ? -d - 1 : d - 1; return m > 0 ? (double)(m * m) : 0.0; };
-  for (int dz = -s; dz <= s; ++dz)
-    for (int dy = -s; dy <= s; ++dy) {
-      int width = -1;
-      for (int dx = 0; dx <= s; ++dx)
-        if ((m2(dx) + m2(dy) + m2(dz)) * f * f < lim) width = dx;
-      w[(dz + s) * W + dy + s] = (int8_t)width;
-    }
-}
-
 int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsrf_min, ps_bins bins,
               const uint32_t* ks, uint32_t n_k, uint64_t* d_rdf, uint64_t* d_knn, uint64_t* d_meta, float* d_kth,
               uint32_t* d_nwithin, cudaStream_t s) {
@@ -1396,13 +1374,12 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
   if (rdf) z.p[1] = d_rdf, z.n[1] = bins.n_bins;
   if (n_k) z.p[2] = d_knn, z.n[2] = n_k * bins.n_bins;
 
-  bool subset = !g->pack_type;
-  for (int w = 0; w < 4; ++w) subset = subset && (ctr_mask[w] & ~g->nbr_mask[w]) == 0;
+  const bool subset = centrals_in_neighbours(g, ctr_mask);
   // the query in passes, and its near kNN pass on the vertex-centred central list (two-cell
   // stencils; the ranks of that counting sort take one word per central of the cell arrays)
   const bool split = g->split && subset && rdf && d_nwithin == nullptr && g->stencil >= 2 && g->dense_min == 0xFFFFFFFFu;
   const bool vertex = split && n_k > 0 && g->stencil == 2 && (uint64_t)g->n <= (uint64_t)g->cell_cap;
-  int rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, true, vertex);
+  int rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, true, vertex, !split || n_k > 0);
   if (rc) return rc;
 
   // staging budget of the CTA kernel: two CTAs per SM
@@ -1454,7 +1431,6 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
     QueryArgs qs = qa;
     qs.n_k = 0;
     SweepArgs sw = sweep_args(g, &g->ctr.geo->sym_next);
-    memcpy(sw.row_w, qa.row_w, sizeof(sw.row_w));
     const double stop = (double)bins.n_bins * bins.dr;
     sw.range = (float)((bins.r0 + stop) * (bins.r0 + stop));
     // direct bins: r0 = 0, the two rows of a warp at most 4 KB, and edges and ranges far from the

@@ -669,14 +669,6 @@ static int launch_grid_for(const ps_grid* g, const void* kern, uint32_t smem, in
   return PS_OK;
 }
 
-// The centrals are neighbour records (the central list then carries the central prefix over the
-// neighbour records, g->cr).
-static bool centrals_in_neighbours(const ps_grid* g, const uint64_t ctr_mask[4]) {
-  bool subset = !g->pack_type;
-  for (int w = 0; w < 4; ++w) subset = subset && (ctr_mask[w] & ~g->nbr_mask[w]) == 0;
-  return subset;
-}
-
 // Owners = the neighbour records: warp items over the non-empty neighbour cells.
 static int nbr_items(ps_grid* g, SoftArgs& sa, cudaStream_t s, uint32_t kid) {
   PS_LAUNCH(kid, s, PS_CUDA(launch_pdl(k_reset_items, 1, 32, 0, s, g->nbr.geo)));

@@ -24,6 +24,9 @@
 
 namespace ps {
 
+constexpr float kMagic = 12582912.0f;           // 1.5 * 2^23: x + kMagic holds floor(x) in its low bits
+constexpr uint32_t kMagicBits = 0x4B400000u;
+
 constexpr uint32_t kSweepRec = 64;        // records staged at a time
 constexpr uint32_t kSweepTile = 64;       // candidates per tile, two per lane
 constexpr uint32_t kCandSingle = 0u, kCandBoth = 1u, kCandOwn = 2u, kCandSelf = 3u;
@@ -40,8 +43,28 @@ struct SweepArgs {
   int8_t row_w[49];     // half-width of each stencil row (dy, dz), at [(dz + s)(2s + 1) + dy + s]; -1: none
 };
 
+// Row widths of a stencil of s cells for cells of edge h >= r_cut * cs * (1 + 2^-10) (plus the
+// grid's rounding margin extent * 2^-20, which covers the float32 rounding of the cell index).
+// Two points whose cells are |d| >= 2 apart along an axis are more than (|d| - 1) r_cut cs apart
+// along it, so cell offset (dx, dy, dz) can hold a pair within r_cut only if
+// sum_i max(0, |d_i| - 1)^2 (cs (1 + 2^-10))^2 < 1; the test keeps a further 2^-20 margin.
+// Stencils of three cells (cs < 1/2) lose the 4 far corner cells of each octant; two-cell stencils
+// lose corners or rows only for cs above ~0.58.
+inline void row_widths(int s, double cs, int8_t* w) {
+  const int W = 2 * s + 1;
+  const double f = cs * (1.0 + 1.0 / 1024.0), lim = (1.0 + 1.0 / 1048576.0) * (1.0 + 1.0 / 1048576.0);
+  auto m2 = [](int d) { const int m = d < 0 ? -d - 1 : d - 1; return m > 0 ? (double)(m * m) : 0.0; };
+  for (int dz = -s; dz <= s; ++dz)
+    for (int dy = -s; dy <= s; ++dy) {
+      int width = -1;
+      for (int dx = 0; dx <= s; ++dx)
+        if ((m2(dx) + m2(dy) + m2(dz)) * f * f < lim) width = dx;
+      w[(dz + s) * W + dy + s] = (int8_t)width;
+    }
+}
+
 // The arguments over the last build's neighbour records and the central list's prefix over them;
-// the caller fills in row_w and range.
+// the caller fills in range.
 inline SweepArgs sweep_args(const ps_grid* g, uint32_t* next) {
   SweepArgs a = {};
   a.nrec = g->nbr.rec;
@@ -51,6 +74,7 @@ inline SweepArgs sweep_args(const ps_grid* g, uint32_t* next) {
   a.next = next;
   a.stencil = g->stencil;
   a.one = 1.0f;
+  row_widths(g->stencil, g->cell_scale, a.row_w);
   return a;
 }
 

@@ -47,3 +47,23 @@ def test_lattice_edges_and_coincident_ions(ps, orc, spec):
             g = run_gpu(ps, xyz, t, d, "all", "all", dmin, bins, [], cell_scale=0.5, split=True)
             r = orc.spatstat(xyz, t, d, "all", "all", dmin, *bins, [])
             assert_same(g, r, [])
+
+
+@pytest.mark.parametrize("R,w,nv", [(1.5, 0.1, 30), (1.5, 0.1, 31), (1.0, 0.25, 8), (1.0, 0.25, 7), (1.2, 3.0, 1)])
+@pytest.mark.parametrize("lattice", [False, True])
+def test_distribution_map_mirrored(ps, orc, spec, R, w, nv, lattice):
+    """The map from unordered pairs: mirrored voxels, odd cubes (a voxel that is its own mirror
+    image), displacements on voxel edges, one or both ends central, coincident ions."""
+    if lattice:
+        xyz, t, d = spec.simple_cubic(11, 0.25, 0.125)
+    else:
+        xyz, t, d = spec.cube(77, 1500, 4.0, (0.5, 0.5))
+    xyz, t, d = np.concatenate([xyz, xyz[:20]]), np.concatenate([t, t[:20]]), np.concatenate([d, d[:20]])
+    X, T, D = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (xyz, t, d))
+    for cs, dmin, ctr in ((1.0, 0.5, "all"), (0.5, 0.3, [0])):
+        g = ps.Grid(X.shape[0], cs).build(X, T, "all", R * (1 + 1e-6))
+        out = ps.sdm(g, D, ctr, dmin, R, w, nv)
+        H, m = orc.sdm(xyz, t, d, ctr, "all", dmin, R, w, nv)
+        np.testing.assert_array_equal(out["meta"].cpu().numpy()[:3].astype(np.uint64), m)
+        np.testing.assert_array_equal(out["H"].cpu().numpy().astype(np.uint64), H)
+        g.close()
