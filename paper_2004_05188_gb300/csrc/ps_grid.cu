@@ -884,8 +884,8 @@ int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4]
     uint32_t* pfx = reinterpret_cast<uint32_t*>(g->cr);  // 2 n_max words, n_records + 1 needed
     PS_LAUNCH(PS_KID_CENTRAL, s,
               PS_CUDA(launch_pdl(k_central_subset, grid_blocks(g, 1), kScanThreads, 0, s, g->nbr.rec, g->nbr.geo,
-                                 g->ctr.geo, g->type, dsrf, m, dsrf_min, g->ctr.rec, pfx, g->scan_state, g->scan_ctr, z,
-                                 (uint32_t*)nullptr)));
+                                 g->ctr.geo, g->type, dsrf, m, dsrf_min, items ? g->ctr.rec : (float4*)nullptr, pfx, g->scan_state,
+                                 g->scan_ctr, z, (uint32_t*)nullptr)));
     if (items)
       PS_LAUNCH(PS_KID_SCAN, s,
               PS_CUDA(launch_pdl(k_central_items, grid_blocks(g, 4), kThreads, 0, s, g->nbr.start, pfx, g->ctr.geo,

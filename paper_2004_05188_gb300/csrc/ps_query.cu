@@ -936,17 +936,6 @@ __global__ void __launch_bounds__(256) k_query_cta(const QueryArgs a) {
 // ---------------------------------------------------------------------------
 constexpr float kBinBias = 1.0f / 2097152.0f;   // 2^-21
 
-__device__ __forceinline__ float sqrt_fast(float x) {
-  float r;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ unsigned long long f2_fma_down(unsigned long long a, unsigned long long b,
-                                                          unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
 __device__ __forceinline__ void red_shared_inc(uint32_t addr) {
   asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr));
 }

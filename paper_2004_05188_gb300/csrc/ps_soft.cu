@@ -16,24 +16,18 @@
 // and odd about c_m, i.e. a relative error ~1e-7 that averages out.
 // Adjoint: W, W', W'' are tabulated on the same fine grid (FP64, stored as
 // float) and evaluated per pair by the same second-order expansion.  Pairs are
-// recomputed, never stored.  Record k's gradient gathers every pair it is in,
-// W s (x_k - x_m)/d, once for each role: as the central (m a neighbour) and as
-// the neighbour (m a central).  When the centrals are neighbour records, one
-// pass has every neighbour record own its gradient, with the pair weighted by
-// the central flags of both ends (0, 1 or 2); otherwise pass A (one lane per
-// central) writes and pass B (one lane per neighbour, candidates = centrals)
-// adds.  Each gradient has one owner: no atomics on the gradient.  dL/ds sums
-// W d over the pairs with a central owner.
-// Both kernels test the candidates two at a time with packed float32.  The
-// forward over unordered pairs takes the neighbour cells one by one: the half
-// stencil's records are the lanes and the cell's records are read from shared
-// memory by every lane at once; the in-range pairs are compacted into a warp
-// list that all lanes bin.  The adjoint runs the pair code under a branch per
-// candidate (its per-pair work needs the owner's accumulators).
+// recomputed, never stored.  Where the centrals are neighbour records, forward and
+// adjoint meet every unordered pair once (sweep_pairs), weighted by the central
+// flags of both ends, and the adjoint adds a pair's force at both of them.
+// Otherwise the forward has one lane per central, and the adjoint's pass A (one
+// lane per central) writes and pass B (one lane per neighbour, candidates =
+// centrals) adds: each gradient then has one owner.  dL/ds sums W d over the
+// pairs, once per central end.
 #include <cmath>
 #include <cstring>
 
 #include "ps_internal.cuh"
+#include "ps_sweep.cuh"
 
 namespace ps {
 
@@ -61,7 +55,6 @@ struct SoftArgs {
   double* M2;
   // adjoint
   const float* T;          // [3][n_fine]: W, W', W'' at the fine-bin centres
-  const uint32_t* pfx;     // one-pass adjoint: central prefix over the neighbour records
   float* grad;             // [n][3]
   double* grad_s;
   int pass_b;              // 0: owners are centrals (write), 1: owners are neighbours (add, sign flipped)
@@ -83,40 +76,11 @@ __device__ __forceinline__ void soft_run(const SoftArgs& a, const Geo& ng, uint3
   }
 }
 
-// Half stencil of cell c for the forward over unordered pairs, run r of (2s+1)s + s + 1: the
-// rows above (dz > 0, every dy), the rows ahead in the same plane (dz = 0, dy > 0), both over
-// cx-s .. cx+s, and the cells after c in its own row (cx+1 .. cx+s).  With the pairs inside the
-// cell (j > i) every unordered pair within the stencil is met once.
-__device__ __forceinline__ void soft_half_run(const SoftArgs& a, const Geo& ng, uint32_t c, uint32_t r,
-                                              uint32_t& src, uint32_t& len) {
-  const int s = a.stencil, wd = 2 * s + 1;
-  const uint32_t cx = c % ng.dims[0], cy = (c / ng.dims[0]) % ng.dims[1], cz = c / (ng.dims[0] * ng.dims[1]);
-  src = 0;
-  len = 0;
-  int dy, dz;
-  uint32_t xlo = cx >= (uint32_t)s ? cx - s : 0;
-  const uint32_t xhi = cx + s < ng.dims[0] ? cx + s : ng.dims[0] - 1;
-  if ((int)r < s * wd) {
-    dz = 1 + (int)r / wd, dy = (int)r % wd - s;
-  } else if ((int)r < s * wd + s) {
-    dz = 0, dy = 1 + (int)r - s * wd;
-  } else if ((int)r == s * wd + s) {
-    dz = 0, dy = 0, xlo = cx + 1;
-  } else {
-    return;
-  }
-  const int y = (int)cy + dy, z = (int)cz + dz;
-  if (y < 0 || y >= (int)ng.dims[1] || z >= (int)ng.dims[2] || xlo > xhi) return;
-  const uint32_t row = ((uint32_t)z * ng.dims[1] + (uint32_t)y) * ng.dims[0];
-  src = a.nstart[row + xlo];
-  len = a.nstart[row + xhi + 1] - src;
-}
-
 // Iterates the items of the owner list (the centrals; candidates: their full stencil of
 // neighbours, whose staged .w is the ion index so that the owner itself is skipped) with the
 // candidates staged 32 at a time as interleaved pairs (xa xb ya yb za zb wa wb) and tested two at
 // a time with packed float32 math; the in-range pairs of every half-batch of 16 candidates go to
-// a warp list that all lanes then process: hit(d2, 1) for each.  item_hook(cnt, n_cand) runs once
+// a warp list that all lanes then process: hit(d2) for each.  item_hook(cnt, n_cand) runs once
 // per item.
 template <class H, class I>
 __device__ __forceinline__ void soft_items_listed(const SoftArgs& a, float* bf, uint32_t* rsrc, uint32_t* rpre,
@@ -184,142 +148,17 @@ __device__ __forceinline__ void soft_items_listed(const SoftArgs& a, float* bf, 
           nh += __popc(bb);
         }
         __syncwarp();
-        for (uint32_t h = lane; h < nh; h += 32) hit(wlist[h], 1.f);
+        for (uint32_t h = lane; h < nh; h += 32) hit(wlist[h]);
         __syncwarp();
-      }
-    }
-  }
-}
-
-// The forward over unordered pairs, cell by cell: a warp takes a share of the cells left (at
-// most 32, at least 1, from the counter a.ogeo->work_next2) and, for each non-empty cell, tests
-// the half stencil's records (the lanes, 32 per load, each in registers) against the cell's
-// records (staged in shared memory up to 64 at a time as interleaved pairs xa xb ya yb za zb ea
-// eb and read by every lane at once, two per packed test), so that the lanes stay busy whatever
-// the cell's record count; the pairs inside the cell (j > i) are tested by each lane on its own.
-// A record's e (and a candidate's) is rc^2 for a central and -1 otherwise: a pair is in range
-// below max(e_rec, e_cand), weight 2 (the sign bit of its listed d2) when both are central.
-// hit(d2, weight) per in-range pair; cell_hook(m, n_cand) once per cell before its pairs.
-template <class H, class C>
-__device__ __forceinline__ void soft_cells_sym(const SoftArgs& a, float* gf, uint32_t* rsrc, uint32_t* rpre,
-                                               uint32_t* wlist, H&& hit, C&& cell_hook) {
-  const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
-  const Geo ng = *a.ngeo;
-  const uint32_t n_cells = ng.n_cells;
-  const int s = a.stencil, n_runs = s * (2 * s + 1) + s + 1;
-  const float E = a.rc2u;
-  const uint32_t n_warps = gridDim.x * (blockDim.x >> 5);
-  for (;;) {
-    uint32_t base = 0, take = 0;
-    if (lane == 0) {
-      const uint32_t cur = *reinterpret_cast<volatile uint32_t*>(&a.ogeo->work_next2);
-      const uint32_t left = cur < n_cells ? n_cells - cur : 0u;
-      take = min(32u, max(1u, left / (8 * n_warps)));
-      base = atomicAdd(&a.ogeo->work_next2, take);
-    }
-    base = __shfl_sync(0xffffffffu, base, 0);
-    take = __shfl_sync(0xffffffffu, take, 0);
-    if (base >= n_cells) break;
-    uint32_t s0 = 0, s1 = 0;
-    if (lane < take && base + lane < n_cells) s0 = a.ostart[base + lane], s1 = a.ostart[base + lane + 1];
-    uint32_t todo = __ballot_sync(0xffffffffu, s1 > s0);
-    while (todo) {
-      const int src_lane = __ffs(todo) - 1;
-      todo &= todo - 1u;
-      const uint32_t c = base + (uint32_t)src_lane;
-      const uint32_t a0 = __shfl_sync(0xffffffffu, s0, src_lane), a1 = __shfl_sync(0xffffffffu, s1, src_lane);
-      const uint32_t n_cand = run_table(lane, n_runs, rsrc, rpre, [&](uint32_t r, uint32_t& src, uint32_t& len) {
-        soft_half_run(a, ng, c, r, src, len);
-      });
-      cell_hook(a1 - a0, n_cand + (a1 - a0));
-      // pairs inside the cell
-      for (uint32_t i0 = a0; i0 < a1; i0 += 32) {
-        const uint32_t i = i0 + lane;
-        if (i < a1) {
-          const float4 p = __ldg(a.orec + i);
-          const float ci = (float)(__ldg(a.pfx + i + 1) - __ldg(a.pfx + i));
-          for (uint32_t j = i + 1; j < a1; ++j) {
-            const float4 q = __ldg(a.orec + j);
-            const float d2 = dist2(p.x, p.y, p.z, q.x, q.y, q.z);
-            const float wt = ci + (float)(__ldg(a.pfx + j + 1) - __ldg(a.pfx + j));
-            if (d2 < E && wt > 0.f) hit(d2, wt);
-          }
-        }
-      }
-      if (n_cand == 0) continue;
-      for (uint32_t g0 = a0; g0 < a1; g0 += 64) {
-        const uint32_t m = min(64u, a1 - g0), n_pr = (m + 1) >> 1;
-        __syncwarp();
-#pragma unroll
-        for (uint32_t h = 0; h < 64; h += 32) {
-          const uint32_t r = h + lane;
-          if (r < 2 * n_pr) {
-            float4 q = make_float4(INFINITY, INFINITY, INFINITY, -1.f);  // the pad of an odd group never hits
-            if (r < m) {
-              q = __ldg(a.orec + g0 + r);
-              q.w = __ldg(a.pfx + g0 + r + 1) > __ldg(a.pfx + g0 + r) ? E : -1.f;
-            }
-            float* d = gf + (r >> 1) * 8 + (r & 1);
-            d[0] = q.x, d[2] = q.y, d[4] = q.z, d[6] = q.w;
-          }
-        }
-        __syncwarp();
-        int rr = 0;
-        auto fetch = [&](uint32_t pos) -> float4 {
-          if (pos >= n_cand) return make_float4(INFINITY, INFINITY, INFINITY, -1.f);
-          while (pos >= rpre[rr + 1]) ++rr;
-          const uint32_t j = rsrc[rr] + (pos - rpre[rr]);
-          float4 q = __ldg(a.nrec + j);
-          q.w = __ldg(a.pfx + j + 1) > __ldg(a.pfx + j) ? E : -1.f;
-          return q;
-        };
-        float4 nxt = fetch(lane);
-        for (uint32_t b = 0; b < n_cand; b += 32) {
-          const float4 q = nxt;
-          nxt = fetch(b + 32 + lane);
-          const unsigned long long qx = f2_pack(q.x, q.x), qy = f2_pack(q.y, q.y), qz = f2_pack(q.z, q.z);
-          const float eq = q.w;
-          const uint32_t w2q = eq > 0.f ? 0x80000000u : 0u;
-          for (uint32_t k0 = 0; k0 < n_pr; k0 += 8) {
-            const uint32_t k1 = min(n_pr, k0 + 8);
-            uint32_t nh = 0;
-#pragma unroll 4
-            for (uint32_t k = k0; k < k1; ++k) {
-              const ulonglong2 xy = reinterpret_cast<const ulonglong2*>(gf)[2 * k];
-              const ulonglong2 zw = reinterpret_cast<const ulonglong2*>(gf)[2 * k + 1];
-              float d2a, d2b, ea, eb;
-              dist2_x2(xy.x, xy.y, zw.x, qx, qy, qz, d2a, d2b);
-              f2_unpack(zw.y, ea, eb);
-              const bool ha = d2a < fmaxf(eq, ea), hb = d2b < fmaxf(eq, eb);
-              const uint32_t va = __float_as_uint(d2a) | (~__float_as_uint(ea) & w2q);
-              const uint32_t vb = __float_as_uint(d2b) | (~__float_as_uint(eb) & w2q);
-              const uint32_t ba = __ballot_sync(0xffffffffu, ha);
-              wlist[ha ? nh + __popc(ba & lt) : 512 + lane] = va;
-              nh += __popc(ba);
-              const uint32_t bb = __ballot_sync(0xffffffffu, hb);
-              wlist[hb ? nh + __popc(bb & lt) : 512 + lane] = vb;
-              nh += __popc(bb);
-            }
-            __syncwarp();
-            for (uint32_t h = lane; h < nh; h += 32) {
-              const uint32_t v = wlist[h];
-              hit(__uint_as_float(v & 0x7FFFFFFFu), (v >> 31) ? 2.f : 1.f);
-            }
-            __syncwarp();
-          }
-        }
       }
     }
   }
 }
 
 // Same iteration for the adjoint, where every in-range pair updates its owner lane's
-// accumulators: f(p, qx, qy, qz, qw, d2) under a branch per candidate (queueing the pairs
-// first measured slower).  ONE: owners and candidates are the neighbour records and the staged
-// .w is the candidate's central flag (from the central prefix); a pair counts when d2 > 0 and
-// either end is central.  Otherwise .w is the ion index and the owner itself is skipped.
-// begin_owner(valid, p, c_own) / end_owner(valid, p) bracket each owner.
-template <bool ONE, class F, class B, class E>
+// accumulators: f(p, qx, qy, qz, d2) under a branch per candidate (queueing the pairs first
+// measured slower).  begin_owner() / end_owner(valid, p) bracket each owner.
+template <class F, class B, class E>
 __device__ __forceinline__ void soft_items_owned(const SoftArgs& a, float* bf, uint32_t* rsrc, uint32_t* rpre,
                                                  F&& f, B&& begin_owner, E&& end_owner) {
   const uint32_t lane = threadIdx.x & 31;
@@ -339,28 +178,18 @@ __device__ __forceinline__ void soft_items_owned(const SoftArgs& a, float* bf, u
     });
     const bool valid = lane < cnt;
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-    float c_own = 0.f;
-    if (valid) {
-      p = a.orec[c0 + lane];
-      if (ONE) c_own = (float)(__ldg(a.pfx + c0 + lane + 1) - __ldg(a.pfx + c0 + lane));
-    }
+    if (valid) p = a.orec[c0 + lane];
     const uint32_t pidx = valid ? __float_as_uint(p.w) : ~0u;
     const float emax = valid ? a.rc2u : -INFINITY;
     const unsigned long long px = f2_pack(p.x, p.x), py = f2_pack(p.y, p.y), pz = f2_pack(p.z, p.z);
-    begin_owner(valid, p, c_own);
+    begin_owner();
     int rr = 0;
     auto fetch = [&](uint32_t pos) -> float4 {
-      if (pos >= n_cand) return make_float4(INFINITY, INFINITY, INFINITY, ONE ? 0.f : __uint_as_float(~0u));
+      if (pos >= n_cand) return make_float4(INFINITY, INFINITY, INFINITY, __uint_as_float(~0u));
       while (pos >= rpre[rr + 1]) ++rr;
-      const uint32_t j = rsrc[rr] + (pos - rpre[rr]);
-      float4 q = __ldg(a.nrec + j);
-      if (ONE) q.w = (float)(__ldg(a.pfx + j + 1) - __ldg(a.pfx + j));
-      return q;
+      return __ldg(a.nrec + rsrc[rr] + (pos - rpre[rr]));
     };
-    auto hit = [&](float d2, float w) -> bool {
-      if (ONE) return d2 < emax && d2 > 0.f && c_own + w > 0.f;
-      return d2 < emax && __float_as_uint(w) != pidx;
-    };
+    auto hit = [&](float d2, float w) -> bool { return d2 < emax && __float_as_uint(w) != pidx; };
     float4 nxt = fetch(lane);
     for (uint32_t b = 0; b < n_cand; b += 32) {
       __syncwarp();
@@ -379,11 +208,11 @@ __device__ __forceinline__ void soft_items_owned(const SoftArgs& a, float* bf, u
         f2_unpack(zw.y, wa, wb);
         if (hit(d2a, wa)) {
           f2_unpack(xy.x, xa, xb), f2_unpack(xy.y, ya, yb), f2_unpack(zw.x, za, zb);
-          f(p, xa, ya, za, wa, d2a);
+          f(p, xa, ya, za, d2a);
         }
         if (hit(d2b, wb)) {
           f2_unpack(xy.x, xa, xb), f2_unpack(xy.y, ya, yb), f2_unpack(zw.x, za, zb);
-          f(p, xb, yb, zb, wb, d2b);
+          f(p, xb, yb, zb, d2b);
         }
       }
     }
@@ -394,7 +223,6 @@ __device__ __forceinline__ void soft_items_owned(const SoftArgs& a, float* bf, u
 // ---------------------------------------------------------------------------
 // forward: fine-grid moments
 // ---------------------------------------------------------------------------
-template <bool SYM>
 __global__ void __launch_bounds__(256) k_soft_fwd(const SoftArgs a) {
   griddep_wait();
   griddep_launch();
@@ -402,8 +230,8 @@ __global__ void __launch_bounds__(256) k_soft_fwd(const SoftArgs a) {
   __shared__ float4 s_grp[8][64];        // per warp: staged records (the cell's, or a batch of candidates)
   __shared__ float s_hits[8][512 + 32];  // per warp: one half-batch's in-range d2 + a trash row
   __shared__ uint32_t s_rsrc[8][kSoftRuns], s_rpre[8][kSoftRuns + 1];
-  // 32-bit counts per CTA; a warp whose item could push the CTA past 2^31 (weighted) pairs writes
-  // to global instead
+  // 32-bit counts per CTA; a warp whose item could push the CTA past 2^31 pairs writes to global
+  // instead
   uint32_t* sM0 = reinterpret_cast<uint32_t*>(smem);
   float* sM1 = reinterpret_cast<float*>(smem + a.n_fine * 4);
   float* sM2 = reinterpret_cast<float*>(smem + a.n_fine * 8);
@@ -415,36 +243,31 @@ __global__ void __launch_bounds__(256) k_soft_fwd(const SoftArgs a) {
   const uint32_t w = threadIdx.x >> 5;
   const float s = a.scale, inv_w = a.inv_w, wf = a.w, rc = a.rc;
   const uint32_t nf = a.n_fine;
-  // one pair at distance sqrt(d2) with weight wt (1 or 2) into the fine-grid moments
-  auto pair = [&](float d2, float wt) {
+  // one pair at distance sqrt(d2) into the fine-grid moments
+  auto pair = [&](float d2) {
     const float u = s * (d2 > 0.f ? d2 * rsqrtf(d2) : 0.f);
     if (!(u < rc)) return;
     uint32_t m = (uint32_t)(u * inv_w);
     m = m < nf ? m : nf - 1;
     const float delta = u - ((float)m + 0.5f) * wf;
-    const float wd = wt * delta;
     if (glob) {
-      atomicAdd(&a.M0[m], (unsigned long long)wt);
-      atomicAdd(&a.M1[m], (double)wd);
-      atomicAdd(&a.M2[m], (double)wd * (double)delta);
+      atomicAdd(&a.M0[m], 1ull);
+      atomicAdd(&a.M1[m], (double)delta);
+      atomicAdd(&a.M2[m], (double)delta * (double)delta);
     } else {
-      atomicAdd(&sM0[m], (uint32_t)wt);
-      atomicAdd(&sM1[m], wd);
-      atomicAdd(&sM2[m], wd * delta);
+      atomicAdd(&sM0[m], 1u);
+      atomicAdd(&sM1[m], delta);
+      atomicAdd(&sM2[m], delta * delta);
     }
   };
   auto bound = [&](uint32_t cnt, uint32_t n_cand) {
     unsigned long long old = 0;
-    const unsigned long long inc = (unsigned long long)cnt * n_cand * (SYM ? 2u : 1u);
+    const unsigned long long inc = (unsigned long long)cnt * n_cand;
     if ((threadIdx.x & 31) == 0) old = atomicAdd(&s_pairs, inc);
     old = __shfl_sync(0xffffffffu, old, 0);
     glob = old + inc >= (1ull << 31);
   };
-  if (SYM)
-    soft_cells_sym(a, reinterpret_cast<float*>(s_grp[w]), s_rsrc[w], s_rpre[w], reinterpret_cast<uint32_t*>(s_hits[w]),
-                   pair, bound);
-  else
-    soft_items_listed(a, reinterpret_cast<float*>(s_grp[w]), s_rsrc[w], s_rpre[w], s_hits[w], pair, bound);
+  soft_items_listed(a, reinterpret_cast<float*>(s_grp[w]), s_rsrc[w], s_rpre[w], s_hits[w], pair, bound);
   __syncthreads();
   for (uint32_t m = threadIdx.x; m < nf; m += blockDim.x) {
     if (sM0[m]) {
@@ -453,6 +276,140 @@ __global__ void __launch_bounds__(256) k_soft_fwd(const SoftArgs a) {
       atomicAdd(&a.M2[m], (double)sM2[m]);
     }
   }
+}
+
+// Pairs of the sweep as packed distances: the range test is u < rc (u = scale * distance), the fine
+// bin floor(u / w).  w has 11 significant bits and n_fine < 2^13, so that the bin centres (m + 1/2) w
+// are exact in float32 and the remainder u - (m + 1/2) w carries only the rounding of u.
+struct SoftFine {
+  unsigned long long scale2, inv_w2, w2, half_w2, magic2;
+  __device__ explicit SoftFine(const SoftArgs& a) {
+    scale2 = f2_pack(a.scale, a.scale);
+    inv_w2 = f2_pack(a.inv_w, a.inv_w);
+    w2 = f2_pack(a.w, a.w);
+    half_w2 = f2_pack(0.5f * a.w, 0.5f * a.w);
+    magic2 = f2_pack(kMagic, kMagic);
+  }
+  // u -> floor(u / w) in the low bits of m, and the remainder about the bin centre
+  __device__ __forceinline__ void split(unsigned long long u2, unsigned long long& m2, unsigned long long& delta2) const {
+    m2 = f2_fma_down(u2, inv_w2, magic2);
+    delta2 = f2_sub(u2, f2_fma(f2_sub(m2, magic2), w2, half_w2));
+  }
+};
+
+// (subnormal squared distances count as 0, i.e. as coincident ions)
+__device__ __forceinline__ float rsqrt_fast(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ unsigned long long soft_d2(unsigned long long dx, unsigned long long dy,
+                                                      unsigned long long dz) {
+  return f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
+}
+
+// The forward's moments of a fine bin in integers: the weights, the remainders in units of w / 2^13
+// (half of float32's step of u at 2 nm and sigma = 0.05 nm) and their squares in units of w^2 / 2^13.
+// Integer shared-memory atomics run at the rate of the plain count (measured, 2 of 5 lanes active
+// at random places, cycles per warp and SM: one count 4.5, three integers 5.4, a count and two
+// floats 12.1), and the sums do not round.  A bin's sums stay inside 32 bits while its weight is
+// below 2^19: a warp looks the counts over after every 2^14 that it may have added, and drains the
+// rows to the global moments when one has reached 2^18 (8 warps: below 2^18 + 8 (2^14 + 2^13)).
+constexpr float kSoftQ = 8192.0f;
+constexpr uint32_t kSoftLook = 1u << 14, kSoftDrain = 1u << 18;
+
+// Forward where the centrals are neighbour records: every unordered pair once (sweep_pairs), its
+// moments straight from the testing lane into the CTA's shared fine grid.  Bound by the shared-
+// memory pipe (three scattered atomics per in-range pair) and issue.  Measured, 1e7-ion needle on
+// half-size cells / 2e5 cylinder on full-size cells (ms): 36.8 -> 19.4 / 14.5 -> 1.13 (before: a warp list of
+// the hits of every candidate of the half stencil, a float sum per moment, cells not split; 27.4 /
+// 1.25 with the sweep and float sums).
+__global__ void __launch_bounds__(256, 4) k_soft_fwd_sym(const SoftArgs a, const __grid_constant__ SweepArgs sw,
+                                                         double unit1, double unit2) {
+  griddep_wait();
+  griddep_launch();
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ SweepBuf s_sweep[8];
+  const uint32_t nf = a.n_fine, row = (nf + 3u) & ~3u, lane = threadIdx.x & 31;
+  uint32_t* sM = reinterpret_cast<uint32_t*>(smem);  // [3][row]
+  for (uint32_t m = threadIdx.x; m < 3 * row; m += blockDim.x) sM[m] = 0;
+  __syncthreads();
+  SweepBuf& buf = s_sweep[threadIdx.x >> 5];
+  const SoftFine fine(a);
+  const float rc = a.rc, q1 = kSoftQ * a.inv_w, q2 = kSoftQ * a.inv_w * a.inv_w;
+  const unsigned long long q1_2 = f2_pack(q1, q1), q2_2 = f2_pack(q2, q2);
+  const uint32_t base = smem_u32(sM) - 4u * kMagicBits;
+  uint32_t added = 0;  // bound on the weights this warp has added since it last looked (uniform)
+  // the rows' bins i, i + step, ... to the global moments
+  auto drain = [&](uint32_t i, uint32_t step) {
+    for (; i < nf; i += step) {
+      const int32_t v0 = (int32_t)atomicExch(&sM[i], 0u), v1 = (int32_t)atomicExch(&sM[row + i], 0u),
+                    v2 = (int32_t)atomicExch(&sM[2 * row + i], 0u);
+      // (a count may stand below zero when its self pairs were drained before they were taken out)
+      if (v0) atomicAdd(&a.M0[i], (unsigned long long)(long long)v0);
+      if (v1) atomicAdd(&a.M1[i], (double)v1 * unit1);
+      if (v2) atomicAdd(&a.M2[i], (double)v2 * unit2);
+    }
+  };
+  sweep_pairs<false>(sw, buf, [&](uint32_t n_pr, uint32_t m, uint32_t nc, bool) __attribute__((always_inline)) {
+    const float4 far = make_float4(INFINITY, INFINITY, INFINITY, __uint_as_float(kCandSingle));
+    const float4 c0 = lane < nc ? buf.cand[lane] : far, c1 = lane + 32 < nc ? buf.cand[lane + 32] : far;
+    const uint32_t k0 = __float_as_uint(c0.w), k1 = __float_as_uint(c1.w);
+    const uint32_t w0 = k0 == kCandBoth ? 2u : 1u, w1 = k1 == kCandBoth ? 2u : 1u;
+    const unsigned long long x0 = f2_pack(c0.x, c0.x), y0 = f2_pack(c0.y, c0.y), z0 = f2_pack(c0.z, c0.z);
+    const unsigned long long x1 = f2_pack(c1.x, c1.x), y1 = f2_pack(c1.y, c1.y), z1 = f2_pack(c1.z, c1.z);
+    auto deposit = [&](unsigned long long d2, uint32_t wt) __attribute__((always_inline)) {
+      float da, db, u[2], mm[2], r1[2], r2[2];
+      f2_unpack(d2, da, db);
+      const unsigned long long u2 = f2_mul(f2_pack(sqrt_fast(da), sqrt_fast(db)), fine.scale2);
+      unsigned long long m2, dl2;
+      fine.split(u2, m2, dl2);
+      f2_unpack(u2, u[0], u[1]), f2_unpack(m2, mm[0], mm[1]);
+      f2_unpack(f2_fma(dl2, q1_2, fine.magic2), r1[0], r1[1]);  // rounded to the nearest unit
+      f2_unpack(f2_fma(f2_mul(dl2, dl2), q2_2, fine.magic2), r2[0], r2[1]);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        if (u[e] < rc) {
+          const uint32_t at = __float_as_uint(mm[e]) * 4u + base;
+          asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at), "r"(wt));
+          asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at + 4u * row), "r"((__float_as_uint(r1[e]) - kMagicBits) * wt));
+          asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at + 8u * row), "r"((__float_as_uint(r2[e]) - kMagicBits) * wt));
+        }
+      }
+    };
+    const ulonglong2* rxy = reinterpret_cast<const ulonglong2*>(buf.rxy);
+    const unsigned long long* rz = reinterpret_cast<const unsigned long long*>(buf.rz);
+#pragma unroll 1
+    for (uint32_t k = 0; k < n_pr; ++k) {
+      const ulonglong2 xy = rxy[k];
+      const unsigned long long zz = rz[k];
+      deposit(soft_d2(f2_sub(x0, xy.x), f2_sub(y0, xy.y), f2_sub(z0, zz)), w0);
+      deposit(soft_d2(f2_sub(x1, xy.x), f2_sub(y1, xy.y), f2_sub(z1, zz)), w1);
+    }
+    // the staged records met themselves once each, at u = 0: taken out of bin 0 (remainder -w / 2)
+    const uint32_t self = __popc(__ballot_sync(0xffffffffu, k0 == kCandSelf)) +
+                          __popc(__ballot_sync(0xffffffffu, k1 == kCandSelf));
+    if (self && lane == 0) {
+      atomicAdd(&sM[0], 0u - self);
+      atomicAdd(&sM[row], self * (uint32_t)(kSoftQ / 2));
+      atomicAdd(&sM[2 * row], 0u - self * (uint32_t)(kSoftQ / 4));
+    }
+    added += 2u * kSweepTile * m;
+    if (added >= kSoftLook) {
+      added = 0;
+      uint32_t top = 0;
+      for (uint32_t i = lane; i < row / 4; i += 32) {
+        uint4 v;
+        asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                     : "r"(smem_u32(sM) + 16u * i));
+        top = max(max(top, max(v.x, v.y)), max(v.z, v.w));
+      }
+      if (__any_sync(0xffffffffu, top >= kSoftDrain)) drain(lane, 32);
+    }
+  });
+  __syncthreads();
+  drain(threadIdx.x, blockDim.x);
 }
 
 // d^n/du^n of Phi((e - u)/sigma), n = 0..3, in FP64
@@ -495,7 +452,7 @@ __global__ void __launch_bounds__(256) k_soft_finalize(const unsigned long long*
   }
 }
 
-// T[0][m] = W(c_m), T[1][m] = W'(c_m), T[2][m] = W''(c_m) for W(u) = sum_b G[b] K_b'(u)
+// T[2m] = W(c_m), T[2m + 1] = W'(c_m), T[2 n_fine + m] = W''(c_m) / 2 for W(u) = sum_b G[b] K_b'(u)
 __global__ void __launch_bounds__(256) k_soft_table(const float* __restrict__ G, uint32_t n_bins, uint32_t n_fine,
                                                     double w, double r0, double dr, double sigma,
                                                     float* __restrict__ T) {
@@ -516,19 +473,16 @@ __global__ void __launch_bounds__(256) k_soft_table(const float* __restrict__ G,
     a3 += g * (ph[3] - pl[3]);
     for (int k = 0; k < 4; ++k) pl[k] = ph[k];
   }
-  T[m] = (float)a1;
-  T[n_fine + m] = (float)a2;
-  T[2 * n_fine + m] = (float)a3;
+  T[2 * m] = (float)a1;
+  T[2 * m + 1] = (float)a2;
+  T[2 * n_fine + m] = (float)(0.5 * a3);
 }
 
 // ---------------------------------------------------------------------------
 // adjoint passes
 // ---------------------------------------------------------------------------
-// ONE: a single pass over the neighbour records when the centrals are among them; every record
-// owns its gradient, W s (x_o - x_c)/d times the pair's weight (central flags of both ends
-// added), and the central owners accumulate dL/ds.  Otherwise pass A (owners = centrals, write)
-// and pass B (owners = neighbours, add).
-template <bool ONE>
+// Pass A (owners = centrals, write) and pass B (owners = neighbours, add), for central types that are
+// not all neighbour types.
 __global__ void __launch_bounds__(256) k_soft_bwd(const SoftArgs a) {
   griddep_wait();
   griddep_launch();
@@ -542,11 +496,11 @@ __global__ void __launch_bounds__(256) k_soft_bwd(const SoftArgs a) {
   const uint32_t w = threadIdx.x >> 5;
   const float s = a.scale, inv_w = a.inv_w, wf = a.w, rc = a.rc;
   const uint32_t nf = a.n_fine;
-  float gx = 0.f, gy = 0.f, gz = 0.f, c_self = 0.f;
+  float gx = 0.f, gy = 0.f, gz = 0.f;
   double gs_lane = 0.0;
   float gs_item = 0.f;
-  auto begin = [&](bool, const float4&, float c_own) { gx = gy = gz = 0.f, gs_item = 0.f, c_self = c_own; };
-  auto pair = [&](const float4& p, float qx, float qy, float qz, float qw, float d2) {
+  auto begin = [&]() { gx = gy = gz = 0.f, gs_item = 0.f; };
+  auto pair = [&](const float4& p, float qx, float qy, float qz, float d2) {
     const float rs = d2 > 0.f ? rsqrtf(d2) : 0.f;
     const float d = d2 * rs;
     const float u = s * d;
@@ -554,18 +508,18 @@ __global__ void __launch_bounds__(256) k_soft_bwd(const SoftArgs a) {
     uint32_t m = (uint32_t)(u * inv_w);
     m = m < nf ? m : nf - 1;
     const float delta = u - ((float)m + 0.5f) * wf;
-    const float W = sT[m] + delta * (sT[nf + m] + 0.5f * delta * sT[2 * nf + m]);
-    const float f = W * s * rs * (ONE ? c_self + qw : 1.f);  // W s / d (0 for coincident ions), weighted
+    const float W = sT[2 * m] + delta * (sT[2 * m + 1] + delta * sT[2 * nf + m]);
+    const float f = W * s * rs;  // W s / d (0 for coincident ions)
     gx += f * (p.x - qx);
     gy += f * (p.y - qy);
     gz += f * (p.z - qz);
-    if (!ONE || c_self > 0.f) gs_item += W * d;
+    gs_item += W * d;
   };
   auto end = [&](bool valid, const float4& p) {
     if (!valid) return;
     const uint32_t idx = __float_as_uint(p.w);
     float* g = a.grad + 3 * (int64_t)idx;
-    if (!ONE && a.pass_b) {
+    if (a.pass_b) {
       // owners are neighbours j: dL/dx_j = -sum W s (x_i - x_j)/d, here p = x_j, q = x_i
       g[0] += gx, g[1] += gy, g[2] += gz;
     } else {
@@ -573,8 +527,8 @@ __global__ void __launch_bounds__(256) k_soft_bwd(const SoftArgs a) {
       gs_lane += (double)gs_item;
     }
   };
-  soft_items_owned<ONE>(a, reinterpret_cast<float*>(s_buf[w]), s_rsrc[w], s_rpre[w], pair, begin, end);
-  if (ONE || !a.pass_b) {
+  soft_items_owned(a, reinterpret_cast<float*>(s_buf[w]), s_rsrc[w], s_rpre[w], pair, begin, end);
+  if (!a.pass_b) {
     for (int o = 16; o > 0; o >>= 1) gs_lane += __shfl_xor_sync(0xffffffffu, gs_lane, o);
     if ((threadIdx.x & 31) == 0) s_gs[w] = gs_lane;
     __syncthreads();
@@ -583,6 +537,157 @@ __global__ void __launch_bounds__(256) k_soft_bwd(const SoftArgs a) {
       for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += s_gs[i];
       atomicAdd(a.grad_s, t);
     }
+  }
+}
+
+// Sums v[0..11] over the warp: afterwards lane l holds, in v[0], the sum of value
+// sum_slot(l) (lanes that differ in bit 0 alone hold the same one).  13 exchanges instead of 60:
+// each step sends away the half of the values that the partner keeps.
+template <int N>
+__device__ __forceinline__ void warp_sum_step(float (&v)[12], uint32_t lane, uint32_t o) {
+  const bool up = (lane & o) != 0u;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const float keep = up ? v[i + N] : v[i], send = up ? v[i] : v[i + N];
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+  }
+}
+__device__ __forceinline__ void warp_sum12(float (&v)[12], uint32_t lane) {
+  warp_sum_step<6>(v, lane, 16);
+  warp_sum_step<3>(v, lane, 8);
+  v[3] = 0.f;  // the fourth value of each lane is empty
+  warp_sum_step<2>(v, lane, 4);
+  warp_sum_step<1>(v, lane, 2);
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+// the value that lane l ends up with, or 12 (none)
+__device__ __forceinline__ uint32_t sum_slot(uint32_t lane) {
+  const uint32_t k = ((lane >> 2) & 1u) * 2u + ((lane >> 1) & 1u);  // of the three left after two steps
+  return k == 3u ? 12u : ((lane >> 4) & 1u) * 6u + ((lane >> 3) & 1u) * 3u + k;
+}
+
+__device__ __forceinline__ void red_global_v4(float4* p, float x, float y, float z) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x), "f"(y), "f"(z), "f"(0.f)
+               : "memory");
+}
+
+// Adjoint where the centrals are neighbour records: every unordered pair once (sweep_pairs), its
+// force f (x_j - x_i) added at both ends.  The candidate end sums over the staged records in
+// its lane's registers; the record end is summed over the lanes (warp_sum12, four records at a
+// time) into shared memory; both go to the record-ordered gradient `acc` with one 16-byte
+// reduction per record and tile (neighbouring candidates are neighbouring records), which
+// k_soft_grad_out scatters to the ions.  Bound by issue (~30 instructions per 32 tests) and by
+// the table's shared-memory reads.  Measured, 1e7-ion needle on half-size cells / 2e5 cylinder on
+// full-size cells (ms): 75.4 -> 23.8 / 3.56 -> 1.60 (before: every record a lane of its own, each pair tested
+// and evaluated from both ends); 128 or 64 registers a thread: 29.1 and 23.7 ms.
+__global__ void __launch_bounds__(256, 3) k_soft_bwd_sym(const SoftArgs a, const __grid_constant__ SweepArgs sw,
+                                                         float4* __restrict__ acc) {
+  griddep_wait();
+  griddep_launch();
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ SweepBuf s_sweep[8];
+  __shared__ float s_rec[8][kSweepRec * 3];  // per warp: gradients of the staged records
+  __shared__ double s_gs[8];
+  float* sT = reinterpret_cast<float*>(smem);
+  const uint32_t nf = a.n_fine, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (uint32_t m = threadIdx.x; m < 3 * nf; m += blockDim.x) sT[m] = a.T[m];
+  for (uint32_t i = lane; i < kSweepRec * 3; i += 32) s_rec[w][i] = 0.f;
+  __syncthreads();
+  SweepBuf& buf = s_sweep[w];
+  float* grec = s_rec[w];
+  const SoftFine fine(a);
+  const float rc = a.rc, s = a.scale;
+  const float2* T01 = reinterpret_cast<const float2*>(sT);
+  const float* T2 = sT + 2 * nf;
+  const uint32_t slot = sum_slot(lane);
+  double gs_lane = 0.0;
+  sweep_pairs<true>(
+      sw, buf,
+      [&](uint32_t n_pr, uint32_t, uint32_t nc, bool) __attribute__((always_inline)) {
+        const float4 far = make_float4(INFINITY, INFINITY, INFINITY, __uint_as_float(kCandSingle));
+        float4 c[2] = {lane < nc ? buf.cand[lane] : far, lane + 32 < nc ? buf.cand[lane + 32] : far};
+        float ws[2], g[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}}, gs = 0.f;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) ws[h] = __float_as_uint(c[h].w) == kCandBoth ? 2.f : 1.f;
+        const ulonglong2* rxy = reinterpret_cast<const ulonglong2*>(buf.rxy);
+        const unsigned long long* rz = reinterpret_cast<const unsigned long long*>(buf.rz);
+#pragma unroll 1
+        for (uint32_t k = 0; k < n_pr; k += 2) {  // four records
+          float r[12];
+#pragma unroll
+          for (int i = 0; i < 12; ++i) r[i] = 0.f;
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const ulonglong2 xy = rxy[k + q];
+            const unsigned long long zz = rz[k + q];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const unsigned long long dx2 = f2_sub(f2_pack(c[h].x, c[h].x), xy.x),
+                                       dy2 = f2_sub(f2_pack(c[h].y, c[h].y), xy.y),
+                                       dz2 = f2_sub(f2_pack(c[h].z, c[h].z), zz);
+              float da, db;
+              const unsigned long long d2 = soft_d2(dx2, dy2, dz2);
+              f2_unpack(d2, da, db);
+              const unsigned long long rs2 = f2_pack(rsqrt_fast(da), rsqrt_fast(db)), dd2 = f2_mul(d2, rs2),
+                                       u2 = f2_mul(dd2, fine.scale2);  // NaN at d = 0: no pair
+              unsigned long long m2, dl2;
+              fine.split(u2, m2, dl2);
+              float u[2], mm[2], dl[2], rs[2], dd[2], dx[2], dy[2], dz[2];
+              f2_unpack(u2, u[0], u[1]), f2_unpack(m2, mm[0], mm[1]), f2_unpack(dl2, dl[0], dl[1]);
+              f2_unpack(rs2, rs[0], rs[1]), f2_unpack(dd2, dd[0], dd[1]);
+              f2_unpack(dx2, dx[0], dx[1]), f2_unpack(dy2, dy[0], dy[1]), f2_unpack(dz2, dz[0], dz[1]);
+#pragma unroll
+              for (int e = 0; e < 2; ++e) {
+                if (u[e] < rc) {
+                  const uint32_t m = __float_as_uint(mm[e]) - kMagicBits;
+                  const float2 t = T01[m];
+                  const float W = (t.x + dl[e] * (t.y + dl[e] * T2[m])) * ws[h];
+                  const float f = W * s * rs[e];
+                  gs += W * dd[e];
+                  const float fx = f * dx[e], fy = f * dy[e], fz = f * dz[e];
+                  g[h][0] += fx, g[h][1] += fy, g[h][2] += fz;
+                  r[6 * q + 3 * e] -= fx, r[6 * q + 3 * e + 1] -= fy, r[6 * q + 3 * e + 2] -= fz;
+                }
+              }
+            }
+          }
+          warp_sum12(r, lane);
+          // value 6 q + 3 e + axis: record 2 (k + q) + e
+          if (slot < 12u && !(lane & 1u)) grec[6 * k + slot] += r[0];
+        }
+        gs_lane += (double)gs;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (lane + 32 * h < nc) red_global_v4(acc + buf.cidx[lane + 32 * h], g[h][0], g[h][1], g[h][2]);
+      },
+      [&](uint32_t m, bool) __attribute__((always_inline)) {
+        __syncwarp();
+        for (uint32_t r = lane; r < m; r += 32) {
+          red_global_v4(acc + buf.ridx[r], grec[3 * r], grec[3 * r + 1], grec[3 * r + 2]);
+          grec[3 * r] = grec[3 * r + 1] = grec[3 * r + 2] = 0.f;
+        }
+        __syncwarp();
+      });
+  for (int o = 16; o > 0; o >>= 1) gs_lane += __shfl_xor_sync(0xffffffffu, gs_lane, o);
+  if (lane == 0) s_gs[w] = gs_lane;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += s_gs[i];
+    atomicAdd(a.grad_s, t);
+  }
+}
+
+// the record-ordered gradient to the ions
+__global__ void __launch_bounds__(256) k_soft_grad_out(const float4* __restrict__ nrec, const float4* __restrict__ acc,
+                                                       const Geo* __restrict__ geo, float* __restrict__ grad) {
+  griddep_wait();
+  griddep_launch();
+  const uint32_t n = geo->n_sel;
+  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    const float4 v = acc[j];
+    float* g = grad + 3 * (int64_t)__float_as_uint(__ldg(nrec + j).w);
+    g[0] = v.x, g[1] = v.y, g[2] = v.z;
   }
 }
 
@@ -625,12 +730,6 @@ __global__ void k_reset_items(Geo* geo) {
   if (threadIdx.x == 0) geo->work_n2 = 0, geo->work_n3 = 0, geo->work_next2 = 0;
 }
 
-__global__ void k_reset_counter(Geo* geo) {
-  griddep_wait();
-  griddep_launch();
-  if (threadIdx.x == 0) geo->work_next2 = 0;
-}
-
 __global__ void k_soft_gs_out(const double* __restrict__ gs, float* __restrict__ out) {
   griddep_wait();
   griddep_launch();
@@ -644,10 +743,16 @@ static int soft_setup(ps_grid* g, float sigma, float scale, ps_bins bins, SoftAr
   const double rc = stop + 6.0 * (double)sigma;
   if ((double)g->r_cut * (double)scale < rc * (1.0 + 1e-6))
     return fail(PS_ERR_INVALID_ARG, "smoothed RDF: grid r_cut * scale must cover stop + 6 sigma");
-  double w = (double)sigma / 40.0;
-  if (rc / w > (double)kSoftFineMax) w = rc / (double)kSoftFineMax;
-  sa.n_fine = (uint32_t)std::ceil(rc / w);
-  if (sa.n_fine > kSoftFineMax) sa.n_fine = kSoftFineMax;
+  // fine width: at most sigma / 40, 11 significant bits (rounded down), and one spare bin for the
+  // rounding of floor(rc / w); wider (rounded up) where that takes more than kSoftFineMax bins
+  auto bits11 = [](double x, bool up) {
+    int e;
+    const double f = std::frexp(x, &e) * 2048.0;
+    return std::ldexp(up ? std::ceil(f) : std::floor(f), e - 11);
+  };
+  double w = bits11((double)sigma / 40.0, false);
+  if (rc / w > (double)(kSoftFineMax - 2)) w = bits11(rc / (double)(kSoftFineMax - 2), true);
+  sa.n_fine = (uint32_t)std::ceil(rc / w) + 1;
   sa.w = (float)w;
   sa.inv_w = (float)(1.0 / w);
   sa.scale = scale;
@@ -693,7 +798,8 @@ int soft_forward(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], floa
   z.p[1] = reinterpret_cast<uint64_t*>(g->soft_m1);
   z.p[2] = reinterpret_cast<uint64_t*>(g->soft_m2);
   z.n[0] = z.n[1] = z.n[2] = sa.n_fine;
-  rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z);
+  const bool sym = centrals_in_neighbours(g, ctr_mask);
+  rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, false, false, !sym);
   if (rc) return rc;
   sa.nrec = g->nbr.rec;
   sa.nstart = g->nbr.start;
@@ -701,28 +807,26 @@ int soft_forward(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], floa
   sa.M0 = g->soft_m0;
   sa.M1 = g->soft_m1;
   sa.M2 = g->soft_m2;
-  const uint32_t smem = sa.n_fine * 12;
   int blocks = 0;
-  if (centrals_in_neighbours(g, ctr_mask)) {
-    // unordered pairs of neighbour records, weighted by the central flags of both ends
-    rc = launch_grid_for(g, (const void*)k_soft_fwd<true>, smem, &blocks);
+  if (sym) {
+    const uint32_t smem = ((sa.n_fine + 3u) & ~3u) * 12;
+    rc = launch_grid_for(g, (const void*)k_soft_fwd_sym, smem, &blocks);
     if (rc) return rc;
-    // cells taken from the neighbour list's counter (owners = candidates = neighbour records)
-    PS_LAUNCH(PS_KID_SOFT_FWD, s, PS_CUDA(launch_pdl(k_reset_items, 1, 32, 0, s, g->nbr.geo)));
-    sa.orec = g->nbr.rec;
-    sa.ostart = g->nbr.start;
-    sa.ogeo = g->nbr.geo;
-    sa.pfx = reinterpret_cast<const uint32_t*>(g->cr);
-    PS_LAUNCH(PS_KID_SOFT_FWD, s, PS_CUDA(launch_pdl(k_soft_fwd<true>, blocks, 256, smem, s, sa)));
+    SweepArgs sw = sweep_args(g, &g->ctr.geo->sym_next);
+    sw.range = sa.rc2u;
+    PS_LAUNCH(PS_KID_SOFT_FWD, s,
+              PS_CUDA(launch_pdl(k_soft_fwd_sym, blocks, 256, smem, s, sa, sw, w / (double)kSoftQ,
+                                 w * w / (double)kSoftQ)));
   } else {
-    rc = launch_grid_for(g, (const void*)k_soft_fwd<false>, smem, &blocks);
+    const uint32_t smem = sa.n_fine * 12;
+    rc = launch_grid_for(g, (const void*)k_soft_fwd, smem, &blocks);
     if (rc) return rc;
     sa.orec = g->ctr.rec;
     sa.ostart = g->ctr.start;
     sa.oitem = g->ctr.witem;
     sa.ocap = g->item_cap;
     sa.ogeo = g->ctr.geo;
-    PS_LAUNCH(PS_KID_SOFT_FWD, s, PS_CUDA(launch_pdl(k_soft_fwd<false>, blocks, 256, smem, s, sa)));
+    PS_LAUNCH(PS_KID_SOFT_FWD, s, PS_CUDA(launch_pdl(k_soft_fwd, blocks, 256, smem, s, sa)));
   }
   PS_LAUNCH(PS_KID_SOFT_FWD, s,
             PS_CUDA(launch_pdl(k_soft_finalize, bins.n_bins, 256, 0, s, g->soft_m0, g->soft_m1, g->soft_m2, sa.n_fine, w, bins.r0,
@@ -738,7 +842,8 @@ int soft_backward(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], flo
   double w = 0.0;
   int rc = soft_setup(g, sigma, scale, bins, sa, w);
   if (rc) return rc;
-  rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s);
+  const bool sym = centrals_in_neighbours(g, ctr_mask);
+  rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, ZeroOut(), false, false, !sym);
   if (rc) return rc;
   PS_CUDA(cudaMemsetAsync(d_grad, 0, (size_t)g->n * 3 * sizeof(float), s));
   PS_CUDA(cudaMemsetAsync(g->soft_gs, 0, sizeof(double), s));
@@ -750,20 +855,19 @@ int soft_backward(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], flo
   sa.grad_s = g->soft_gs;
   const uint32_t smem = sa.n_fine * 12;
   int blocks = 0;
-  if (centrals_in_neighbours(g, ctr_mask)) {
-    // one pass: the central prefix over the neighbour records (built with the central list) gives
-    // every record's central flag
-    rc = launch_grid_for(g, (const void*)k_soft_bwd<true>, smem, &blocks);
+  if (sym) {
+    // the record-ordered gradient takes the place of the central records, which the sweep does not use
+    rc = launch_grid_for(g, (const void*)k_soft_bwd_sym, smem, &blocks);
     if (rc) return rc;
-    rc = nbr_items(g, sa, s, PS_KID_SOFT_BWD);
-    if (rc) return rc;
-    sa.nrec = g->nbr.rec;
-    sa.nstart = g->nbr.start;
-    sa.ngeo = g->nbr.geo;
-    sa.pfx = reinterpret_cast<const uint32_t*>(g->cr);
-    PS_LAUNCH(PS_KID_SOFT_BWD, s, PS_CUDA(launch_pdl(k_soft_bwd<true>, blocks, 256, smem, s, sa)));
+    float4* acc = g->ctr.rec;
+    PS_CUDA(cudaMemsetAsync(acc, 0, (size_t)g->n * sizeof(float4), s));
+    SweepArgs sw = sweep_args(g, &g->ctr.geo->sym_next);
+    sw.range = sa.rc2u;
+    PS_LAUNCH(PS_KID_SOFT_BWD, s, PS_CUDA(launch_pdl(k_soft_bwd_sym, blocks, 256, smem, s, sa, sw, acc)));
+    PS_LAUNCH(PS_KID_SOFT_BWD, s,
+              PS_CUDA(launch_pdl(k_soft_grad_out, g->num_sms * 8, 256, 0, s, g->nbr.rec, acc, g->nbr.geo, d_grad)));
   } else {
-    rc = launch_grid_for(g, (const void*)k_soft_bwd<false>, smem, &blocks);
+    rc = launch_grid_for(g, (const void*)k_soft_bwd, smem, &blocks);
     if (rc) return rc;
     // pass A: owners = centrals, candidates = neighbours
     sa.orec = g->ctr.rec;
@@ -775,7 +879,7 @@ int soft_backward(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], flo
     sa.nstart = g->nbr.start;
     sa.ngeo = g->nbr.geo;
     sa.pass_b = 0;
-    PS_LAUNCH(PS_KID_SOFT_BWD, s, PS_CUDA(launch_pdl(k_soft_bwd<false>, blocks, 256, smem, s, sa)));
+    PS_LAUNCH(PS_KID_SOFT_BWD, s, PS_CUDA(launch_pdl(k_soft_bwd, blocks, 256, smem, s, sa)));
     // pass B: owners = neighbours, candidates = centrals
     rc = nbr_items(g, sa, s, PS_KID_SOFT_BWD);
     if (rc) return rc;
@@ -783,7 +887,7 @@ int soft_backward(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], flo
     sa.nstart = g->ctr.start;
     sa.ngeo = g->nbr.geo;
     sa.pass_b = 1;
-    PS_LAUNCH(PS_KID_SOFT_BWD, s, PS_CUDA(launch_pdl(k_soft_bwd<false>, blocks, 256, smem, s, sa)));
+    PS_LAUNCH(PS_KID_SOFT_BWD, s, PS_CUDA(launch_pdl(k_soft_bwd, blocks, 256, smem, s, sa)));
   }
   PS_LAUNCH(PS_KID_SOFT_BWD, s, PS_CUDA(launch_pdl(k_soft_gs_out, 1, 32, 0, s, g->soft_gs, d_grad_s)));
   PS_CUDA(cudaGetLastError());

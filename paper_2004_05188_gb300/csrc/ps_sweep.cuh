@@ -31,6 +31,25 @@ constexpr uint32_t kSweepRec = 64;        // records staged at a time
 constexpr uint32_t kSweepTile = 64;       // candidates per tile, two per lane
 constexpr uint32_t kCandSingle = 0u, kCandBoth = 1u, kCandOwn = 2u, kCandSelf = 3u;
 
+__device__ __forceinline__ float sqrt_fast(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
+                                                     unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// rounded down: with c = kMagic the floor of a * b in the low bits
+__device__ __forceinline__ unsigned long long f2_fma_down(unsigned long long a, unsigned long long b,
+                                                          unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 struct SweepArgs {
   const float4* nrec;
   const uint32_t* nstart;
@@ -87,12 +106,6 @@ struct SweepBuf {
   uint32_t ridx[kSweepRec];                // record numbers of the staged records (likewise)
 };
 
-__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
-                                                     unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
 // Two squared distances as dist2(): packed throughout.  The sums are x * one + y with one = 1.0f
 // passed at run time: x * 1 + y rounds once, exactly as x + y does, and the compiler cannot fuse
 // the squares into it (a packed add it does fuse).
@@ -117,9 +130,9 @@ __device__ __forceinline__ void sweep_shape(const Geo& g, uint32_t n_warps, uint
 
 // Runs every unit.  tile(n_pr, m, nc, central): the staged records (m of them, n_pr pairs, n_pr even,
 // padded with far records), all central or all not, against nc <= 64 candidates in buf.cand.
-// INDEX: fill buf.cidx / buf.ridx.
-template <bool INDEX, class Tile>
-__device__ __forceinline__ void sweep_pairs(const SweepArgs& a, SweepBuf& buf, Tile&& tile) {
+// INDEX: fill buf.cidx / buf.ridx.  done(m, central) follows the last tile of the staged records.
+template <bool INDEX, class Tile, class Done>
+__device__ __forceinline__ void sweep_pairs(const SweepArgs& a, SweepBuf& buf, Tile&& tile, Done&& done) {
   const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
   const Geo g = *a.ngeo;
   const int s = a.stencil, W = 2 * s + 1, inv_w = 65536 / W + 1;
@@ -308,10 +321,16 @@ __device__ __forceinline__ void sweep_pairs(const SweepArgs& a, SweepBuf& buf, T
               __syncwarp();
             }
           }
+          done(m, central != 0u);
         }
       }
     }
   }
+}
+
+template <bool INDEX, class Tile>
+__device__ __forceinline__ void sweep_pairs(const SweepArgs& a, SweepBuf& buf, Tile&& tile) {
+  sweep_pairs<INDEX>(a, buf, tile, [](uint32_t, bool) {});
 }
 
 }  // namespace ps

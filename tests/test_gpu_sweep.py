@@ -67,3 +67,39 @@ def test_distribution_map_mirrored(ps, orc, spec, R, w, nv, lattice):
         np.testing.assert_array_equal(out["meta"].cpu().numpy()[:3].astype(np.uint64), m)
         np.testing.assert_array_equal(out["H"].cpu().numpy().astype(np.uint64), H)
         g.close()
+
+
+@pytest.mark.parametrize("m,copies", [(12, 1), (12, 3), (24, 40)])
+def test_smoothed_rdf_of_lattice_shells(ps, spec, m, copies):
+    """Smoothed RDF and dL/dscale of coincident copies of a simple-cubic block against the closed form
+    over its shells (FP64): every pair of a shell falls into one fine bin, up to 2e8 of them (the
+    integer moments are drained on the way), and coincident ions count at u = 0 but the ion itself
+    does not.  Tolerance: the library's stated 1e-5 of h; the force of each interior ion cancels."""
+    from math import erf, exp, pi, sqrt
+
+    a, sig, bins = 0.25, 0.05, (0.0, 0.02, 30)
+    xyz, t, d = spec.simple_cubic(m, a, 0.125)
+    xyz, t, d = (np.repeat(v, copies, axis=0) for v in (xyz, t, d))
+    rc = 0.6 + 6 * sig
+    dmin = 0.95
+    X, T, D = (torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (xyz, t, d))
+    g = ps.Grid(X.shape[0], 0.5).build(X, T, "all", ps.soft_r_cut(bins, sig, 1.0))
+    h = ps.soft_rdf_fwd(g, D, "all", dmin, sig, 1.0, bins).cpu().numpy().astype(np.float64)
+    G = np.random.default_rng(5).normal(size=bins[2])
+    gx, gs = ps.soft_rdf_bwd(g, D, "all", dmin, sig, 1.0, bins, torch.from_numpy(G.astype(np.float32)).cuda())
+    n_c = int((d >= dmin).sum())
+    assert n_c > 0
+    k = np.arange(-4, 5)
+    I, J, K = np.meshgrid(k, k, k, indexing="ij")
+    u = a * np.sqrt((I**2 + J**2 + K**2).ravel())
+    u = u[u < rc]
+    e = np.arange(bins[2] + 1) * bins[1]
+    Phi = np.array([[0.5 * (1 + erf((x - y) / sig / sqrt(2))) for x in e] for y in u])
+    pdf = np.array([[exp(-0.5 * ((x - y) / sig) ** 2) / sig / sqrt(2 * pi) for x in e] for y in u])
+    mult = np.where(u > 0, copies, copies - 1).astype(np.float64)
+    ref = n_c * (mult[:, None] * np.diff(Phi, axis=1)).sum(0)
+    assert np.linalg.norm(h - ref) <= 1e-5 * np.linalg.norm(ref)
+    W = -(np.diff(pdf, axis=1) * G.astype(np.float32)).sum(1)
+    gs_ref = n_c * (mult * W * u).sum()
+    assert abs(float(gs[0]) - gs_ref) <= 1e-4 * n_c * (mult * np.abs(W) * u).sum()
+    g.close()
