@@ -134,9 +134,11 @@ int ps_grid_create(int64_t n_max, const ps_grid_opts* opts, ps_grid** out) {
   const int64_t cap0 = g->stencil >= 2 ? g->n_max : g->n_max / 8;
   const int64_t cap = cap0 > 65536 ? cap0 : 65536;
   g->cell_cap = (uint32_t)(cap < (int64_t)1 << 31 ? cap : (int64_t)1 << 31);
+  // the count arrays also hold the sub-cells of dense cells (at most n / 4, see sub_cells)
+  g->fine_cap = (uint32_t)((int64_t)g->cell_cap > g->n_max / 4 ? (int64_t)g->cell_cap : g->n_max / 4);
   // scan tiles of 4096 cells or 4096 records (the central list's record compaction)
   g->scan_tiles_cap = (uint32_t)(((int64_t)g->cell_cap > g->n_max + 1 ? (int64_t)g->cell_cap : g->n_max + 1) + 4095) / 4096;
-  const size_t nm = (size_t)g->n_max, cc = g->cell_cap;
+  const size_t nm = (size_t)g->n_max, cc = g->cell_cap, fc = g->fine_cap;
   size_t off = 0;
   auto take = [&](size_t bytes) {
     const size_t o = off;
@@ -144,8 +146,8 @@ int ps_grid_create(int64_t n_max, const ps_grid_opts* opts, ps_grid** out) {
     return o;
   };
   const size_t o_sel = take(nm * 4), o_cr = take(nm * 8);
-  const size_t o_ncount = take(cc * 4), o_nstart = take((cc + 1) * 4), o_nrec = take(nm * 16);
-  const size_t o_ccount = take(cc * 4), o_cstart = take((cc + 1) * 4), o_crec = take(nm * 16), o_cwork = take(cc * 4);
+  const size_t o_ncount = take(fc * 4), o_nstart = take((cc + 1) * 4), o_nrec = take(nm * 16);
+  const size_t o_ccount = take(fc * 4), o_cstart = take((cc + 1) * 4), o_crec = take(nm * 16), o_cwork = take(cc * 4);
   g->item_cap = (uint32_t)(cc + nm / 8 + 2);  // batches of >= 8 centrals (4 lanes per central) + one per cell
   const size_t o_witem = take((size_t)g->item_cap * 8), o_nwitem = take((size_t)g->item_cap * 8);
   const size_t o_sm0 = take(kSoftFineMax * 8), o_sm1 = take(kSoftFineMax * 8), o_sm2 = take(kSoftFineMax * 8);

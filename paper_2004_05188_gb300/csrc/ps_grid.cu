@@ -111,7 +111,7 @@ __global__ void k_reset(Geo* geo) {
     geo->status = 0;
     geo->work_n = geo->work_n2 = geo->work_n3 = geo->work_n4 = 0;
     geo->work_next = geo->work_next2 = geo->work_next3 = 0;
-    geo->work_next2b = geo->work_next3b = geo->sym_next = geo->list_n = 0;
+    geo->work_next2b = geo->work_next3b = geo->sym_next = geo->list_n = geo->sub = 0;
   }
 }
 
@@ -242,15 +242,17 @@ __device__ void compute_geometry(const Geo& in, float r_cut, float cell_scale, u
 
 // One thread per block computes the geometry; block 0 publishes it; all zero the counts.
 __global__ void __launch_bounds__(kThreads) k_geometry_zero(Geo* geo, float r_cut, float cell_scale, uint32_t cell_cap,
-                                                            uint32_t* __restrict__ count) {
+                                                            uint32_t fine_cap, uint32_t* __restrict__ count) {
   griddep_wait();
   griddep_launch();
   __shared__ uint32_t s_nc;
   if (threadIdx.x == 0) {
     Geo g = *geo;
     compute_geometry(g, r_cut, cell_scale, cell_cap, g);
-    s_nc = g.n_cells;
+    const uint32_t sub = sub_cells(g.n_sel, g.n_cells, fine_cap);
+    s_nc = g.n_cells << (3 * sub);
     if (blockIdx.x == 0) {
+      geo->sub = sub;
       for (int a = 0; a < 3; ++a) geo->origin[a] = g.origin[a], geo->dims[a] = g.dims[a];
       geo->h = g.h;
       geo->inv_h = g.inv_h;
@@ -271,7 +273,7 @@ __global__ void __launch_bounds__(kThreads) k_count(const float* __restrict__ xy
   const Geo g = *geo;
   for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < g.n_sel; s += gridDim.x * blockDim.x) {
     const uint32_t i = sel[s];
-    const uint32_t c = cell_of(g, xyz[3 * (int64_t)i], xyz[3 * (int64_t)i + 1], xyz[3 * (int64_t)i + 2]);
+    const uint32_t c = fine_of(g, g.sub, xyz[3 * (int64_t)i], xyz[3 * (int64_t)i + 1], xyz[3 * (int64_t)i + 2]);
     cr[s] = make_uint2(c, atomicAdd(&count[c], 1u));
   }
 }
@@ -287,6 +289,7 @@ __global__ void __launch_bounds__(kThreads) k_central_select_count(const float* 
   griddep_launch();
   __shared__ uint32_t s_aw[kThreads / 32], s_ax[kThreads / 32], s_abase;
   const Geo g = *ngeo;
+  const uint32_t sub = cgeo->sub;
   bool bad = false;
   const int64_t groups = (n + kGroup - 1) / kGroup;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -331,7 +334,7 @@ __global__ void __launch_bounds__(kThreads) k_central_select_count(const float* 
       const int64_t i = i0 + k;
       const float x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
       bad |= !finite3(x, y, z);
-      const uint32_t c = cell_of(g, x, y, z);
+      const uint32_t c = fine_of(g, sub, x, y, z);
       sel[slot] = (uint32_t)i;
       cr[slot] = make_uint2(c, atomicAdd(&count[c], 1u));
       ++slot;
@@ -342,10 +345,12 @@ __global__ void __launch_bounds__(kThreads) k_central_select_count(const float* 
 
 // Resets the central list (copies the neighbour geometry, zeroes the counters
 // and cell counts) and zeroes the query's output arrays.
-__global__ void k_central_reset(const Geo* __restrict__ ngeo, Geo* cgeo, uint32_t* __restrict__ count, ZeroOut z) {
+__global__ void k_central_reset(const Geo* __restrict__ ngeo, Geo* cgeo, uint32_t* __restrict__ count, ZeroOut z,
+                                uint64_t n, uint32_t fine_cap) {
   griddep_wait();
   griddep_launch();
-  const uint32_t nc = ngeo->n_cells;
+  // (the centrals are not counted yet: their sub-cells by the number of ions)
+  const uint32_t sub = sub_cells(n, ngeo->n_cells, fine_cap), nc = ngeo->n_cells << (3 * sub);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *cgeo = *ngeo;
     cgeo->n_sel = 0;
@@ -353,6 +358,7 @@ __global__ void k_central_reset(const Geo* __restrict__ ngeo, Geo* cgeo, uint32_
     cgeo->work_n = cgeo->work_n2 = cgeo->work_n3 = cgeo->work_n4 = 0;
     cgeo->work_next = cgeo->work_next2 = cgeo->work_next3 = 0;
     cgeo->work_next2b = cgeo->work_next3b = cgeo->sym_next = cgeo->list_n = 0;
+    cgeo->sub = sub;
   }
   const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
   for (uint32_t c = tid; c < nc; c += stride) count[c] = 0;
@@ -521,8 +527,9 @@ __device__ __forceinline__ void emit_items(const uint32_t (&v)[kScanItems], uint
     if (dense) work[s1] = c0 + k;
     const uint32_t cand = (!dense && v[k] > 0 && nstart != nullptr) ? stencil_count(nstart, geo, c0 + k, stencil) : 0u;
     sparse[k] = !dense && v[k] > 0 && v[k] < kHeavy && nstart != nullptr && cand <= kSparseCand;
-    lanes[k] = (split && nstart != nullptr && !sparse[k] && v[k] > 3) ? lanes_per_central(cand, n_nbr, nc, stencil)
-                                                                        : 1u;
+    lanes[k] = (split && nstart != nullptr && !sparse[k] && v[k] > 3)
+                   ? max(lanes_per_central(cand, n_nbr, nc, stencil), fill_lanes(geo->n_sel))
+                   : 1u;
     cands[k] = cand;
     if (!dense && sparse[k]) n_back += items_of(v[k], lanes[k]);
     if (!dense && !sparse[k]) {
@@ -559,10 +566,10 @@ __device__ __forceinline__ void emit_items(const uint32_t (&v)[kScanItems], uint
   }
 }
 
-// Single-pass exclusive scan of the cell counts (decoupled look-back).  Also
-// writes the end sentinel and, for the central list (`work` given), the work
-// lists (emit_items).
-__global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t* __restrict__ count, Geo* geo,
+// Single-pass exclusive scan of the cell (or sub-cell) counts (decoupled look-back): the cells' starts
+// and the end sentinel; the counts of sub-cells are replaced by their starts, which the scatter
+// reads.  With `work` given (no sub-cells), also the work lists (emit_items).
+__global__ void __launch_bounds__(kScanThreads) k_scan(uint32_t* __restrict__ count, Geo* geo,
                                                        uint32_t* __restrict__ start, uint32_t* __restrict__ work,
                                                        uint2* __restrict__ witem, uint32_t dense_min, uint32_t cap,
                                                        unsigned long long* state, uint32_t* ctr,
@@ -572,7 +579,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t* __restric
   griddep_launch();
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_tile, s_prefix;
-  const uint32_t nc = geo->n_cells;
+  const uint32_t sub3 = 3 * geo->sub, nc = geo->n_cells << sub3, in_cell = (1u << sub3) - 1u;
   const uint32_t tiles = (nc + kScanTile - 1) / kScanTile;
   for (;;) {
     if (threadIdx.x == 0) s_tile = atomicAdd(&ctr[0], 1u);
@@ -592,14 +599,17 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t* __restric
       const uint32_t prefix = tile_lookback(t, total, state, &geo->status);
       if (lane_id() == 0) {
         s_prefix = prefix;
-        if (t == tiles - 1) start[nc] = prefix + total;  // end sentinel: number of records
+        if (t == tiles - 1) start[nc >> sub3] = prefix + total;  // end sentinel: number of records
       }
     }
     __syncthreads();
     uint32_t run = s_prefix + excl;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-      if (c0 + k < nc) start[c0 + k] = run;
+      if (c0 + k < nc) {
+        if (((c0 + k) & in_cell) == 0u) start[(c0 + k) >> sub3] = run;
+        if (sub3) count[c0 + k] = run;
+      }
       run += v[k];
     }
     if (work != nullptr) emit_items(v, c0, nc, geo, work, witem, dense_min, cap, nstart, stencil, split, whi);
@@ -644,7 +654,7 @@ __global__ void __launch_bounds__(kScanThreads) k_central_subset(const float4* _
     cgeo->status = 0;
     cgeo->work_n = cgeo->work_n2 = cgeo->work_n3 = cgeo->work_n4 = 0;
     cgeo->work_next = cgeo->work_next2 = cgeo->work_next3 = 0;
-    cgeo->work_next2b = cgeo->work_next3b = cgeo->sym_next = cgeo->list_n = 0;
+    cgeo->work_next2b = cgeo->work_next3b = cgeo->sym_next = cgeo->list_n = cgeo->sub = 0;
     if (nr == 0) pfx[0] = 0, cgeo->n_sel = 0;
   }
   {
@@ -698,9 +708,9 @@ __global__ void __launch_bounds__(kScanThreads) k_central_subset(const float4* _
   scan_finish(state, ctr, tiles);
 }
 
-// Central list of a central type set contained in the neighbour set, step 2 of 2:
-// cell starts from the record prefix (a cell's centrals are the flagged records
-// among its neighbour records), the end sentinel and the work lists.
+// Work lists of the central list.  Central type set contained in the neighbour set (`pfx` given),
+// step 2 of 2: also the cell starts from the record prefix (a cell's centrals are the flagged
+// records among its neighbour records) and the end sentinel; otherwise from the cell starts.
 __global__ void __launch_bounds__(kThreads) k_central_items(const uint32_t* __restrict__ nstart,
                                                             const uint32_t* __restrict__ pfx, Geo* cgeo,
                                                             uint32_t* __restrict__ start, uint32_t* __restrict__ work,
@@ -721,10 +731,12 @@ __global__ void __launch_bounds__(kThreads) k_central_items(const uint32_t* __re
       v[k] = 0;
       const uint32_t c = c0 + k;
       if (c < nc) {
-        const uint32_t b = pfx[nstart[c]], e = pfx[nstart[c + 1]];
-        start[c] = b;
+        const uint32_t b = pfx ? pfx[nstart[c]] : start[c], e = pfx ? pfx[nstart[c + 1]] : start[c + 1];
         v[k] = (ok && e >= b) ? e - b : 0u;
-        if (c == nc - 1) start[nc] = e;
+        if (pfx) {
+          start[c] = b;
+          if (c == nc - 1) start[nc] = e;
+        }
       }
     }
     emit_items(v, c0, nc, cgeo, work, witem, dense_min, cap, nstart, stencil, split, whi);
@@ -774,12 +786,14 @@ __global__ void __launch_bounds__(kThreads) k_vertex_scatter(const float4* __res
 // Scatter the selected ions to their sorted slot.  The record's 4th word is the
 // ion index, or (index << 8 | type) when `type` is given (clouds of < 2^24 ions).
 __global__ void __launch_bounds__(kThreads) k_scatter(const float* __restrict__ xyz, const uint32_t* __restrict__ sel,
-                                                      const uint2* __restrict__ cr, const uint32_t* __restrict__ start,
+                                                      const uint2* __restrict__ cr, const uint32_t* __restrict__ cell_start,
+                                                      const uint32_t* __restrict__ sub_start,
                                                       const Geo* __restrict__ cnt, float4* __restrict__ rec,
                                                       const uint8_t* __restrict__ type) {
   griddep_wait();
   griddep_launch();
   const uint32_t ns = cnt->n_sel;
+  const uint32_t* start = cnt->sub ? sub_start : cell_start;
   for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < ns; s += gridDim.x * blockDim.x) {
     const uint32_t i = sel[s];
     const uint2 c = cr[s];
@@ -820,14 +834,16 @@ int wait_selftest(uint64_t limit_ns, unsigned long long* d_work, cudaStream_t s)
 
 static int grid_blocks(const ps_grid* g, int per_sm) { return g->num_sms * per_sm; }
 
+// sub-cells only where a cell is as wide as the search range (two- and three-cell stencils are fine enough)
+static uint32_t fine_cap(const ps_grid* g) { return g->stencil == 1 ? g->fine_cap : 0u; }
+
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-static int scan_cells(ps_grid* g, CellList& L, Geo* geo, bool with_work, cudaStream_t s, bool split = false) {
+static int scan_cells(ps_grid* g, CellList& L, Geo* geo, cudaStream_t s) {
   PS_LAUNCH(PS_KID_SCAN, s,
-            PS_CUDA(launch_pdl(k_scan, grid_blocks(g, 1), kScanThreads, 0, s, L.count, geo, L.start, with_work ? L.work : nullptr,
-                                                               L.witem, g->dense_min, g->item_cap, g->scan_state,
-                                                               g->scan_ctr, with_work ? g->nbr.start : nullptr,
-                                                               g->stencil, split, split ? g->nbr_witem : nullptr)));
+            PS_CUDA(launch_pdl(k_scan, grid_blocks(g, 1), kScanThreads, 0, s, L.count, geo, L.start, (uint32_t*)nullptr,
+                               L.witem, g->dense_min, g->item_cap, g->scan_state, g->scan_ctr, (const uint32_t*)nullptr,
+                               g->stencil, false, (uint2*)nullptr)));
   PS_CUDA(cudaGetLastError());
   return PS_OK;
 }
@@ -842,12 +858,12 @@ int build_neighbour_grid(ps_grid* g, const uint64_t nbr_mask[4], float r_cut, cu
     PS_LAUNCH(PS_KID_SELECT, s,
               PS_CUDA(launch_pdl(k_select_bbox, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->type, g->n, m, vec, g->sel, geo)));
   PS_LAUNCH(PS_KID_GEOMETRY, s,
-            PS_CUDA(launch_pdl(k_geometry_zero, grid_blocks(g, 4), kThreads, 0, s, geo, r_cut, g->cell_scale, g->cell_cap, g->nbr.count)));
+            PS_CUDA(launch_pdl(k_geometry_zero, grid_blocks(g, 4), kThreads, 0, s, geo, r_cut, g->cell_scale, g->cell_cap, fine_cap(g), g->nbr.count)));
   PS_LAUNCH(PS_KID_COUNT, s, PS_CUDA(launch_pdl(k_count, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->sel, geo, g->nbr.count, g->cr)));
-  int rc = scan_cells(g, g->nbr, geo, false, s);
+  int rc = scan_cells(g, g->nbr, geo, s);
   if (rc) return rc;
   PS_LAUNCH(PS_KID_SCATTER, s,
-            PS_CUDA(launch_pdl(k_scatter, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->sel, g->cr, g->nbr.start, geo, g->nbr.rec,
+            PS_CUDA(launch_pdl(k_scatter, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->sel, g->cr, g->nbr.start, g->nbr.count, geo, g->nbr.rec,
                                                              g->pack_type ? g->type : nullptr)));
   PS_CUDA(cudaGetLastError());
   return PS_OK;
@@ -888,7 +904,7 @@ int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4]
                                  g->scan_ctr, z, (uint32_t*)nullptr)));
     if (items)
       PS_LAUNCH(PS_KID_SCAN, s,
-              PS_CUDA(launch_pdl(k_central_items, grid_blocks(g, 4), kThreads, 0, s, g->nbr.start, pfx, g->ctr.geo,
+              PS_CUDA(launch_pdl(k_central_items, grid_blocks(g, 4), kThreads, 0, s, g->nbr.start, (const uint32_t*)pfx, g->ctr.geo,
                                  g->ctr.start, g->ctr.work, g->ctr.witem, g->dense_min, g->item_cap, g->stencil, split,
                                  split ? g->nbr_witem : nullptr)));
     PS_CUDA(cudaGetLastError());
@@ -896,16 +912,20 @@ int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4]
   }
   const bool vec = aligned16(g->type) && aligned16(g->xyz) && (dsrf == nullptr || aligned16(dsrf));
   PS_LAUNCH(PS_KID_CENTRAL, s,
-            PS_CUDA(launch_pdl(k_central_reset, grid_blocks(g, 4), kThreads, 0, s, g->nbr.geo, g->ctr.geo, g->ctr.count, z)));
+            PS_CUDA(launch_pdl(k_central_reset, grid_blocks(g, 4), kThreads, 0, s, g->nbr.geo, g->ctr.geo, g->ctr.count, z, (uint64_t)g->n, fine_cap(g))));
   if (g->n > 0)
     PS_LAUNCH(PS_KID_CENTRAL, s,
               PS_CUDA(launch_pdl(k_central_select_count, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->type, dsrf, g->n, m, dsrf_min,
                                                                               vec, g->nbr.geo, g->ctr.geo, g->ctr.count,
                                                                               g->sel, g->cr)));
-  int rc = scan_cells(g, g->ctr, g->ctr.geo, true, s, split);
+  int rc = scan_cells(g, g->ctr, g->ctr.geo, s);
   if (rc) return rc;
+  PS_LAUNCH(PS_KID_SCAN, s,
+            PS_CUDA(launch_pdl(k_central_items, grid_blocks(g, 4), kThreads, 0, s, g->nbr.start, (const uint32_t*)nullptr,
+                               g->ctr.geo, g->ctr.start, g->ctr.work, g->ctr.witem, g->dense_min, g->item_cap,
+                               g->stencil, split, split ? g->nbr_witem : nullptr)));
   PS_LAUNCH(PS_KID_SCATTER, s,
-            PS_CUDA(launch_pdl(k_scatter, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->sel, g->cr, g->ctr.start, g->ctr.geo, g->ctr.rec,
+            PS_CUDA(launch_pdl(k_scatter, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->sel, g->cr, g->ctr.start, g->ctr.count, g->ctr.geo, g->ctr.rec,
                                                              g->pack_type ? g->type : nullptr)));
   PS_CUDA(cudaGetLastError());
   return PS_OK;

@@ -85,7 +85,20 @@ struct Geo {
   uint32_t work_next3b;
   uint32_t sym_next;     // cells taken by the symmetric RDF pass (32 at a time)
   uint32_t list_n;       // centrals listed by the near kNN pass for the full-radius search
+  uint32_t sub;          // the records of a cell are ordered by its 2^sub x 2^sub x 2^sub sub-cells
 };
+
+// Sub-cells: a cell of many records is searched in groups (32 centrals of an item, 64 records of
+// a sweep), and the candidates that a group has to test are those within range of its bounding
+// box, so the groups should be compact.  Ordering the records of a cell by its octants (2 nm cells
+// at 30 ions/nm^3: 240 records, 30 per octant) shrinks a group's box from the cell to about two
+// octants, the volume within 2 nm of it from 165 to 106 nm^3.  Cells of 48 records on average are
+// split once, of 512 twice; sparser ones are a group or two anyway.  `cap` entries of counts (0: no sub-cells).
+__host__ __device__ __forceinline__ uint32_t sub_cells(uint64_t n_rec, uint64_t n_cells, uint64_t cap) {
+  uint32_t s = n_rec >= 512 * n_cells ? 2u : (n_rec >= 48 * n_cells ? 1u : 0u);
+  while (s && (n_cells << (3 * s)) > cap) --s;
+  return s;
+}
 
 // Warp items with at least this many centrals per cell are listed first (largest work first).
 constexpr uint32_t kHeavy = 16;
@@ -106,12 +119,23 @@ __host__ __device__ __forceinline__ uint32_t lanes_per_central(uint32_t n_cand, 
   return lhs >= 32 * unit ? 4u : (lhs >= 16 * unit ? 2u : 1u);
 }
 
-// Lanes per central of a warp item of the exact query with cnt (4..32) centrals: the largest
-// power of two, at most 8, with cnt * L <= 32.  A full item of a cell split by
+// Small clouds: enough lanes per central that the query has as many items as the chip takes warps
+// (about 3,600 on 152 SMs): an item tests its thousands of candidates one after the other, and too few
+// items leave the chip idle for the length of that chain.  2e4-ion cylinder, one pass: 0.317 -> 0.140 ms;
+// 3e4 ions, per-ion outputs: 0.64 ms for 912 items, 0.40 for 1824, 0.28 for 3648 and 0.27 for 7296 (which
+// costs the 1e5-ion cloud 10 %: more lanes per central share less of a candidate's load).
+constexpr uint32_t kFillItems = 3648;
+__host__ __device__ __forceinline__ uint32_t fill_lanes(uint32_t n_ctr) {
+  const uint32_t want = kFillItems * 32u;
+  return n_ctr * 8u <= want ? 8u : (n_ctr * 4u <= want ? 4u : (n_ctr * 2u <= want ? 2u : 1u));
+}
+
+// Lanes per central of a warp item of the exact query with cnt (1..32) centrals: the largest
+// power of two with cnt * L <= 32, at most 8 (16 for one or two centrals).  A full item of a cell split by
 // lanes_per_central (32 / L centrals) gets that L back; a cell's last, partial item gets more
 // lanes, so that its warp is not left mostly idle.
 __host__ __device__ __forceinline__ uint32_t item_lanes(uint32_t cnt) {
-  return cnt <= 4u ? 8u : (cnt <= 8u ? 4u : (cnt <= 16u ? 2u : 1u));
+  return cnt <= 2u ? 16u : (cnt <= 4u ? 8u : (cnt <= 8u ? 4u : (cnt <= 16u ? 2u : 1u)));
 }
 
 // A warp item of the exact query is "very heavy" when each of its lanes tests at least 8 times
@@ -130,7 +154,7 @@ __device__ __forceinline__ uint2 work_item(const uint2* witem, uint32_t cap, uin
 
 // A sorted cell list: count / start per cell and the sorted records.
 struct CellList {
-  uint32_t* count = nullptr;   // [cell_cap]
+  uint32_t* count = nullptr;   // [fine_cap]: records per (sub-)cell, then where each sub-cell starts
   uint32_t* start = nullptr;   // [cell_cap + 1]
   float4* rec = nullptr;       // [n_max]: x, y, z, original index bits
   uint32_t* work = nullptr;    // [cell_cap]: dense cells
@@ -143,6 +167,7 @@ struct CellList {
 struct ps_grid {
   int64_t n_max = 0;
   uint32_t cell_cap = 0;
+  uint32_t fine_cap = 0;       // (sub-)cells that the count arrays hold
   float cell_scale = 1.0f;
   uint32_t block = 0;
   int device = 0;
@@ -252,6 +277,21 @@ __device__ __forceinline__ uint32_t cell_of(const Geo& g, float x, float y, floa
   const uint32_t cy = cell_axis(y, g.origin[1], g.inv_h, g.dims[1]);
   const uint32_t cz = cell_axis(z, g.origin[2], g.inv_h, g.dims[2]);
   return (cz * g.dims[1] + cy) * g.dims[0] + cx;
+}
+
+// sub-cell of a point, numbered cell by cell (see sub_cells): the cell where sub = 0
+__device__ __forceinline__ uint32_t fine_of(const Geo& g, uint32_t sub, float x, float y, float z) {
+  const uint32_t c = cell_of(g, x, y, z);
+  if (sub == 0u) return c;
+  const float q = (float)(1u << sub), p[3] = {x, y, z};
+  uint32_t f = 0;
+#pragma unroll
+  for (int a = 2; a >= 0; --a) {
+    const float u = __fmul_rn(__fsub_rn(p[a], g.origin[a]), g.inv_h);
+    const int s = __float2int_rd((u - (float)cell_axis(p[a], g.origin[a], g.inv_h, g.dims[a])) * q);
+    f = (f << sub) | (uint32_t)min(max(s, 0), (int)(1u << sub) - 1);
+  }
+  return (c << (3 * sub)) | f;
 }
 
 __device__ __forceinline__ bool finite3(float x, float y, float z) {

@@ -41,9 +41,19 @@ namespace ps {
 
 constexpr int kMaxRuns = 49;  // (2 * stencil + 1)^2 for stencil <= 3
 
+// One-pass queries whose centrals are neighbour records: in dense clouds the RDF is left to the sweep
+// over unordered pairs (half the tests, no kNN beside them), in sparse ones the blocks of the
+// sweep are nearly empty and the query's own pass over each central is the better one.  The cloud's
+// density is known on the device only, where both kernels apply this rule.  Measured (query and sweep,
+// one box): 8e6-ion needle, Sc-Sc + Si-Si (1 to 2 records per cell) 0.165 ms in one pass, 0.348 ms with
+// the sweep; 1e5-ion cylinder, all-all (223 per cell, RDF and k = 1, 4, 10) 0.73 -> 0.37 ms; 2e4-ion cylinder
+// (68 per cell) 0.140 -> 0.106 ms.
+__device__ __forceinline__ bool sweep_pays(const Geo& g) { return (uint64_t)g.n_sel >= 8ull * g.n_cells; }
+
 struct QueryArgs {
   const float4* nrec;
   const uint32_t* nstart;
+  const uint32_t* nsub;  // sub-cell starts (where the cells have sub-cells)
   const Geo* ngeo;
   const float4* crec;
   const uint32_t* cstart;
@@ -72,7 +82,12 @@ struct QueryArgs {
   int fallback;           // 1: only the centrals marked in need[] (the full-radius kNN pass)
   uint32_t* next_front;   // work counters of the front (heavy) and back (light) items
   uint32_t* next_light;
-  int vertex;             // near kNN pass on the vertex-centred central list (see vertex_run)
+  // whether a central is among its own candidates: every one (self_all), or by its type
+  int self_all;
+  const uint8_t* type;
+  Mask nbr;
+  float one;  // 1.0f, opaque to the compiler (see dist2_x2_fma)
+  int sweep;  // 1: the RDF of a dense cloud is left to k_rdf_sym (see sweep_pays)
   // bin lookup table (lut_shift = 0: none): cell c covers the float32 bit patterns
   // [(lut_base + c) << lut_shift, (lut_base + c + 1) << lut_shift), at most one interior edge each
   uint32_t lut_shift, lut_base, lut_n;
@@ -114,6 +129,29 @@ __device__ __forceinline__ uint32_t bin_index(float d2, const float* sE, uint32_
   return (uint32_t)b;
 }
 
+// Insertion queue of a lane: a column of a [row][32 lanes] array, `at` the shared address of its next
+// slot.  Every value is stored and the slot taken only if it is below thr: no branch, and one
+// predicated add per value.
+__device__ __forceinline__ void queue_push(uint32_t& at, float v, float thr) {
+  asm volatile(
+      "{\n .reg .pred p;\n st.shared.f32 [%0], %1;\n setp.lt.f32 p, %1, %2;\n @p add.u32 %0, %0, 128;\n}"
+      : "+r"(at)
+      : "f"(v), "f"(thr));
+}
+// the same for a candidate of index word j, other than the lane's central (index word own)
+__device__ __forceinline__ void queue_push_other(uint32_t& at, float v, float thr, uint32_t j, uint32_t own) {
+  asm volatile(
+      "{\n .reg .pred p;\n st.shared.f32 [%0], %1;\n setp.ne.u32 p, %3, %4;\n setp.lt.and.f32 p, %1, %2, p;\n"
+      " @p add.u32 %0, %0, 128;\n}"
+      : "+r"(at)
+      : "f"(v), "f"(thr), "r"(j), "r"(own));
+}
+__device__ __forceinline__ float queue_at(uint32_t first, uint32_t q) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(first + 128u * q));
+  return v;
+}
+
 struct SmemLayout {
   uint32_t off_E, off_lut, off_rdf, off_knn, off_kmeta, off_stage, total;
   bool priv;
@@ -134,7 +172,8 @@ __host__ __device__ inline SmemLayout smem_layout(uint32_t n_bins, uint32_t n_k,
   o += rdf ? lut_n * 4 : 0;
   o = (o + 7u) & ~7u;
   L.off_rdf = o;
-  o += rdf ? (L.priv ? 8 * n_bins * 4 : n_bins * 8) : 0;
+  o += rdf ? (L.priv ? 8 * (n_bins + 1) * 4 : n_bins * 8) : 0;  // (bin n_bins: see FastBins)
+  o = (o + 7u) & ~7u;
   L.off_knn = o;
   o += n_k * n_bins * 4;
   L.off_kmeta = o;
@@ -151,7 +190,9 @@ template <bool RDF>
 struct Hist {
   float* sE;
   unsigned long long* s_rdf;  // CTA row, 64-bit: per-CTA pair counts can pass 2^32 on large clouds
-  uint32_t* s_rdfw;           // or one 32-bit row per warp (priv), flushed by its warp before it could wrap
+  // or one 32-bit row per warp (priv), flushed by its warp before it could pass 2^31; bin 0 may stand
+  // below zero between a flush and the removal of the centrals that met themselves
+  uint32_t* s_rdfw;
   bool priv;
   uint32_t* s_knn;            // per-CTA central counts stay below n < 2^32
   uint32_t* s_kmeta;
@@ -169,7 +210,7 @@ struct Hist {
     lut_mask = (1u << lut_shift) - 1u;
     priv = L.priv;
     s_rdf = reinterpret_cast<unsigned long long*>(smem + L.off_rdf);
-    s_rdfw = reinterpret_cast<uint32_t*>(smem + L.off_rdf) + (threadIdx.x >> 5) * a.n_bins;
+    s_rdfw = reinterpret_cast<uint32_t*>(smem + L.off_rdf) + (threadIdx.x >> 5) * (a.n_bins + 1);
     s_knn = reinterpret_cast<uint32_t*>(smem + L.off_knn);
     s_kmeta = reinterpret_cast<uint32_t*>(smem + L.off_kmeta);
     nb = a.n_bins;
@@ -180,7 +221,7 @@ struct Hist {
     }
     if (RDF) {
       if (priv)
-        for (uint32_t b = threadIdx.x; b < 8 * nb; b += blockDim.x) reinterpret_cast<uint32_t*>(s_rdf)[b] = 0;
+        for (uint32_t b = threadIdx.x; b < 8 * (nb + 1); b += blockDim.x) reinterpret_cast<uint32_t*>(s_rdf)[b] = 0;
       else
         for (uint32_t b = threadIdx.x; b < nb; b += blockDim.x) s_rdf[b] = 0ull;
     }
@@ -282,8 +323,9 @@ struct Hist {
     unsigned long long tot = 0;
     for (uint32_t b = threadIdx.x & 31; b < nb; b += 32)
       if (s_rdfw[b]) {
-        tot += s_rdfw[b];
-        atomicAdd((unsigned long long*)&a.rdf[b], (unsigned long long)s_rdfw[b]);
+        const unsigned long long v = (unsigned long long)(long long)(int32_t)s_rdfw[b];
+        tot += v;
+        atomicAdd((unsigned long long*)&a.rdf[b], v);
         s_rdfw[b] = 0;
       }
 #pragma unroll
@@ -302,7 +344,7 @@ struct Hist {
       const uint32_t nw = blockDim.x >> 5;
       for (uint32_t b = threadIdx.x; b < nb; b += blockDim.x) {
         unsigned long long sum = 0;
-        for (uint32_t w = 0; w < nw; ++w) sum += rows[w * nb + b], rows[w * nb + b] = 0;
+        for (uint32_t w = 0; w < nw; ++w) sum += (unsigned long long)(long long)(int32_t)rows[w * (nb + 1) + b], rows[w * (nb + 1) + b] = 0;
         if (sum) atomicAdd((unsigned long long*)&a.rdf[b], sum);
         tot += sum;
       }
@@ -389,6 +431,50 @@ __device__ __forceinline__ void cell_run(const QueryArgs& a, const Geo& ng, uint
   row_run(a, ng, cx, (int)cy + dy, (int)cz + dz, row_width(a, dy, dz), src, len);
 }
 
+// Run r of the candidates of an item whose box, in cell edges, is ulo .. uhi.  Cells without sub-cells:
+// the own cell, the own row to its left and to its right, then rows 1 .. of the stencil (nearest
+// first).  With them (27-cell stencils), the x-rods of 2^sub sub-cells, cell by cell from the own row
+// outwards, those out of reach left empty: a 2 nm cell's 27 cells hold 216 octants, an octant's
+// items reach 105 of them within 2 nm and about 27 within a 10th-neighbour distance.
+__device__ __forceinline__ uint32_t item_runs(const QueryArgs& a, const Geo& ng) {
+  const uint32_t W = 2 * a.stencil + 1;
+  return ng.sub ? W * W * W << (2 * ng.sub) : W * W + 2;
+}
+__device__ __forceinline__ void item_run(const QueryArgs& a, const Geo& ng, uint32_t c, uint32_t r, const float (&ulo)[3],
+                                         const float (&uhi)[3], float lim_u, uint32_t& src, uint32_t& len) {
+  src = 0, len = 0;
+  if (r >= item_runs(a, ng)) return;
+  if (ng.sub) {
+    const uint32_t W = 2 * a.stencil + 1, cell = r >> (2 * ng.sub), yz = r & ((1u << (2 * ng.sub)) - 1u);
+    const int row = (int)(cell / W), q = (int)(cell - row * W), dx = q & 1 ? -((q + 1) >> 1) : q >> 1;  // 0 -1 1 -2 2 ..
+    const int x = (int)(c % ng.dims[0]) + dx, y = (int)((c / ng.dims[0]) % ng.dims[1]) + c_row_dy[row],
+              z = (int)(c / (ng.dims[0] * ng.dims[1])) + c_row_dz[row];
+    if (x < 0 || y < 0 || z < 0 || x >= (int)ng.dims[0] || y >= (int)ng.dims[1] || z >= (int)ng.dims[2]) return;
+    const float e = 1.0f / (float)(1u << ng.sub);
+    const float y0 = (float)y + e * (float)(yz & ((1u << ng.sub) - 1u)), z0 = (float)z + e * (float)(yz >> ng.sub);
+    const float gx = fmaxf(0.f, fmaxf((float)x - uhi[0], ulo[0] - (float)(x + 1)));
+    const float gy = fmaxf(0.f, fmaxf(y0 - uhi[1], ulo[1] - (y0 + e)));
+    const float gz = fmaxf(0.f, fmaxf(z0 - uhi[2], ulo[2] - (z0 + e)));
+    if (gx * gx + gy * gy + gz * gz > lim_u) return;  // (a NaN box keeps the rod)
+    const uint32_t cc = ((uint32_t)z * ng.dims[1] + (uint32_t)y) * ng.dims[0] + (uint32_t)x;
+    const uint32_t f = (cc << (3 * ng.sub)) | (yz << ng.sub), f1 = f + (1u << ng.sub);
+    src = a.nsub[f];
+    len = (f1 == ng.n_cells << (3 * ng.sub) ? ng.n_sel : a.nsub[f1]) - src;
+    return;
+  }
+  if (r >= 3) {
+    cell_run(a, ng, c, r - 2, src, len);
+    return;
+  }
+  const uint32_t row = c - c % ng.dims[0], cx = c - row, w = (uint32_t)row_width(a, 0, 0);
+  const uint32_t lo = r == 0 ? cx : (r == 1 ? (cx >= w ? cx - w : 0u) : cx + 1);
+  const uint32_t hi = r == 0 ? cx + 1 : (r == 1 ? cx : min(cx + w, ng.dims[0] - 1) + 1);
+  if (lo < hi) {
+    src = a.nstart[row + lo];
+    len = a.nstart[row + hi] - src;
+  }
+}
+
 // Near kNN pass of the query in passes (vertex != 0): the central list is sorted by the grid
 // of cells centred on the vertices of the neighbour grid (vg: origin half a cell lower, one more
 // cell per axis), so the centrals of item cell c are those nearest to vertex V = c's coordinates,
@@ -444,50 +530,121 @@ __device__ __forceinline__ void list_append(const QueryArgs& a, bool miss, uint3
 __device__ __forceinline__ float4 far_record() { return make_float4(INFINITY, INFINITY, INFINITY, __uint_as_float(~0u)); }
 
 // ---------------------------------------------------------------------------
+// direct bins (r0 = 0)
+// ---------------------------------------------------------------------------
+constexpr float kBinBias = 1.0f / 2097152.0f;   // 2^-21
+
+__device__ __forceinline__ void red_shared_inc(uint32_t addr) {
+  asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr));
+}
+__device__ __forceinline__ void red_shared(uint32_t addr, uint32_t v) {
+  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v));
+}
+
+// Bins of the direct form (r0 = 0).  With s = sqrt.approx(d2) and inv = (1 +- 2^-21) / dr, the true
+// quotient sqrt(d2) / dr lies between s * inv- and s * inv+ (the root is good to 2^-23, inv to 2^-24,
+// the edge table to 2^-25 of the distance).  The bin is floor(s * inv+), or the one below where the two floors
+// differ (2 in 10^4 pairs at 200 bins): those compare d2 with that edge.  Pairs out of range are
+// clamped into the unused bin n_bins, so that every lane increments and no instruction is
+// predicated: the compiler branches around a predicated shared-memory increment.  Measured on the
+// pair loop alone (cycles per 32 tests and scheduler): 23 with a predicated increment and the excess over
+// the edge computed, 17 in this form, of which 14.5 are the distance, root and floor; no table load per pair, so
+// the shared-memory pipe is left to the increments (increments by one merge in a bin).
+struct FastBins {
+  const float* sE;
+  unsigned long long hi2, lo2, magic2;
+  float s_far;
+  __device__ void init(const QueryArgs& a, const float* edges) {
+    sE = edges;
+    const float hi = (float)((1.0 + (double)kBinBias) / a.dr), lo = (float)((1.0 - (double)kBinBias) / a.dr);
+    hi2 = f2_pack(hi, hi);
+    lo2 = f2_pack(lo, lo);
+    magic2 = f2_pack(kMagic, kMagic);
+    s_far = (float)(((double)a.n_bins + 0.5) * a.dr);
+  }
+  // counts two pairs in the row at shared address `base` (bin b at base + 4 (kMagicBits + b));
+  // returns 0 unless one of them may lie under the edge of its bin
+  __device__ __forceinline__ uint32_t count2(unsigned long long d2, uint32_t base) const {
+    float da, db, ma, mb, la, lb;
+    f2_unpack(d2, da, db);
+    const unsigned long long s2 = f2_pack(fminf(sqrt_fast(da), s_far), fminf(sqrt_fast(db), s_far));
+    f2_unpack(f2_fma_down(s2, hi2, magic2), ma, mb);
+    f2_unpack(f2_fma_down(s2, lo2, magic2), la, lb);
+    red_shared_inc(__float_as_uint(ma) * 4u + base);
+    red_shared_inc(__float_as_uint(mb) * 4u + base);
+    return (__float_as_uint(ma) ^ __float_as_uint(la)) | (__float_as_uint(mb) ^ __float_as_uint(lb));
+  }
+  // a counted pair that may lie under the edge of its bin: moved to the bin below if it does
+  __device__ __forceinline__ void settle(float d2, uint32_t base) const {
+    float m, x;
+    f2_unpack(f2_fma_down(f2_pack(fminf(sqrt_fast(d2), s_far), 0.f), hi2, magic2), m, x);
+    const uint32_t addr = __float_as_uint(m) * 4u + base;
+    if (d2 < sE[__float_as_uint(m) - kMagicBits]) {
+      red_shared(addr, ~0u);
+      red_shared_inc(addr - 4u);
+    }
+  }
+  __device__ __forceinline__ void settle2(unsigned long long d2, uint32_t base) const {
+    float da, db;
+    f2_unpack(d2, da, db);
+    settle(da, base);
+    settle(db, base);
+  }
+};
+
+// ---------------------------------------------------------------------------
 // warp kernel
-//   heavy items (cells with >= kHeavy centrals, batches of 4..32 centrals): one
-//     to eight lanes per central (item_lanes), the candidates staged 32 at a
-//     time in the warp's shared buffer and tested two at a time with packed
-//     float32 math;
+//   heavy items (cells with >= kHeavy centrals, batches of 4..32 centrals): one to eight lanes per
+//     central (item_lanes).  The candidates are read 32 at a time, the stencil's rows nearest
+//     first, and kept only within range of the bounding box of the item's centrals (the
+//     histogram's range, or for kNN alone the largest k-th distance so far); the kept ones are
+//     compacted into a ring of 64 in shared memory as interleaved pairs and tested 32 at a time, two
+//     per packed test.  Candidates further from the box than every current k-th distance skip
+//     the kNN part of the test.
 //   light items (cells with < kHeavy centrals): the warp takes 32 items at a
 //     time and gives each of their centrals a thread of its own that walks its
 //     own stencil (the records of neighbouring centrals' cells hit in L1).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kHalf = 16;                 // candidates per staging half-batch
 constexpr uint32_t kRowLaneCap = 1u << 25;     // per-central increments of the 32-bit warp row, then global
+constexpr uint32_t kRing = 128;                // candidates kept for testing (a batch of 64 and 32 more)
+constexpr int kNoRdf = 0, kRdfGeneral = 1, kRdfDirect = 2;
 
-// VX: the near kNN pass on the vertex-centred central list (a.vertex; kNN only), compiled apart
-// so that the other forms carry none of its code
-template <int KMAX, bool RDF, bool VX = false>
-__global__ void __launch_bounds__(256) k_query_warp(const QueryArgs a) {
+// Bound by instruction issue, and on small or clustered clouds by the chain of one item.  Where the
+// RDF is left to the sweep (a.sweep, dense clouds) only the kNN is done here: k = 10, 1e5-ion
+// cylinder, 2 nm cells, 0.325 ms walking every record of the 27 cells, 0.163 ms with the sub-cells out of
+// reach left out.
+template <int KMAX, int MODE>
+__global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __grid_constant__ QueryArgs a) {
+  constexpr bool RDF = MODE != kNoRdf;
   griddep_wait();
   griddep_launch();
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ float4 s_buf[8][32];
-  __shared__ float s_hits[8][32 * kHalf + 32];  // per warp: the in-range hits of one half-batch + a trash row
+  __shared__ float4 s_buf[8][kRing];            // per warp: ring of kept candidates, as interleaved pairs
   __shared__ float s_kq[8][32 * kHalf + 32];    // per warp: kNN insertion queue, [slot][lane] + a spare row
-  __shared__ uint32_t s_rsrc[8][kMaxRuns], s_rpre[8][kMaxRuns + 1];
   constexpr int KK = KMAX > 0 ? KMAX : 1;
-  Hist<RDF> H;
+  if (KMAX == 0 && a.sweep && sweep_pays(*a.ngeo)) return;  // nothing is left to do here
+  Hist<RDF> H{};
   H.init(a, smem, 0, true);
+  FastBins fb;
+  if (MODE == kRdfDirect) fb.init(a, H.sE);
+  const uint32_t row_base = smem_u32(H.s_rdfw) - 4u * kMagicBits;
+  const unsigned long long one2 = f2_pack(a.one, a.one);
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint64_t wcount = 0;  // increments of this warp's private row since its last flush (uniform)
   const Geo ng = *a.ngeo;
   const uint32_t n_hi = a.cgeo->work_n4, n_front = n_hi + a.cgeo->work_n2, n_light = a.cgeo->work_n3;
-  const int n_runs = VX ? 4 : (2 * a.stencil + 1) * (2 * a.stencil + 1);
+  const int n_runs = (int)item_runs(a, ng);
+  const float u_slack = (float)max(ng.dims[0], max(ng.dims[1], ng.dims[2])) * 5.0e-7f + 1.0e-6f;  // rounding of (x - origin) inv_h
+  const bool swept = a.sweep && sweep_pays(ng);  // RDF and in-range counts are the sweep's
+  const bool rdf_here = RDF && !swept;
+  uint32_t* const nwithin = swept ? nullptr : a.nwithin;
   const float erange = a.emax_near > 0.f ? a.emax_near : H.Emax;  // squared search range of this pass
-  // vertex mode: the item cells are those of the vertex-centred grid (a.cgeo); rounding slack of
-  // a cell coordinate (cells) and the cell edge for vertex_reach
-  const Geo vg = *a.cgeo;
-  const float v_slack = (float)max(ng.dims[0], max(ng.dims[1], ng.dims[2])) * 5.0e-7f + 1.0e-6f;
-  const float v_heff = __fmul_rn(__fdiv_rn(1.0f, ng.inv_h), 1.0f - 1.0f / 4096.0f);
   uint64_t my_binned = 0;  // pairs counted straight into the global histogram
   uint32_t my_below = 0;   // pairs below E[0]
-  float4* buf = s_buf[w];
-  float* wlist = s_hits[w];
+  float* bf = reinterpret_cast<float*>(s_buf[w]);
   float* kq = s_kq[w];
-  uint32_t* rsrc = s_rsrc[w];
-  uint32_t* rpre = s_rpre[w];
+  const uint32_t q0 = smem_u32(kq + lane);
 
   // ---- items from the front: dense cells, the very heavy ones first ----
   for (;;) {
@@ -498,230 +655,239 @@ __global__ void __launch_bounds__(256) k_query_warp(const QueryArgs a) {
     const uint2 it = item < n_hi ? a.whi[item] : a.witem[item - n_hi];
     const uint32_t c = it.x, first = it.y >> 6, cnt = it.y & 63u;
     const uint32_t c0 = a.cstart[c] + first;
-    // run table: sources and prefix counts of the candidate runs
-    const uint32_t n_cand = run_table(lane, n_runs, rsrc, rpre, [&](uint32_t r, uint32_t& src, uint32_t& len) {
-      if (VX)
-        vertex_run(a, ng, vg, c, r, src, len);
-      else
-        cell_run(a, ng, c, r, src, len);
-    });
-
-    // record at virtual candidate position pos (runs concatenated); rr is a run hint, nondecreasing in pos
-    auto fetch = [&](uint32_t pos, int& rr) -> float4 {
-      if (pos >= n_cand) return far_record();
-      while (pos >= rpre[rr + 1]) ++rr;
-      return __ldg(a.nrec + rsrc[rr] + (pos - rpre[rr]));
-    };
-
-    if (cnt > 3) {
-      // 32 candidates per coalesced load, staged as 16 interleaved pairs (xa xb ya yb za zb wa wb)
-      // and tested two at a time.  In-range hits go to a warp-wide list (ballot + popc give each
-      // hit its slot) binned by all 32 lanes together; kNN candidates below the lane's current
-      // k-th distance go to the lane's column of the insertion queue, drained after each half-batch
-      // (the sorted insertion then runs with most lanes active instead of once per candidate
-      // whenever any lane needs it).
-      // L lanes per central (items of dense clusters, a cell's partial last item): lane sub of a
-      // central tests the pairs t = sub mod L
-      const uint32_t L = item_lanes(cnt);
-      const uint32_t lg = L == 8u ? 3u : (L == 4u ? 2u : (L == 2u ? 1u : 0u));
-      const uint32_t sub = lane & (L - 1u), ci = lane >> lg;
-      const uint32_t n_it = 8u >> lg;  // pair tests per lane per half-batch
-      bool valid = ci < cnt;
-      if (a.fallback && valid) valid = a.need[c0 + ci] != 0u;
-      if (a.fallback && __ballot_sync(0xffffffffu, valid) == 0u) continue;  // no central of this item to redo
-      float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (valid) p = a.crec[c0 + ci];
-      const uint32_t pidx = valid ? __float_as_uint(p.w) : ~0u;
-      // lanes without a central never hit; vertex mode: each central's own reach
-      const float emax = valid ? (VX ? vertex_reach(ng, vg, c, p, v_slack, v_heff, H.Emax) : erange) : -INFINITY;
-      const unsigned long long px = f2_pack(p.x, p.x), py = f2_pack(p.y, p.y), pz = f2_pack(p.z, p.z);
-      const uint32_t lt = (1u << lane) - 1u;
-      float top[KK];
+    // L lanes per central (items of dense clusters, small clouds, a cell's partial last item): lane
+    // sub of a central tests the pairs t = sub mod L
+    const uint32_t L = item_lanes(cnt);
+    const uint32_t lg = 31u - __clz(L);
+    const uint32_t sub = lane & (L - 1u), ci = lane >> lg;
+    bool valid = ci < cnt;
+    if (a.fallback && valid) valid = a.need[c0 + ci] != 0u;
+    if (a.fallback && __ballot_sync(0xffffffffu, valid) == 0u) continue;  // no central of this item to redo
+    // lanes without a central never hit (their distances are infinite or NaN)
+    float4 p = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+    if (valid) p = a.crec[c0 + ci];
+    const uint32_t pidx = valid ? __float_as_uint(p.w) : ~0u;
+    const float emax = erange;
+    const unsigned long long px = f2_pack(p.x, p.x), py = f2_pack(p.y, p.y), pz = f2_pack(p.z, p.z);
+    // bounding box of the centrals as mid +- half (half rounded up)
+    float mid[3], half[3], ulo[3], uhi[3];
+    {
+      const float pc[3] = {p.x, p.y, p.z};
 #pragma unroll
-      for (int t = 0; t < KK; ++t) top[t] = INFINITY;
-      uint32_t within = 0;
-      int rr = 0;
-      float4 nxt = fetch(lane, rr);
-      float* bf = reinterpret_cast<float*>(buf);
-      for (uint32_t b = 0; b < n_cand; b += 32) {
-        __syncwarp();
-        {
-          float* d = bf + (lane >> 1) * 8 + (lane & 1);
-          d[0] = nxt.x, d[2] = nxt.y, d[4] = nxt.z, d[6] = nxt.w;
+      for (int ax = 0; ax < 3; ++ax) {
+        const float lo = key2f(__reduce_min_sync(0xffffffffu, f2key(valid ? pc[ax] : INFINITY)));
+        const float hi = key2f(__reduce_max_sync(0xffffffffu, f2key(valid ? pc[ax] : -INFINITY)));
+        mid[ax] = 0.5f * (lo + hi);
+        half[ax] = fmaxf(hi - mid[ax], mid[ax] - lo) * 1.000001f + fabsf(mid[ax]) * 2.4e-7f;
+        ulo[ax] = (lo - ng.origin[ax]) * ng.inv_h - u_slack, uhi[ax] = (hi - ng.origin[ax]) * ng.inv_h + u_slack;
+      }
+    }
+    float top[KK];
+#pragma unroll
+    for (int t = 0; t < KK; ++t) top[t] = INFINITY;
+    uint32_t within = 0;
+    // bound of the kNN insertions: the range and the k-th distance of the lane's central
+    float thr = KMAX > 0 ? emax : -INFINITY;
+    float near_max = fmaxf(thr, 0.f);  // the largest over the warp
+    const bool all = rdf_here || nwithin != nullptr;  // every in-range pair counts, not the nearest alone
+    // ring of kept candidates: slots [head, tail); those from near_to on are beyond near_max.  Items
+    // whose lanes share centrals take 64 at a time, so that each lane has enough of them.
+    const uint32_t nb = L > 1u ? 64u : 32u;
+    uint32_t head = 0, tail = 0, near_to = 0;
+
+    // tests the nb ring slots from `head`, of which n hold candidates
+    auto batch = [&](uint32_t n) __attribute__((always_inline)) {
+      const ulonglong2* ring = reinterpret_cast<const ulonglong2*>(bf) + (head & (kRing - 1u));
+      const uint32_t n_pr = (n + 1) >> 1;
+      if (all) {
+        // two pairs of candidates at a time (beyond the last there are far ones to the end of the batch)
+#pragma unroll 1
+        for (uint32_t t0 = 0; t0 < n_pr; t0 += 2 * L) {
+          const uint32_t t = t0 + sub;
+          const ulonglong2 xy0 = ring[2 * t], xy1 = ring[2 * (t + L)];
+          const unsigned long long z0 = ring[2 * t + 1].x, z1 = ring[2 * (t + L) + 1].x;
+          const unsigned long long d20 = dist2_x2_fma(px, py, pz, xy0.x, xy0.y, z0, one2);
+          const unsigned long long d21 = dist2_x2_fma(px, py, pz, xy1.x, xy1.y, z1, one2);
+          float d[4];
+          f2_unpack(d20, d[0], d[1]);
+          f2_unpack(d21, d[2], d[3]);
+          if (MODE == kRdfDirect && rdf_here) {
+            const uint32_t x = fb.count2(d20, row_base) | fb.count2(d21, row_base);
+            if (__any_sync(0xffffffffu, x != 0u)) {
+              fb.settle2(d20, row_base);
+              fb.settle2(d21, row_base);
+            }
+          }
+          if (MODE == kRdfGeneral && rdf_here) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (d[e] < emax && __float_as_uint(bf[4 * (head & (kRing - 1u)) + (t + (e >> 1) * L) * 8 + 6 + (e & 1)]) != pidx)
+                H.pair(a, d[e], my_below);
+          }
+          if (nwithin != nullptr)
+            within += (uint32_t)(d[0] < emax) + (uint32_t)(d[1] < emax) + (uint32_t)(d[2] < emax) + (uint32_t)(d[3] < emax);
         }
         __syncwarp();
-        nxt = fetch(b + 32 + lane, rr);
+      }
+      if (KMAX > 0 && (int32_t)(near_to - head) > 0) {
+        // candidates below the lane's bound go to its queue column (unconditional stores at the next
+        // slot, kept only if counted), inserted every 16 pairs of the lanes
 #pragma unroll 1
-        for (int half = 0; half < 2; ++half) {
-          uint32_t nh = 0;  // hits in the warp list (uniform)
-          uint32_t qn = 0;  // entries in this lane's queue column
-          const float thr = top[KK - 1];
-          // vertex mode: no in-range count, one bound for the queue (the reach and the k-th distance)
-          const float thr_e = fminf(thr, emax);
+        for (uint32_t t0 = 0; t0 < n_pr; t0 += 8 * L) {
+          uint32_t qa = q0;
+          const uint32_t t1 = min(n_pr, t0 + 8 * L);
 #pragma unroll 2
-          for (uint32_t u = 0; u < n_it; ++u) {
-            const uint32_t t = 8 * half + u * L + sub;
-            const ulonglong2 xy = reinterpret_cast<const ulonglong2*>(bf)[2 * t];
-            const ulonglong2 zw = reinterpret_cast<const ulonglong2*>(bf)[2 * t + 1];
-            float d2a, d2b;
-            dist2_x2(px, py, pz, xy.x, xy.y, zw.x, d2a, d2b);
-            float wa, wb;
+          for (uint32_t t = t0 + sub; t < t1; t += L) {
+            const ulonglong2 xy = ring[2 * t], zw = ring[2 * t + 1];
+            float da, db, wa, wb;
+            f2_unpack(dist2_x2_fma(px, py, pz, xy.x, xy.y, zw.x, one2), da, db);
             f2_unpack(zw.y, wa, wb);
-            if constexpr (VX) {
-              const bool qa = d2a < thr_e && __float_as_uint(wa) != pidx;
-              const bool qb = d2b < thr_e && __float_as_uint(wb) != pidx;
-              kq[qn * 32 + lane] = d2a;
-              qn += (uint32_t)qa;
-              kq[qn * 32 + lane] = d2b;
-              qn += (uint32_t)qb;
-              continue;
-            }
-            const bool ha = d2a < emax && __float_as_uint(wa) != pidx;
-            const bool hb = d2b < emax && __float_as_uint(wb) != pidx;
-            within += (uint32_t)ha + (uint32_t)hb;
-            if (KMAX > 0) {
-              // unconditional stores at the queue's next slot (row qn <= 16 of 17), kept only if counted
-              const bool qa = ha && d2a < thr, qb = hb && d2b < thr;
-              kq[qn * 32 + lane] = d2a;
-              qn += (uint32_t)qa;
-              kq[qn * 32 + lane] = d2b;
-              qn += (uint32_t)qb;
-            }
-            if (RDF) {
-              // every lane stores (no branch): a hit at its compacted slot, a miss in the trash row
-              const uint32_t ba = __ballot_sync(0xffffffffu, ha);
-              wlist[ha ? nh + __popc(ba & lt) : 32 * kHalf + lane] = d2a;
-              nh += __popc(ba);
-              const uint32_t bb = __ballot_sync(0xffffffffu, hb);
-              wlist[hb ? nh + __popc(bb & lt) : 32 * kHalf + lane] = d2b;
-              nh += __popc(bb);
-            }
+            queue_push_other(qa, da, thr, __float_as_uint(wa), pidx);
+            queue_push_other(qa, db, thr, __float_as_uint(wb), pidx);
           }
-          if (KMAX > 0) {
-            const uint32_t m = __reduce_max_sync(0xffffffffu, qn);
-            for (uint32_t q = 0; q < m; ++q)
-              if (q < qn) topk_insert(top, kq[q * 32 + lane]);
-          }
-          if (RDF) {
-            __syncwarp();
-            for (uint32_t h = lane; h < nh; h += 32) H.pair(a, wlist[h], my_below);
-            __syncwarp();
-            wcount += nh;
-            if (wcount >= (1ull << 31)) {
-              H.flush_warp(a);
-              wcount = 0;
-            }
-          }
-        }
-      }
-      // merge the partial lists of the L lanes of each central (disjoint candidate subsets); the
-      // partner's sorted list is read from the warp's queue buffer in a rolled loop, which keeps
-      // the kernel's code small (its speed depends on the instruction cache)
-      for (uint32_t o = 1; o < L; o <<= 1) {
-        within += __shfl_xor_sync(0xffffffffu, within, o);
-        if constexpr (KMAX > 0 && KK * 32 <= 32 * kHalf) {
           __syncwarp();
-#pragma unroll
-          for (int t = 0; t < KK; ++t) kq[t * 32 + lane] = top[t];
-          __syncwarp();
-          const float* ot = kq + (lane ^ o);
-#pragma unroll 1
-          for (int t = 0; t < KK; ++t) {
-            const float v = ot[t * 32];
-            if (!(v < top[KK - 1])) break;  // the partner's list is sorted
-            topk_insert(top, v);
-          }
-        } else if constexpr (KMAX > 0) {
-          float other[KK];
-#pragma unroll
-          for (int t = 0; t < KK; ++t) other[t] = __shfl_xor_sync(0xffffffffu, top[t], o);
-#pragma unroll
-          for (int t = 0; t < KK; ++t) {
-            if (!(other[t] < top[KK - 1])) break;  // the partner's list is sorted
-            topk_insert(top, other[t]);
-          }
+          const uint32_t qn = (qa - q0) >> 7, m = __reduce_max_sync(0xffffffffu, qn);
+          for (uint32_t q = 0; q < m; ++q)
+            if (q < qn) topk_insert(top, queue_at(q0, q));
+          float kth = top[KK - 1];  // an upper bound of the central's k-th distance in each of its lanes
+          for (uint32_t o = 1; o < L; o <<= 1) kth = fminf(kth, __shfl_xor_sync(0xffffffffu, kth, o));
+          thr = fminf(kth, emax);
         }
+        near_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(valid ? thr : 0.f)));
       }
-      bool miss = false;
-      if (valid && sub == 0) {
-        if (a.nwithin) a.nwithin[pidx] = within;
-        if (KMAX > 0) {
-          const float kd = topk_get(top, a.k_need - 1);
-          const bool found = VX ? kd < emax : (!(a.emax_near > 0.f) || kd < a.emax_near);
-          if (VX)
-            miss = !found;
-          else if (a.emax_near > 0.f)
-            a.need[c0 + ci] = found ? 0u : 1u;
-          if (found)
-            for (uint32_t q = 0; q < a.n_k; ++q) H.kth(a, q, topk_get(top, a.ks[q] - 1), pidx);
-        }
-      }
-      if (VX) list_append(a, miss, c0 + ci, lane);
-    } else {
-      // few centrals, many candidates: the lanes split the candidates of each central and
-      // merge their sorted lists by shuffles
-      for (uint32_t ci = 0; ci < cnt; ++ci) {
-        if (a.fallback && a.need[c0 + ci] == 0u) continue;  // warp-uniform
-        const float4 p = a.crec[c0 + ci];
-        const uint32_t pidx = __float_as_uint(p.w);
-        const float er = VX ? vertex_reach(ng, vg, c, p, v_slack, v_heff, H.Emax) : erange;
-        float top[KK];
-#pragma unroll
-        for (int t = 0; t < KK; ++t) top[t] = INFINITY;
-        uint32_t within = 0;
-        int rr = 0;
-        for (uint32_t b = 0; b < n_cand; b += 32) {
-          const float4 q = fetch(b + lane, rr);
-          const float d2 = dist2(p.x, p.y, p.z, q.x, q.y, q.z);
-          if (d2 < er && __float_as_uint(q.w) != pidx) {
-            ++within;
-            H.pair(a, d2, my_below);
-            if (KMAX > 0) topk_insert(top, d2);
-          }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) within += __shfl_xor_sync(0xffffffffu, within, o);
-        if (lane == 0 && a.nwithin) a.nwithin[pidx] = within;
-        wcount += within;
-        if (wcount >= (1ull << 31)) {
+      if (RDF && H.priv) {
+        wcount += 32u * 64u;
+        if (wcount >= (1ull << 30)) {
           H.flush_warp(a);
           wcount = 0;
         }
-        if (KMAX > 0) {
-          // merge the 32 sorted lane lists: pop the warp minimum k_need times (ranks kept in kq)
-          float m = INFINITY;
-          for (uint32_t rank = 0; rank < a.k_need; ++rank) {
-            m = top[0];
+      }
+    };
+
+    for (int r0 = 0; r0 < n_runs; r0 += 32) {
+      // lane r: run r0 + r
+      uint32_t rs = 0, rl = 0;
+      item_run(a, ng, c, (uint32_t)r0 + lane, ulo, uhi, (all ? emax : near_max) * 1.0001f * ng.inv_h * ng.inv_h, rs, rl);
+      // the runs as one list: lane r holds the position at which run r starts and, less that, its first
+      // record; a position's run is found by bisection over the lanes (runs of sparse sets hold a few
+      // records each, and a round of 32 loads per run would be mostly idle)
+      uint32_t pre = rl;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            const uint32_t bal = __ballot_sync(0xffffffffu, top[0] == m);
-            if (lane == (uint32_t)(__ffs(bal) - 1)) {
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, pre, o);
+        if (lane >= (uint32_t)o) pre += y;
+      }
+      const uint32_t n_list = __shfl_sync(0xffffffffu, pre, 31);
+      pre -= rl;
+      const uint32_t first = rs - pre;
+      auto fetch = [&](uint32_t pos) -> float4 {
+        uint32_t r = 0;
 #pragma unroll
-              for (int t = 0; t < KK - 1; ++t) top[t] = top[t + 1];
-              top[KK - 1] = INFINITY;
-            }
-            if (lane == 0) kq[rank] = m;
-          }
+        for (uint32_t st = 16; st > 0; st >>= 1)
+          if (__shfl_sync(0xffffffffu, pre, r + st) <= pos) r += st;
+        const uint32_t j = __shfl_sync(0xffffffffu, first, r) + pos;
+        return pos < n_list ? __ldg(a.nrec + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+      };
+      // one candidate per lane: into the ring if it is within reach
+      auto offer = [&](const float4& q, bool ok) {
+        const float ex = fmaxf(fabsf(q.x - mid[0]) - half[0], 0.f);
+        const float ey = fmaxf(fabsf(q.y - mid[1]) - half[1], 0.f);
+        const float ez = fmaxf(fabsf(q.z - mid[2]) - half[2], 0.f);
+        // (the factor covers the rounding of both distances)
+        const float e2 = __fmaf_rn(ez, ez, __fmaf_rn(ey, ey, ex * ex)) * 0.99999f;
+        const bool close = ok && e2 < near_max;
+        const bool keep = all ? ok && e2 < emax : close;
+        const uint32_t bal = __ballot_sync(0xffffffffu, keep);
+        if (keep) {
+          const uint32_t slot = (tail + __popc(bal & ((1u << lane) - 1u))) & (kRing - 1u);
+          float* d = bf + (slot >> 1) * 8 + (slot & 1u);
+          d[0] = q.x, d[2] = q.y, d[4] = q.z, d[6] = q.w;
+        }
+        tail += __popc(bal);
+        if (__any_sync(0xffffffffu, close)) near_to = tail;
+      };
+      float4 n0 = fetch(lane), n1 = fetch(32 + lane);
+      for (uint32_t o = 0; o < n_list; o += 64) {
+        const float4 c0 = n0, c1 = n1;
+        n0 = fetch(o + 64 + lane);
+        if (o + 96 < n_list) n1 = fetch(o + 96 + lane);
+        offer(c0, o + lane < n_list);
+        if (o + 32 < n_list) offer(c1, o + 32 + lane < n_list);
+        while (tail - head >= nb) {
           __syncwarp();
-          if (lane == 0) {
-            const bool found = VX ? m < er : (!(a.emax_near > 0.f) || m < a.emax_near);
-            if (VX) {
-              if (!found) a.need[atomicAdd(&a.cgeo->list_n, 1u)] = c0 + ci;
-            } else if (a.emax_near > 0.f) {
-              a.need[c0 + ci] = found ? 0u : 1u;
-            }
-            if (found)
-              for (uint32_t q = 0; q < a.n_k; ++q) H.kth(a, q, kq[a.ks[q] - 1], pidx);
-          }
+          batch(nb);
+          head += nb;
           __syncwarp();
         }
+      }
+    }
+    if (tail != head) {
+      // the last, partial batch: far records to its end
+      const uint32_t n = tail - head;
+      for (uint32_t h = lane; h < nb; h += 32)
+        if (h >= n) {
+          const uint32_t slot = (head + h) & (kRing - 1u);
+          float* d = bf + (slot >> 1) * 8 + (slot & 1u);
+          d[0] = INFINITY, d[2] = INFINITY, d[4] = INFINITY, d[6] = __uint_as_float(~0u);
+        }
+      __syncwarp();
+      batch(n);
+      __syncwarp();
+    }
+    if (all) {
+      // the centrals met themselves once each, at d2 = 0 (a non-finite one did not)
+      bool self = valid && sub == 0 && dist2(p.x, p.y, p.z, p.x, p.y, p.z) == 0.f;
+      if (self && !a.self_all) self = in_mask(a.nbr, a.type[pidx]);
+      within -= (uint32_t)self;
+      if (MODE == kRdfDirect && rdf_here) {
+        const uint32_t n_self = __popc(__ballot_sync(0xffffffffu, self));
+        if (lane == 0 && n_self) red_shared(row_base + 4u * kMagicBits, 0u - n_self);
+      }
+    }
+    // merge the partial lists of the L lanes of each central (disjoint candidate subsets); the
+    // partner's sorted list is read from the warp's queue buffer in a rolled loop, which keeps
+    // the kernel's code small (its speed depends on the instruction cache)
+    for (uint32_t o = 1; o < L; o <<= 1) {
+      within += __shfl_xor_sync(0xffffffffu, within, o);
+      if constexpr (KMAX > 0 && KK * 32 <= 32 * kHalf) {
+        __syncwarp();
+#pragma unroll
+        for (int t = 0; t < KK; ++t) kq[t * 32 + lane] = top[t];
+        __syncwarp();
+        const float* ot = kq + (lane ^ o);
+#pragma unroll 1
+        for (int t = 0; t < KK; ++t) {
+          const float v = ot[t * 32];
+          if (!(v < top[KK - 1])) break;  // the partner's list is sorted
+          topk_insert(top, v);
+        }
+      } else if constexpr (KMAX > 0) {
+        float other[KK];
+#pragma unroll
+        for (int t = 0; t < KK; ++t) other[t] = __shfl_xor_sync(0xffffffffu, top[t], o);
+#pragma unroll
+        for (int t = 0; t < KK; ++t) {
+          if (!(other[t] < top[KK - 1])) break;  // the partner's list is sorted
+          topk_insert(top, other[t]);
+        }
+      }
+    }
+    if (valid && sub == 0) {
+      if (nwithin) nwithin[pidx] = within;
+      if (KMAX > 0) {
+        const float kd = topk_get(top, a.k_need - 1);
+        const bool found = !(a.emax_near > 0.f) || kd < a.emax_near;
+        if (a.emax_near > 0.f) a.need[c0 + ci] = found ? 0u : 1u;
+        if (found)
+          for (uint32_t q = 0; q < a.n_k; ++q) H.kth(a, q, topk_get(top, a.ks[q] - 1), pidx);
       }
     }
   }
 
   // ---- items from the back: sparse cells, one thread per central ----
   // central record and cell of the taken items' centrals (<= 32 * 15, kHeavy - 1 per item)
-  uint32_t* cl_rec = reinterpret_cast<uint32_t*>(s_hits[w]);
+  static_assert(32 * (kHeavy - 1) <= 4 * kRing && 32 * (kHeavy - 1) <= 32 * kHalf + 32, "light items taken at once");
+  uint32_t* cl_rec = reinterpret_cast<uint32_t*>(s_buf[w]);
   uint32_t* cl_cell = reinterpret_cast<uint32_t*>(s_kq[w]);
   const int st = a.stencil;
   // items per take: enough that every warp of the grid gets work when the list is short
@@ -772,7 +938,7 @@ __global__ void __launch_bounds__(256) k_query_warp(const QueryArgs a) {
               const float d2 = dist2(p.x, p.y, p.z, q.x, q.y, q.z);
               if (d2 < erange && __float_as_uint(q.w) != pidx) {
                 ++within;
-                if (RDF) {
+                if (rdf_here) {
                   if (within <= kRowLaneCap)
                     H.pair(a, d2, my_below);
                   else
@@ -783,7 +949,7 @@ __global__ void __launch_bounds__(256) k_query_warp(const QueryArgs a) {
             }
           }
         rowc = within < kRowLaneCap ? within : kRowLaneCap;
-        if (a.nwithin) a.nwithin[pidx] = within;
+        if (nwithin) nwithin[pidx] = within;
         if (KMAX > 0) {
           const bool found = !(a.emax_near > 0.f) || topk_get(top, a.k_need - 1) < a.emax_near;
           if (a.emax_near > 0.f) a.need[cl_rec[r0 + lane]] = found ? 0u : 1u;
@@ -792,9 +958,9 @@ __global__ void __launch_bounds__(256) k_query_warp(const QueryArgs a) {
         }
       }
       if (RDF) {
-        // a round adds at most 32 * 2^25 = 2^30 to the row: flushed at 2^31, it never wraps
+        // a round adds at most 32 * 2^25 = 2^30 to the row: flushed at 2^30, it stays below 2^31
         wcount += __reduce_add_sync(0xffffffffu, rowc);
-        if (wcount >= (1ull << 31)) {
+        if (wcount >= (1ull << 30)) {
           H.flush_warp(a);
           wcount = 0;
         }
@@ -934,66 +1100,6 @@ __global__ void __launch_bounds__(256) k_query_cta(const QueryArgs a) {
 // ---------------------------------------------------------------------------
 // symmetric RDF pass: every unordered pair of neighbour records once (sweep_pairs)
 // ---------------------------------------------------------------------------
-constexpr float kBinBias = 1.0f / 2097152.0f;   // 2^-21
-
-__device__ __forceinline__ void red_shared_inc(uint32_t addr) {
-  asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr));
-}
-__device__ __forceinline__ void red_shared(uint32_t addr, uint32_t v) {
-  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v));
-}
-
-// Bins of the direct form (r0 = 0).  With s = sqrt.approx(d2) and inv = (1 +- 2^-21) / dr, the true
-// quotient sqrt(d2) / dr lies between s * inv- and s * inv+ (the root is good to 2^-23, inv to 2^-24,
-// the edge table to 2^-25 of the distance).  The bin is floor(s * inv+), or the one below where the two floors
-// differ (2 in 10^4 pairs at 200 bins): those compare d2 with that edge.  Pairs out of range are
-// clamped into the unused bin n_bins, so that every lane increments and no instruction is
-// predicated: the compiler branches around a predicated shared-memory increment.  Measured on the
-// pair loop alone (cycles per 32 tests and scheduler): 23 with a predicated increment and the excess over
-// the edge computed, 17 in this form, of which 14.5 are the distance, root and floor; no table load per pair, so
-// the shared-memory pipe is left to the increments (increments by one merge in a bin).
-struct FastBins {
-  const float* sE;
-  unsigned long long hi2, lo2, magic2;
-  float s_far;
-  __device__ void init(const QueryArgs& a, const float* edges) {
-    sE = edges;
-    const float hi = (float)((1.0 + (double)kBinBias) / a.dr), lo = (float)((1.0 - (double)kBinBias) / a.dr);
-    hi2 = f2_pack(hi, hi);
-    lo2 = f2_pack(lo, lo);
-    magic2 = f2_pack(kMagic, kMagic);
-    s_far = (float)(((double)a.n_bins + 0.5) * a.dr);
-  }
-  // counts two pairs in the row at shared address `base` (bin b at base + 4 (kMagicBits + b));
-  // returns 0 unless one of them may lie under the edge of its bin
-  __device__ __forceinline__ uint32_t count2(unsigned long long d2, uint32_t base) const {
-    float da, db, ma, mb, la, lb;
-    f2_unpack(d2, da, db);
-    const unsigned long long s2 = f2_pack(fminf(sqrt_fast(da), s_far), fminf(sqrt_fast(db), s_far));
-    f2_unpack(f2_fma_down(s2, hi2, magic2), ma, mb);
-    f2_unpack(f2_fma_down(s2, lo2, magic2), la, lb);
-    red_shared_inc(__float_as_uint(ma) * 4u + base);
-    red_shared_inc(__float_as_uint(mb) * 4u + base);
-    return (__float_as_uint(ma) ^ __float_as_uint(la)) | (__float_as_uint(mb) ^ __float_as_uint(lb));
-  }
-  // a counted pair that may lie under the edge of its bin: moved to the bin below if it does
-  __device__ __forceinline__ void settle(float d2, uint32_t base) const {
-    float m, x;
-    f2_unpack(f2_fma_down(f2_pack(fminf(sqrt_fast(d2), s_far), 0.f), hi2, magic2), m, x);
-    const uint32_t addr = __float_as_uint(m) * 4u + base;
-    if (d2 < sE[__float_as_uint(m) - kMagicBits]) {
-      red_shared(addr, ~0u);
-      red_shared_inc(addr - 4u);
-    }
-  }
-  __device__ __forceinline__ void settle2(unsigned long long d2, uint32_t base) const {
-    float da, db;
-    f2_unpack(d2, da, db);
-    settle(da, base);
-    settle(db, base);
-  }
-};
-
 // Bound by instruction issue and the shared-memory pipe (ncu, 2e5 cylinder: 77 % of the issue slots,
 // two bank cycles per increment).  FAST (r0 = 0, at most kPrivBins bins; the host's rule in run_query):
 // two 32-bit rows per warp, for pairs of weight 1 and 2, and one increment per test by every
@@ -1002,13 +1108,17 @@ struct FastBins {
 // Measured, all-all, one box (ms): 1e8-ion needle 192.8 -> 76.7, 8e6-ion needle 14.95 -> 5.85,
 // 2e5 cylinder 0.504 -> 0.232 (before: full half stencils, warp list of hits, bin table).
 // Otherwise (r0 > 0 or more bins): the general bins of Hist, a branch per hit.
-template <bool FAST>
-__global__ void __launch_bounds__(256, 4) k_rdf_sym(const QueryArgs a, const __grid_constant__ SweepArgs sw) {
+// WITHIN (direct bins): also the in-range neighbours of every record, in record order, into `wacc`: a
+// candidate's lane counts its hits, the hits of a staged record are counted over the warp.
+template <bool FAST, bool WITHIN>
+__global__ void __launch_bounds__(256, WITHIN ? 3 : 4) k_rdf_sym(const QueryArgs a, const __grid_constant__ SweepArgs sw,
+                                                                 uint32_t* __restrict__ wacc) {
   griddep_wait();
   griddep_launch();
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ SweepBuf s_sweep[8];
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (a.sweep && !sweep_pays(*a.ngeo)) return;
   SweepBuf& buf = s_sweep[w];
   uint64_t wcount = 0;  // bound on the increments of this warp's rows since their last flush (uniform)
   if constexpr (FAST) {
@@ -1026,7 +1136,11 @@ __global__ void __launch_bounds__(256, 4) k_rdf_sym(const QueryArgs a, const __g
     uint32_t* row1 = rows + 2 * w * stride;
     const uint32_t a1 = smem_u32(row1), base1 = a1 - 4u * kMagicBits, base2 = base1 + 4u * stride;
     const unsigned long long one2 = f2_pack(sw.one, sw.one);
-    sweep_pairs<false>(sw, buf, [&](uint32_t n_pr, uint32_t, uint32_t nc, bool) __attribute__((always_inline)) {
+    const float Emax = sE[nb];
+    uint32_t* wrec = rows + 16 * stride + w * kSweepRec;  // WITHIN: hits of the staged records
+    if (WITHIN)
+      for (uint32_t r = lane; r < kSweepRec; r += 32) wrec[r] = 0;
+    auto tile = [&](uint32_t n_pr, uint32_t, uint32_t nc, bool) __attribute__((always_inline)) {
       const float4 far = make_float4(INFINITY, INFINITY, INFINITY, __uint_as_float(kCandSingle));
       const float4 c0 = lane < nc ? buf.cand[lane] : far, c1 = lane + 32 < nc ? buf.cand[lane + 32] : far;
       const uint32_t k0 = __float_as_uint(c0.w), k1 = __float_as_uint(c1.w);
@@ -1035,6 +1149,7 @@ __global__ void __launch_bounds__(256, 4) k_rdf_sym(const QueryArgs a, const __g
       const unsigned long long x1 = f2_pack(c1.x, c1.x), y1 = f2_pack(c1.y, c1.y), z1 = f2_pack(c1.z, c1.z);
       const ulonglong2* rxy = reinterpret_cast<const ulonglong2*>(buf.rxy);
       const ulonglong2* rz = reinterpret_cast<const ulonglong2*>(buf.rz);
+      uint32_t hits0 = 0, hits1 = 0;
 #pragma unroll 1
       for (uint32_t k = 0; k < n_pr; k += 2) {  // 4 records against the lane's 2 candidates
         const ulonglong2 xy = rxy[k], xy2 = rxy[k + 1], zz = rz[k >> 1];
@@ -1049,11 +1164,30 @@ __global__ void __launch_bounds__(256, 4) k_rdf_sym(const QueryArgs a, const __g
           fb.settle2(d2, b0);
           fb.settle2(d3, b1);
         }
+        if (WITHIN) {
+          // of each of the four records, and of the lane's two candidates
+          float e0[4], e1[4];
+          f2_unpack(d0, e0[0], e0[1]), f2_unpack(d2, e0[2], e0[3]);
+          f2_unpack(d1, e1[0], e1[1]), f2_unpack(d3, e1[2], e1[3]);
+          uint32_t n = 0;
+#pragma unroll
+          for (uint32_t i = 0; i < 4; ++i) {
+            const bool h0 = e0[i] < Emax, h1 = e1[i] < Emax;
+            hits0 += h0, hits1 += h1;
+            const uint32_t v = __popc(__ballot_sync(0xffffffffu, h0)) + __popc(__ballot_sync(0xffffffffu, h1));
+            if (lane == i) n = v;
+          }
+          if (lane < 4) wrec[2 * k + lane] += n;
+        }
       }
       // the staged records met themselves once each, at d2 = 0
       const uint32_t self = __popc(__ballot_sync(0xffffffffu, k0 == kCandSelf)) +
                             __popc(__ballot_sync(0xffffffffu, k1 == kCandSelf));
       if (self && lane == 0) red_shared(a1, 0u - self);
+      if (WITHIN) {  // (the block's own records count their neighbours in it as staged records)
+        if (lane < nc && (k0 == kCandBoth || k0 == kCandSingle) && hits0) atomicAdd(wacc + buf.cidx[lane], hits0);
+        if (lane + 32 < nc && (k1 == kCandBoth || k1 == kCandSingle) && hits1) atomicAdd(wacc + buf.cidx[lane + 32], hits1);
+      }
       wcount += 2u * kSweepTile * n_pr;
       if (wcount >= (1ull << 31)) {
         __syncwarp();
@@ -1068,7 +1202,18 @@ __global__ void __launch_bounds__(256, 4) k_rdf_sym(const QueryArgs a, const __g
         __syncwarp();
         wcount = 0;
       }
-    });
+    };
+    if constexpr (WITHIN)
+      sweep_pairs<true>(sw, buf, tile, [&](uint32_t m, bool) __attribute__((always_inline)) {
+        __syncwarp();
+        for (uint32_t r = lane; r < kSweepRec; r += 32) {
+          if (r < m && wrec[r]) atomicAdd(wacc + buf.ridx[r], wrec[r]);
+          wrec[r] = 0;
+        }
+        __syncwarp();
+      });
+    else
+      sweep_pairs<false>(sw, buf, tile);
     __syncthreads();
     unsigned long long tot = 0;
     for (uint32_t b = threadIdx.x; b < nb; b += blockDim.x) {
@@ -1099,7 +1244,7 @@ __global__ void __launch_bounds__(256, 4) k_rdf_sym(const QueryArgs a, const __g
       }
       __syncwarp();
       wcount += 2u * kSweepTile * m;
-      if (wcount >= (1ull << 31)) {
+      if (wcount >= (1ull << 30)) {
         H.flush_warp(a);
         wcount = 0;
       }
@@ -1109,15 +1254,190 @@ __global__ void __launch_bounds__(256, 4) k_rdf_sym(const QueryArgs a, const __g
   }
 }
 
-template <bool FAST>
-static int launch_rdf_sym(const ps_grid* g, const QueryArgs& qa, const SweepArgs& sw, uint32_t smem, cudaStream_t s) {
-  auto k = k_rdf_sym<FAST>;
+// in-range neighbours of the central records (record order; each met itself once) to their ions
+__global__ void __launch_bounds__(256) k_within_out(const QueryArgs a, const uint32_t* __restrict__ pfx,
+                                                    const uint32_t* __restrict__ wacc) {
+  griddep_wait();
+  griddep_launch();
+  if (!sweep_pays(*a.ngeo)) return;
+  const uint32_t n = a.ngeo->n_sel;
+  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    if (pfx[j + 1] == pfx[j]) continue;
+    const float4 p = __ldg(a.nrec + j);
+    const bool self = dist2(p.x, p.y, p.z, p.x, p.y, p.z) == 0.f;
+    a.nwithin[__float_as_uint(p.w)] = wacc[j] - (uint32_t)self;
+  }
+}
+
+template <bool FAST, bool WITHIN>
+static int launch_rdf_sym(const ps_grid* g, const QueryArgs& qa, const SweepArgs& sw, uint32_t smem, uint32_t* wacc,
+                          cudaStream_t s) {
+  auto k = k_rdf_sym<FAST, WITHIN>;
   PS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem));
   if (per_sm < 1) return fail(PS_ERR_UNSUPPORTED, "symmetric RDF kernel does not fit on an SM");
-  PS_LAUNCH(PS_KID_RDF_SYM, s, PS_CUDA(launch_pdl(k, g->num_sms * per_sm, 256, smem, s, qa, sw)));
+  PS_LAUNCH(PS_KID_RDF_SYM, s, PS_CUDA(launch_pdl(k, g->num_sms * per_sm, 256, smem, s, qa, sw, wacc)));
+  if (WITHIN)
+    PS_LAUNCH(PS_KID_RDF_SYM, s, PS_CUDA(launch_pdl(k_within_out, g->num_sms * 8, 256, 0, s, qa, sw.pfx, (const uint32_t*)wacc)));
   return PS_OK;
+}
+
+// ---------------------------------------------------------------------------
+// near kNN pass on the vertex-centred central list
+// ---------------------------------------------------------------------------
+constexpr uint32_t kQueue = 40;  // queue rows per lane; inserted when fewer than 16 are free
+
+// One warp per item (up to 32 centrals of a vertex cell, one to eight lanes each), its candidates the
+// records of the 2 x 2 x 2 cells around the vertex, staged 32 at a time as interleaved pairs.  A sorted
+// insertion costs ~25 instructions for the whole warp whichever lanes need it, so the candidates
+// are filtered first: by the central's reach and by the radius that holds k + 3 sqrt(k) records
+// at the block's density (about 20 of 240 candidates at k = 10), and the few left are queued and
+// inserted together.  A central with fewer than k records there is listed for the full search, as
+// one whose k-th distance is beyond its reach.  The central itself stays in (distance 0): the
+// list is one longer and rank k is its entry k, so that no test compares indexes.  KMAX > k_need.
+// Bound by issue (ncu, 8e6-ion needle: 81 % of the slots).  All-all, k = 10, one box (ms): 8e6-ion needle
+// 1.94 -> 1.65, the 1e8-ion one 25.4 -> 21.5 (before: an insertion queue drained every 16 candidates, the
+// central compared by index).
+template <int KMAX>
+__global__ void __launch_bounds__(256, KMAX <= 13 ? 4 : 2) k_knn_vertex(const __grid_constant__ QueryArgs a) {
+  griddep_wait();
+  griddep_launch();
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ float4 s_xy[8][16];
+  __shared__ float2 s_z[8][16];
+  __shared__ float s_kq[8][(kQueue + 1) * 32];
+  Hist<false> H{};
+  H.init(a, smem, 0, true);
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float* kq = s_kq[w];
+  const uint32_t q0 = smem_u32(kq + lane);
+  const Geo ng = *a.ngeo, vg = *a.cgeo;
+  const uint32_t n_items = vg.work_n2;
+  const unsigned long long one2 = f2_pack(a.one, a.one);
+  // rounding slack of a cell coordinate (cells) and the cell edge for vertex_reach
+  const float slack = (float)max(ng.dims[0], max(ng.dims[1], ng.dims[2])) * 5.0e-7f + 1.0e-6f;
+  const float h_eff = __fmul_rn(__fdiv_rn(1.0f, ng.inv_h), 1.0f - 1.0f / 4096.0f);
+  const float k_f = (float)a.k_need, want = (k_f + 3.f * sqrtf(k_f) + 1.f) * 0.238732415f;  // 3 / (4 pi)
+  for (;;) {
+    uint32_t item = 0;
+    if (lane == 0) item = atomicAdd(a.next_front, 1u);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if (item >= n_items) break;
+    const uint2 it = a.witem[item];
+    const uint32_t c = it.x, cnt = it.y & 63u, c0 = a.cstart[c] + (it.y >> 6);
+    const uint32_t L = item_lanes(cnt), lg = 31u - __clz(L);
+    const uint32_t sub = lane & (L - 1u), ci = lane >> lg;
+    const bool valid = ci < cnt;
+    // the four runs of the block: their records as one list
+    uint32_t rs = 0, rl = 0;
+    vertex_run(a, ng, vg, c, lane, rs, rl);
+    const uint32_t s0 = __shfl_sync(0xffffffffu, rs, 0), s1 = __shfl_sync(0xffffffffu, rs, 1),
+                   s2 = __shfl_sync(0xffffffffu, rs, 2), s3 = __shfl_sync(0xffffffffu, rs, 3);
+    const uint32_t e0 = __shfl_sync(0xffffffffu, rl, 0), e1 = e0 + __shfl_sync(0xffffffffu, rl, 1),
+                   e2 = e1 + __shfl_sync(0xffffffffu, rl, 2), n_cand = e2 + __shfl_sync(0xffffffffu, rl, 3);
+    auto fetch = [&](uint32_t pos) -> float4 {
+      if (pos >= n_cand) return make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+      const uint32_t j = pos < e1 ? (pos < e0 ? s0 + pos : s1 + (pos - e0)) : (pos < e2 ? s2 + (pos - e1) : s3 + (pos - e2));
+      return __ldg(a.nrec + j);
+    };
+    float4 nxt = fetch(lane);
+    float4 p = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+    float thr = 0.f;
+    if (valid) {
+      p = a.crec[c0 + ci];
+      // (cells of the block inside the grid: at least 1 of 8)
+      const float r0 = ng.h * cbrtf(want * 8.f / (float)max(n_cand, 1u));
+      thr = fminf(vertex_reach(ng, vg, c, p, slack, h_eff, H.Emax), r0 * r0);
+    }
+    const unsigned long long px = f2_pack(p.x, p.x), py = f2_pack(p.y, p.y), pz = f2_pack(p.z, p.z);
+    float top[KMAX];
+#pragma unroll
+    for (int t = 0; t < KMAX; ++t) top[t] = INFINITY;
+    uint32_t qa = q0;  // the next slot of this lane's queue column
+    auto insert = [&](uint32_t m) __attribute__((always_inline)) {
+      const uint32_t qn = (qa - q0) >> 7;
+#pragma unroll 1
+      for (uint32_t q = 0; q < m; ++q)
+        if (q < qn) topk_insert(top, queue_at(q0, q));
+      qa = q0;
+    };
+    float* sxy = reinterpret_cast<float*>(s_xy[w]);
+    float* sz = reinterpret_cast<float*>(s_z[w]);
+    for (uint32_t b = 0; b < n_cand; b += 32) {
+      __syncwarp();
+      {
+        float* d = sxy + (lane >> 1) * 4 + (lane & 1u);
+        d[0] = nxt.x, d[2] = nxt.y, sz[lane] = nxt.z;
+      }
+      __syncwarp();
+      nxt = fetch(b + 32 + lane);
+#pragma unroll 1
+      for (uint32_t hb = 0; hb < 16; hb += 8) {
+#pragma unroll 4
+        for (uint32_t t = hb + sub; t < hb + 8; t += L) {
+          const ulonglong2 xy = *reinterpret_cast<const ulonglong2*>(&s_xy[w][t]);
+          const unsigned long long zz = *reinterpret_cast<const unsigned long long*>(&s_z[w][t]);
+          float da, db;
+          f2_unpack(dist2_x2_fma(px, py, pz, xy.x, xy.y, zz, one2), da, db);
+          queue_push(qa, da, thr);
+          queue_push(qa, db, thr);
+        }
+        const uint32_t m = __reduce_max_sync(0xffffffffu, qa - q0) >> 7;
+        if (m > kQueue - 16u) {
+          insert(m);
+          thr = fminf(thr, top[KMAX - 1]);
+        }
+      }
+    }
+    insert(__reduce_max_sync(0xffffffffu, qa - q0) >> 7);
+    // merge the partial lists of the L lanes of each central (disjoint candidate subsets)
+    for (uint32_t o = 1; o < L; o <<= 1) {
+      __syncwarp();
+#pragma unroll
+      for (int t = 0; t < KMAX; ++t) kq[t * 32 + lane] = top[t];
+      __syncwarp();
+      const float* ot = kq + (lane ^ o);
+#pragma unroll 1
+      for (int t = 0; t < KMAX; ++t) {
+        const float v = ot[t * 32];
+        if (!(v < top[KMAX - 1])) break;  // the partner's list is sorted
+        topk_insert(top, v);
+      }
+    }
+    __syncwarp();
+    bool miss = false;
+    if (valid && sub == 0) {
+      miss = !(topk_get(top, a.k_need) < INFINITY);  // entry 0 is the central itself
+      if (!miss)
+        for (uint32_t q = 0; q < a.n_k; ++q) H.kth(a, q, topk_get(top, a.ks[q]), __float_as_uint(p.w));
+    }
+    list_append(a, miss, c0 + ci, lane);
+  }
+  H.flush(a);
+}
+
+template <int KMAX>
+static int launch_knn_vertex(const ps_grid* g, const QueryArgs& qa, uint32_t smem, cudaStream_t s) {
+  auto k = k_knn_vertex<KMAX>;
+  int per_sm = 0;
+  PS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem));
+  if (per_sm < 1) return fail(PS_ERR_UNSUPPORTED, "near kNN kernel does not fit on an SM");
+  PS_LAUNCH(PS_KID_QUERY, s, PS_CUDA(launch_pdl(k, g->num_sms * per_sm, 256, smem, s, qa)));
+  return PS_OK;
+}
+
+static int dispatch_knn_vertex(const ps_grid* g, const QueryArgs& qa, uint32_t smem, cudaStream_t s) {
+  const uint32_t k = qa.k_need;
+  if (k <= 1) return launch_knn_vertex<2>(g, qa, smem, s);
+  if (k <= 2) return launch_knn_vertex<3>(g, qa, smem, s);
+  if (k <= 4) return launch_knn_vertex<5>(g, qa, smem, s);
+  if (k <= 8) return launch_knn_vertex<9>(g, qa, smem, s);
+  if (k <= 10) return launch_knn_vertex<11>(g, qa, smem, s);
+  if (k <= 12) return launch_knn_vertex<13>(g, qa, smem, s);
+  if (k <= 16) return launch_knn_vertex<17>(g, qa, smem, s);
+  return launch_knn_vertex<33>(g, qa, smem, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -1256,10 +1576,11 @@ __global__ void k_query_epilogue(const Geo* __restrict__ ngeo, const Geo* __rest
   }
 }
 
-template <int KMAX, bool RDF>
+template <int KMAX, int MODE>
 static int launch_query(const ps_grid* g, const QueryArgs& qa, uint32_t smem_cta, uint32_t smem_warp, cudaStream_t s) {
   const uint32_t kid = qa.fallback ? PS_KID_KNN_FULL : PS_KID_QUERY;
-  auto kw = (!RDF && qa.vertex) ? k_query_warp<KMAX, RDF, !RDF> : k_query_warp<KMAX, RDF>;
+  constexpr bool RDF = MODE != kNoRdf;
+  auto kw = k_query_warp<KMAX, MODE>;
   PS_CUDA(cudaFuncSetAttribute(kw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_warp));
   int per_sm_w = 0;
   PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_w, kw, 256, smem_warp));
@@ -1277,18 +1598,18 @@ static int launch_query(const ps_grid* g, const QueryArgs& qa, uint32_t smem_cta
   return PS_OK;
 }
 
-template <bool RDF>
+template <int MODE>
 static int dispatch_k(const ps_grid* g, const QueryArgs& qa, uint32_t sc, uint32_t sw, cudaStream_t s) {
   const uint32_t k = qa.k_need;
-  if (k == 0) return RDF ? launch_query<0, RDF>(g, qa, sc, sw, s) : PS_OK;
-  if (k <= 1) return launch_query<1, RDF>(g, qa, sc, sw, s);
-  if (k <= 2) return launch_query<2, RDF>(g, qa, sc, sw, s);
-  if (k <= 4) return launch_query<4, RDF>(g, qa, sc, sw, s);
-  if (k <= 8) return launch_query<8, RDF>(g, qa, sc, sw, s);
-  if (k <= 10) return launch_query<10, RDF>(g, qa, sc, sw, s);
-  if (k <= 12) return launch_query<12, RDF>(g, qa, sc, sw, s);
-  if (k <= 16) return launch_query<16, RDF>(g, qa, sc, sw, s);
-  return launch_query<32, RDF>(g, qa, sc, sw, s);
+  if (k == 0) return MODE != kNoRdf ? launch_query<0, MODE>(g, qa, sc, sw, s) : PS_OK;
+  if (k <= 1) return launch_query<1, MODE>(g, qa, sc, sw, s);
+  if (k <= 2) return launch_query<2, MODE>(g, qa, sc, sw, s);
+  if (k <= 4) return launch_query<4, MODE>(g, qa, sc, sw, s);
+  if (k <= 8) return launch_query<8, MODE>(g, qa, sc, sw, s);
+  if (k <= 10) return launch_query<10, MODE>(g, qa, sc, sw, s);
+  if (k <= 12) return launch_query<12, MODE>(g, qa, sc, sw, s);
+  if (k <= 16) return launch_query<16, MODE>(g, qa, sc, sw, s);
+  return launch_query<32, MODE>(g, qa, sc, sw, s);
 }
 
 // Parameters of the bin lookup table: a bit shift S <= 16 at which the interior edges
@@ -1327,6 +1648,7 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
   memset(&qa, 0, sizeof(qa));
   qa.nrec = g->nbr.rec;
   qa.nstart = g->nbr.start;
+  qa.nsub = g->nbr.count;
   qa.ngeo = g->nbr.geo;
   qa.crec = g->ctr.rec;
   qa.cstart = g->ctr.start;
@@ -1357,6 +1679,10 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
   choose_lut(bins, qa);
 
   const bool rdf = d_rdf != nullptr;
+  // direct bins: r0 = 0, a warp's row of counts at most 2 KB, and edges and range far from the limits
+  // of float32 (the approximate root flushes subnormals)
+  const double stop = bins.r0 + (double)bins.n_bins * bins.dr;
+  const bool direct = bins.r0 == 0.0 && bins.n_bins <= kPrivBins && bins.dr > 1e-15 && stop < 1e15;
   ZeroOut z;  // the outputs are zeroed by the central-list reset kernel
   z.p[0] = d_meta;
   z.n[0] = PS_META_LEN(n_k);
@@ -1364,6 +1690,10 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
   if (n_k) z.p[2] = d_knn, z.n[2] = n_k * bins.n_bins;
 
   const bool subset = centrals_in_neighbours(g, ctr_mask);
+  qa.self_all = subset;
+  qa.type = g->type;
+  for (int w = 0; w < 4; ++w) qa.nbr.w[w] = g->nbr_mask[w];
+  qa.one = 1.0f;
   // the query in passes, and its near kNN pass on the vertex-centred central list (two-cell
   // stencils; the ranks of that counting sort take one word per central of the cell arrays)
   const bool split = g->split && subset && rdf && d_nwithin == nullptr && g->stencil >= 2 && g->dense_min == 0xFFFFFFFFu;
@@ -1382,6 +1712,20 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
   qa.stage_cap = (stage_bytes / 16) & ~7u;
   const uint32_t smem_cta = smem_layout(bins.n_bins, n_k, rdf, qa.stage_cap, false, qa.lut_n).total;
   const uint32_t smem_warp = smem_layout(bins.n_bins, n_k, rdf, 0, true, qa.lut_n).total;
+  // the RDF over unordered pairs
+  auto run_rdf_sym = [&]() -> int {
+    QueryArgs qs = qa;
+    qs.n_k = 0;
+    SweepArgs sw = sweep_args(g, &g->ctr.geo->sym_next);
+    sw.range = (float)(stop * stop);
+    if (!direct)
+      return launch_rdf_sym<false, false>(g, qs, sw, smem_layout(bins.n_bins, 0, true, 0, true, qa.lut_n).total, nullptr, s);
+    const uint32_t smem = (bins.n_bins + 1) * 4 * 17;
+    if (d_nwithin == nullptr) return launch_rdf_sym<true, false>(g, qs, sw, smem, nullptr, s);
+    // the counts in record order take the counting sort's index list, free until the next build
+    PS_CUDA(cudaMemsetAsync(g->sel, 0, (size_t)g->n * sizeof(uint32_t), s));
+    return launch_rdf_sym<true, true>(g, qs, sw, smem + 8 * kSweepRec * 4, g->sel, s);
+  };
   if (split) {
     // the query in passes: (1) kNN near each central, centrals with fewer than k_need
     // neighbours there set apart; (2) their full-radius kNN; (3) the RDF over unordered pairs
@@ -1391,21 +1735,19 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
       const uint32_t smem_knn = smem_layout(bins.n_bins, n_k, false, 0, true).total;
       if (vertex) {
         // the 2 x 2 x 2 cells around each central's nearest vertex, each central within its own
-        // reach (k_query_warp, vertex mode); the others listed for k_knn_list
-        qn.vertex = 1;
-        rc = dispatch_k<false>(g, qn, smem_cta, smem_knn, s);
+        // reach; the others listed for k_knn_list
+        rc = dispatch_knn_vertex(g, qn, smem_knn, s);
         if (rc) return rc;
         rc = dispatch_knn_list(g, qn, smem_knn, s);
         if (rc) return rc;
       } else {
         // the 27 cells around each central's cell, within the cell edge
         const double rk = (double)g->r_cut * (double)g->cell_scale;
-        double e = bins.r0 + (double)bins.n_bins * bins.dr;
-        const float Emax = (float)(e * e), Ek = (float)(rk * rk);
+        const float Emax = (float)(stop * stop), Ek = (float)(rk * rk);
         qn.emax_near = Ek < Emax ? Ek : Emax;
         qn.stencil = 1;
         row_widths(1, 1.0, qn.row_w);
-        rc = dispatch_k<false>(g, qn, smem_cta, smem_layout(bins.n_bins, n_k, false, 0, true).total, s);
+        rc = dispatch_k<kNoRdf>(g, qn, smem_cta, smem_layout(bins.n_bins, n_k, false, 0, true).total, s);
         if (rc) return rc;
         // the full radius for the centrals it marked
         QueryArgs qf = qa;
@@ -1413,23 +1755,21 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
         qf.need = g->sel;
         qf.next_front = &g->ctr.geo->work_next2b;
         qf.next_light = &g->ctr.geo->work_next3b;
-        rc = dispatch_k<false>(g, qf, smem_cta, smem_layout(bins.n_bins, n_k, false, 0, true).total, s);
+        rc = dispatch_k<kNoRdf>(g, qf, smem_cta, smem_layout(bins.n_bins, n_k, false, 0, true).total, s);
         if (rc) return rc;
       }
     }
-    QueryArgs qs = qa;
-    qs.n_k = 0;
-    SweepArgs sw = sweep_args(g, &g->ctr.geo->sym_next);
-    const double stop = (double)bins.n_bins * bins.dr;
-    sw.range = (float)((bins.r0 + stop) * (bins.r0 + stop));
-    // direct bins: r0 = 0, the two rows of a warp at most 4 KB, and edges and ranges far from the
-    // limits of float32 (the approximate root flushes subnormals)
-    const bool fast = bins.r0 == 0.0 && bins.n_bins <= kPrivBins && bins.dr > 1e-15 && stop < 1e15;
-    rc = fast ? launch_rdf_sym<true>(g, qs, sw, (bins.n_bins + 1) * 4 * 17, s)
-              : launch_rdf_sym<false>(g, qs, sw, smem_layout(bins.n_bins, 0, true, 0, true, qa.lut_n).total, s);
+    rc = run_rdf_sym();
     if (rc) return rc;
   } else if (n_k > 0 || rdf) {
-    rc = rdf ? dispatch_k<true>(g, qa, smem_cta, smem_warp, s) : dispatch_k<false>(g, qa, smem_cta, smem_warp, s);
+    if (rdf && subset && g->dense_min == 0xFFFFFFFFu && (direct || d_nwithin == nullptr)) {
+      qa.sweep = 1;
+      rc = run_rdf_sym();
+      if (rc) return rc;
+    }
+    rc = !rdf    ? dispatch_k<kNoRdf>(g, qa, smem_cta, smem_warp, s)
+         : direct ? dispatch_k<kRdfDirect>(g, qa, smem_cta, smem_warp, s)
+                  : dispatch_k<kRdfGeneral>(g, qa, smem_cta, smem_warp, s);
     if (rc) return rc;
   }
   PS_LAUNCH(PS_KID_EPILOGUE, s, PS_CUDA(launch_pdl(k_query_epilogue, 1, 32, 0, s, g->nbr.geo, g->ctr.geo, d_meta)));

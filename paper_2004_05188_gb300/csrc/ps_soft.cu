@@ -692,7 +692,7 @@ __global__ void __launch_bounds__(256) k_soft_grad_out(const float4* __restrict_
 }
 
 // warp items (cell, first << 6 | count) over every non-empty cell of a list
-__global__ void __launch_bounds__(256) k_make_items(const uint32_t* __restrict__ count, Geo* geo,
+__global__ void __launch_bounds__(256) k_make_items(const uint32_t* __restrict__ start, Geo* geo,
                                                     uint2* __restrict__ item) {
   griddep_wait();
   griddep_launch();
@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(256) k_make_items(const uint32_t* __restrict__
   const uint32_t lane = threadIdx.x & 31;
   for (uint32_t base = blockIdx.x * blockDim.x; base < nc; base += gridDim.x * blockDim.x) {
     const uint32_t c = base + threadIdx.x;
-    const uint32_t v = c < nc ? count[c] : 0u;
+    const uint32_t v = c < nc ? start[c + 1] - start[c] : 0u;
     const uint32_t m = v == 0 ? 0u : (v + 31u) / 32u;
     uint32_t x = m;
     for (int o = 1; o < 32; o <<= 1) {
@@ -777,7 +777,7 @@ static int launch_grid_for(const ps_grid* g, const void* kern, uint32_t smem, in
 // Owners = the neighbour records: warp items over the non-empty neighbour cells.
 static int nbr_items(ps_grid* g, SoftArgs& sa, cudaStream_t s, uint32_t kid) {
   PS_LAUNCH(kid, s, PS_CUDA(launch_pdl(k_reset_items, 1, 32, 0, s, g->nbr.geo)));
-  PS_LAUNCH(kid, s, PS_CUDA(launch_pdl(k_make_items, g->num_sms * 4, 256, 0, s, g->nbr.count, g->nbr.geo, g->nbr_witem)));
+  PS_LAUNCH(kid, s, PS_CUDA(launch_pdl(k_make_items, g->num_sms * 4, 256, 0, s, g->nbr.start, g->nbr.geo, g->nbr_witem)));
   sa.orec = g->nbr.rec;
   sa.ostart = g->nbr.start;
   sa.oitem = g->nbr_witem;

@@ -100,6 +100,7 @@ extern "C" int ps_spatstat_static(const float* xyz, const uint8_t* type, const f
   ps_grid g;  // a grid whose scratch is the static array (nothing to free)
   g.n_max = (int64_t)kN;
   g.cell_cap = (uint32_t)kCells;
+  g.fine_cap = (uint32_t)kCells;
   g.cell_scale = 1.0f;
   g.stencil = 1;
   g.item_cap = (uint32_t)kItems;

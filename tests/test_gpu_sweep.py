@@ -103,3 +103,20 @@ def test_smoothed_rdf_of_lattice_shells(ps, spec, m, copies):
     gs_ref = n_c * (mult * W * u).sum()
     assert abs(float(gs[0]) - gs_ref) <= 1e-4 * n_c * (mult * np.abs(W) * u).sum()
     g.close()
+
+
+@pytest.mark.parametrize("n,L", [(40, 9.0), (900, 9.0), (5000, 9.0), (12000, 7.0), (9000, 3.5), (30, 1.0)])
+@pytest.mark.parametrize("bins", [(0.0, 0.01, 200), (0.3, 0.05, 34)])
+def test_default_grid_over_its_densities(ps, orc, spec, n, L, bins):
+    """Default options from a record per cell to hundreds (RDF and in-range counts in the query or in
+    the sweep, cells without sub-cells, with 8 and with 64), centrals among the neighbours or not,
+    one to sixteen lanes per central, a blob that fills single cells."""
+    xyz, t, d = spec.cube(400 + n, n, L, (0.5, 0.3, 0.2))
+    blob = (np.array([L / 3, L / 2, L / 2]) + np.random.default_rng(n).normal(0, 0.05, (n // 10, 3))).astype(np.float32)
+    xyz = np.concatenate([xyz, blob, xyz[:3]])
+    t, d = np.resize(t, xyz.shape[0]), np.resize(d, xyz.shape[0])
+    for ctr, nbr, dmin, ks in (("all", "all", 0.0, [1, 3, 32]), ([0], [0, 1], 0.4, [10]), ([0, 2], [1], 0.0, [2, 5]),
+                               ("all", "all", 0.6, [])):
+        g = run_gpu(ps, xyz, t, d, ctr, nbr, dmin, bins, ks, per_central=True)
+        r = orc.spatstat(xyz, t, d, ctr, nbr, dmin, *bins, ks, per_central=True)
+        assert_same(g, r, ks, per_central=True)
