@@ -117,7 +117,7 @@ def query_sources_sha256() -> str:
     import re
 
     h = hashlib.sha256()
-    for f in ("ps_query.cu", "ps_sweep.cuh", "ps_internal.cuh"):
+    for f in ("ps_query.cu", "ps_items.cuh", "ps_sweep.cuh", "ps_internal.cuh"):
         with open(os.path.join(ROOT, "paper_2004_05188_gb300", "csrc", f), encoding="utf-8") as fh:
             for line in fh:
                 code = re.sub(r"//.*$", "", line).rstrip()

@@ -16,24 +16,27 @@
 //     ion type; a hit counts for the pairs whose central and neighbour sets hold
 //     both ends).
 // Work: one queue over all ROIs, items (cell, <= 32 centrals) in ROI order,
-// padded per ROI to whole chunks of 8 so a CTA (8 warps) always works on one
-// ROI and can keep that ROI's RDF counts in shared memory.  kNN counts go to
-// global memory (one update per central, k and pair).
+// padded per ROI to whole chunks of 16 so a CTA (8 warps, which share out a chunk)
+// always works on one ROI and can keep that ROI's RDF counts in shared memory.  Pairs
+// of the same neighbour set whose central sets are disjoint are searched together (a
+// pass: every lane has one pair); kNN counts go to global memory (one update per
+// central, k and pair).
 #include <cmath>
 #include <cstring>
 #include <new>
 #include <vector>
 
 #include "ps_internal.cuh"
+#include "ps_items.cuh"
 
 namespace ps {
 
-constexpr int kChunk = 8;        // items per CTA fetch (one per warp)
-constexpr int kBatchRuns = 25;
+constexpr int kChunk = 16;       // items per CTA fetch
 
 struct BRoi {
   const float4* nrec;
   const uint32_t* nstart;
+  const uint32_t* nsub;
   const Geo* ngeo;
   const float4* crec;
   const uint32_t* cstart;
@@ -52,11 +55,12 @@ struct BatchArgs {
   double r0, dr;
   uint32_t n_bins;           // bins at the largest r_max
   uint32_t n_pairs, n_cls, k_max;
-  uint32_t n_lists;
-  uint32_t list_of[4];       // pair -> top-k list
+  uint32_t n_pass;
+  uint32_t pass_pairs[4];    // bit p: pair p is searched in this pass
   uint64_t ctr_mask[4][4];
-  uint64_t nbr_mask[4][4];
-  uint64_t list_mask[2][4];  // neighbour set of each list
+  Mask nbr[4];               // neighbour set of each pass
+  float one;                 // 1.0f, opaque to the compiler (see dist2_x2_fma)
+  int8_t row_w[kMaxRuns];
   float cls_min[4];          // d_srf class lower bounds (ascending)
   unsigned long long* acc;   // per ROI accumulators, acc_len each
   uint32_t acc_len;
@@ -68,82 +72,62 @@ __host__ __device__ inline uint32_t acc_block(uint32_t nb, uint32_t kmax) { retu
 
 __device__ __forceinline__ bool mask_has(const uint64_t* m, uint32_t t) { return (m[t >> 6] >> (t & 63)) & 1ull; }
 
-template <int K>
-__device__ __forceinline__ void tk_insert(float (&top)[K], float x) {
-  if (x < top[K - 1]) {
-#pragma unroll
-    for (int t = K - 1; t > 0; --t) top[t] = fminf(top[t], fmaxf(x, top[t - 1]));
-    top[0] = fminf(top[0], x);
-  }
-}
-
-template <int K>
-__device__ __forceinline__ float tk_get(const float (&top)[K], uint32_t idx) {
-  float v = INFINITY;
-#pragma unroll
-  for (int t = 0; t < K; ++t)
-    if ((uint32_t)t == idx) v = top[t];
-  return v;
-}
-
-__device__ __forceinline__ uint32_t bbin(float d2, const float* sE, uint32_t nb, float r0f, float inv_dr) {
-  const float d = d2 > 0.f ? d2 * rsqrtf(d2) : 0.f;
-  int b = (int)((d - r0f) * inv_dr);
-  b = b < 0 ? 0 : (b >= (int)nb ? (int)nb - 1 : b);
-  if (d2 < sE[b] || d2 >= sE[b + 1]) {
-    while (b > 0 && d2 < sE[b]) --b;
-    while (b + 1 < (int)nb && d2 >= sE[b + 1]) ++b;
-  }
-  return (uint32_t)b;
-}
-
-template <int KMAX, int NL>
-__global__ void __launch_bounds__(256, 3) k_batch_query(const BatchArgs a) {
+// One item per warp, its passes one after the other: the candidates of the pass's neighbour set near
+// the item's box (item_scan), every in-range pair into the bin row of its central's pair and class,
+// those that can still enter a k list into the lane's queue.  DIRECT (r0 = 0): direct bins, an
+// increment per test by every lane; otherwise a branch per hit, and the pairs below r0 in bin
+// n_bins.  Rows are 32-bit and shared by the CTA: a warp drains them before it has added 2^28 since
+// its last drain.  Bound by instruction issue.  24 ROIs (2e6 ions, k = 1 .. 20, r_max = 3 nm, 3 pairs, 3
+// thresholds), whole pass: 75 -> 18.7 ms (before: every
+// record of the 125 cells, a sorted insertion under a branch per candidate, 64-bit counters).
+template <int KMAX, bool DIRECT>
+__global__ void __launch_bounds__(256, KMAX <= 20 ? 3 : 2) k_batch_query(const __grid_constant__ BatchArgs a) {
   griddep_wait();
   griddep_launch();
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ float4 s_buf[8][32];
-  __shared__ float s_hd[8][512];
-  __shared__ uint32_t s_ht[8][512];
-  __shared__ uint32_t s_rsrc[8][kBatchRuns], s_rpre[8][kBatchRuns + 1];
-  __shared__ uint32_t s_chunk, s_roi;
-  __shared__ uint32_t s_tinfo[256];  // per type: bit l = in list l's neighbour set, bit 2 + p = in pair p's
+  __shared__ float4 s_buf[8][kRing];
+  constexpr uint32_t kRows = (KMAX > (int)kHalf ? KMAX : (int)kHalf) + 1;  // of the insertion queue, and of the lists' merge
+  __shared__ uint32_t s_chunk, s_roi, s_next;
 
   const uint32_t nb = a.n_bins, P = a.n_pairs, C = a.n_cls;
-  // 64-bit pair counters (a CTA may count more than 2^32 pairs of one ROI), 32-bit central counts
   float* sE = reinterpret_cast<float*>(smem);
-  unsigned long long* s_rdf = reinterpret_cast<unsigned long long*>(smem + ((nb + 1) * 4 + 15) / 16 * 16);  // [P][C][nb+1]
-  uint32_t* s_nc = reinterpret_cast<uint32_t*>(s_rdf + P * C * (nb + 1));                                   // [P][C]
-  const uint32_t n_rdf = P * C * (nb + 1);  // per (p, c): nb bins then the below-range count
+  uint32_t* s_rdf = reinterpret_cast<uint32_t*>(sE + nb + 1);  // [P][C][nb + 1]
+  uint32_t* s_nc = s_rdf + P * C * (nb + 1);                   // [P][C]
+  const uint32_t n_rdf = P * C * (nb + 1);
   for (uint32_t b = threadIdx.x; b <= nb; b += blockDim.x) {
     const double e = __dadd_rn(a.r0, __dmul_rn((double)b, a.dr));
     sE[b] = __double2float_rn(__dmul_rn(e, e));
   }
-  for (uint32_t i = threadIdx.x; i < n_rdf; i += blockDim.x) s_rdf[i] = 0ull;
-  for (uint32_t i = threadIdx.x; i < P * C; i += blockDim.x) s_nc[i] = 0;
-  for (uint32_t t = threadIdx.x; t < 256; t += blockDim.x) {
-    uint32_t v = 0;
-    for (uint32_t l = 0; l < (uint32_t)NL; ++l) v |= (mask_has(a.list_mask[l], t) ? 1u : 0u) << l;
-    for (uint32_t pp = 0; pp < P; ++pp) v |= (mask_has(a.nbr_mask[pp], t) ? 1u : 0u) << (2 + pp);
-    s_tinfo[t] = v;
-  }
+  for (uint32_t i = threadIdx.x; i < n_rdf + P * C; i += blockDim.x) s_rdf[i] = 0;
   __syncthreads();
   const float Emax = sE[nb], E0 = sE[0], r0f = (float)a.r0, inv_dr = (float)(1.0 / a.dr);
+  FastBins fb;
+  if (DIRECT) fb.init(nb, a.dr, sE);
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t total = a.item_off[a.n_roi];
   const uint32_t blk = acc_block(nb, a.k_max);
+  const unsigned long long one2 = f2_pack(a.one, a.one);
+  float* bf = reinterpret_cast<float*>(s_buf[w]);
+  float* kq = reinterpret_cast<float*>(s_nc + P * C) + w * kRows * 32;
+  const uint32_t q0 = smem_u32(kq + lane), rows = smem_u32(s_rdf) - 4u * kMagicBits;
+  uint32_t added = 0;  // bound on this warp's increments since it last drained the rows (uniform)
   int cur = -1;
 
+  // the rows' entries i, i + step, ... to ROI roi's accumulators: bin b (or the count below r0, bin nb)
+  // of block pc.  A bin 0 may stand below zero while centrals that met themselves are still to be
+  // taken out; the direct bins' bin nb holds the pairs out of range.
+  auto drain = [&](int roi, uint32_t i, uint32_t step) {
+    unsigned long long* A = a.acc + (size_t)roi * a.acc_len;
+    for (; i < n_rdf; i += step) {
+      const int32_t v = (int32_t)atomicExch(&s_rdf[i], 0u);
+      const uint32_t b = i % (nb + 1);
+      if (v && !(DIRECT && b == nb)) atomicAdd(&A[(i / (nb + 1)) * blk + b], (unsigned long long)(long long)v);
+    }
+  };
   auto flush = [&](int roi) {
     __syncthreads();
+    drain(roi, threadIdx.x, blockDim.x);
     unsigned long long* A = a.acc + (size_t)roi * a.acc_len;
-    for (uint32_t i = threadIdx.x; i < n_rdf; i += blockDim.x) {
-      const unsigned long long v = s_rdf[i];
-      if (!v) continue;
-      // rdf[b] at offset b of block pc, the below-range count at offset nb
-      atomicAdd(&A[(i / (nb + 1)) * blk + i % (nb + 1)], v);
-      s_rdf[i] = 0ull;
-    }
     for (uint32_t i = threadIdx.x; i < P * C; i += blockDim.x) {
       if (s_nc[i]) atomicAdd(&A[i * blk + nb + 1], (unsigned long long)s_nc[i]);
       s_nc[i] = 0;
@@ -155,6 +139,7 @@ __global__ void __launch_bounds__(256, 3) k_batch_query(const BatchArgs a) {
     if (threadIdx.x == 0) {
       const uint32_t ch = atomicAdd(a.next, (uint32_t)kChunk);
       s_chunk = ch;
+      s_next = 0;
       uint32_t lo = 0, hi = a.n_roi;  // item_off[lo] <= ch < item_off[hi]
       if (ch < total)
         while (hi - lo > 1) {
@@ -174,147 +159,142 @@ __global__ void __launch_bounds__(256, 3) k_batch_query(const BatchArgs a) {
       cur = (int)roi;
     }
     const BRoi R = a.roi[roi];
-    const uint32_t l_item = chunk + w - a.item_off[roi];
+    const Geo ng = *R.ngeo;
+    const Search S{R.nrec, R.nstart, R.nsub, a.stencil, a.row_w};
+    const float slack = item_slack(ng);
     const uint32_t n_front = R.cgeo->work_n2, n_items = n_front + R.cgeo->work_n3;
     unsigned long long* A = a.acc + (size_t)roi * a.acc_len;
-    if (l_item < n_items) {
-      const Geo ng = *R.ngeo;
+    for (;;) {
+      uint32_t l_item = 0;
+      if (lane == 0) l_item = atomicAdd(&s_next, 1u);
+      l_item = __shfl_sync(0xffffffffu, l_item, 0);
+      if (l_item >= (uint32_t)kChunk) break;
+      l_item += chunk - a.item_off[roi];
+      if (l_item >= n_items) break;
       const uint2 it = work_item(R.witem, R.cap, n_front, l_item);
-      const uint32_t c = it.x, first = it.y >> 6, cnt = it.y & 63u;
-      const uint32_t c0 = R.cstart[c] + first;
-      // run table
-      uint32_t src = 0, len = 0;
-      {
-        const int s = a.stencil, wd = 2 * s + 1;
-        const uint32_t cx = c % ng.dims[0], cy = (c / ng.dims[0]) % ng.dims[1], cz = c / (ng.dims[0] * ng.dims[1]);
-        const int y = (int)cy + (int)(lane % wd) - s, z = (int)cz + (int)(lane / wd) - s;
-        if ((int)lane < wd * wd && y >= 0 && z >= 0 && y < (int)ng.dims[1] && z < (int)ng.dims[2]) {
-          const uint32_t xlo = cx >= (uint32_t)s ? cx - s : 0;
-          const uint32_t xhi = cx + s < ng.dims[0] ? cx + s : ng.dims[0] - 1;
-          const uint32_t row = ((uint32_t)z * ng.dims[1] + (uint32_t)y) * ng.dims[0];
-          src = R.nstart[row + xlo];
-          len = R.nstart[row + xhi + 1] - src;
-        }
-      }
-      uint32_t pre = len;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, pre, o);
-        if (lane >= (uint32_t)o) pre += y;
-      }
-      const uint32_t n_cand = __shfl_sync(0xffffffffu, pre, 31);
-      uint32_t* rsrc = s_rsrc[w];
-      uint32_t* rpre = s_rpre[w];
-      __syncwarp();
-      if (lane < (uint32_t)kBatchRuns) {
-        rsrc[lane] = src;
-        rpre[lane + 1] = pre;
-      }
-      if (lane == 0) rpre[0] = 0;
-      __syncwarp();
-
-      // this lane's central: type, class, pair membership
-      const bool valid = lane < cnt;
-      float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-      uint32_t pw = ~0u, cls = 0, pmask = 0;
-      if (valid) {
-        p = R.crec[c0 + lane];
-        pw = __float_as_uint(p.w);
-        const uint32_t ti = pw & 0xFFu;
-        const float di = R.dsrf ? R.dsrf[pw >> 8] : INFINITY;
+      const uint32_t c = it.x, cnt = it.y & 63u, c0 = R.cstart[c] + (it.y >> 6);
+      const uint32_t L = item_lanes(cnt), lg = 31u - __clz(L), sub = lane & (L - 1u), ci = lane >> lg;
+      const uint32_t nbat = L > 1u ? 64u : 32u;
+      float4 rec = make_float4(INFINITY, INFINITY, INFINITY, __uint_as_float(~0u));
+      uint32_t cls = 0;
+      if (ci < cnt) {
+        rec = R.crec[c0 + ci];
+        const float di = R.dsrf ? R.dsrf[__float_as_uint(rec.w) >> 8] : INFINITY;
         for (uint32_t q = 1; q < C; ++q)
           if (di >= a.cls_min[q]) cls = q;
-        for (uint32_t pp = 0; pp < P; ++pp)
-          if (mask_has(a.ctr_mask[pp], ti)) pmask |= 1u << pp;
       }
-      const float emax = valid ? Emax : -INFINITY;
-      const uint32_t lt = (1u << lane) - 1u;
-      float top[NL][KMAX];
+      const uint32_t pw = __float_as_uint(rec.w);
+#pragma unroll 1
+      for (uint32_t ps = 0; ps < a.n_pass; ++ps) {
+        // the lane's pair in this pass (the central sets of a pass are disjoint)
+        uint32_t pair = ~0u;
+        if (ci < cnt)
+          for (uint32_t pp = 0; pp < P; ++pp)
+            if (((a.pass_pairs[ps] >> pp) & 1u) && mask_has(a.ctr_mask[pp], pw & 0xFFu)) pair = pp;
+        const bool valid = pair != ~0u;
+        if (__ballot_sync(0xffffffffu, valid) == 0u) continue;
+        const uint32_t pc = valid ? pair * C + cls : 0u, row = rows + 4u * pc * (nb + 1);
+        // lanes without a central never hit (their distances are infinite or NaN)
+        const float4 p = valid ? rec : make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+        const unsigned long long px = f2_pack(p.x, p.x), py = f2_pack(p.y, p.y), pz = f2_pack(p.z, p.z);
+        ItemBox box;
+        box.set(p, valid, ng, slack);
+        float top[KMAX];
 #pragma unroll
-      for (int l = 0; l < NL; ++l)
+        for (int t = 0; t < KMAX; ++t) top[t] = INFINITY;
+        float thr = Emax, near_max = Emax;
+        ItemRing ring{bf, 0, 0, 0};
+        auto batch = [&](uint32_t n) __attribute__((always_inline)) {
+          const ulonglong2* rp = reinterpret_cast<const ulonglong2*>(bf) + (ring.head & (kRing - 1u));
+          const uint32_t n_pr = (n + 1) >> 1;
+#pragma unroll 1
+          for (uint32_t t0 = 0; t0 < n_pr; t0 += 2 * L) {
+            const uint32_t t = t0 + sub;
+            const ulonglong2 xy0 = rp[2 * t], xy1 = rp[2 * (t + L)], zw0 = rp[2 * t + 1], zw1 = rp[2 * (t + L) + 1];
+            const unsigned long long d20 = dist2_x2_fma(px, py, pz, xy0.x, xy0.y, zw0.x, one2);
+            const unsigned long long d21 = dist2_x2_fma(px, py, pz, xy1.x, xy1.y, zw1.x, one2);
+            if (DIRECT) {
+              const uint32_t x = fb.count2(d20, row) | fb.count2(d21, row);
+              if (__any_sync(0xffffffffu, x != 0u)) {
+                fb.settle2(d20, row);
+                fb.settle2(d21, row);
+              }
+            } else {
+              float d[4], wv[4];
+              f2_unpack(d20, d[0], d[1]), f2_unpack(d21, d[2], d[3]);
+              f2_unpack(zw0.y, wv[0], wv[1]), f2_unpack(zw1.y, wv[2], wv[3]);
 #pragma unroll
-        for (int t = 0; t < KMAX; ++t) top[l][t] = INFINITY;
-      const unsigned long long px = f2_pack(p.x, p.x), py = f2_pack(p.y, p.y), pz = f2_pack(p.z, p.z);
-      float* hd = s_hd[w];
-      uint32_t* ht = s_ht[w];
-      float* bf = reinterpret_cast<float*>(s_buf[w]);
-      int rr = 0;
-      auto fetch = [&](uint32_t pos) -> float4 {
-        if (pos >= n_cand) return make_float4(INFINITY, INFINITY, INFINITY, __uint_as_float(~0u));
-        while (pos >= rpre[rr + 1]) ++rr;
-        return __ldg(R.nrec + rsrc[rr] + (pos - rpre[rr]));
-      };
-      float4 nxt = fetch(lane);
-      for (uint32_t b0 = 0; b0 < n_cand; b0 += 32) {
-        __syncwarp();
-        {
-          float* d = bf + (lane >> 1) * 8 + (lane & 1);
-          d[0] = nxt.x, d[2] = nxt.y, d[4] = nxt.z, d[6] = nxt.w;
-        }
-        __syncwarp();
-        nxt = fetch(b0 + 32 + lane);
-        for (int half = 0; half < 2; ++half) {
-          uint32_t nh = 0;
+              for (int e = 0; e < 4; ++e)
+                if (d[e] < Emax && __float_as_uint(wv[e]) != pw) {
+                  const uint32_t bn = d[e] < E0 ? nb : bin_index(d[e], sE, nb, r0f, inv_dr);
+                  red_shared_inc(row + 4u * (kMagicBits + bn));
+                }
+            }
+          }
+          __syncwarp();
+          if ((int32_t)(ring.near_to - ring.head) > 0) {
+#pragma unroll 1
+            for (uint32_t t0 = 0; t0 < n_pr; t0 += 8 * L) {
+              uint32_t qa = q0;
+              const uint32_t t1 = min(n_pr, t0 + 8 * L);
 #pragma unroll 2
-          for (int t = half * 8; t < half * 8 + 8; ++t) {
-            const ulonglong2 xy = reinterpret_cast<const ulonglong2*>(bf)[2 * t];
-            const ulonglong2 zw = reinterpret_cast<const ulonglong2*>(bf)[2 * t + 1];
-            float d2v[2], wv[2];
-            dist2_x2(px, py, pz, xy.x, xy.y, zw.x, d2v[0], d2v[1]);
-            f2_unpack(zw.y, wv[0], wv[1]);
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const uint32_t qw = __float_as_uint(wv[e]);
-              const bool hit = d2v[e] < emax && qw != pw;
-              uint32_t tag = 0;
-              if (hit) {
-                const uint32_t ti = s_tinfo[qw & 0xFFu];
-#pragma unroll
-                for (int l = 0; l < NL; ++l)
-                  if (((ti >> l) & 1u) && d2v[e] < top[l][KMAX - 1]) tk_insert(top[l], d2v[e]);
-                tag = (ti >> 2) & pmask;
+              for (uint32_t t = t0 + sub; t < t1; t += L) {
+                const ulonglong2 xy = rp[2 * t], zw = rp[2 * t + 1];
+                float da, db, wa, wb;
+                f2_unpack(dist2_x2_fma(px, py, pz, xy.x, xy.y, zw.x, one2), da, db);
+                f2_unpack(zw.y, wa, wb);
+                queue_push_other(qa, da, thr, __float_as_uint(wa), pw);
+                queue_push_other(qa, db, thr, __float_as_uint(wb), pw);
               }
-              const bool rec = tag != 0;
-              const uint32_t bal = __ballot_sync(0xffffffffu, rec);
-              if (rec) {
-                const uint32_t slot = nh + __popc(bal & lt);
-                hd[slot] = d2v[e];
-                ht[slot] = tag | (cls << 8);
-              }
-              nh += __popc(bal);
+              __syncwarp();
+              const uint32_t qn = (qa - q0) >> 7, m = __reduce_max_sync(0xffffffffu, qn);
+#pragma unroll 1
+              for (uint32_t q = 0; q < m; ++q)
+                if (q < qn) topk_insert(top, queue_at(q0, q));
+              float kth = top[KMAX - 1];  // an upper bound of the central's k-th distance in each of its lanes
+              for (uint32_t o = 1; o < L; o <<= 1) kth = fminf(kth, __shfl_xor_sync(0xffffffffu, kth, o));
+              thr = fminf(kth, Emax);
             }
+            near_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(valid ? thr : 0.f)));
           }
-          __syncwarp();
-          for (uint32_t h = lane; h < nh; h += 32) {
-            const float d2 = hd[h];
-            const uint32_t tg = ht[h], cc = tg >> 8;
-            const bool below = d2 < E0;
-            const uint32_t bn = below ? 0u : bbin(d2, sE, nb, r0f, inv_dr);
-            for (uint32_t pp = 0; pp < P; ++pp) {
-              if (!((tg >> pp) & 1u)) continue;
-              atomicAdd(&s_rdf[(pp * C + cc) * (nb + 1) + (below ? nb : bn)], 1ull);
-            }
+          added += 32u * 64u;
+          if (added >= (1u << 28) - 4096u) {
+            __syncwarp();
+            drain(cur, lane, 32);
+            added = 0;
           }
+        };
+        const Mask nm = a.nbr[ps];
+        item_scan(S, ng, c, box, ring, nbat, true, Emax, near_max, batch,
+                  [&](float qw) { return in_mask(nm, __float_as_uint(qw) & 0xFFu); });
+        // the centrals whose type is in the neighbour set met themselves once each, at d2 = 0
+        if (DIRECT && valid && sub == 0 && in_mask(nm, pw & 0xFFu) && dist2(p.x, p.y, p.z, p.x, p.y, p.z) == 0.f)
+          red_shared(row + 4u * kMagicBits, ~0u);
+        // merge the partial lists of the L lanes of each central (disjoint candidate subsets)
+        for (uint32_t o = 1; o < L; o <<= 1) {
           __syncwarp();
+#pragma unroll
+          for (int t = 0; t < KMAX; ++t) kq[t * 32 + lane] = top[t];
+          __syncwarp();
+          const float* ot = kq + (lane ^ o);
+#pragma unroll 1
+          for (int t = 0; t < KMAX; ++t) {
+            const float v = ot[t * 32];
+            if (!(v < top[KMAX - 1])) break;  // the partner's list is sorted
+            topk_insert(top, v);
+          }
         }
-      }
-      // per central: counts and the k-th distances of every pair
-      if (valid) {
-        for (uint32_t pp = 0; pp < P; ++pp) {
-          if (!((pmask >> pp) & 1u)) continue;
-          const uint32_t pc = pp * C + cls;
+        __syncwarp();
+        if (valid && sub == 0) {
           atomicAdd(&s_nc[pc], 1u);
-          const uint32_t l = a.list_of[pp];
-          for (uint32_t k = 0; k < a.k_max; ++k) {
-            float D = INFINITY;
 #pragma unroll
-            for (int ll = 0; ll < NL; ++ll)
-              if ((uint32_t)ll == l) D = tk_get(top[ll], k);
-            if (!(D < Emax)) continue;  // not found: derived from the counts
+          for (int t = 0; t < KMAX; ++t) {
+            const float D = top[t];
+            if ((uint32_t)t >= a.k_max || !(D < Emax)) break;  // not found: derived from the counts
             if (D < E0)
-              atomicAdd(&A[pc * blk + nb + 2 + a.k_max * nb + k], 1ull);
+              atomicAdd(&A[pc * blk + nb + 2 + a.k_max * nb + t], 1ull);
             else
-              atomicAdd(&A[pc * blk + nb + 2 + k * nb + bbin(D, sE, nb, r0f, inv_dr)], 1ull);
+              atomicAdd(&A[pc * blk + nb + 2 + t * nb + bin_index(D, sE, nb, r0f, inv_dr)], 1ull);
           }
         }
       }
@@ -410,17 +390,20 @@ struct ps_batch {
   uint32_t* d_next = nullptr;
   uint32_t* d_rbins = nullptr;
   unsigned long long* d_acc = nullptr;
-  uint32_t acc_len = 0, n_lists = 0, list_of[4] = {0, 0, 0, 0};
-  uint64_t list_mask[2][4];
+  uint32_t acc_len = 0, n_pass = 0, pass_pairs[4] = {0, 0, 0, 0};
+  uint64_t pass_nbr[4][4];
   uint64_t nbr_union[4], ctr_union[4];
   float r_cut = 0.f;
 };
 
 using namespace ps;
 
-template <int KMAX, int NL>
-static int launch_batch(const ps_batch* b, const BatchArgs& a, uint32_t smem, int sms, cudaStream_t st) {
-  auto kern = k_batch_query<KMAX, NL>;
+template <int KMAX, bool DIRECT>
+static int launch_batch(const BatchArgs& a, int sms, cudaStream_t st) {
+  auto kern = k_batch_query<KMAX, DIRECT>;
+  // edges, bin rows, central counts, insertion queues
+  const uint32_t smem = (a.n_bins + 1) * 4 + a.n_pairs * a.n_cls * ((a.n_bins + 1) * 4 + 4) +
+                        8u * ((KMAX > (int)kHalf ? KMAX : (int)kHalf) + 1) * 32u * 4u;
   PS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem));
@@ -430,6 +413,13 @@ static int launch_batch(const ps_batch* b, const BatchArgs& a, uint32_t smem, in
   return PS_OK;
 }
 
+template <bool DIRECT>
+static int dispatch_batch(const BatchArgs& a, int sms, cudaStream_t st) {
+  return a.k_max <= 8    ? launch_batch<8, DIRECT>(a, sms, st)
+         : a.k_max <= 16 ? launch_batch<16, DIRECT>(a, sms, st)
+         : a.k_max <= 20 ? launch_batch<20, DIRECT>(a, sms, st)
+                         : launch_batch<32, DIRECT>(a, sms, st);
+}
 
 extern "C" {
 
@@ -458,20 +448,26 @@ int ps_batch_create(const ps_dataset* ds, int n_ds, const ps_sweep* sw, ps_batch
   ps_batch* b = new (std::nothrow) ps_batch();
   if (!b) return fail(PS_ERR_OOM, "host allocation failed");
   b->sw = s;
-  // distinct neighbour sets -> top-k lists
+  // at most two distinct neighbour sets; passes: pairs of one neighbour set with disjoint central sets
+  uint32_t n_sets = 0;
   for (uint32_t p = 0; p < s.n_pairs; ++p) {
-    int found = -1;
-    for (uint32_t l = 0; l < b->n_lists; ++l)
-      if (!memcmp(b->list_mask[l], s.nbr_mask[p], sizeof(uint64_t) * 4)) found = (int)l;
-    if (found < 0) {
-      if (b->n_lists == 2) {
-        delete b;
-        return fail(PS_ERR_UNSUPPORTED, "ps_batch_create: at most 2 distinct neighbour type sets");
-      }
-      memcpy(b->list_mask[b->n_lists], s.nbr_mask[p], sizeof(uint64_t) * 4);
-      found = (int)b->n_lists++;
+    bool known = false;
+    for (uint32_t q = 0; q < p; ++q) known = known || !memcmp(s.nbr_mask[q], s.nbr_mask[p], sizeof(uint64_t) * 4);
+    n_sets += known ? 0u : 1u;
+    if (n_sets > 2) {
+      delete b;
+      return fail(PS_ERR_UNSUPPORTED, "ps_batch_create: at most 2 distinct neighbour type sets");
     }
-    b->list_of[p] = (uint32_t)found;
+    uint32_t ps = 0;
+    for (; ps < b->n_pass; ++ps) {
+      bool fits = !memcmp(b->pass_nbr[ps], s.nbr_mask[p], sizeof(uint64_t) * 4);
+      for (uint32_t q = 0; q < p; ++q)
+        if ((b->pass_pairs[ps] >> q) & 1u)
+          for (int w = 0; w < 4; ++w) fits = fits && (s.ctr_mask[q][w] & s.ctr_mask[p][w]) == 0;
+      if (fits) break;
+    }
+    if (ps == b->n_pass) memcpy(b->pass_nbr[b->n_pass++], s.nbr_mask[p], sizeof(uint64_t) * 4);
+    b->pass_pairs[ps] |= 1u << p;
   }
   for (int w = 0; w < 4; ++w) {
     b->nbr_union[w] = b->ctr_union[w] = 0;
@@ -518,7 +514,7 @@ int ps_batch_create(const ps_dataset* ds, int n_ds, const ps_sweep* sw, ps_batch
   std::vector<BRoi> h(n_ds);
   for (int i = 0; i < n_ds; ++i) {
     ps_grid* g = b->grids[i];
-    h[i] = BRoi{g->nbr.rec, g->nbr.start, g->nbr.geo, g->ctr.rec,       g->ctr.start,
+    h[i] = BRoi{g->nbr.rec, g->nbr.start, g->nbr.count, g->nbr.geo, g->ctr.rec, g->ctr.start,
                 g->ctr.witem, g->ctr.geo,  ds[i].dsrf, g->item_cap};
   }
   e = cudaMemcpy(b->d_roi, h.data(), sizeof(BRoi) * n_ds, cudaMemcpyHostToDevice);
@@ -575,30 +571,23 @@ int ps_batch_run(ps_batch* b, uint64_t* d_out, void* stream) {
   a.n_pairs = s.n_pairs;
   a.n_cls = s.n_dsrf;
   a.k_max = s.k_max;
-  a.n_lists = b->n_lists;
-  for (uint32_t p = 0; p < s.n_pairs; ++p) {
-    a.list_of[p] = b->list_of[p];
-    for (int w = 0; w < 4; ++w) a.ctr_mask[p][w] = s.ctr_mask[p][w], a.nbr_mask[p][w] = s.nbr_mask[p][w];
+  a.n_pass = b->n_pass;
+  a.one = 1.0f;
+  row_widths(b->grids[0]->stencil, b->grids[0]->cell_scale, a.row_w);
+  for (uint32_t p = 0; p < s.n_pairs; ++p)
+    for (int w = 0; w < 4; ++w) a.ctr_mask[p][w] = s.ctr_mask[p][w];
+  for (uint32_t ps = 0; ps < b->n_pass; ++ps) {
+    a.pass_pairs[ps] = b->pass_pairs[ps];
+    for (int w = 0; w < 4; ++w) a.nbr[ps].w[w] = b->pass_nbr[ps][w];
   }
-  for (uint32_t l = 0; l < b->n_lists; ++l)
-    for (int w = 0; w < 4; ++w) a.list_mask[l][w] = b->list_mask[l][w];
   for (uint32_t q = 0; q < s.n_dsrf; ++q) a.cls_min[q] = s.dsrf_min[q];
   a.acc = b->d_acc;
   a.acc_len = b->acc_len;
-  const uint32_t smem = ((s.bins.n_bins + 1) * 4 + 15) / 16 * 16 + s.n_pairs * s.n_dsrf * ((s.bins.n_bins + 1) * 8 + 4);
   const int sms = b->grids[0]->num_sms;
-  int rc;
-  const uint32_t k = s.k_max;
-  if (b->n_lists == 1)
-    rc = k <= 8 ? launch_batch<8, 1>(b, a, smem, sms, st)
-         : k <= 16 ? launch_batch<16, 1>(b, a, smem, sms, st)
-         : k <= 20 ? launch_batch<20, 1>(b, a, smem, sms, st)
-                   : launch_batch<32, 1>(b, a, smem, sms, st);
-  else
-    rc = k <= 8 ? launch_batch<8, 2>(b, a, smem, sms, st)
-         : k <= 16 ? launch_batch<16, 2>(b, a, smem, sms, st)
-         : k <= 20 ? launch_batch<20, 2>(b, a, smem, sms, st)
-                   : launch_batch<32, 2>(b, a, smem, sms, st);
+  // direct bins: r0 = 0 and edges far from the limits of float32 (as the exact query; at most 512 bins)
+  const double stop = (double)s.bins.n_bins * s.bins.dr;
+  const bool direct = s.bins.r0 == 0.0 && s.bins.dr > 1e-15 && stop < 1e15;
+  const int rc = direct ? dispatch_batch<true>(a, sms, st) : dispatch_batch<false>(a, sms, st);
   if (rc) return rc;
   const uint32_t n_out = n_roi * s.n_pairs * s.n_rmax * s.n_dsrf;
   PS_LAUNCH(PS_KID_BATCH, st,

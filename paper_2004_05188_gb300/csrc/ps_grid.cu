@@ -834,9 +834,6 @@ int wait_selftest(uint64_t limit_ns, unsigned long long* d_work, cudaStream_t s)
 
 static int grid_blocks(const ps_grid* g, int per_sm) { return g->num_sms * per_sm; }
 
-// sub-cells only where a cell is as wide as the search range (two- and three-cell stencils are fine enough)
-static uint32_t fine_cap(const ps_grid* g) { return g->stencil == 1 ? g->fine_cap : 0u; }
-
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 static int scan_cells(ps_grid* g, CellList& L, Geo* geo, cudaStream_t s) {
@@ -858,7 +855,7 @@ int build_neighbour_grid(ps_grid* g, const uint64_t nbr_mask[4], float r_cut, cu
     PS_LAUNCH(PS_KID_SELECT, s,
               PS_CUDA(launch_pdl(k_select_bbox, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->type, g->n, m, vec, g->sel, geo)));
   PS_LAUNCH(PS_KID_GEOMETRY, s,
-            PS_CUDA(launch_pdl(k_geometry_zero, grid_blocks(g, 4), kThreads, 0, s, geo, r_cut, g->cell_scale, g->cell_cap, fine_cap(g), g->nbr.count)));
+            PS_CUDA(launch_pdl(k_geometry_zero, grid_blocks(g, 4), kThreads, 0, s, geo, r_cut, g->cell_scale, g->cell_cap, g->fine_cap, g->nbr.count)));
   PS_LAUNCH(PS_KID_COUNT, s, PS_CUDA(launch_pdl(k_count, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->sel, geo, g->nbr.count, g->cr)));
   int rc = scan_cells(g, g->nbr, geo, s);
   if (rc) return rc;
@@ -912,7 +909,7 @@ int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4]
   }
   const bool vec = aligned16(g->type) && aligned16(g->xyz) && (dsrf == nullptr || aligned16(dsrf));
   PS_LAUNCH(PS_KID_CENTRAL, s,
-            PS_CUDA(launch_pdl(k_central_reset, grid_blocks(g, 4), kThreads, 0, s, g->nbr.geo, g->ctr.geo, g->ctr.count, z, (uint64_t)g->n, fine_cap(g))));
+            PS_CUDA(launch_pdl(k_central_reset, grid_blocks(g, 4), kThreads, 0, s, g->nbr.geo, g->ctr.geo, g->ctr.count, z, (uint64_t)g->n, g->fine_cap)));
   if (g->n > 0)
     PS_LAUNCH(PS_KID_CENTRAL, s,
               PS_CUDA(launch_pdl(k_central_select_count, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->type, dsrf, g->n, m, dsrf_min,

@@ -93,7 +93,7 @@ struct Geo {
 // box, so the groups should be compact.  Ordering the records of a cell by its octants (2 nm cells
 // at 30 ions/nm^3: 240 records, 30 per octant) shrinks a group's box from the cell to about two
 // octants, the volume within 2 nm of it from 165 to 106 nm^3.  Cells of 48 records on average are
-// split once, of 512 twice; sparser ones are a group or two anyway.  `cap` entries of counts (0: no sub-cells).
+// split once, of 512 twice; sparser ones are a group or two anyway.  `cap` entries of counts.
 __host__ __device__ __forceinline__ uint32_t sub_cells(uint64_t n_rec, uint64_t n_cells, uint64_t cap) {
   uint32_t s = n_rec >= 512 * n_cells ? 2u : (n_rec >= 48 * n_cells ? 1u : 0u);
   while (s && (n_cells << (3 * s)) > cap) --s;

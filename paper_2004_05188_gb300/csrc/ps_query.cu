@@ -35,11 +35,10 @@
 #include <vector>
 
 #include "ps_internal.cuh"
+#include "ps_items.cuh"
 #include "ps_sweep.cuh"
 
 namespace ps {
-
-constexpr int kMaxRuns = 49;  // (2 * stencil + 1)^2 for stencil <= 3
 
 // One-pass queries whose centrals are neighbour records: in dense clouds the RDF is left to the sweep
 // over unordered pairs (half the tests, no kNN beside them), in sparse ones the blocks of the
@@ -97,60 +96,7 @@ struct QueryArgs {
   int8_t row_w[kMaxRuns];
 };
 
-template <int K>
-__device__ __forceinline__ void topk_insert(float (&top)[K], float x) {
-  if (x < top[K - 1]) {
-#pragma unroll
-    for (int t = K - 1; t > 0; --t) top[t] = fminf(top[t], fmaxf(x, top[t - 1]));
-    top[0] = fminf(top[0], x);
-  }
-}
-
-template <int K>
-__device__ __forceinline__ float topk_get(const float (&top)[K], uint32_t idx) {
-  float v = INFINITY;
-#pragma unroll
-  for (int t = 0; t < K; ++t)
-    if ((uint32_t)t == idx) v = top[t];
-  return v;
-}
-
-// bin b in [0, nb) with sE[b] <= d2 < sE[b+1]; caller guarantees sE[0] <= d2 < sE[nb].
-// The guess from an approximate square root is checked against the exact edge
-// table; the (rare) wrong guess is walked to the right bin.
-__device__ __forceinline__ uint32_t bin_index(float d2, const float* sE, uint32_t nb, float r0f, float inv_dr) {
-  const float d = d2 > 0.f ? d2 * rsqrtf(d2) : 0.f;
-  int b = (int)((d - r0f) * inv_dr);
-  b = b < 0 ? 0 : (b >= (int)nb ? (int)nb - 1 : b);
-  if (d2 < sE[b] || d2 >= sE[b + 1]) {
-    while (b > 0 && d2 < sE[b]) --b;
-    while (b + 1 < (int)nb && d2 >= sE[b + 1]) ++b;
-  }
-  return (uint32_t)b;
-}
-
-// Insertion queue of a lane: a column of a [row][32 lanes] array, `at` the shared address of its next
-// slot.  Every value is stored and the slot taken only if it is below thr: no branch, and one
-// predicated add per value.
-__device__ __forceinline__ void queue_push(uint32_t& at, float v, float thr) {
-  asm volatile(
-      "{\n .reg .pred p;\n st.shared.f32 [%0], %1;\n setp.lt.f32 p, %1, %2;\n @p add.u32 %0, %0, 128;\n}"
-      : "+r"(at)
-      : "f"(v), "f"(thr));
-}
-// the same for a candidate of index word j, other than the lane's central (index word own)
-__device__ __forceinline__ void queue_push_other(uint32_t& at, float v, float thr, uint32_t j, uint32_t own) {
-  asm volatile(
-      "{\n .reg .pred p;\n st.shared.f32 [%0], %1;\n setp.ne.u32 p, %3, %4;\n setp.lt.and.f32 p, %1, %2, p;\n"
-      " @p add.u32 %0, %0, 128;\n}"
-      : "+r"(at)
-      : "f"(v), "f"(thr), "r"(j), "r"(own));
-}
-__device__ __forceinline__ float queue_at(uint32_t first, uint32_t q) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(first + 128u * q));
-  return v;
-}
+__device__ __forceinline__ Search search_of(const QueryArgs& a) { return Search{a.nrec, a.nstart, a.nsub, a.stencil, a.row_w}; }
 
 struct SmemLayout {
   uint32_t off_E, off_lut, off_rdf, off_knn, off_kmeta, off_stage, total;
@@ -390,91 +336,6 @@ __device__ __forceinline__ void add_pair_counters(const QueryArgs& a, uint64_t b
   }
 }
 
-// Rows of the stencil, nearest first: (dy, dz) ordered by dy^2 + dz^2 (the first 9 entries are
-// the 3 x 3 rows of the 27-cell stencil, the first 25 the 5 x 5 rows).  Walking the central row
-// first lets the k-th distance of every central settle early, so later candidates rarely enter
-// the top-k lists.
-__constant__ signed char c_row_dy[kMaxRuns] = {0, -1, 1, 0, 0, -1, 1, -1, 1, -2, 2, 0, 0, -2, 2, -2, 2,
-                                               -1, 1, -1, 1, -2, 2, -2, 2, 0, 0, -3, 3, -1, 1, -1, 1,
-                                               -3, 3, -3, 3, -2, 2, -2, 2, -3, 3, -3, 3, -3, 3, -3, 3};
-__constant__ signed char c_row_dz[kMaxRuns] = {0, 0, 0, -1, 1, -1, -1, 1, 1, 0, 0, -2, 2, -1, -1, 1, 1,
-                                               -2, -2, 2, 2, -2, -2, 2, 2, -3, 3, 0, 0, -3, -3, 3, 3,
-                                               -1, -1, 1, 1, -3, -3, 3, 3, -2, -2, 2, 2, -3, -3, 3, 3};
-
-__device__ __forceinline__ int row_width(const QueryArgs& a, int dy, int dz) {
-  const int s = a.stencil;
-  return a.row_w[(dz + s) * (2 * s + 1) + dy + s];
-}
-
-// x-run of cells cx - w .. cx + w (clipped to the grid) of row (y, z): its records
-__device__ __forceinline__ void row_run(const QueryArgs& a, const Geo& ng, uint32_t cx, int y, int z, int w,
-                                        uint32_t& src, uint32_t& len) {
-  src = 0;
-  len = 0;
-  if (w < 0 || y < 0 || z < 0 || y >= (int)ng.dims[1] || z >= (int)ng.dims[2]) return;
-  const uint32_t xlo = cx >= (uint32_t)w ? cx - w : 0;
-  const uint32_t xhi = cx + w < ng.dims[0] ? cx + w : ng.dims[0] - 1;
-  const uint32_t row = ((uint32_t)z * ng.dims[1] + (uint32_t)y) * ng.dims[0];
-  src = a.nstart[row + xlo];
-  len = a.nstart[row + xhi + 1] - src;
-}
-
-// cell c -> run r of its stencil: the x-contiguous records of cells (cx-w .. cx+w, cy+dy, cz+dz)
-__device__ __forceinline__ void cell_run(const QueryArgs& a, const Geo& ng, uint32_t c, uint32_t r, uint32_t& src,
-                                         uint32_t& len) {
-  const int s = a.stencil, w = 2 * s + 1;
-  const uint32_t cx = c % ng.dims[0], cy = (c / ng.dims[0]) % ng.dims[1], cz = c / (ng.dims[0] * ng.dims[1]);
-  src = 0;
-  len = 0;
-  if ((int)r >= w * w) return;
-  const int dy = c_row_dy[r], dz = c_row_dz[r];
-  row_run(a, ng, cx, (int)cy + dy, (int)cz + dz, row_width(a, dy, dz), src, len);
-}
-
-// Run r of the candidates of an item whose box, in cell edges, is ulo .. uhi.  Cells without sub-cells:
-// the own cell, the own row to its left and to its right, then rows 1 .. of the stencil (nearest
-// first).  With them (27-cell stencils), the x-rods of 2^sub sub-cells, cell by cell from the own row
-// outwards, those out of reach left empty: a 2 nm cell's 27 cells hold 216 octants, an octant's
-// items reach 105 of them within 2 nm and about 27 within a 10th-neighbour distance.
-__device__ __forceinline__ uint32_t item_runs(const QueryArgs& a, const Geo& ng) {
-  const uint32_t W = 2 * a.stencil + 1;
-  return ng.sub ? W * W * W << (2 * ng.sub) : W * W + 2;
-}
-__device__ __forceinline__ void item_run(const QueryArgs& a, const Geo& ng, uint32_t c, uint32_t r, const float (&ulo)[3],
-                                         const float (&uhi)[3], float lim_u, uint32_t& src, uint32_t& len) {
-  src = 0, len = 0;
-  if (r >= item_runs(a, ng)) return;
-  if (ng.sub) {
-    const uint32_t W = 2 * a.stencil + 1, cell = r >> (2 * ng.sub), yz = r & ((1u << (2 * ng.sub)) - 1u);
-    const int row = (int)(cell / W), q = (int)(cell - row * W), dx = q & 1 ? -((q + 1) >> 1) : q >> 1;  // 0 -1 1 -2 2 ..
-    const int x = (int)(c % ng.dims[0]) + dx, y = (int)((c / ng.dims[0]) % ng.dims[1]) + c_row_dy[row],
-              z = (int)(c / (ng.dims[0] * ng.dims[1])) + c_row_dz[row];
-    if (x < 0 || y < 0 || z < 0 || x >= (int)ng.dims[0] || y >= (int)ng.dims[1] || z >= (int)ng.dims[2]) return;
-    const float e = 1.0f / (float)(1u << ng.sub);
-    const float y0 = (float)y + e * (float)(yz & ((1u << ng.sub) - 1u)), z0 = (float)z + e * (float)(yz >> ng.sub);
-    const float gx = fmaxf(0.f, fmaxf((float)x - uhi[0], ulo[0] - (float)(x + 1)));
-    const float gy = fmaxf(0.f, fmaxf(y0 - uhi[1], ulo[1] - (y0 + e)));
-    const float gz = fmaxf(0.f, fmaxf(z0 - uhi[2], ulo[2] - (z0 + e)));
-    if (gx * gx + gy * gy + gz * gz > lim_u) return;  // (a NaN box keeps the rod)
-    const uint32_t cc = ((uint32_t)z * ng.dims[1] + (uint32_t)y) * ng.dims[0] + (uint32_t)x;
-    const uint32_t f = (cc << (3 * ng.sub)) | (yz << ng.sub), f1 = f + (1u << ng.sub);
-    src = a.nsub[f];
-    len = (f1 == ng.n_cells << (3 * ng.sub) ? ng.n_sel : a.nsub[f1]) - src;
-    return;
-  }
-  if (r >= 3) {
-    cell_run(a, ng, c, r - 2, src, len);
-    return;
-  }
-  const uint32_t row = c - c % ng.dims[0], cx = c - row, w = (uint32_t)row_width(a, 0, 0);
-  const uint32_t lo = r == 0 ? cx : (r == 1 ? (cx >= w ? cx - w : 0u) : cx + 1);
-  const uint32_t hi = r == 0 ? cx + 1 : (r == 1 ? cx : min(cx + w, ng.dims[0] - 1) + 1);
-  if (lo < hi) {
-    src = a.nstart[row + lo];
-    len = a.nstart[row + hi] - src;
-  }
-}
-
 // Near kNN pass of the query in passes (vertex != 0): the central list is sorted by the grid
 // of cells centred on the vertices of the neighbour grid (vg: origin half a cell lower, one more
 // cell per axis), so the centrals of item cell c are those nearest to vertex V = c's coordinates,
@@ -530,69 +391,6 @@ __device__ __forceinline__ void list_append(const QueryArgs& a, bool miss, uint3
 __device__ __forceinline__ float4 far_record() { return make_float4(INFINITY, INFINITY, INFINITY, __uint_as_float(~0u)); }
 
 // ---------------------------------------------------------------------------
-// direct bins (r0 = 0)
-// ---------------------------------------------------------------------------
-constexpr float kBinBias = 1.0f / 2097152.0f;   // 2^-21
-
-__device__ __forceinline__ void red_shared_inc(uint32_t addr) {
-  asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr));
-}
-__device__ __forceinline__ void red_shared(uint32_t addr, uint32_t v) {
-  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v));
-}
-
-// Bins of the direct form (r0 = 0).  With s = sqrt.approx(d2) and inv = (1 +- 2^-21) / dr, the true
-// quotient sqrt(d2) / dr lies between s * inv- and s * inv+ (the root is good to 2^-23, inv to 2^-24,
-// the edge table to 2^-25 of the distance).  The bin is floor(s * inv+), or the one below where the two floors
-// differ (2 in 10^4 pairs at 200 bins): those compare d2 with that edge.  Pairs out of range are
-// clamped into the unused bin n_bins, so that every lane increments and no instruction is
-// predicated: the compiler branches around a predicated shared-memory increment.  Measured on the
-// pair loop alone (cycles per 32 tests and scheduler): 23 with a predicated increment and the excess over
-// the edge computed, 17 in this form, of which 14.5 are the distance, root and floor; no table load per pair, so
-// the shared-memory pipe is left to the increments (increments by one merge in a bin).
-struct FastBins {
-  const float* sE;
-  unsigned long long hi2, lo2, magic2;
-  float s_far;
-  __device__ void init(const QueryArgs& a, const float* edges) {
-    sE = edges;
-    const float hi = (float)((1.0 + (double)kBinBias) / a.dr), lo = (float)((1.0 - (double)kBinBias) / a.dr);
-    hi2 = f2_pack(hi, hi);
-    lo2 = f2_pack(lo, lo);
-    magic2 = f2_pack(kMagic, kMagic);
-    s_far = (float)(((double)a.n_bins + 0.5) * a.dr);
-  }
-  // counts two pairs in the row at shared address `base` (bin b at base + 4 (kMagicBits + b));
-  // returns 0 unless one of them may lie under the edge of its bin
-  __device__ __forceinline__ uint32_t count2(unsigned long long d2, uint32_t base) const {
-    float da, db, ma, mb, la, lb;
-    f2_unpack(d2, da, db);
-    const unsigned long long s2 = f2_pack(fminf(sqrt_fast(da), s_far), fminf(sqrt_fast(db), s_far));
-    f2_unpack(f2_fma_down(s2, hi2, magic2), ma, mb);
-    f2_unpack(f2_fma_down(s2, lo2, magic2), la, lb);
-    red_shared_inc(__float_as_uint(ma) * 4u + base);
-    red_shared_inc(__float_as_uint(mb) * 4u + base);
-    return (__float_as_uint(ma) ^ __float_as_uint(la)) | (__float_as_uint(mb) ^ __float_as_uint(lb));
-  }
-  // a counted pair that may lie under the edge of its bin: moved to the bin below if it does
-  __device__ __forceinline__ void settle(float d2, uint32_t base) const {
-    float m, x;
-    f2_unpack(f2_fma_down(f2_pack(fminf(sqrt_fast(d2), s_far), 0.f), hi2, magic2), m, x);
-    const uint32_t addr = __float_as_uint(m) * 4u + base;
-    if (d2 < sE[__float_as_uint(m) - kMagicBits]) {
-      red_shared(addr, ~0u);
-      red_shared_inc(addr - 4u);
-    }
-  }
-  __device__ __forceinline__ void settle2(unsigned long long d2, uint32_t base) const {
-    float da, db;
-    f2_unpack(d2, da, db);
-    settle(da, base);
-    settle(db, base);
-  }
-};
-
-// ---------------------------------------------------------------------------
 // warp kernel
 //   heavy items (cells with >= kHeavy centrals, batches of 4..32 centrals): one to eight lanes per
 //     central (item_lanes).  The candidates are read 32 at a time, the stencil's rows nearest
@@ -605,9 +403,7 @@ struct FastBins {
 //     time and gives each of their centrals a thread of its own that walks its
 //     own stencil (the records of neighbouring centrals' cells hit in L1).
 // ---------------------------------------------------------------------------
-constexpr uint32_t kHalf = 16;                 // candidates per staging half-batch
 constexpr uint32_t kRowLaneCap = 1u << 25;     // per-central increments of the 32-bit warp row, then global
-constexpr uint32_t kRing = 128;                // candidates kept for testing (a batch of 64 and 32 more)
 constexpr int kNoRdf = 0, kRdfGeneral = 1, kRdfDirect = 2;
 
 // Bound by instruction issue, and on small or clustered clouds by the chain of one item.  Where the
@@ -627,15 +423,15 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __
   Hist<RDF> H{};
   H.init(a, smem, 0, true);
   FastBins fb;
-  if (MODE == kRdfDirect) fb.init(a, H.sE);
+  if (MODE == kRdfDirect) fb.init(a.n_bins, a.dr, H.sE);
   const uint32_t row_base = smem_u32(H.s_rdfw) - 4u * kMagicBits;
   const unsigned long long one2 = f2_pack(a.one, a.one);
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint64_t wcount = 0;  // increments of this warp's private row since its last flush (uniform)
   const Geo ng = *a.ngeo;
   const uint32_t n_hi = a.cgeo->work_n4, n_front = n_hi + a.cgeo->work_n2, n_light = a.cgeo->work_n3;
-  const int n_runs = (int)item_runs(a, ng);
-  const float u_slack = (float)max(ng.dims[0], max(ng.dims[1], ng.dims[2])) * 5.0e-7f + 1.0e-6f;  // rounding of (x - origin) inv_h
+  const Search S = search_of(a);
+  const float u_slack = item_slack(ng);
   const bool swept = a.sweep && sweep_pays(ng);  // RDF and in-range counts are the sweep's
   const bool rdf_here = RDF && !swept;
   uint32_t* const nwithin = swept ? nullptr : a.nwithin;
@@ -669,19 +465,8 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __
     const uint32_t pidx = valid ? __float_as_uint(p.w) : ~0u;
     const float emax = erange;
     const unsigned long long px = f2_pack(p.x, p.x), py = f2_pack(p.y, p.y), pz = f2_pack(p.z, p.z);
-    // bounding box of the centrals as mid +- half (half rounded up)
-    float mid[3], half[3], ulo[3], uhi[3];
-    {
-      const float pc[3] = {p.x, p.y, p.z};
-#pragma unroll
-      for (int ax = 0; ax < 3; ++ax) {
-        const float lo = key2f(__reduce_min_sync(0xffffffffu, f2key(valid ? pc[ax] : INFINITY)));
-        const float hi = key2f(__reduce_max_sync(0xffffffffu, f2key(valid ? pc[ax] : -INFINITY)));
-        mid[ax] = 0.5f * (lo + hi);
-        half[ax] = fmaxf(hi - mid[ax], mid[ax] - lo) * 1.000001f + fabsf(mid[ax]) * 2.4e-7f;
-        ulo[ax] = (lo - ng.origin[ax]) * ng.inv_h - u_slack, uhi[ax] = (hi - ng.origin[ax]) * ng.inv_h + u_slack;
-      }
-    }
+    ItemBox box;
+    box.set(p, valid, ng, u_slack);
     float top[KK];
 #pragma unroll
     for (int t = 0; t < KK; ++t) top[t] = INFINITY;
@@ -690,22 +475,21 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __
     float thr = KMAX > 0 ? emax : -INFINITY;
     float near_max = fmaxf(thr, 0.f);  // the largest over the warp
     const bool all = rdf_here || nwithin != nullptr;  // every in-range pair counts, not the nearest alone
-    // ring of kept candidates: slots [head, tail); those from near_to on are beyond near_max.  Items
-    // whose lanes share centrals take 64 at a time, so that each lane has enough of them.
+    // items whose lanes share centrals take 64 candidates at a time, so that each lane has enough of them
     const uint32_t nb = L > 1u ? 64u : 32u;
-    uint32_t head = 0, tail = 0, near_to = 0;
+    ItemRing ring{bf, 0, 0, 0};
 
-    // tests the nb ring slots from `head`, of which n hold candidates
+    // tests the nb ring slots from the head, of which n hold candidates
     auto batch = [&](uint32_t n) __attribute__((always_inline)) {
-      const ulonglong2* ring = reinterpret_cast<const ulonglong2*>(bf) + (head & (kRing - 1u));
+      const ulonglong2* rp = reinterpret_cast<const ulonglong2*>(bf) + (ring.head & (kRing - 1u));
       const uint32_t n_pr = (n + 1) >> 1;
       if (all) {
         // two pairs of candidates at a time (beyond the last there are far ones to the end of the batch)
 #pragma unroll 1
         for (uint32_t t0 = 0; t0 < n_pr; t0 += 2 * L) {
           const uint32_t t = t0 + sub;
-          const ulonglong2 xy0 = ring[2 * t], xy1 = ring[2 * (t + L)];
-          const unsigned long long z0 = ring[2 * t + 1].x, z1 = ring[2 * (t + L) + 1].x;
+          const ulonglong2 xy0 = rp[2 * t], xy1 = rp[2 * (t + L)];
+          const unsigned long long z0 = rp[2 * t + 1].x, z1 = rp[2 * (t + L) + 1].x;
           const unsigned long long d20 = dist2_x2_fma(px, py, pz, xy0.x, xy0.y, z0, one2);
           const unsigned long long d21 = dist2_x2_fma(px, py, pz, xy1.x, xy1.y, z1, one2);
           float d[4];
@@ -721,7 +505,7 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __
           if (MODE == kRdfGeneral && rdf_here) {
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-              if (d[e] < emax && __float_as_uint(bf[4 * (head & (kRing - 1u)) + (t + (e >> 1) * L) * 8 + 6 + (e & 1)]) != pidx)
+              if (d[e] < emax && __float_as_uint(bf[4 * (ring.head & (kRing - 1u)) + (t + (e >> 1) * L) * 8 + 6 + (e & 1)]) != pidx)
                 H.pair(a, d[e], my_below);
           }
           if (nwithin != nullptr)
@@ -729,7 +513,7 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __
         }
         __syncwarp();
       }
-      if (KMAX > 0 && (int32_t)(near_to - head) > 0) {
+      if (KMAX > 0 && (int32_t)(ring.near_to - ring.head) > 0) {
         // candidates below the lane's bound go to its queue column (unconditional stores at the next
         // slot, kept only if counted), inserted every 16 pairs of the lanes
 #pragma unroll 1
@@ -738,7 +522,7 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __
           const uint32_t t1 = min(n_pr, t0 + 8 * L);
 #pragma unroll 2
           for (uint32_t t = t0 + sub; t < t1; t += L) {
-            const ulonglong2 xy = ring[2 * t], zw = ring[2 * t + 1];
+            const ulonglong2 xy = rp[2 * t], zw = rp[2 * t + 1];
             float da, db, wa, wb;
             f2_unpack(dist2_x2_fma(px, py, pz, xy.x, xy.y, zw.x, one2), da, db);
             f2_unpack(zw.y, wa, wb);
@@ -764,76 +548,7 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __
       }
     };
 
-    for (int r0 = 0; r0 < n_runs; r0 += 32) {
-      // lane r: run r0 + r
-      uint32_t rs = 0, rl = 0;
-      item_run(a, ng, c, (uint32_t)r0 + lane, ulo, uhi, (all ? emax : near_max) * 1.0001f * ng.inv_h * ng.inv_h, rs, rl);
-      // the runs as one list: lane r holds the position at which run r starts and, less that, its first
-      // record; a position's run is found by bisection over the lanes (runs of sparse sets hold a few
-      // records each, and a round of 32 loads per run would be mostly idle)
-      uint32_t pre = rl;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, pre, o);
-        if (lane >= (uint32_t)o) pre += y;
-      }
-      const uint32_t n_list = __shfl_sync(0xffffffffu, pre, 31);
-      pre -= rl;
-      const uint32_t first = rs - pre;
-      auto fetch = [&](uint32_t pos) -> float4 {
-        uint32_t r = 0;
-#pragma unroll
-        for (uint32_t st = 16; st > 0; st >>= 1)
-          if (__shfl_sync(0xffffffffu, pre, r + st) <= pos) r += st;
-        const uint32_t j = __shfl_sync(0xffffffffu, first, r) + pos;
-        return pos < n_list ? __ldg(a.nrec + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-      };
-      // one candidate per lane: into the ring if it is within reach
-      auto offer = [&](const float4& q, bool ok) {
-        const float ex = fmaxf(fabsf(q.x - mid[0]) - half[0], 0.f);
-        const float ey = fmaxf(fabsf(q.y - mid[1]) - half[1], 0.f);
-        const float ez = fmaxf(fabsf(q.z - mid[2]) - half[2], 0.f);
-        // (the factor covers the rounding of both distances)
-        const float e2 = __fmaf_rn(ez, ez, __fmaf_rn(ey, ey, ex * ex)) * 0.99999f;
-        const bool close = ok && e2 < near_max;
-        const bool keep = all ? ok && e2 < emax : close;
-        const uint32_t bal = __ballot_sync(0xffffffffu, keep);
-        if (keep) {
-          const uint32_t slot = (tail + __popc(bal & ((1u << lane) - 1u))) & (kRing - 1u);
-          float* d = bf + (slot >> 1) * 8 + (slot & 1u);
-          d[0] = q.x, d[2] = q.y, d[4] = q.z, d[6] = q.w;
-        }
-        tail += __popc(bal);
-        if (__any_sync(0xffffffffu, close)) near_to = tail;
-      };
-      float4 n0 = fetch(lane), n1 = fetch(32 + lane);
-      for (uint32_t o = 0; o < n_list; o += 64) {
-        const float4 c0 = n0, c1 = n1;
-        n0 = fetch(o + 64 + lane);
-        if (o + 96 < n_list) n1 = fetch(o + 96 + lane);
-        offer(c0, o + lane < n_list);
-        if (o + 32 < n_list) offer(c1, o + 32 + lane < n_list);
-        while (tail - head >= nb) {
-          __syncwarp();
-          batch(nb);
-          head += nb;
-          __syncwarp();
-        }
-      }
-    }
-    if (tail != head) {
-      // the last, partial batch: far records to its end
-      const uint32_t n = tail - head;
-      for (uint32_t h = lane; h < nb; h += 32)
-        if (h >= n) {
-          const uint32_t slot = (head + h) & (kRing - 1u);
-          float* d = bf + (slot >> 1) * 8 + (slot & 1u);
-          d[0] = INFINITY, d[2] = INFINITY, d[4] = INFINITY, d[6] = __uint_as_float(~0u);
-        }
-      __syncwarp();
-      batch(n);
-      __syncwarp();
-    }
+    item_scan(S, ng, c, box, ring, nb, all, emax, near_max, batch, [](float) { return true; });
     if (all) {
       // the centrals met themselves once each, at d2 = 0 (a non-finite one did not)
       bool self = valid && sub == 0 && dist2(p.x, p.y, p.z, p.x, p.y, p.z) == 0.f;
@@ -931,7 +646,7 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __
         for (int dz = -st; dz <= st; ++dz)
           for (int dy = -st; dy <= st; ++dy) {
             uint32_t j0 = 0, nj = 0;
-            row_run(a, ng, cx, (int)cy + dy, (int)cz + dz, row_width(a, dy, dz), j0, nj);
+            row_run(S, ng, cx, (int)cy + dy, (int)cz + dz, row_width(S, dy, dz), j0, nj);
             const uint32_t j1 = j0 + nj;
             for (uint32_t j = j0; j < j1; ++j) {
               const float4 q = __ldg(a.nrec + j);
@@ -976,9 +691,10 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __
 // CTA kernel: one CTA per dense cell, runs staged in shared memory by bulk copies
 // ---------------------------------------------------------------------------
 template <int KMAX, bool RDF>
-__global__ void __launch_bounds__(256) k_query_cta(const QueryArgs a) {
+__global__ void __launch_bounds__(256) k_query_cta(const __grid_constant__ QueryArgs a) {
   griddep_wait();
   griddep_launch();
+  const Search S = search_of(a);
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ uint64_t bar;
   __shared__ uint32_t s_item;
@@ -1010,7 +726,7 @@ __global__ void __launch_bounds__(256) k_query_cta(const QueryArgs a) {
     if (item >= work_n || s_timeout) break;
     const uint32_t c = a.cwork[item];
     const uint32_t c0 = a.cstart[c], n_c = a.cstart[c + 1] - c0;
-    if (tid < n_runs) cell_run(a, ng, c, tid, s_run_src[tid], s_run_len[tid]);
+    if (tid < n_runs) cell_run(S, ng, c, tid, s_run_src[tid], s_run_len[tid]);
     __syncthreads();
 
     for (uint32_t cb = 0; cb < n_c; cb += blockDim.x) {
@@ -1132,7 +848,7 @@ __global__ void __launch_bounds__(256, WITHIN ? 3 : 4) k_rdf_sym(const QueryArgs
     for (uint32_t b = threadIdx.x; b < 16 * stride; b += blockDim.x) rows[b] = 0;
     __syncthreads();
     FastBins fb;
-    fb.init(a, sE);
+    fb.init(a.n_bins, a.dr, sE);
     uint32_t* row1 = rows + 2 * w * stride;
     const uint32_t a1 = smem_u32(row1), base1 = a1 - 4u * kMagicBits, base2 = base1 + 4u * stride;
     const unsigned long long one2 = f2_pack(sw.one, sw.one);
@@ -1451,9 +1167,10 @@ static int dispatch_knn_vertex(const ps_grid* g, const QueryArgs& qa, uint32_t s
 // first) with the k_need smallest d2 below E[nb] kept through the per-lane queue; fewer than k of
 // them: not found (INF).
 template <int KMAX>
-__global__ void __launch_bounds__(256) k_knn_list(const QueryArgs a) {
+__global__ void __launch_bounds__(256) k_knn_list(const __grid_constant__ QueryArgs a) {
   griddep_wait();
   griddep_launch();
+  const Search S = search_of(a);
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ float s_kq[8][17 * 32];
   Hist<false> H{};
@@ -1526,12 +1243,12 @@ __global__ void __launch_bounds__(256) k_knn_list(const QueryArgs a) {
     if (__ballot_sync(0xffffffffu, more)) {
       // tier B: the outer cells of the inner rows, then the outer rows, each within its width
       for (int r = 0; r < 9; ++r) {
-        const int dy = c_row_dy[r], dz = c_row_dz[r], wd = valid ? row_width(a, dy, dz) : -1;
+        const int dy = c_row_dy[r], dz = c_row_dz[r], wd = valid ? row_width(S, dy, dz) : -1;
         walk(more && wd >= 2, cc[1] + dy, cc[2] + dz, cc[0] - wd, cc[0] - 2);
         walk(more && wd >= 2, cc[1] + dy, cc[2] + dz, cc[0] + 2, cc[0] + wd);
       }
       for (int r = 9; r < n_rows; ++r) {
-        const int dy = c_row_dy[r], dz = c_row_dz[r], wd = valid ? row_width(a, dy, dz) : -1;
+        const int dy = c_row_dy[r], dz = c_row_dz[r], wd = valid ? row_width(S, dy, dz) : -1;
         walk(more && wd >= 0, cc[1] + dy, cc[2] + dz, cc[0] - wd, cc[0] + wd);
       }
     }

@@ -96,3 +96,25 @@ def test_batched_256_rois_full_size_sampled(ps, spec):
         np.testing.assert_array_equal(meta, o["meta"].cpu().numpy())
         g.close()
     b.close()
+
+
+@pytest.mark.parametrize("bins,k_max", [((0.0, 0.05, 30), 1), ((0.0, 0.004, 400), 32), ((0.3, 0.04, 30), 17)])
+@pytest.mark.parametrize("pairs", [[("all", "all"), ([1], "all"), ([0, 2], "all"), ([2], [1])],
+                                   [([0], [1]), ([1], [1]), ([0, 1], [1]), ([0, 1, 2], [0])]])
+def test_batched_pairs_that_share_a_neighbour_set(ps, orc, spec, bins, k_max, pairs):
+    """Overlapping and disjoint central sets on one neighbour set (searched apart and together),
+    r0 > 0, the shortest and longest k lists, coincident ions."""
+    xyz, t, d = spec.cube(91, 2500, 4.5, (0.6, 0.25, 0.15))
+    xyz, t, d = (np.concatenate([v, v[:30]]) for v in (xyz, t, d))
+    roi = tuple(torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (xyz, t, d))
+    nb = bins[2]
+    b = ps.Batch([roi], bins, [nb // 2, nb], [0.0, 0.7], pairs, k_max)
+    rdf, knn, meta = b.split(b.run().cpu().numpy())
+    for p, (ctr, nbr) in enumerate(pairs):
+        for q, dmin in enumerate([0.0, 0.7]):
+            r = orc.spatstat(xyz, t, d, ctr, nbr, dmin, *bins, list(range(1, k_max + 1)))
+            np.testing.assert_array_equal(rdf[0, p, 1, q].astype(np.uint64), r["rdf"])
+            np.testing.assert_array_equal(knn[0, p, 1, q].astype(np.uint64), r["knn"])
+            assert meta[0, p, 1, q, 0] == r["n_central"]
+            np.testing.assert_array_equal(meta[0, p, 1, q, 4::2].astype(np.uint64), r["not_found"])
+    b.close()
