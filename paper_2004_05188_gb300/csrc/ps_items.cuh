@@ -307,32 +307,30 @@ __device__ __forceinline__ void item_scan(const Search& S, const Geo& ng, uint32
       if (__any_sync(0xffffffffu, close)) R.near_to = R.tail;
     };
     float4 n0 = fetch(lane), n1 = fetch(32 + lane);
-    for (uint32_t o = 0; o < n_list; o += 64) {
+    const bool last = r0 + 32 >= n_runs;
+    for (uint32_t o = 0; o < n_list || (last && o == 0u); o += 64) {
       const float4 c0 = n0, c1 = n1;
       n0 = fetch(o + 64 + lane);
       if (o + 96 < n_list) n1 = fetch(o + 96 + lane);
       offer(c0, o + lane < n_list);
       if (o + 32 < n_list) offer(c1, o + 32 + lane < n_list);
-      while (R.tail - R.head >= nb) {
+      // full batches, and at the very end the rest (one call of batch: the kernels' speed depends on
+      // their code size)
+      const bool end = last && o + 64 >= n_list;
+      while (R.tail - R.head >= nb || (end && R.tail != R.head)) {
+        const uint32_t n = min(R.tail - R.head, nb);
+        for (uint32_t h = n + lane; h < nb; h += 32) {  // far records to the end of the last batch
+          const uint32_t slot = (R.head + h) & (kRing - 1u);
+          float* d = R.bf + (slot >> 1) * 8 + (slot & 1u);
+          d[0] = INFINITY, d[2] = INFINITY, d[4] = INFINITY, d[6] = __uint_as_float(~0u);
+        }
         __syncwarp();
-        batch(nb);
+        batch(n);
         R.head += nb;
         __syncwarp();
+        if (n < nb) R.tail = R.head;
       }
     }
-  }
-  if (R.tail != R.head) {
-    // the last, partial batch: far records to its end
-    const uint32_t n = R.tail - R.head;
-    for (uint32_t h = lane; h < nb; h += 32)
-      if (h >= n) {
-        const uint32_t slot = (R.head + h) & (kRing - 1u);
-        float* d = R.bf + (slot >> 1) * 8 + (slot & 1u);
-        d[0] = INFINITY, d[2] = INFINITY, d[4] = INFINITY, d[6] = __uint_as_float(~0u);
-      }
-    __syncwarp();
-    batch(n);
-    __syncwarp();
   }
 }
 
