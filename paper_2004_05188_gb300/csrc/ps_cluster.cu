@@ -5,11 +5,14 @@
 //
 // Ions of the grid's set are linked when d2 <= (float)(d_max^2); the clusters
 // are the connected components with at least N_min ions.  GPU form: a
-// lock-free union-find over the grid's sorted records.  Every record tests the
-// later records of its stencil; a link hooks the larger root under the smaller
-// one with a compare-and-swap (a failed swap means another thread hooked that
-// root, so every retry follows someone's progress), so each component ends
-// rooted at its smallest record.  Then the paths are compressed and every
+// lock-free union-find over the grid's sorted records.  Every record first hooks
+// itself under the first record within reach (earlier than itself; no other thread
+// writes that parent), and the trees that this gives, a few links deep, are
+// flattened: most neighbours then share their root.  Then every record tests the
+// earlier records of its stencil again; a link between different roots hooks the
+// larger under the smaller one with a compare-and-swap (a failed swap means another
+// thread hooked that root, so every retry follows someone's progress), so each
+// component ends rooted at its smallest record.  Then the paths are compressed and every
 // root gathers its size, the smallest original index of its ions (the
 // cluster's label) and the smallest d_srf of its ions (interior test).
 // Scratch: the grid's central-list records (unused between queries).
@@ -84,47 +87,86 @@ __device__ __forceinline__ uint32_t rec_index(const ClusterArgs& a, float w) {
   return a.packed ? (u >> 8) : u;
 }
 
-__global__ void __launch_bounds__(256) k_cl_init(const ClusterArgs a) {
+// f(j, d2) for the records j < s of the stencil of record s, in ascending order while it returns true
+template <class F>
+__device__ __forceinline__ void cl_earlier(const ClusterArgs& a, const Geo& g, uint32_t s, F&& f) {
+  const int st = a.stencil;
+  const float4 p = __ldg(a.rec + s);
+  const uint32_t c = cell_of(g, p.x, p.y, p.z);
+  const uint32_t cx = c % g.dims[0], cy = (c / g.dims[0]) % g.dims[1], cz = c / (g.dims[0] * g.dims[1]);
+  const uint32_t xlo = cx >= (uint32_t)st ? cx - st : 0;
+  const uint32_t xhi = cx + st < g.dims[0] ? cx + st : g.dims[0] - 1;
+  const int ylo = max((int)cy - st, 0), zlo = max((int)cz - st, 0);
+  for (int z = zlo; z <= (int)cz; ++z) {
+    const int yhi = z == (int)cz ? (int)cy : min((int)cy + st, (int)g.dims[1] - 1);
+    for (int y = ylo; y <= yhi; ++y) {
+      const uint32_t row = ((uint32_t)z * g.dims[1] + (uint32_t)y) * g.dims[0];
+      const uint32_t j1 = min(a.start[row + xhi + 1], s);
+      for (uint32_t j = a.start[row + xlo]; j < j1; ++j) {
+        const float4 q = __ldg(a.rec + j);
+        if (!f(j, dist2(p.x, p.y, p.z, q.x, q.y, q.z))) return;
+      }
+    }
+  }
+}
+
+// every record under the first record within d_max of it, if there is an earlier one (parent written by
+// its own thread alone; the rest of the init beside it)
+__global__ void __launch_bounds__(256) k_cl_hook(const ClusterArgs a) {
   griddep_wait();
   griddep_launch();
-  const uint32_t ns = a.geo->n_sel;
+  const Geo g = *a.geo;
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t s = tid; s < ns; s += stride) {
-    a.parent[s] = (uint32_t)s;
+  for (uint64_t s = tid; s < g.n_sel; s += stride) {
+    uint32_t first = (uint32_t)s;
+    cl_earlier(a, g, (uint32_t)s, [&](uint32_t j, float d2) {
+      if (!(d2 <= a.D)) return true;
+      first = j;
+      return false;
+    });
+    a.parent[s] = first;
     a.size[s] = 0;
     a.cmin[s] = 0xFFFFFFFFu;
     a.dkey[s] = f2key(INFINITY);
   }
-  for (uint64_t i = tid; i < (uint64_t)a.n; i += stride) a.label[i] = 0xFFFFFFFFu;
+  // outputs: four labels at a time
+  const uint64_t n4 = (reinterpret_cast<uintptr_t>(a.label) & 15u) == 0 ? (uint64_t)a.n / 4 : 0;
+  for (uint64_t i = tid; i < n4; i += stride) reinterpret_cast<uint4*>(a.label)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+  for (uint64_t i = 4 * n4 + tid; i < (uint64_t)a.n; i += stride) a.label[i] = 0xFFFFFFFFu;
   for (uint64_t b = tid; b < a.hist_len; b += stride) a.size_hist[b] = 0ull, a.interior_hist[b] = 0ull;
   if (tid < PS_CLUSTER_META_LEN) a.meta[tid] = 0ull;
 }
 
-// every record links to the later records of its stencil within d_max
+// flattens the trees: every record under its root (a thread that reads a parent another one has
+// already replaced by the root only gets there sooner)
+__global__ void __launch_bounds__(256) k_cl_flatten(const ClusterArgs a) {
+  griddep_wait();
+  griddep_launch();
+  const uint32_t ns = a.geo->n_sel;
+  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < ns; s += gridDim.x * blockDim.x) {
+    uint32_t r = ld_rlx(a.parent + s), p = ld_rlx(a.parent + r);
+    while (p != r) r = p, p = ld_rlx(a.parent + r);
+    st_rlx(a.parent + s, r);
+  }
+}
+
+// every record links to the earlier records of its stencil within d_max whose root differs.  Bound by the
+// latency of the dependent loads of one record's walk.  8e6-ion needle, Sc, d_max = 0.5 nm (us): 236 -> 105 for the
+// links (with every record its own root at first, each link climbed and hooked trees hundreds of
+// links deep), the whole pass 334 -> 186.
 __global__ void __launch_bounds__(256) k_cl_link(const ClusterArgs a) {
   griddep_wait();
   griddep_launch();
   const Geo g = *a.geo;
-  const int st = a.stencil;
   for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < g.n_sel; s += gridDim.x * blockDim.x) {
-    const float4 p = __ldg(a.rec + s);
-    const uint32_t c = cell_of(g, p.x, p.y, p.z);
-    const uint32_t cx = c % g.dims[0], cy = (c / g.dims[0]) % g.dims[1], cz = c / (g.dims[0] * g.dims[1]);
-    const uint32_t xlo = cx >= (uint32_t)st ? cx - st : 0;
-    const uint32_t xhi = cx + st < g.dims[0] ? cx + st : g.dims[0] - 1;
-    const int ylo = max((int)cy - st, 0), yhi = min((int)cy + st, (int)g.dims[1] - 1);
-    const int zlo = max((int)cz - st, 0), zhi = min((int)cz + st, (int)g.dims[2] - 1);
-    for (int z = zlo; z <= zhi; ++z)
-      for (int y = ylo; y <= yhi; ++y) {
-        const uint32_t row = ((uint32_t)z * g.dims[1] + (uint32_t)y) * g.dims[0];
-        const uint32_t j1 = a.start[row + xhi + 1];
-        uint32_t j = a.start[row + xlo];
-        j = j > s ? j : s + 1;
-        for (; j < j1; ++j) {
-          const float4 q = __ldg(a.rec + j);
-          if (dist2(p.x, p.y, p.z, q.x, q.y, q.z) <= a.D) cl_unite(a.parent, s, j);
-        }
+    uint32_t root = cl_find(a.parent, s);
+    cl_earlier(a, g, s, [&](uint32_t j, float d2) {
+      if (d2 <= a.D && ld_rlx(a.parent + j) != root) {
+        cl_unite(a.parent, s, j);
+        root = cl_find(a.parent, s);
       }
+      return true;
+    });
   }
 }
 
@@ -209,7 +251,8 @@ int run_cluster(ps_grid* g, const float* dsrf, ps_cluster_spec spec, uint32_t* d
   a.interior_hist = reinterpret_cast<unsigned long long*>(d_interior_hist);
   a.meta = reinterpret_cast<unsigned long long*>(d_meta);
   const int blocks = g->num_sms * 8;
-  PS_LAUNCH(PS_KID_CLUSTER, s, PS_CUDA(launch_pdl(k_cl_init, blocks, 256, 0, s, a)));
+  PS_LAUNCH(PS_KID_CLUSTER, s, PS_CUDA(launch_pdl(k_cl_hook, blocks, 256, 0, s, a)));
+  PS_LAUNCH(PS_KID_CLUSTER, s, PS_CUDA(launch_pdl(k_cl_flatten, blocks, 256, 0, s, a)));
   PS_LAUNCH(PS_KID_CLUSTER, s, PS_CUDA(launch_pdl(k_cl_link, blocks, 256, 0, s, a)));
   PS_LAUNCH(PS_KID_CLUSTER, s, PS_CUDA(launch_pdl(k_cl_gather, blocks, 256, 0, s, a)));
   PS_LAUNCH(PS_KID_CLUSTER, s, PS_CUDA(launch_pdl(k_cl_final, blocks, 256, 0, s, a)));

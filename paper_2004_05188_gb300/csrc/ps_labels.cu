@@ -42,16 +42,24 @@ __global__ void __launch_bounds__(256) k_shuffle_labels(const uint8_t* __restric
   griddep_launch();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t domain = 1ull << (2 * key.h);
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    uint64_t y = feistel4(i, key);
-    // cycle walking: the cycle through i returns below n within `domain` steps
-    for (uint64_t w = 0; y >= n && w < domain; ++w) y = feistel4(y, key);
-    if (y >= n) {  // not reachable for a permutation; never read out of bounds
+  // One step of the permutation per turn: a thread whose value is below n writes it and goes on to its
+  // next ion, one whose value is not walks on along the cycle.  The lanes of a warp so never wait for
+  // the longest walk among them (up to 3 of 4 values are walked on).
+  uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, y = i, walked = 0;
+  while (i < n) {
+    y = feistel4(y, key);
+    // the cycle through i returns below n within `domain` steps
+    if (y >= n && ++walked > domain) {  // not reachable for a permutation; never read out of bounds
       if (status) atomicCAS(status, 0, (int)PS_ERR_INVALID_INPUT);
       y = i;
     }
-    out[i] = in[y];
-    if (perm) perm[i] = (uint32_t)y;
+    if (y < n) {
+      out[i] = in[y];
+      if (perm) perm[i] = (uint32_t)y;
+      i += stride;
+      y = i;
+      walked = 0;
+    }
   }
 }
 
