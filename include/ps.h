@@ -413,7 +413,7 @@ PS_API int ps_spatstat_static(const float* xyz, const uint8_t* type, const float
  *                     ps_prof_enable; waits for the recorded events.
  */
 typedef enum {
-  PS_KID_RESET = 1,      /* grid reset */
+  PS_KID_RESET = 1,      /* no launches of its own (the resets ride on the build kernels) */
   PS_KID_SELECT = 2,     /* neighbour-set selection + bounding box */
   PS_KID_GEOMETRY = 3,   /* cell geometry + zeroing of the counts */
   PS_KID_COUNT = 4,      /* cell index + rank of the neighbours */

@@ -9,7 +9,7 @@
 // spatial splitting"), records sorted by cell as float4 (x, y, z, index).
 //
 // Pipeline (all on the device, no host synchronisation):
-//   reset -> select + bounding box -> geometry + zero counts -> count ranks
+//   select + bounding box -> geometry + zero counts -> count ranks
 //   -> single-pass exclusive scan (decoupled look-back) -> scatter
 // The selection kernels read 16 type labels per thread (one 16-byte load).
 #include <cstring>
@@ -108,22 +108,6 @@ __device__ __forceinline__ void load_types16(const uint8_t* __restrict__ type, i
   }
 }
 
-__global__ void k_reset(Geo* geo) {
-  griddep_wait();
-  griddep_launch();
-  if (threadIdx.x == 0) {
-    for (int a = 0; a < 3; ++a) {
-      geo->bbox_key[a] = f2key(INFINITY);
-      geo->bbox_key[3 + a] = f2key(-INFINITY);
-    }
-    geo->n_sel = 0;
-    geo->status = 0;
-    geo->work_n = geo->work_n2 = geo->work_n3 = geo->work_n4 = 0;
-    geo->work_next = geo->work_next2 = geo->work_next3 = 0;
-    geo->work_next2b = geo->work_next3b = geo->sym_next = geo->list_n = geo->sub = 0;
-  }
-}
-
 __device__ __forceinline__ void box_add(float (&lo)[3], float (&hi)[3], bool& bad, float x, float y, float z) {
   if (finite3(x, y, z)) {
     lo[0] = fminf(lo[0], x), hi[0] = fmaxf(hi[0], x);
@@ -156,7 +140,7 @@ __global__ void __launch_bounds__(kThreads) k_select_bbox(const float* __restric
       for (int k = 0; k < kGroup; ++k) m |= (in_mask(mask, t[k]) ? 1u : 0u) << k;
       m &= valid;
     }
-    const uint32_t total = tile_list(s_list, m, &geo->n_sel);
+    const uint32_t total = tile_list(s_list, m, &geo->acc_sel);
     const int64_t i0 = base * kGroup;
 #pragma unroll 4
     for (uint32_t q = threadIdx.x; q < total; q += kThreads) {
@@ -186,11 +170,11 @@ __global__ void __launch_bounds__(kThreads) k_select_bbox(const float* __restric
     float l = INFINITY, h = -INFINITY;
     for (int w = 0; w < kThreads / 32; ++w) l = fminf(l, s_lo[a][w]), h = fmaxf(h, s_hi[a][w]);
     if (l <= h) {
-      atomicMin(&geo->bbox_key[a], f2key(l));
-      atomicMax(&geo->bbox_key[3 + a], f2key(h));
+      atomicMax(&geo->acc_box[a], ~((uint32_t)f2key(l) ^ 0x80000000u));
+      atomicMax(&geo->acc_box[3 + a], (uint32_t)f2key(h) ^ 0x80000000u);
     }
   }
-  if (threadIdx.x == 0 && s_bad) atomicCAS(&geo->status, 0, (int)PS_ERR_INVALID_INPUT);
+  if (threadIdx.x == 0 && s_bad) atomicCAS(&geo->acc_status, 0, (int)PS_ERR_INVALID_INPUT);
 }
 
 // Cell geometry from the bounding box.  The cell edge carries a margin so that
@@ -199,10 +183,10 @@ __global__ void __launch_bounds__(kThreads) k_select_bbox(const float* __restric
 // extent * 2^-20 (cell_scale >= 1/stencil).
 __device__ void compute_geometry(const Geo& in, float r_cut, float cell_scale, uint32_t cell_cap, Geo& out) {
   double lo[3], hi[3];
-  const bool empty = in.n_sel == 0 || in.bbox_key[0] > in.bbox_key[3];
+  const bool empty = in.acc_sel == 0 || in.acc_box[0] == 0;
   for (int a = 0; a < 3; ++a) {
-    lo[a] = empty ? 0.0 : (double)key2f(in.bbox_key[a]);
-    hi[a] = empty ? 0.0 : (double)key2f(in.bbox_key[3 + a]);
+    lo[a] = empty ? 0.0 : (double)key2f((int32_t)(~in.acc_box[a] ^ 0x80000000u));
+    hi[a] = empty ? 0.0 : (double)key2f((int32_t)(in.acc_box[3 + a] ^ 0x80000000u));
   }
   double ext = 0.0;
   for (int a = 0; a < 3; ++a) ext = fmax(ext, hi[a] - lo[a]);
@@ -240,10 +224,15 @@ __global__ void __launch_bounds__(kThreads) k_geometry_zero(Geo* geo, float r_cu
   if (threadIdx.x == 0) {
     Geo g = *geo;
     compute_geometry(g, r_cut, cell_scale, cell_cap, g);
-    const uint32_t sub = sub_cells(g.n_sel, g.n_cells, fine_cap);
+    const uint32_t sub = sub_cells(g.acc_sel, g.n_cells, fine_cap);
     s_nc = g.n_cells << (3 * sub);
     if (blockIdx.x == 0) {
       geo->sub = sub;
+      geo->n_sel = g.acc_sel;
+      geo->status = g.acc_status;
+      geo->work_n = geo->work_n2 = geo->work_n3 = geo->work_n4 = 0;
+      geo->work_next = geo->work_next2 = geo->work_next3 = 0;
+      geo->work_next2b = geo->work_next3b = geo->sym_next = geo->list_n = 0;
       for (int a = 0; a < 3; ++a) geo->origin[a] = g.origin[a], geo->dims[a] = g.dims[a];
       geo->h = g.h;
       geo->inv_h = g.inv_h;
@@ -257,11 +246,19 @@ __global__ void __launch_bounds__(kThreads) k_geometry_zero(Geo* geo, float r_cu
 
 // Cell index and rank (arrival order within the cell) of every selected ion.
 __global__ void __launch_bounds__(kThreads) k_count(const float* __restrict__ xyz, const uint32_t* __restrict__ sel,
-                                                    const Geo* __restrict__ geo, uint32_t* __restrict__ count,
+                                                    Geo* geo, uint32_t* __restrict__ count,
                                                     uint2* __restrict__ cr) {
   griddep_wait();
   griddep_launch();
   const Geo g = *geo;
+  if (blockIdx.x == 0 && threadIdx.x < 8) {  // the selection's accumulators, for the next build
+    if (threadIdx.x < 6)
+      geo->acc_box[threadIdx.x] = 0;
+    else if (threadIdx.x == 6)
+      geo->acc_sel = 0;
+    else
+      geo->acc_status = 0;
+  }
   for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < g.n_sel; s += gridDim.x * blockDim.x) {
     const uint32_t i = sel[s];
     const uint32_t c = fine_of(g, g.sub, xyz[3 * (int64_t)i], xyz[3 * (int64_t)i + 1], xyz[3 * (int64_t)i + 2]);
@@ -352,7 +349,7 @@ __global__ void k_central_reset(const Geo* __restrict__ ngeo, Geo* cgeo, uint32_
   }
   const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
   for (uint32_t c = tid; c < nc; c += stride) count[c] = 0;
-  for (int k = 0; k < 3; ++k)
+  for (int k = 0; k < 4; ++k)
     if (z.p[k])
       for (uint32_t i = tid; i < z.n[k]; i += stride) z.p[k][i] = 0ull;
 }
@@ -557,9 +554,15 @@ __device__ __forceinline__ void emit_items(const uint32_t (&v)[N], uint32_t c0, 
   }
 }
 
+// Where the work lists of a counting-sorted central list are made: large grids in the scan, which holds
+// the counts already (1.1e7-ion cylinder, 1.2e7 cells: 0.44 ms against 0.64 with a second pass over
+// the cells), small ones and those with sub-cells, one cell per thread, by k_central_items.
+__device__ __forceinline__ bool emit_in_scan(const Geo& g) { return g.sub == 0u && g.n_cells >= (1u << 18); }
+
 // Single-pass exclusive scan of the cell (or sub-cell) counts (decoupled look-back): the cells' starts
 // and the end sentinel; the counts of sub-cells are replaced by their starts, which the scatter
-// reads.  With `work` given (no sub-cells), also the work lists (emit_items).
+// reads.  With `work` given, also the work lists (emit_items;
+// for a central list with a neighbour grid `nstart` where emit_in_scan says so).
 __global__ void __launch_bounds__(kScanThreads) k_scan(uint32_t* __restrict__ count, Geo* geo,
                                                        uint32_t* __restrict__ start, uint32_t* __restrict__ work,
                                                        uint2* __restrict__ witem, uint32_t dense_min, uint32_t cap,
@@ -603,7 +606,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(uint32_t* __restrict__ co
       }
       run += v[k];
     }
-    if (work != nullptr) emit_items(v, c0, nc, geo, work, witem, dense_min, cap, nstart, stencil, split, whi);
+    if (work != nullptr && (nstart == nullptr || emit_in_scan(*geo)))
+      emit_items(v, c0, nc, geo, work, witem, dense_min, cap, nstart, stencil, split, whi);
     __syncthreads();  // s_tile and s_prefix are rewritten next
   }
   scan_finish(state, ctr, tiles);
@@ -638,7 +642,6 @@ __global__ void __launch_bounds__(kScanThreads) k_central_subset(const float4* _
     const float half = vcount ? __fmul_rn(0.5f, ngeo->h) : 0.0f;
     for (int a = 0; a < 3; ++a)
       cgeo->origin[a] = __fsub_rn(ngeo->origin[a], half), cgeo->dims[a] = ngeo->dims[a] + (vcount ? 1u : 0u);
-    for (int a = 0; a < 6; ++a) cgeo->bbox_key[a] = ngeo->bbox_key[a];
     cgeo->inv_h = ngeo->inv_h;
     cgeo->h = ngeo->h;
     cgeo->n_cells = vcount ? nvc : ngeo->n_cells;
@@ -650,7 +653,7 @@ __global__ void __launch_bounds__(kScanThreads) k_central_subset(const float4* _
   }
   {
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < 4; ++k)
       if (z.p[k])
         for (uint32_t i = tid; i < z.n[k]; i += stride) z.p[k][i] = 0ull;
     if (vcount)
@@ -709,6 +712,7 @@ __global__ void __launch_bounds__(kThreads) k_central_items(const uint32_t* __re
                                                             int stencil, bool split, uint2* __restrict__ whi) {
   griddep_wait();
   griddep_launch();
+  if (!pfx && emit_in_scan(*cgeo)) return;
   const uint32_t nc = cgeo->n_cells;
   // after a look-back that gave up (status set) the prefixes may be inconsistent: no work items
   const bool ok = cgeo->status == 0;
@@ -825,11 +829,12 @@ static int grid_blocks(const ps_grid* g, int per_sm) { return g->num_sms * per_s
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-static int scan_cells(ps_grid* g, CellList& L, Geo* geo, cudaStream_t s) {
+static int scan_cells(ps_grid* g, CellList& L, Geo* geo, bool with_work, cudaStream_t s, bool split = false) {
   PS_LAUNCH(PS_KID_SCAN, s,
-            PS_CUDA(launch_pdl(k_scan, grid_blocks(g, 1), kScanThreads, 0, s, L.count, geo, L.start, (uint32_t*)nullptr,
-                               L.witem, g->dense_min, g->item_cap, g->scan_state, g->scan_ctr, (const uint32_t*)nullptr,
-                               g->stencil, false, (uint2*)nullptr)));
+            PS_CUDA(launch_pdl(k_scan, grid_blocks(g, 1), kScanThreads, 0, s, L.count, geo, L.start,
+                               with_work ? L.work : (uint32_t*)nullptr, L.witem, g->dense_min, g->item_cap, g->scan_state,
+                               g->scan_ctr, with_work ? g->nbr.start : (uint32_t*)nullptr, g->stencil, split,
+                               split ? g->nbr_witem : (uint2*)nullptr)));
   PS_CUDA(cudaGetLastError());
   return PS_OK;
 }
@@ -839,14 +844,13 @@ int build_neighbour_grid(ps_grid* g, const uint64_t nbr_mask[4], float r_cut, cu
   for (int w = 0; w < 4; ++w) m.w[w] = nbr_mask[w], g->nbr_mask[w] = nbr_mask[w];
   Geo* geo = g->nbr.geo;
   const bool vec = aligned16(g->type) && aligned16(g->xyz);
-  PS_LAUNCH(PS_KID_RESET, s, PS_CUDA(launch_pdl(k_reset, 1, 32, 0, s, geo)));
   if (g->n > 0)
     PS_LAUNCH(PS_KID_SELECT, s,
               PS_CUDA(launch_pdl(k_select_bbox, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->type, g->n, m, vec, g->sel, geo)));
   PS_LAUNCH(PS_KID_GEOMETRY, s,
             PS_CUDA(launch_pdl(k_geometry_zero, grid_blocks(g, 4), kThreads, 0, s, geo, r_cut, g->cell_scale, g->cell_cap, g->fine_cap, g->nbr.count)));
   PS_LAUNCH(PS_KID_COUNT, s, PS_CUDA(launch_pdl(k_count, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->sel, geo, g->nbr.count, g->cr)));
-  int rc = scan_cells(g, g->nbr, geo, s);
+  int rc = scan_cells(g, g->nbr, geo, false, s);
   if (rc) return rc;
   PS_LAUNCH(PS_KID_SCATTER, s,
             PS_CUDA(launch_pdl(k_scatter, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->sel, g->cr, g->nbr.start, g->nbr.count, geo, g->nbr.rec,
@@ -904,7 +908,7 @@ int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4]
               PS_CUDA(launch_pdl(k_central_select_count, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->type, dsrf, g->n, m, dsrf_min,
                                                                               vec, g->nbr.geo, g->ctr.geo, g->ctr.count,
                                                                               g->sel, g->cr)));
-  int rc = scan_cells(g, g->ctr, g->ctr.geo, s);
+  int rc = scan_cells(g, g->ctr, g->ctr.geo, true, s, split);
   if (rc) return rc;
   PS_LAUNCH(PS_KID_SCAN, s,
             PS_CUDA(launch_pdl(k_central_items, grid_blocks(g, 4), kThreads, 0, s, g->nbr.start, (const uint32_t*)nullptr,

@@ -72,7 +72,11 @@ struct Geo {
   uint32_t dims[3];
   uint32_t n_cells;
   uint32_t n_sel;   // ions in the set
-  int32_t bbox_key[6];  // order-preserving int keys of min xyz, max xyz
+  // the selection's accumulators, zero between builds (the count kernel clears them for the next one):
+  // largest ~key of min xyz and key of max xyz, ordered as unsigned (0: none), ions, status
+  uint32_t acc_box[6];
+  uint32_t acc_sel;
+  int32_t acc_status;
   int32_t status;   // device-side ps_status
   uint32_t work_n;     // dense cells in work[] (CTA-staged kernel)
   uint32_t work_n2;    // warp items from the front of witem[] (warp kernel)
@@ -231,8 +235,8 @@ int check_spatstat_args(const char* who, const uint64_t* ctr_mask, float dsrf_mi
 int build_neighbour_grid(ps_grid* g, const uint64_t nbr_mask[4], float r_cut, cudaStream_t s);
 // output arrays a central-list reset also zeroes (null pointers are skipped)
 struct ZeroOut {
-  uint64_t* p[3] = {nullptr, nullptr, nullptr};
-  uint32_t n[3] = {0, 0, 0};
+  uint64_t* p[4] = {nullptr, nullptr, nullptr, nullptr};
+  uint32_t n[4] = {0, 0, 0, 0};
 };
 // split: size the warp items of dense cells for lanes_per_central (the exact query's staged path);
 // vertex: centrals among the neighbour records sorted by the vertex-centred grid (the query in

@@ -205,6 +205,16 @@ struct FastBins {
     red_shared_inc(__float_as_uint(mb) * 4u + base);
     return (__float_as_uint(ma) ^ __float_as_uint(la)) | (__float_as_uint(mb) ^ __float_as_uint(lb));
   }
+  // counts one pair in range
+  __device__ __forceinline__ void count1(float d2, uint32_t base) const {
+    float m, l, x;
+    const unsigned long long s2 = f2_pack(sqrt_fast(d2), 0.f);
+    f2_unpack(f2_fma_down(s2, hi2, magic2), m, x);
+    f2_unpack(f2_fma_down(s2, lo2, magic2), l, x);
+    uint32_t b = __float_as_uint(m);
+    if (b != __float_as_uint(l) && d2 < sE[b - kMagicBits]) --b;
+    red_shared_inc(b * 4u + base);
+  }
   // a counted pair that may lie under the edge of its bin: moved to the bin below if it does
   __device__ __forceinline__ void settle(float d2, uint32_t base) const {
     float m, x;

@@ -411,7 +411,7 @@ constexpr int kNoRdf = 0, kRdfGeneral = 1, kRdfDirect = 2;
 // cylinder, 2 nm cells, 0.325 ms walking every record of the 27 cells, 0.163 ms with the sub-cells out of
 // reach left out.
 template <int KMAX, int MODE>
-__global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __grid_constant__ QueryArgs a) {
+__global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : 2) k_query_warp(const __grid_constant__ QueryArgs a) {
   constexpr bool RDF = MODE != kNoRdf;
   griddep_wait();
   griddep_launch();
@@ -654,8 +654,12 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 3 : 2) k_query_warp(const __
               if (d2 < erange && __float_as_uint(q.w) != pidx) {
                 ++within;
                 if (rdf_here) {
-                  if (within <= kRowLaneCap)
-                    H.pair(a, d2, my_below);
+                  if (within <= kRowLaneCap) {
+                    if (MODE == kRdfDirect)
+                      fb.count1(d2, row_base);
+                    else
+                      H.pair(a, d2, my_below);
+                  }
                   else
                     H.pair_global(a, d2, 1u, my_binned, my_below);
                 }
@@ -970,21 +974,6 @@ __global__ void __launch_bounds__(256, WITHIN ? 3 : 4) k_rdf_sym(const QueryArgs
   }
 }
 
-// in-range neighbours of the central records (record order; each met itself once) to their ions
-__global__ void __launch_bounds__(256) k_within_out(const QueryArgs a, const uint32_t* __restrict__ pfx,
-                                                    const uint32_t* __restrict__ wacc) {
-  griddep_wait();
-  griddep_launch();
-  if (!sweep_pays(*a.ngeo)) return;
-  const uint32_t n = a.ngeo->n_sel;
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    if (pfx[j + 1] == pfx[j]) continue;
-    const float4 p = __ldg(a.nrec + j);
-    const bool self = dist2(p.x, p.y, p.z, p.x, p.y, p.z) == 0.f;
-    a.nwithin[__float_as_uint(p.w)] = wacc[j] - (uint32_t)self;
-  }
-}
-
 template <bool FAST, bool WITHIN>
 static int launch_rdf_sym(const ps_grid* g, const QueryArgs& qa, const SweepArgs& sw, uint32_t smem, uint32_t* wacc,
                           cudaStream_t s) {
@@ -994,8 +983,6 @@ static int launch_rdf_sym(const ps_grid* g, const QueryArgs& qa, const SweepArgs
   PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem));
   if (per_sm < 1) return fail(PS_ERR_UNSUPPORTED, "symmetric RDF kernel does not fit on an SM");
   PS_LAUNCH(PS_KID_RDF_SYM, s, PS_CUDA(launch_pdl(k, g->num_sms * per_sm, 256, smem, s, qa, sw, wacc)));
-  if (WITHIN)
-    PS_LAUNCH(PS_KID_RDF_SYM, s, PS_CUDA(launch_pdl(k_within_out, g->num_sms * 8, 256, 0, s, qa, sw.pfx, (const uint32_t*)wacc)));
   return PS_OK;
 }
 
@@ -1281,11 +1268,24 @@ static int dispatch_knn_list(const ps_grid* g, const QueryArgs& qa, uint32_t sme
   return launch_knn_list<32>(g, qa, smem, s);
 }
 
-// Writes n_central and the device status into the meta array.
-__global__ void k_query_epilogue(const Geo* __restrict__ ngeo, const Geo* __restrict__ cgeo, uint64_t* meta) {
+// Writes n_central and the device status into the meta array, and the in-range counts that the sweep
+// took (wacc, record order; each central met itself once) to their ions.
+__global__ void __launch_bounds__(256) k_query_epilogue(const Geo* __restrict__ ngeo, const Geo* __restrict__ cgeo,
+                                                        uint64_t* meta, const float4* __restrict__ nrec,
+                                                        const uint32_t* __restrict__ pfx,
+                                                        const uint32_t* __restrict__ wacc, uint32_t* __restrict__ nwithin) {
   griddep_wait();
   griddep_launch();
-  if (threadIdx.x == 0) {
+  if (wacc != nullptr && sweep_pays(*ngeo)) {
+    const uint32_t n = ngeo->n_sel;
+    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+      if (pfx[j + 1] == pfx[j]) continue;
+      const float4 p = __ldg(nrec + j);
+      const bool self = dist2(p.x, p.y, p.z, p.x, p.y, p.z) == 0.f;
+      nwithin[__float_as_uint(p.w)] = wacc[j] - (uint32_t)self;
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
     meta[PS_META_N_CENTRAL] = cgeo->n_sel;
     int st = cgeo->status;
     if (st == 0) st = ngeo->status;
@@ -1405,6 +1405,14 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
   z.n[0] = PS_META_LEN(n_k);
   if (rdf) z.p[1] = d_rdf, z.n[1] = bins.n_bins;
   if (n_k) z.p[2] = d_knn, z.n[2] = n_k * bins.n_bins;
+  // one-pass queries: the sweep takes dense clouds (sweep_pays); its in-range counts, in record order, in
+  // the counting sort's index list, free until the next build
+  const bool in_passes = g->split && centrals_in_neighbours(g, ctr_mask) && rdf && d_nwithin == nullptr && g->stencil >= 2 &&
+                         g->dense_min == 0xFFFFFFFFu;
+  const bool sweep = !in_passes && rdf && centrals_in_neighbours(g, ctr_mask) && g->dense_min == 0xFFFFFFFFu &&
+                     (direct || d_nwithin == nullptr);
+  uint32_t* wacc = sweep && d_nwithin != nullptr ? g->sel : nullptr;
+  if (wacc) z.p[3] = reinterpret_cast<uint64_t*>(wacc), z.n[3] = (uint32_t)(((uint64_t)g->n + 1) / 2);
 
   const bool subset = centrals_in_neighbours(g, ctr_mask);
   qa.self_all = subset;
@@ -1413,7 +1421,7 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
   qa.one = 1.0f;
   // the query in passes, and its near kNN pass on the vertex-centred central list (two-cell
   // stencils; the ranks of that counting sort take one word per central of the cell arrays)
-  const bool split = g->split && subset && rdf && d_nwithin == nullptr && g->stencil >= 2 && g->dense_min == 0xFFFFFFFFu;
+  const bool split = in_passes;
   const bool vertex = split && n_k > 0 && g->stencil == 2 && (uint64_t)g->n <= (uint64_t)g->cell_cap;
   int rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, true, vertex, !split || n_k > 0);
   if (rc) return rc;
@@ -1439,8 +1447,6 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
       return launch_rdf_sym<false, false>(g, qs, sw, smem_layout(bins.n_bins, 0, true, 0, true, qa.lut_n).total, nullptr, s);
     const uint32_t smem = (bins.n_bins + 1) * 4 * 17;
     if (d_nwithin == nullptr) return launch_rdf_sym<true, false>(g, qs, sw, smem, nullptr, s);
-    // the counts in record order take the counting sort's index list, free until the next build
-    PS_CUDA(cudaMemsetAsync(g->sel, 0, (size_t)g->n * sizeof(uint32_t), s));
     return launch_rdf_sym<true, true>(g, qs, sw, smem + 8 * kSweepRec * 4, g->sel, s);
   };
   if (split) {
@@ -1479,7 +1485,7 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
     rc = run_rdf_sym();
     if (rc) return rc;
   } else if (n_k > 0 || rdf) {
-    if (rdf && subset && g->dense_min == 0xFFFFFFFFu && (direct || d_nwithin == nullptr)) {
+    if (sweep) {
       qa.sweep = 1;
       rc = run_rdf_sym();
       if (rc) return rc;
@@ -1489,7 +1495,9 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
                   : dispatch_k<kRdfGeneral>(g, qa, smem_cta, smem_warp, s);
     if (rc) return rc;
   }
-  PS_LAUNCH(PS_KID_EPILOGUE, s, PS_CUDA(launch_pdl(k_query_epilogue, 1, 32, 0, s, g->nbr.geo, g->ctr.geo, d_meta)));
+  PS_LAUNCH(PS_KID_EPILOGUE, s,
+            PS_CUDA(launch_pdl(k_query_epilogue, wacc ? g->num_sms * 8 : 1, wacc ? 256 : 32, 0, s, g->nbr.geo, g->ctr.geo, d_meta,
+                               g->nbr.rec, reinterpret_cast<const uint32_t*>(g->cr), (const uint32_t*)wacc, d_nwithin)));
   PS_CUDA(cudaGetLastError());
   return PS_OK;
 }
