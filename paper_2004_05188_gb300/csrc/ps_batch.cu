@@ -207,10 +207,10 @@ __global__ void __launch_bounds__(256, KMAX <= 20 ? 3 : 2) k_batch_query(const _
         auto batch = [&](uint32_t n) __attribute__((always_inline)) {
           const ulonglong2* rp = reinterpret_cast<const ulonglong2*>(bf) + (ring.head & (kRing - 1u));
           const uint32_t n_pr = (n + 1) >> 1;
+          const ulonglong2 *pa = rp + 2 * sub, *pb = pa + 2 * L;
 #pragma unroll 1
-          for (uint32_t t0 = 0; t0 < n_pr; t0 += 2 * L) {
-            const uint32_t t = t0 + sub;
-            const ulonglong2 xy0 = rp[2 * t], xy1 = rp[2 * (t + L)], zw0 = rp[2 * t + 1], zw1 = rp[2 * (t + L) + 1];
+          for (uint32_t t0 = 0; t0 < n_pr; t0 += 2 * L, pa += 4 * L, pb += 4 * L) {
+            const ulonglong2 xy0 = pa[0], xy1 = pb[0], zw0 = pa[1], zw1 = pb[1];
             const unsigned long long d20 = dist2_x2_fma(px, py, pz, xy0.x, xy0.y, zw0.x, one2);
             const unsigned long long d21 = dist2_x2_fma(px, py, pz, xy1.x, xy1.y, zw1.x, one2);
             if (DIRECT) {
@@ -237,9 +237,10 @@ __global__ void __launch_bounds__(256, KMAX <= 20 ? 3 : 2) k_batch_query(const _
             for (uint32_t t0 = 0; t0 < n_pr; t0 += 8 * L) {
               uint32_t qa = q0;
               const uint32_t t1 = min(n_pr, t0 + 8 * L);
+          const ulonglong2* pk = rp + 2 * (t0 + sub);
 #pragma unroll 2
-              for (uint32_t t = t0 + sub; t < t1; t += L) {
-                const ulonglong2 xy = rp[2 * t], zw = rp[2 * t + 1];
+              for (uint32_t t = t0 + sub; t < t1; t += L, pk += 2 * L) {
+                const ulonglong2 xy = pk[0], zw = pk[1];
                 float da, db, wa, wb;
                 f2_unpack(dist2_x2_fma(px, py, pz, xy.x, xy.y, zw.x, one2), da, db);
                 f2_unpack(zw.y, wa, wb);

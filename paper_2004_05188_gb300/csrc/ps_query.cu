@@ -485,11 +485,11 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : 2) k_query_warp(const __
       const uint32_t n_pr = (n + 1) >> 1;
       if (all) {
         // two pairs of candidates at a time (beyond the last there are far ones to the end of the batch)
+        const ulonglong2 *pa = rp + 2 * sub, *pb = pa + 2 * L;
 #pragma unroll 1
-        for (uint32_t t0 = 0; t0 < n_pr; t0 += 2 * L) {
-          const uint32_t t = t0 + sub;
-          const ulonglong2 xy0 = rp[2 * t], xy1 = rp[2 * (t + L)];
-          const unsigned long long z0 = rp[2 * t + 1].x, z1 = rp[2 * (t + L) + 1].x;
+        for (uint32_t t0 = 0; t0 < n_pr; t0 += 2 * L, pa += 4 * L, pb += 4 * L) {
+          const ulonglong2 xy0 = pa[0], xy1 = pb[0];
+          const unsigned long long z0 = pa[1].x, z1 = pb[1].x;
           const unsigned long long d20 = dist2_x2_fma(px, py, pz, xy0.x, xy0.y, z0, one2);
           const unsigned long long d21 = dist2_x2_fma(px, py, pz, xy1.x, xy1.y, z1, one2);
           float d[4];
@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : 2) k_query_warp(const __
           if (MODE == kRdfGeneral && rdf_here) {
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-              if (d[e] < emax && __float_as_uint(bf[4 * (ring.head & (kRing - 1u)) + (t + (e >> 1) * L) * 8 + 6 + (e & 1)]) != pidx)
+              if (d[e] < emax && __float_as_uint(reinterpret_cast<const float*>(e < 2 ? pa : pb)[6 + (e & 1)]) != pidx)
                 H.pair(a, d[e], my_below);
           }
           if (nwithin != nullptr)
@@ -520,9 +520,10 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : 2) k_query_warp(const __
         for (uint32_t t0 = 0; t0 < n_pr; t0 += 8 * L) {
           uint32_t qa = q0;
           const uint32_t t1 = min(n_pr, t0 + 8 * L);
+          const ulonglong2* pk = rp + 2 * (t0 + sub);
 #pragma unroll 2
-          for (uint32_t t = t0 + sub; t < t1; t += L) {
-            const ulonglong2 xy = rp[2 * t], zw = rp[2 * t + 1];
+          for (uint32_t t = t0 + sub; t < t1; t += L, pk += 2 * L) {
+            const ulonglong2 xy = pk[0], zw = pk[1];
             float da, db, wa, wb;
             f2_unpack(dist2_x2_fma(px, py, pz, xy.x, xy.y, zw.x, one2), da, db);
             f2_unpack(zw.y, wa, wb);
@@ -1077,14 +1078,20 @@ __global__ void __launch_bounds__(256, KMAX <= 13 ? 4 : 2) k_knn_vertex(const __
       nxt = fetch(b + 32 + lane);
 #pragma unroll 1
       for (uint32_t hb = 0; hb < 16; hb += 8) {
-#pragma unroll 4
-        for (uint32_t t = hb + sub; t < hb + 8; t += L) {
+        auto test = [&](uint32_t t) __attribute__((always_inline)) {
           const ulonglong2 xy = *reinterpret_cast<const ulonglong2*>(&s_xy[w][t]);
           const unsigned long long zz = *reinterpret_cast<const unsigned long long*>(&s_z[w][t]);
           float da, db;
           f2_unpack(dist2_x2_fma(px, py, pz, xy.x, xy.y, zz, one2), da, db);
           queue_push(qa, da, thr);
           queue_push(qa, db, thr);
+        };
+        if (L == 1u) {  // constant offsets: half the instructions of the loop below
+#pragma unroll
+          for (uint32_t t = 0; t < 8; ++t) test(hb + t);
+        } else {
+#pragma unroll 1
+          for (uint32_t t = hb + sub; t < hb + 8; t += L) test(t);
         }
         const uint32_t m = __reduce_max_sync(0xffffffffu, qa - q0) >> 7;
         if (m > kQueue - 16u) {
