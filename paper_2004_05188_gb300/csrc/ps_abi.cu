@@ -151,7 +151,7 @@ int ps_grid_create(int64_t n_max, const ps_grid_opts* opts, ps_grid** out) {
   g->item_cap = (uint32_t)(cc + nm / 8 + 2);  // batches of >= 8 centrals (4 lanes per central) + one per cell
   const size_t o_witem = take((size_t)g->item_cap * 8), o_nwitem = take((size_t)g->item_cap * 8);
   const size_t o_sm0 = take(kSoftFineMax * 8), o_sm1 = take(kSoftFineMax * 8), o_sm2 = take(kSoftFineMax * 8);
-  const size_t o_sT = take(3 * kSoftFineMax * 4), o_sgs = take(8);
+  const size_t o_sT = take(kSoftFineMax * 16), o_sgs = take(8);
   const size_t o_part = take((size_t)g->scan_tiles_cap * 8), o_sctr = take(8);
   const size_t o_ngeo = take(sizeof(Geo)), o_cgeo = take(sizeof(Geo));
   void* base = nullptr;

@@ -54,7 +54,7 @@ struct SoftArgs {
   double* M1;
   double* M2;
   // adjoint
-  const float* T;          // [3][n_fine]: W, W', W'' at the fine-bin centres
+  const float4* T;         // [n_fine]: W, W', W'' / 2 at the fine-bin centres, times the scale
   float* grad;             // [n][3]
   double* grad_s;
   int pass_b;              // 0: owners are centrals (write), 1: owners are neighbours (add, sign flipped)
@@ -321,30 +321,31 @@ constexpr uint32_t kSoftLook = 1u << 14, kSoftDrain = 1u << 18;
 // Forward where the centrals are neighbour records: every unordered pair once (sweep_pairs), its
 // moments straight from the testing lane into the CTA's shared fine grid.  Bound by the shared-
 // memory pipe (three scattered atomics per in-range pair) and issue.  Measured, 1e7-ion needle on
-// half-size cells / 2e5 cylinder on full-size cells (ms): 36.8 -> 19.4 / 14.5 -> 1.13 (before: a warp list of
-// the hits of every candidate of the half stencil, a float sum per moment, cells not split; 27.4 /
-// 1.25 with the sweep and float sums).
+// half-size cells / 2e5 cylinder on full-size cells (ms): 36.8 -> 17.7 / 14.5 -> 0.87 (before: a warp
+// list of the hits of every candidate of the half stencil, a float sum per moment, cells not split;
+// 27.4 / 1.25 with the sweep and float sums; 19.4 / 0.92 with a row of bins per moment, which takes
+// two more additions per pair than the three moments of a bin side by side).
 __global__ void __launch_bounds__(256, 4) k_soft_fwd_sym(const SoftArgs a, const __grid_constant__ SweepArgs sw,
                                                          double unit1, double unit2) {
   griddep_wait();
   griddep_launch();
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ SweepBuf s_sweep[8];
-  const uint32_t nf = a.n_fine, row = (nf + 3u) & ~3u, lane = threadIdx.x & 31;
-  uint32_t* sM = reinterpret_cast<uint32_t*>(smem);  // [3][row]
-  for (uint32_t m = threadIdx.x; m < 3 * row; m += blockDim.x) sM[m] = 0;
+  const uint32_t nf = a.n_fine, nf4 = (nf + 3u) & ~3u, lane = threadIdx.x & 31;
+  uint32_t* sM = reinterpret_cast<uint32_t*>(smem);  // [nf4][3]: the three moments of a bin side by side
+  for (uint32_t m = threadIdx.x; m < 3 * nf4; m += blockDim.x) sM[m] = 0;
   __syncthreads();
   SweepBuf& buf = s_sweep[threadIdx.x >> 5];
   const SoftFine fine(a);
   const float rc = a.rc, q1 = kSoftQ * a.inv_w, q2 = kSoftQ * a.inv_w * a.inv_w;
   const unsigned long long q1_2 = f2_pack(q1, q1), q2_2 = f2_pack(q2, q2);
-  const uint32_t base = smem_u32(sM) - 4u * kMagicBits;
+  const uint32_t base = smem_u32(sM) - 12u * kMagicBits;
   uint32_t added = 0;  // bound on the weights this warp has added since it last looked (uniform)
   // the rows' bins i, i + step, ... to the global moments
   auto drain = [&](uint32_t i, uint32_t step) {
     for (; i < nf; i += step) {
-      const int32_t v0 = (int32_t)atomicExch(&sM[i], 0u), v1 = (int32_t)atomicExch(&sM[row + i], 0u),
-                    v2 = (int32_t)atomicExch(&sM[2 * row + i], 0u);
+      const int32_t v0 = (int32_t)atomicExch(&sM[3 * i], 0u), v1 = (int32_t)atomicExch(&sM[3 * i + 1], 0u),
+                    v2 = (int32_t)atomicExch(&sM[3 * i + 2], 0u);
       // (a count may stand below zero when its self pairs were drained before they were taken out)
       if (v0) atomicAdd(&a.M0[i], (unsigned long long)(long long)v0);
       if (v1) atomicAdd(&a.M1[i], (double)v1 * unit1);
@@ -359,6 +360,7 @@ __global__ void __launch_bounds__(256, 4) k_soft_fwd_sym(const SoftArgs a, const
     const unsigned long long x0 = f2_pack(c0.x, c0.x), y0 = f2_pack(c0.y, c0.y), z0 = f2_pack(c0.z, c0.z);
     const unsigned long long x1 = f2_pack(c1.x, c1.x), y1 = f2_pack(c1.y, c1.y), z1 = f2_pack(c1.z, c1.z);
     auto deposit = [&](unsigned long long d2, uint32_t wt) __attribute__((always_inline)) {
+      const uint32_t off = 0u - kMagicBits * wt;
       float da, db, u[2], mm[2], r1[2], r2[2];
       f2_unpack(d2, da, db);
       const unsigned long long u2 = f2_mul(f2_pack(sqrt_fast(da), sqrt_fast(db)), fine.scale2);
@@ -370,10 +372,10 @@ __global__ void __launch_bounds__(256, 4) k_soft_fwd_sym(const SoftArgs a, const
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         if (u[e] < rc) {
-          const uint32_t at = __float_as_uint(mm[e]) * 4u + base;
+          const uint32_t at = __float_as_uint(mm[e]) * 12u + base;
           asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at), "r"(wt));
-          asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at + 4u * row), "r"((__float_as_uint(r1[e]) - kMagicBits) * wt));
-          asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at + 8u * row), "r"((__float_as_uint(r2[e]) - kMagicBits) * wt));
+          asm volatile("red.shared.add.u32 [%0+4], %1;" ::"r"(at), "r"(__float_as_uint(r1[e]) * wt + off));
+          asm volatile("red.shared.add.u32 [%0+8], %1;" ::"r"(at), "r"(__float_as_uint(r2[e]) * wt + off));
         }
       }
     };
@@ -391,20 +393,14 @@ __global__ void __launch_bounds__(256, 4) k_soft_fwd_sym(const SoftArgs a, const
                           __popc(__ballot_sync(0xffffffffu, k1 == kCandSelf));
     if (self && lane == 0) {
       atomicAdd(&sM[0], 0u - self);
-      atomicAdd(&sM[row], self * (uint32_t)(kSoftQ / 2));
-      atomicAdd(&sM[2 * row], 0u - self * (uint32_t)(kSoftQ / 4));
+      atomicAdd(&sM[1], self * (uint32_t)(kSoftQ / 2));
+      atomicAdd(&sM[2], 0u - self * (uint32_t)(kSoftQ / 4));
     }
     added += 2u * kSweepTile * m;
     if (added >= kSoftLook) {
       added = 0;
       uint32_t top = 0;
-      for (uint32_t i = lane; i < row / 4; i += 32) {
-        uint4 v;
-        asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                     : "r"(smem_u32(sM) + 16u * i));
-        top = max(max(top, max(v.x, v.y)), max(v.z, v.w));
-      }
+      for (uint32_t i = lane; i < nf4; i += 32) top = max(top, reinterpret_cast<const volatile uint32_t*>(sM)[3 * i]);
       if (__any_sync(0xffffffffu, top >= kSoftDrain)) drain(lane, 32);
     }
   });
@@ -452,10 +448,10 @@ __global__ void __launch_bounds__(256) k_soft_finalize(const unsigned long long*
   }
 }
 
-// T[2m] = W(c_m), T[2m + 1] = W'(c_m), T[2 n_fine + m] = W''(c_m) / 2 for W(u) = sum_b G[b] K_b'(u)
+// T[m] = W(c_m), W'(c_m), W''(c_m) / 2, all times `scale`, for W(u) = sum_b G[b] K_b'(u)
 __global__ void __launch_bounds__(256) k_soft_table(const float* __restrict__ G, uint32_t n_bins, uint32_t n_fine,
                                                     double w, double r0, double dr, double sigma,
-                                                    float* __restrict__ T) {
+                                                    double scale, float4* __restrict__ T) {
   griddep_wait();
   griddep_launch();
   const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -473,9 +469,7 @@ __global__ void __launch_bounds__(256) k_soft_table(const float* __restrict__ G,
     a3 += g * (ph[3] - pl[3]);
     for (int k = 0; k < 4; ++k) pl[k] = ph[k];
   }
-  T[2 * m] = (float)a1;
-  T[2 * m + 1] = (float)a2;
-  T[2 * n_fine + m] = (float)(0.5 * a3);
+  T[m] = make_float4((float)(scale * a1), (float)(scale * a2), (float)(0.5 * scale * a3), 0.f);
 }
 
 // ---------------------------------------------------------------------------
@@ -490,8 +484,8 @@ __global__ void __launch_bounds__(256) k_soft_bwd(const SoftArgs a) {
   __shared__ float4 s_buf[8][32];
   __shared__ uint32_t s_rsrc[8][kSoftRuns], s_rpre[8][kSoftRuns + 1];
   __shared__ double s_gs[8];
-  float* sT = reinterpret_cast<float*>(smem);
-  for (uint32_t m = threadIdx.x; m < 3 * a.n_fine; m += blockDim.x) sT[m] = a.T[m];
+  float4* sT = reinterpret_cast<float4*>(smem);
+  for (uint32_t m = threadIdx.x; m < a.n_fine; m += blockDim.x) sT[m] = a.T[m];
   __syncthreads();
   const uint32_t w = threadIdx.x >> 5;
   const float s = a.scale, inv_w = a.inv_w, wf = a.w, rc = a.rc;
@@ -508,8 +502,9 @@ __global__ void __launch_bounds__(256) k_soft_bwd(const SoftArgs a) {
     uint32_t m = (uint32_t)(u * inv_w);
     m = m < nf ? m : nf - 1;
     const float delta = u - ((float)m + 0.5f) * wf;
-    const float W = sT[2 * m] + delta * (sT[2 * m + 1] + delta * sT[2 * nf + m]);
-    const float f = W * s * rs;  // W s / d (0 for coincident ions)
+    const float4 t = sT[m];
+    const float W = t.x + delta * (t.y + delta * t.z);  // times s
+    const float f = W * rs;                             // W s / d (0 for coincident ions)
     gx += f * (p.x - qx);
     gy += f * (p.y - qy);
     gz += f * (p.z - qz);
@@ -535,7 +530,7 @@ __global__ void __launch_bounds__(256) k_soft_bwd(const SoftArgs a) {
     if (threadIdx.x == 0) {
       double t = 0.0;
       for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += s_gs[i];
-      atomicAdd(a.grad_s, t);
+      atomicAdd(a.grad_s, t / (double)a.scale);
     }
   }
 }
@@ -578,8 +573,9 @@ __device__ __forceinline__ void red_global_v4(float4* p, float x, float y, float
 // reduction per record and tile (neighbouring candidates are neighbouring records), which
 // k_soft_grad_out scatters to the ions.  Bound by issue (~30 instructions per 32 tests) and by
 // the table's shared-memory reads.  Measured, 1e7-ion needle on half-size cells / 2e5 cylinder on
-// full-size cells (ms): 75.4 -> 23.8 / 3.56 -> 1.60 (before: every record a lane of its own, each pair tested
-// and evaluated from both ends); 128 or 64 registers a thread: 29.1 and 23.7 ms.
+// full-size cells (ms): 75.4 -> 23.3 / 3.56 -> 1.36 (before: every record a lane of its own, each
+// pair tested and evaluated from both ends); 128 or 64 registers a thread: 29.1 and 23.7 ms; the
+// table as a pair and a single value per bin instead of one 16-byte entry: 23.8 ms.
 __global__ void __launch_bounds__(256, 3) k_soft_bwd_sym(const SoftArgs a, const __grid_constant__ SweepArgs sw,
                                                          float4* __restrict__ acc) {
   griddep_wait();
@@ -588,17 +584,16 @@ __global__ void __launch_bounds__(256, 3) k_soft_bwd_sym(const SoftArgs a, const
   __shared__ SweepBuf s_sweep[8];
   __shared__ float s_rec[8][kSweepRec * 3];  // per warp: gradients of the staged records
   __shared__ double s_gs[8];
-  float* sT = reinterpret_cast<float*>(smem);
+  float4* sT = reinterpret_cast<float4*>(smem);
   const uint32_t nf = a.n_fine, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (uint32_t m = threadIdx.x; m < 3 * nf; m += blockDim.x) sT[m] = a.T[m];
+  for (uint32_t m = threadIdx.x; m < nf; m += blockDim.x) sT[m] = a.T[m];
   for (uint32_t i = lane; i < kSweepRec * 3; i += 32) s_rec[w][i] = 0.f;
   __syncthreads();
   SweepBuf& buf = s_sweep[w];
   float* grec = s_rec[w];
   const SoftFine fine(a);
-  const float rc = a.rc, s = a.scale;
-  const float2* T01 = reinterpret_cast<const float2*>(sT);
-  const float* T2 = sT + 2 * nf;
+  const float rc = a.rc;
+  const uint32_t table = smem_u32(sT) - 16u * kMagicBits;
   const uint32_t slot = sum_slot(lane);
   double gs_lane = 0.0;
   sweep_pairs<true>(
@@ -639,14 +634,18 @@ __global__ void __launch_bounds__(256, 3) k_soft_bwd_sym(const SoftArgs a, const
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
                 if (u[e] < rc) {
-                  const uint32_t m = __float_as_uint(mm[e]) - kMagicBits;
-                  const float2 t = T01[m];
-                  const float W = (t.x + dl[e] * (t.y + dl[e] * T2[m])) * ws[h];
-                  const float f = W * s * rs[e];
+                  float t0, t1, t2;  // (the fourth value pads the entry to one 16-byte load)
+                  asm("{.reg .f32 pad; ld.shared.v4.f32 {%0, %1, %2, pad}, [%3];}"
+                      : "=f"(t0), "=f"(t1), "=f"(t2)
+                      : "r"(__float_as_uint(mm[e]) * 16u + table));
+                  const float W = (t0 + dl[e] * (t1 + dl[e] * t2)) * ws[h];
+                  const float f = W * rs[e];
                   gs += W * dd[e];
-                  const float fx = f * dx[e], fy = f * dy[e], fz = f * dz[e];
-                  g[h][0] += fx, g[h][1] += fy, g[h][2] += fz;
-                  r[6 * q + 3 * e] -= fx, r[6 * q + 3 * e + 1] -= fy, r[6 * q + 3 * e + 2] -= fz;
+                  g[h][0] = __fmaf_rn(f, dx[e], g[h][0]), g[h][1] = __fmaf_rn(f, dy[e], g[h][1]),
+                  g[h][2] = __fmaf_rn(f, dz[e], g[h][2]);
+                  r[6 * q + 3 * e] = __fmaf_rn(-f, dx[e], r[6 * q + 3 * e]);
+                  r[6 * q + 3 * e + 1] = __fmaf_rn(-f, dy[e], r[6 * q + 3 * e + 1]);
+                  r[6 * q + 3 * e + 2] = __fmaf_rn(-f, dz[e], r[6 * q + 3 * e + 2]);
                 }
               }
             }
@@ -674,7 +673,7 @@ __global__ void __launch_bounds__(256, 3) k_soft_bwd_sym(const SoftArgs a, const
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += s_gs[i];
-    atomicAdd(a.grad_s, t);
+    atomicAdd(a.grad_s, t / (double)a.scale);
   }
 }
 
@@ -849,11 +848,11 @@ int soft_backward(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], flo
   PS_CUDA(cudaMemsetAsync(g->soft_gs, 0, sizeof(double), s));
   PS_LAUNCH(PS_KID_SOFT_BWD, s,
             PS_CUDA(launch_pdl(k_soft_table, (sa.n_fine + 255) / 256, 256, 0, s, d_G, bins.n_bins, sa.n_fine, w, bins.r0, bins.dr,
-                                                                 (double)sigma, g->soft_T)));
-  sa.T = g->soft_T;
+                                                                 (double)sigma, (double)scale, reinterpret_cast<float4*>(g->soft_T))));
+  sa.T = reinterpret_cast<const float4*>(g->soft_T);
   sa.grad = d_grad;
   sa.grad_s = g->soft_gs;
-  const uint32_t smem = sa.n_fine * 12;
+  const uint32_t smem = sa.n_fine * 16;
   int blocks = 0;
   if (sym) {
     // the record-ordered gradient takes the place of the central records, which the sweep does not use
