@@ -77,9 +77,11 @@ __device__ __forceinline__ bool mask_has(const uint64_t* m, uint32_t t) { return
 // those that can still enter a k list into the lane's queue.  DIRECT (r0 = 0): direct bins, an
 // increment per test by every lane; otherwise a branch per hit, and the pairs below r0 in bin
 // n_bins.  Rows are 32-bit and shared by the CTA: a warp drains them before it has added 2^28 since
-// its last drain.  Bound by instruction issue.  24 ROIs (2e6 ions, k = 1 .. 20, r_max = 3 nm, 3 pairs, 3
-// thresholds), whole pass: 75 -> 18.7 ms (before: every
-// record of the 125 cells, a sorted insertion under a branch per candidate, 64-bit counters).
+// its last drain.  Bound by instruction issue (~34 per 32 tests, k = 20).  24 ROIs (2e6 ions, k = 1 .. 20,
+// r_max = 3 nm, 3 pairs, 3 thresholds), kernel: 78 -> 17.4 ms (before: every record of the 125 cells, a
+// sorted insertion under a branch per candidate, 64-bit counters; 17.9 with a loop for the bins and
+// one for the queue, which computes the near candidates' distances twice).  The queue's stores stand
+// after the increments: ahead of them the same loop takes 30 ms.
 template <int KMAX, bool DIRECT>
 __global__ void __launch_bounds__(256, KMAX <= 20 ? 3 : 2) k_batch_query(const __grid_constant__ BatchArgs a) {
   griddep_wait();
@@ -207,47 +209,41 @@ __global__ void __launch_bounds__(256, KMAX <= 20 ? 3 : 2) k_batch_query(const _
         auto batch = [&](uint32_t n) __attribute__((always_inline)) {
           const ulonglong2* rp = reinterpret_cast<const ulonglong2*>(bf) + (ring.head & (kRing - 1u));
           const uint32_t n_pr = (n + 1) >> 1;
+          const bool near = (int32_t)(ring.near_to - ring.head) > 0;
           const ulonglong2 *pa = rp + 2 * sub, *pb = pa + 2 * L;
 #pragma unroll 1
-          for (uint32_t t0 = 0; t0 < n_pr; t0 += 2 * L, pa += 4 * L, pb += 4 * L) {
-            const ulonglong2 xy0 = pa[0], xy1 = pb[0], zw0 = pa[1], zw1 = pb[1];
-            const unsigned long long d20 = dist2_x2_fma(px, py, pz, xy0.x, xy0.y, zw0.x, one2);
-            const unsigned long long d21 = dist2_x2_fma(px, py, pz, xy1.x, xy1.y, zw1.x, one2);
-            if (DIRECT) {
-              const uint32_t x = fb.count2(d20, row) | fb.count2(d21, row);
-              if (__any_sync(0xffffffffu, x != 0u)) {
-                fb.settle2(d20, row);
-                fb.settle2(d21, row);
-              }
-            } else {
+          for (uint32_t t0 = 0; t0 < n_pr; t0 += 8 * L) {
+            uint32_t qa = q0;
+            const uint32_t t1 = min(n_pr, t0 + 8 * L);
+#pragma unroll 1
+            for (uint32_t t = t0; t < t1; t += 2 * L, pa += 4 * L, pb += 4 * L) {
+              const ulonglong2 xy0 = pa[0], xy1 = pb[0], zw0 = pa[1], zw1 = pb[1];
+              const unsigned long long d20 = dist2_x2_fma(px, py, pz, xy0.x, xy0.y, zw0.x, one2);
+              const unsigned long long d21 = dist2_x2_fma(px, py, pz, xy1.x, xy1.y, zw1.x, one2);
               float d[4], wv[4];
               f2_unpack(d20, d[0], d[1]), f2_unpack(d21, d[2], d[3]);
               f2_unpack(zw0.y, wv[0], wv[1]), f2_unpack(zw1.y, wv[2], wv[3]);
-#pragma unroll
-              for (int e = 0; e < 4; ++e)
-                if (d[e] < Emax && __float_as_uint(wv[e]) != pw) {
-                  const uint32_t bn = d[e] < E0 ? nb : bin_index(d[e], sE, nb, r0f, inv_dr);
-                  red_shared_inc(row + 4u * (kMagicBits + bn));
+              if (DIRECT) {
+                const uint32_t x = fb.count2(d20, row) | fb.count2(d21, row);
+                if (__any_sync(0xffffffffu, x != 0u)) {
+                  fb.settle2(d20, row);
+                  fb.settle2(d21, row);
                 }
-            }
-          }
-          __syncwarp();
-          if ((int32_t)(ring.near_to - ring.head) > 0) {
-#pragma unroll 1
-            for (uint32_t t0 = 0; t0 < n_pr; t0 += 8 * L) {
-              uint32_t qa = q0;
-              const uint32_t t1 = min(n_pr, t0 + 8 * L);
-          const ulonglong2* pk = rp + 2 * (t0 + sub);
-#pragma unroll 2
-              for (uint32_t t = t0 + sub; t < t1; t += L, pk += 2 * L) {
-                const ulonglong2 xy = pk[0], zw = pk[1];
-                float da, db, wa, wb;
-                f2_unpack(dist2_x2_fma(px, py, pz, xy.x, xy.y, zw.x, one2), da, db);
-                f2_unpack(zw.y, wa, wb);
-                queue_push_other(qa, da, thr, __float_as_uint(wa), pw);
-                queue_push_other(qa, db, thr, __float_as_uint(wb), pw);
+              } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                  if (d[e] < Emax && __float_as_uint(wv[e]) != pw) {
+                    const uint32_t bn = d[e] < E0 ? nb : bin_index(d[e], sE, nb, r0f, inv_dr);
+                    red_shared_inc(row + 4u * (kMagicBits + bn));
+                  }
               }
-              __syncwarp();
+              if (near) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) queue_push_other(qa, d[e], thr, __float_as_uint(wv[e]), pw);
+              }
+            }
+            __syncwarp();
+            if (near) {
               const uint32_t qn = (qa - q0) >> 7, m = __reduce_max_sync(0xffffffffu, qn);
 #pragma unroll 1
               for (uint32_t q = 0; q < m; ++q)
@@ -256,8 +252,8 @@ __global__ void __launch_bounds__(256, KMAX <= 20 ? 3 : 2) k_batch_query(const _
               for (uint32_t o = 1; o < L; o <<= 1) kth = fminf(kth, __shfl_xor_sync(0xffffffffu, kth, o));
               thr = fminf(kth, Emax);
             }
-            near_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(valid ? thr : 0.f)));
           }
+          if (near) near_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(valid ? thr : 0.f)));
           added += 32u * 64u;
           if (added >= (1u << 28) - 4096u) {
             __syncwarp();
