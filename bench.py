@@ -785,8 +785,8 @@ QUERY_FAMS = ("query", "knn_full", "rdf_sym")  # the pair tests: one pass, or th
 BUILD_FAMS = ("select", "geometry", "count", "scan", "scatter", "central")
 
 
-KERNEL_NAMES = {"query": "k_query_warp (one pass, or the near-radius kNN pass)",
-                "knn_full": "k_query_warp (full-radius kNN fallback)", "rdf_sym": "k_rdf_sym (RDF over unordered pairs)"}
+KERNEL_NAMES = {"query": "k_query_warp (one pass) and k_knn_vertex (near-radius kNN pass)",
+                "knn_full": "k_knn_list (full-radius kNN fallback)", "rdf_sym": "k_rdf_sym (RDF over unordered pairs)"}
 
 
 def rooflines(prof, st, steps, peaks, hbm_peak, hbm_src, traffic):
@@ -844,7 +844,9 @@ def rooflines(prof, st, steps, peaks, hbm_peak, hbm_src, traffic):
         "algorithmic_bytes_per_launch": (algorithmic_bytes("query", st, next(c for c in st["combos"]
                                                                             if c["name"] == traffic["combination"]))
                                          if traffic and d.get("traffic") else None),
-        "per_unit": f"{FLOPS_PER_CANDIDATE} FP32 operations per candidate test (3 sub, 3 mul, 2 add, 1 compare)",
+        "per_unit": f"{FLOPS_PER_CANDIDATE} FP32 operations per candidate test (3 sub, 3 mul, 2 add, 1 compare) of "
+                    "the cells' stencils; the kernels leave out the candidates beyond reach of a block's bounding box "
+                    "(about a third on half-size cells), which are counted here all the same",
         "flops_per_launch": d.get("flops_per_launch"), "launches": d.get("launches"),
         "avg_launch_ms": d.get("avg_launch_ms"),
         "by_kernel": by_kernel,

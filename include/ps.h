@@ -112,7 +112,8 @@ typedef struct {
                          cells around its cell) with a full-radius search only for the centrals that
                          have fewer than k neighbours there, and the RDF over unordered pairs (each
                          pair tested once, counted once per central end).  Same results; 0
-                         (default): one combined pass */
+                         (default): one combined pass, which leaves the RDF and the in-range
+                         counts of dense clouds to the pass over unordered pairs as well */
 } ps_grid_opts;
 
 typedef struct ps_grid ps_grid; /* opaque; owns its device scratch */
@@ -430,7 +431,7 @@ typedef enum {
   PS_KID_CLUSTER = 15,   /* maximum-separation clustering */
   PS_KID_FINALISE = 16,  /* g(r) normalisation */
   PS_KID_PEAKS = 17,     /* throughput microbenchmarks (ps_measure_peaks) */
-  PS_KID_RDF_SYM = 18,   /* RDF over unordered pairs (the split query's third pass) */
+  PS_KID_RDF_SYM = 18,   /* RDF over unordered pairs (beside the query where its centrals are neighbour records) */
   PS_KID_KNN_FULL = 19,  /* full-radius kNN of the centrals the near pass left (split query) */
   PS_KID_COUNT_ = 20
 } ps_kernel_id;

@@ -7,30 +7,32 @@
 // cells within `stencil` cells of it (27 cells for cells of edge >= r_cut, 125
 // for cells of edge >= r_cut/2, up to 343 for r_cut/3, less the cells that
 // cannot hold a pair within r_cut), read as x-contiguous runs of sorted records.
-// Two persistent kernels take work from device counters (the dynamic
-// schedule):
+// Dense grids keep a cell's records ordered by sub-cells, whose x-rods are then the
+// runs.  Persistent kernels take work from device counters (the dynamic schedule):
 //
-//   warp kernel  heavy items = (cell with >= 16 centrals, batch of <= 32 of
-//                them): the candidates are read 32 at a time with one coalesced
-//                load into a per-warp shared buffer (the next batch is
-//                prefetched into registers meanwhile); each lane holds one
-//                central and walks the buffer (shared-memory broadcast).
-//                Light items (sparser cells) are taken 32 at a time and each of
-//                their centrals gets one thread that walks its own stencil.
-//   CTA kernel   for cells with >= dense_min centrals (an option): one CTA per
-//                cell; the runs are staged into shared memory with bulk
-//                asynchronous copies (cp.async.bulk, completion on an mbarrier)
-//                and one thread per central walks them.
+//   k_query_warp   heavy items = (cell with >= 16 centrals, batch of <= 32 of
+//                  them): the candidates within reach of the box around the
+//                  item's centrals go through a per-warp shared ring
+//                  (item_scan), each lane holds one central (or shares one) and
+//                  walks the ring (shared-memory broadcast).  Light items
+//                  (sparser cells) are taken 32 at a time and each of their
+//                  centrals gets one thread that walks its own stencil.
+//   k_rdf_sym      the RDF, and the in-range counts, over unordered pairs of
+//                  neighbour records: where every central is one and the cloud
+//                  is dense (sweep_pays), or in passes.
+//   k_query_cta    for cells with >= dense_min centrals (an option): one CTA per
+//                  cell; the runs are staged into shared memory with bulk
+//                  asynchronous copies (cp.async.bulk, completion on an mbarrier)
+//                  and one thread per central walks them.
 //
 // Each thread keeps the k smallest squared distances in registers (sorted
 // insertion).  Counts go to per-CTA shared-memory histograms (the per-thread
 // buffers) added to the uint64 global histograms when the CTA finishes.
 //
-// The query in passes (ps_grid_opts.split) reuses the warp kernel for its near
-// kNN pass (vertex mode: the centrals sorted by the vertex-centred grid, each
-// item against the 2 x 2 x 2 cells around its vertex) and adds k_knn_list (the
-// full-radius kNN of the centrals that pass lists) and k_rdf_sym (the RDF over
-// unordered pairs of neighbour records).
+// The query in passes (ps_grid_opts.split): k_knn_vertex, the near kNN pass (the
+// centrals sorted by the vertex-centred grid, each item against the 2 x 2 x 2
+// cells around its vertex; k_query_warp on third-size cells), k_knn_list (the
+// full-radius kNN of the centrals that pass lists) and k_rdf_sym.
 #include <cstring>
 #include <vector>
 
@@ -396,8 +398,8 @@ __device__ __forceinline__ float4 far_record() { return make_float4(INFINITY, IN
 //     central (item_lanes).  The candidates are read 32 at a time, the stencil's rows nearest
 //     first, and kept only within range of the bounding box of the item's centrals (the
 //     histogram's range, or for kNN alone the largest k-th distance so far); the kept ones are
-//     compacted into a ring of 64 in shared memory as interleaved pairs and tested 32 at a time, two
-//     per packed test.  Candidates further from the box than every current k-th distance skip
+//     compacted into a ring of 128 in shared memory as interleaved pairs and tested 32 or 64 at a
+//     time, two per packed test.  Candidates further from the box than every current k-th distance skip
 //     the kNN part of the test.
 //   light items (cells with < kHeavy centrals): the warp takes 32 items at a
 //     time and gives each of their centrals a thread of its own that walks its
@@ -409,7 +411,10 @@ constexpr int kNoRdf = 0, kRdfGeneral = 1, kRdfDirect = 2;
 // Bound by instruction issue, and on small or clustered clouds by the chain of one item.  Where the
 // RDF is left to the sweep (a.sweep, dense clouds) only the kNN is done here: k = 10, 1e5-ion
 // cylinder, 2 nm cells, 0.325 ms walking every record of the 27 cells, 0.163 ms with the sub-cells out of
-// reach left out.
+// reach left out.  Sparse neighbours (3e6-ion needle, Al about Sc, RDF and k = 10: 0.354 ms, before 0.494):
+// 75 instructions per 32 tests, of which the bins take 16, the near tests 18, the insertions 17.
+// Near candidates are tested a second time for the queue: one loop for both spills at 64 registers
+// (0.347 ms there, but 0.174 -> 0.193 ms where the kNN is alone).
 template <int KMAX, int MODE>
 __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : 2) k_query_warp(const __grid_constant__ QueryArgs a) {
   constexpr bool RDF = MODE != kNoRdf;
@@ -1001,8 +1006,8 @@ constexpr uint32_t kQueue = 40;  // queue rows per lane; inserted when fewer tha
 // one whose k-th distance is beyond its reach.  The central itself stays in (distance 0): the
 // list is one longer and rank k is its entry k, so that no test compares indexes.  KMAX > k_need.
 // Bound by issue (ncu, 8e6-ion needle: 81 % of the slots).  All-all, k = 10, one box (ms): 8e6-ion needle
-// 1.94 -> 1.65, the 1e8-ion one 25.4 -> 21.5 (before: an insertion queue drained every 16 candidates, the
-// central compared by index).
+// 1.94 -> 1.42, the 1e8-ion one 25.4 -> 20.5 (before: an insertion queue drained every 16 candidates, the
+// central compared by index; 1.65 and 21.5 with the strides of shared centrals in the common loop).
 template <int KMAX>
 __global__ void __launch_bounds__(256, KMAX <= 13 ? 4 : 2) k_knn_vertex(const __grid_constant__ QueryArgs a) {
   griddep_wait();

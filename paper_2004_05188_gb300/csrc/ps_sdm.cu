@@ -5,8 +5,10 @@
 // the float32 displacement x_j - x_i is binned into cubic voxels of edge w;
 // the paper's setting is w = 0.025 nm with R = 2 nm (Results, strong scaling).
 //
-// The enumeration is the exact query's: the same cell grid and central list.
-// Each central gets one thread; the centrals of a dense cell's item share the
+// Where the centrals are neighbour records every unordered pair is met once
+// (sweep_pairs) and the pairs with two central ends are mirrored afterwards.
+// Otherwise the enumeration is over the exact query's cell grid and central list:
+// each central gets one thread; the centrals of a dense cell's item share the
 // candidate walk, so their loads of a record broadcast from L1 (cells with at
 // most 3 centrals let the lanes split each central's candidates instead);
 // sparse cells' items are taken 32 at a time.  Voxel edges V[m] = (float)((m - n_vox/2) * w)
@@ -181,7 +183,8 @@ __global__ void __launch_bounds__(256) k_sdm(const SdmArgs a) {
 // The voxel index is floor(d / w + n / 2), taken twice with n / 2 -+ n 2^-21 (the quotient, its
 // product with the rounded 1 / w and the rounded edges are each good to n 2^-24): where the
 // two floors differ on any axis the pair goes through the edge table.
-// Measured on the 8e6-ion needle (all-all, 160^3 voxels): 131 -> 31.7 ms on full-size cells.
+// Measured on the 8e6-ion needle (all-all, 160^3 voxels, full-size cells): 131 -> 27.5 ms (31.7 with cells
+// whose records are not ordered by sub-cells).
 // ---------------------------------------------------------------------------
 struct SdmSymArgs {
   unsigned long long* H;
