@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(256) k_sdm(const SdmArgs a) {
 // The voxel index is floor(d / w + n / 2), taken twice with n / 2 -+ n 2^-21 (the quotient, its
 // product with the rounded 1 / w and the rounded edges are each good to n 2^-24): where the
 // two floors differ on any axis the pair goes through the edge table.
-// Measured on the 8e6-ion needle (all-all, 160^3 voxels, full-size cells): 131 -> 27.5 ms (31.7 with cells
+// Measured on the 8e6-ion needle (all-all, 160^3 voxels, full-size cells): 131 -> 26.8 ms (31.7 with cells
 // whose records are not ordered by sub-cells).
 // ---------------------------------------------------------------------------
 struct SdmSymArgs {

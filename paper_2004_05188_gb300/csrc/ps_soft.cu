@@ -321,7 +321,7 @@ constexpr uint32_t kSoftLook = 1u << 14, kSoftDrain = 1u << 18;
 // Forward where the centrals are neighbour records: every unordered pair once (sweep_pairs), its
 // moments straight from the testing lane into the CTA's shared fine grid.  Bound by the shared-
 // memory pipe (three scattered atomics per in-range pair) and issue.  Measured, 1e7-ion needle on
-// half-size cells / 2e5 cylinder on full-size cells (ms): 36.8 -> 17.7 / 14.5 -> 0.87 (before: a warp
+// half-size cells / 2e5 cylinder on full-size cells (ms): 36.8 -> 17.7 / 14.5 -> 0.79 (before: a warp
 // list of the hits of every candidate of the half stencil, a float sum per moment, cells not split;
 // 27.4 / 1.25 with the sweep and float sums; 19.4 / 0.92 with a row of bins per moment, which takes
 // two more additions per pair than the three moments of a bin side by side).
@@ -573,7 +573,7 @@ __device__ __forceinline__ void red_global_v4(float4* p, float x, float y, float
 // reduction per record and tile (neighbouring candidates are neighbouring records), which
 // k_soft_grad_out scatters to the ions.  Bound by issue (~30 instructions per 32 tests) and by
 // the table's shared-memory reads.  Measured, 1e7-ion needle on half-size cells / 2e5 cylinder on
-// full-size cells (ms): 75.4 -> 23.3 / 3.56 -> 1.36 (before: every record a lane of its own, each
+// full-size cells (ms): 75.4 -> 23.3 / 3.56 -> 1.32 (before: every record a lane of its own, each
 // pair tested and evaluated from both ends); 128 or 64 registers a thread: 29.1 and 23.7 ms; the
 // table as a pair and a single value per bin instead of one 16-byte entry: 23.8 ms.
 __global__ void __launch_bounds__(256, 3) k_soft_bwd_sym(const SoftArgs a, const __grid_constant__ SweepArgs sw,
