@@ -807,14 +807,16 @@ def rooflines(prof, st, steps, peaks, hbm_peak, hbm_src, traffic):
     b_ms = sum(prof[f][1] for f in BUILD_FAMS)
     tot_ms = sum(v[1] for v in prof.values())
 
-    def launching(fam):  # the combinations that launch this family's kernel once per step
+    def launching(fam):  # the combinations whose step has one working launch of this family's kernel
         if fam == "query":
             return [c["name"] for c in st["combos"]]
-        return [c["name"] for c in st["combos"] if c.get("split")]
+        return [c["name"] for c in st["combos"] if c.get("split") or (fam == "rdf_sym" and c.get("swept"))]
 
     by_kernel = {}
     for fam in QUERY_FAMS:
         n, ms = prof[fam]
+        if fam == "rdf_sym":  # one-pass queries of sparse sets launch it, and it returns at once
+            n = min(n, steps * len(launching(fam)))
         if n == 0:
             continue
         tests = None if fam == "knn_full" else sum(c.get("candidates_by_pass", {}).get(fam, 0)
@@ -880,7 +882,7 @@ def combo_stats(ps, g, o, name, ctr, nbr, X, T, D, t_host, wl, stencil, split=Fa
     (split): every central against its near kNN block (its own 2 x 2 x 2 cells on half-size
     cells, the 27 cells around its cell on third-size cells) plus every unordered pair of records
     in each other's stencil once (symmetric RDF), the few full-radius fallback searches not
-    counted."""
+    counted; one pass over a dense cloud leaves the RDF to that pass as well."""
     meta = o["meta"].cpu().numpy()
     if meta[3] != 0:
         raise RuntimeError(f"device status {meta[3]} for {name}")
@@ -901,12 +903,19 @@ def combo_stats(ps, g, o, name, ctr, nbr, X, T, D, t_host, wl, stencil, split=Fa
         sym = (full - info["n_nbr"]) // 2
         by_pass = {"query": near, "rdf_sym": sym}
         cands = near + sym
+        swept = False
+    elif subset and info["n_nbr"] >= 8 * info["n_cells"]:  # the RDF over unordered pairs, the kNN's tests not counted
+        full = candidate_tests(X, T, D, nbr, nbr, wl["dsrf_min"], info, stencil, all_records=True, cell_scale=cs)
+        cands = (full - info["n_nbr"]) // 2
+        by_pass = {"rdf_sym": cands}
+        swept = True
     else:
         cands = candidate_tests(X, T, D, ctr, nbr, wl["dsrf_min"], info, stencil, cell_scale=cs)
         by_pass = {"query": cands}
+        swept = False
     return dict(name=name, n_nbr=info["n_nbr"], n_cells=info["n_cells"], n_central=int(meta[0]),
                 n_ctr_typed=n_typed, n_pairs_local=int(meta[1]), subset=subset, candidates=cands,
-                candidates_by_pass=by_pass, split=bool(split and subset and stencil >= 2))
+                candidates_by_pass=by_pass, split=bool(split and subset and stencil >= 2), swept=swept)
 
 
 def e2e_runner(dev, stream, sets, hosts, step, outs, res_h):
