@@ -153,12 +153,14 @@ __global__ void __launch_bounds__(256) k_cl_flatten(const ClusterArgs a) {
 // every record links to the earlier records of its stencil within d_max whose root differs.  Bound by the
 // latency of the dependent loads of one record's walk.  8e6-ion needle, Sc, d_max = 0.5 nm (us): 236 -> 105 for the
 // links (with every record its own root at first, each link climbed and hooked trees hundreds of
-// links deep), the whole pass 334 -> 186.
+// links deep), the whole call 333 -> 157; 5e6 ions of every type, d_max = 0.127 nm, 16.1 -> 3.3 ms (a record that
+// the first pass left alone is not walked again: 16.0 -> 3.3).
 __global__ void __launch_bounds__(256) k_cl_link(const ClusterArgs a) {
   griddep_wait();
   griddep_launch();
   const Geo g = *a.geo;
   for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < g.n_sel; s += gridDim.x * blockDim.x) {
+    if (ld_rlx(a.parent + s) == s) continue;  // it found no earlier record within d_max (no parent turns back)
     uint32_t root = cl_find(a.parent, s);
     cl_earlier(a, g, s, [&](uint32_t j, float d2) {
       if (d2 <= a.D && ld_rlx(a.parent + j) != root) {
