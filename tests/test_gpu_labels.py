@@ -58,3 +58,15 @@ def test_statistics_on_randomised_labels(ps, orc, spec):
     assert oo["rdf"][:10].sum().item() > 3 * o["rdf"][:10].sum().item()
     for gg in (g, ga, go):
         gg.close()
+
+
+@pytest.mark.parametrize("n", [2, 4, 1023, 65_536, 65_537, 2**24, 2**24 + 1, 2**26 + 1])
+def test_permutation_at_the_table_sizes(ps, orc, n):
+    """Sizes on both sides of a step of the half-block's bits: nothing walked on (n = 4^h), or three of
+    four values; the largest takes the largest tables."""
+    seed = n + 17
+    t = torch.arange(n, device="cuda").to(torch.uint8)
+    out, perm = ps.shuffle_labels(t, seed, with_perm=True)
+    want = torch.from_numpy(orc.label_perm(n, seed).astype(np.int64)).cuda()
+    assert torch.equal(perm.to(torch.int64) & 0xFFFFFFFF, want)
+    assert torch.equal(out, t[want])
