@@ -38,6 +38,27 @@ __device__ __forceinline__ float topk_get(const float (&top)[K], uint32_t idx) {
   return v;
 }
 
+// Bound on the k-th distance (k <= K) of the central that the lane shares with L - 1 others, each
+// holding the K smallest of its part of the candidates: the K-th of any one list, and the largest over
+// the lists of their ceil(K / L)-th values, below or at which the lists together hold K.
+template <int K>
+__device__ __forceinline__ float topk_bound(const float (&top)[K], uint32_t L) {
+  float kth = top[K - 1];
+  if (L > 1u) {
+    float part = top[(K + 15) / 16 - 1];
+    if (L == 2u) part = top[(K + 1) / 2 - 1];
+    if (L == 4u) part = top[(K + 3) / 4 - 1];
+    if (L == 8u) part = top[(K + 7) / 8 - 1];
+#pragma unroll 1
+    for (uint32_t o = 1; o < L; o <<= 1) {
+      kth = fminf(kth, __shfl_xor_sync(0xffffffffu, kth, o));
+      part = fmaxf(part, __shfl_xor_sync(0xffffffffu, part, o));
+    }
+    kth = fminf(kth, part);
+  }
+  return kth;
+}
+
 // bin b in [0, nb) with sE[b] <= d2 < sE[b+1]; caller guarantees sE[0] <= d2 < sE[nb].
 // The guess from an approximate square root is checked against the exact edge
 // table; the (rare) wrong guess is walked to the right bin.

@@ -414,9 +414,13 @@ constexpr int kNoRdf = 0, kRdfGeneral = 1, kRdfDirect = 2;
 // reach left out.  Sparse neighbours (3e6-ion needle, Al about Sc, RDF and k = 10: 0.354 ms, before 0.494):
 // 75 instructions per 32 tests, of which the bins take 16, the near tests 18, the insertions 17.
 // Near candidates are tested a second time for the queue: one loop for both spills at 64 registers
-// (0.347 ms there, but 0.174 -> 0.193 ms where the kNN is alone).
+// (0.347 ms there, but 0.174 -> 0.193 ms where the kNN is alone).  In-range counts without the RDF are
+// taken beside the kNN (5e5-ion needle, k = 16, r = 1 nm: 0.511 -> 0.456 ms).  Lists of more than 12 stop
+// at the tighter bound over a central's lanes (5e4 ions, k = 32: 0.126 -> 0.117 ms; with shorter lists it costs what
+// it saves); those of up to 16 run 3 CTAs per SM (3e6-ion needle, Al about Sc, k = 16: 0.447 -> 0.406 ms),
+// longer ones 2 (5e5-ion needle, k = 32: 0.757 against 0.783 ms with 3).
 template <int KMAX, int MODE>
-__global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : 2) k_query_warp(const __grid_constant__ QueryArgs a) {
+__global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : (KMAX <= 16 ? 3 : 2)) k_query_warp(const __grid_constant__ QueryArgs a) {
   constexpr bool RDF = MODE != kNoRdf;
   griddep_wait();
   griddep_launch();
@@ -488,7 +492,9 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : 2) k_query_warp(const __
     auto batch = [&](uint32_t n) __attribute__((always_inline)) {
       const ulonglong2* rp = reinterpret_cast<const ulonglong2*>(bf) + (ring.head & (kRing - 1u));
       const uint32_t n_pr = (n + 1) >> 1;
-      if (all) {
+      const bool near = KMAX > 0 && (int32_t)(ring.near_to - ring.head) > 0;
+      // without the RDF the near candidates' in-range counts are taken where their kNN is
+      if (all && !(MODE == kNoRdf && near)) {
         // two pairs of candidates at a time (beyond the last there are far ones to the end of the batch)
         const ulonglong2 *pa = rp + 2 * sub, *pb = pa + 2 * L;
 #pragma unroll 1
@@ -518,7 +524,7 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : 2) k_query_warp(const __
         }
         __syncwarp();
       }
-      if (KMAX > 0 && (int32_t)(ring.near_to - ring.head) > 0) {
+      if (near) {
         // candidates below the lane's bound go to its queue column (unconditional stores at the next
         // slot, kept only if counted), inserted every 16 pairs of the lanes
 #pragma unroll 1
@@ -532,6 +538,7 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : 2) k_query_warp(const __
             float da, db, wa, wb;
             f2_unpack(dist2_x2_fma(px, py, pz, xy.x, xy.y, zw.x, one2), da, db);
             f2_unpack(zw.y, wa, wb);
+            if (MODE == kNoRdf && nwithin != nullptr) within += (uint32_t)(da < emax) + (uint32_t)(db < emax);
             queue_push_other(qa, da, thr, __float_as_uint(wa), pidx);
             queue_push_other(qa, db, thr, __float_as_uint(wb), pidx);
           }
@@ -540,7 +547,10 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : 2) k_query_warp(const __
           for (uint32_t q = 0; q < m; ++q)
             if (q < qn) topk_insert(top, queue_at(q0, q));
           float kth = top[KK - 1];  // an upper bound of the central's k-th distance in each of its lanes
-          for (uint32_t o = 1; o < L; o <<= 1) kth = fminf(kth, __shfl_xor_sync(0xffffffffu, kth, o));
+          if constexpr (KK > 12)
+            kth = topk_bound(top, L);
+          else
+            for (uint32_t o = 1; o < L; o <<= 1) kth = fminf(kth, __shfl_xor_sync(0xffffffffu, kth, o));
           thr = fminf(kth, emax);
         }
         near_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(valid ? thr : 0.f)));

@@ -120,3 +120,20 @@ def test_default_grid_over_its_densities(ps, orc, spec, n, L, bins):
         g = run_gpu(ps, xyz, t, d, ctr, nbr, dmin, bins, ks, per_central=True)
         r = orc.spatstat(xyz, t, d, ctr, nbr, dmin, *bins, ks, per_central=True)
         assert_same(g, r, ks, per_central=True)
+
+
+@pytest.mark.parametrize("n,L", [(3, 1.0), (40, 3.0), (2500, 5.0), (6000, 12.0)])
+@pytest.mark.parametrize("cs", [1.0, 0.5])
+@pytest.mark.parametrize("k", [1, 10, 13, 16, 17, 32])
+def test_knn_and_counts_without_the_rdf(ps, orc, spec, n, L, cs, k):
+    """k-th distances and in-range counts alone (both from one distance, near and far candidates),
+    one to sixteen lanes per central, the bound over the lanes of a central for the longer lists."""
+    xyz, t, d = spec.cube(700 + n, n, L, (0.5, 0.5))
+    xyz = np.concatenate([xyz, xyz[:2]])
+    t, d = np.resize(t, xyz.shape[0]), np.resize(d, xyz.shape[0])
+    bins = (0.0, 0.02, 75)
+    for ctr, nbr in (("all", "all"), ([0], [1])):
+        for per_central in (True, False):
+            g = run_gpu(ps, xyz, t, d, ctr, nbr, 0.0, bins, [1, k], per_central=per_central, cell_scale=cs, rdf=False)
+            r = orc.spatstat(xyz, t, d, ctr, nbr, 0.0, *bins, [1, k], per_central=per_central)
+            assert_same(g, r, [1, k], per_central=per_central, rdf=False)
