@@ -132,7 +132,7 @@ int ps_grid_create(int64_t n_max, const ps_grid_opts* opts, ps_grid** out) {
   // cells: a bounding-box grid at the cutoff needs ~n/100 cells for the clouds seen here; the
   // capacity leaves a wide margin (the cell edge grows past it, results do not change)
   const int64_t cap0 = g->stencil >= 2 ? g->n_max : g->n_max / 8;
-  const int64_t cap = cap0 > 65536 ? cap0 : 65536;
+  const int64_t cap = cap0 > (int64_t)kMinCells ? cap0 : (int64_t)kMinCells;
   g->cell_cap = (uint32_t)(cap < (int64_t)1 << 31 ? cap : (int64_t)1 << 31);
   // the count arrays also hold the sub-cells of dense cells (at most n / 4, see sub_cells)
   g->fine_cap = (uint32_t)((int64_t)g->cell_cap > g->n_max / 4 ? (int64_t)g->cell_cap : g->n_max / 4);
@@ -148,7 +148,7 @@ int ps_grid_create(int64_t n_max, const ps_grid_opts* opts, ps_grid** out) {
   const size_t o_sel = take(nm * 4), o_cr = take(nm * 8);
   const size_t o_ncount = take(fc * 4), o_nstart = take((cc + 1) * 4), o_nrec = take(nm * 16);
   const size_t o_ccount = take(fc * 4), o_cstart = take((cc + 1) * 4), o_crec = take(nm * 16), o_cwork = take(cc * 4);
-  g->item_cap = (uint32_t)(cc + nm / 8 + 2);  // batches of >= 8 centrals (4 lanes per central) + one per cell
+  g->item_cap = (uint32_t)item_capacity(cc, nm);
   const size_t o_witem = take((size_t)g->item_cap * 8), o_nwitem = take((size_t)g->item_cap * 8);
   const size_t o_sm0 = take(kSoftFineMax * 8), o_sm1 = take(kSoftFineMax * 8), o_sm2 = take(kSoftFineMax * 8);
   const size_t o_sT = take(kSoftFineMax * 16), o_sgs = take(8);

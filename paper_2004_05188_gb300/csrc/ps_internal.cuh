@@ -130,9 +130,17 @@ __host__ __device__ __forceinline__ uint32_t lanes_per_central(uint32_t n_cand, 
 // costs the 1e5-ion cloud 10 %: more lanes per central share less of a candidate's load).
 constexpr uint32_t kFillItems = 3648;
 __host__ __device__ __forceinline__ uint32_t fill_lanes(uint32_t n_ctr) {
-  const uint32_t want = kFillItems * 32u;
-  return n_ctr * 8u <= want ? 8u : (n_ctr * 4u <= want ? 4u : (n_ctr * 2u <= want ? 2u : 1u));
+  const uint32_t want = kFillItems * 32u;  // (divided: n_ctr times the lanes may pass 2^32)
+  return n_ctr <= want / 8u ? 8u : (n_ctr <= want / 4u ? 4u : (n_ctr <= want / 2u ? 2u : 1u));
 }
+
+// Capacity of the cell arrays (at least) and of the item lists.  A list holds the cells' remainders and light
+// cells, one item each, and the full items: of at least 8 centrals (4 lanes per central), n / 8 of them.  Lists
+// with 8 lanes per central (fill_lanes) have items of 4, but at most 14,592 centrals, so that even one
+// item per central fits in the least number of cells.
+constexpr uint32_t kMinCells = 65536;
+static_assert(kFillItems * 32u / 8u <= kMinCells, "items of 4 centrals fit the item lists");
+constexpr uint64_t item_capacity(uint64_t cells, uint64_t n) { return cells + n / 8 + 2; }
 
 // Lanes per central of a warp item of the exact query with cnt (1..32) centrals: the largest
 // power of two with cnt * L <= 32, at most 8 (16 for one or two centrals).  A full item of a cell split by

@@ -25,9 +25,9 @@ namespace {
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 constexpr size_t kN = PS_STATIC_MAX_IONS;
-constexpr size_t kCells = kN / 8 > 65536 ? kN / 8 : 65536;  // same cell capacity rule as ps_grid_create
+constexpr size_t kCells = kN / 8 > kMinCells ? kN / 8 : kMinCells;  // same cell capacity rule as ps_grid_create
 constexpr size_t kTiles = ((kCells > kN + 1 ? kCells : kN + 1) + 4095) / 4096;  // cells or records
-constexpr size_t kItems = kCells + kN / 8 + 2;  // same item capacity rule as ps_grid_create
+constexpr size_t kItems = item_capacity(kCells, kN);  // same item capacity rule as ps_grid_create
 
 // byte offsets of every scratch buffer inside the array
 constexpr size_t o_sel = 0;
