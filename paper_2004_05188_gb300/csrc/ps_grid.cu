@@ -12,6 +12,7 @@
 //   select + bounding box -> geometry + zero counts -> count ranks
 //   -> single-pass exclusive scan (decoupled look-back) -> scatter
 // The selection kernels read 16 type labels per thread (one 16-byte load).
+#include <cstddef>
 #include <cstring>
 
 #include "ps_internal.cuh"
@@ -844,12 +845,21 @@ int build_neighbour_grid(ps_grid* g, const uint64_t nbr_mask[4], float r_cut, cu
   for (int w = 0; w < 4; ++w) m.w[w] = nbr_mask[w], g->nbr_mask[w] = nbr_mask[w];
   Geo* geo = g->nbr.geo;
   const bool vec = aligned16(g->type) && aligned16(g->xyz);
+  bool recorded = false;  // the clearing below goes into a graph that runs later, if at all
+  if (g->acc_dirty) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    PS_CUDA(cudaStreamIsCapturing(s, &cap));
+    recorded = cap != cudaStreamCaptureStatusNone;
+    PS_CUDA(cudaMemsetAsync(geo->acc_box, 0, offsetof(Geo, acc_status) + sizeof(geo->acc_status) - offsetof(Geo, acc_box), s));
+  }
+  g->acc_dirty = true;  // until the count kernel, which clears the accumulators, is enqueued
   if (g->n > 0)
     PS_LAUNCH(PS_KID_SELECT, s,
               PS_CUDA(launch_pdl(k_select_bbox, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->type, g->n, m, vec, g->sel, geo)));
   PS_LAUNCH(PS_KID_GEOMETRY, s,
             PS_CUDA(launch_pdl(k_geometry_zero, grid_blocks(g, 4), kThreads, 0, s, geo, r_cut, g->cell_scale, g->cell_cap, g->fine_cap, g->nbr.count)));
   PS_LAUNCH(PS_KID_COUNT, s, PS_CUDA(launch_pdl(k_count, grid_blocks(g, 8), kThreads, 0, s, g->xyz, g->sel, geo, g->nbr.count, g->cr)));
+  g->acc_dirty = recorded;
   int rc = scan_cells(g, g->nbr, geo, false, s);
   if (rc) return rc;
   PS_LAUNCH(PS_KID_SCATTER, s,

@@ -72,7 +72,8 @@ struct Geo {
   uint32_t dims[3];
   uint32_t n_cells;
   uint32_t n_sel;   // ions in the set
-  // the selection's accumulators, zero between builds (the count kernel clears them for the next one):
+  // the selection's accumulators, zero between builds (the count kernel clears them for the next one, after a
+  // build that failed before it the next build does, see ps_grid::acc_dirty):
   // largest ~key of min xyz and key of max xyz, ordered as unsigned (0: none), ions, status
   uint32_t acc_box[6];
   uint32_t acc_sel;
@@ -190,6 +191,7 @@ struct ps_grid {
   int64_t n = 0;
   float r_cut = 0.0f;
   bool built = false;
+  bool acc_dirty = false;      // a selection ran (or may have) whose accumulators nothing cleared: a launch failed
   // scratch shared by both builds
   uint32_t dense_min = 0xFFFFFFFFu;  // cells with at least this many centrals go to the CTA-staged kernel
   uint32_t item_cap = 0;       // capacity of the warp item list

@@ -52,6 +52,7 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void* g_addr[kMaxDevices] = {};
 int g_sms[kMaxDevices] = {};
+bool g_acc_dirty[kMaxDevices] = {};  // see ps_grid::acc_dirty
 
 }  // namespace
 
@@ -82,6 +83,7 @@ extern "C" int ps_spatstat_static(const float* xyz, const uint8_t* type, const f
   if (dev < 0 || dev >= kMaxDevices) return fail(PS_ERR_UNSUPPORTED, "ps_spatstat_static: device index too large");
   void* base = nullptr;
   int sms = 0;
+  bool acc_dirty = false;
   {
     std::lock_guard<std::mutex> lk(g_mu);
     if (g_addr[dev] == nullptr) {
@@ -95,6 +97,7 @@ extern "C" int ps_spatstat_static(const float* xyz, const uint8_t* type, const f
     }
     base = g_addr[dev];
     sms = g_sms[dev];
+    acc_dirty = g_acc_dirty[dev];
   }
   char* b = static_cast<char*>(base);
   ps_grid g;  // a grid whose scratch is the static array (nothing to free)
@@ -105,6 +108,7 @@ extern "C" int ps_spatstat_static(const float* xyz, const uint8_t* type, const f
   g.stencil = 1;
   g.item_cap = (uint32_t)kItems;
   g.scan_tiles_cap = (uint32_t)kTiles;
+  g.acc_dirty = acc_dirty;
   g.device = dev;
   g.num_sms = sms;
   g.sel = reinterpret_cast<uint32_t*>(b + o_sel);
@@ -122,9 +126,14 @@ extern "C" int ps_spatstat_static(const float* xyz, const uint8_t* type, const f
   g.ctr.geo = reinterpret_cast<Geo*>(b + o_cgeo);
   g.scan_state = reinterpret_cast<unsigned long long*>(b + o_part);  // zero at load; each scan clears it again
   g.scan_ctr = reinterpret_cast<uint32_t*>(b + o_sctr);
-  // The build kernels clear every counter and geometry field before use, so the
-  // previous call's contents never leak into this one.
+  // Nothing of the previous call leaks into this one: the build's kernels set or clear the counters and the
+  // geometry before they use them, but for the selection's accumulators, which every build leaves at
+  // zero (a failed one marks them, and the next build clears them first).
   rc = ps_grid_build(&g, xyz, type, n, nbr_mask, r_cut, stream);
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    g_acc_dirty[dev] = g.acc_dirty;
+  }
   if (rc) return rc;
   return ps_spatstat(&g, dsrf, ctr_mask, dsrf_min, bins, ks, n_k, d_rdf, d_knn, d_meta, d_kth, d_nwithin, stream);
 }
