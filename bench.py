@@ -882,7 +882,7 @@ def combo_stats(ps, g, o, name, ctr, nbr, X, T, D, t_host, wl, stencil, split=Fa
     (split): every central against its near kNN block (its own 2 x 2 x 2 cells on half-size
     cells, the 27 cells around its cell on third-size cells) plus every unordered pair of records
     in each other's stencil once (symmetric RDF), the few full-radius fallback searches not
-    counted; one pass over a dense cloud leaves the RDF to that pass as well."""
+    counted; one pass over a dense cloud with many centrals leaves the RDF to that pass as well."""
     meta = o["meta"].cpu().numpy()
     if meta[3] != 0:
         raise RuntimeError(f"device status {meta[3]} for {name}")
@@ -904,7 +904,9 @@ def combo_stats(ps, g, o, name, ctr, nbr, X, T, D, t_host, wl, stencil, split=Fa
         by_pass = {"query": near, "rdf_sym": sym}
         cands = near + sym
         swept = False
-    elif subset and info["n_nbr"] >= 8 * info["n_cells"]:  # the RDF over unordered pairs, the kNN's tests not counted
+    elif (subset and info["n_nbr"] >= 8 * info["n_cells"]
+          and 8 * int(meta[0]) >= info["n_nbr"] + 8 * info["n_cells"]):  # (as sweep_pays in ps_internal.cuh)
+        # the RDF over unordered pairs, the kNN's tests not counted
         full = candidate_tests(X, T, D, nbr, nbr, wl["dsrf_min"], info, stencil, all_records=True, cell_scale=cs)
         cands = (full - info["n_nbr"]) // 2
         by_pass = {"rdf_sym": cands}

@@ -105,6 +105,27 @@ __host__ __device__ __forceinline__ uint32_t sub_cells(uint64_t n_rec, uint64_t 
   return s;
 }
 
+// One-pass queries whose centrals are neighbour records: in dense clouds the RDF is left to the sweep
+// over unordered pairs (half the tests, no kNN beside them), in sparse ones the blocks of the
+// sweep are nearly empty and the query's own pass over each central is the better one.  So it is where
+// the centrals are few: the sweep stages every record and walks the candidates of each group that
+// holds a central, the query's pass grows with the centrals.  The counts are known on the device only,
+// where the kernels apply this rule.  Measured (default options, r = 2 nm, one box):
+//   density: 8e6-ion needle, Sc-Sc + Si-Si (1 to 2 records per cell) 0.165 ms in one pass, 0.348 ms with the
+//   sweep; 1e5-ion cylinder, all-all (223 per cell, RDF and k = 1, 4, 10) 0.73 -> 0.37 ms; 2e4-ion cylinder (68 per
+//   cell) 0.140 -> 0.106 ms;
+//   share of the records that are central, one pass / sweep (whole call, k = 1, 5, 10), centrals at random and the
+//   ions furthest from the surface: 4e6-ion needle (104 per cell) 1.32 and 1.69 at 0.35, 1.11 and 1.53 at 0.2, 0.92
+//   and 1.16 at 0.1, 0.71 and 0.96 at 0.05; 1e5-ion cylinder 1.31 and 1.34, 1.01 and 1.13, 0.91 and 0.97, 0.88 and
+//   0.91; 8e6-ion needle, Si about all (0.002) 0.36.  The thinner the cloud the larger the share has to be: 4e6-ion
+//   needle, r = 1 nm (13 per cell) 0.92 and 1.19 at 0.35, 0.78 and 1.05 at 0.2, 0.67 and 0.89 at 0.1.
+__host__ __device__ __forceinline__ bool sweep_pays(uint64_t n_nbr, uint64_t n_cells, uint64_t n_ctr) {
+  return n_nbr >= 8 * n_cells && 8 * n_ctr >= n_nbr + 8 * n_cells;
+}
+__device__ __forceinline__ bool sweep_pays(const Geo& nbr, const Geo& ctr) {
+  return sweep_pays(nbr.n_sel, nbr.n_cells, ctr.n_sel);
+}
+
 // Warp items with at least this many centrals per cell are listed first (largest work first).
 constexpr uint32_t kHeavy = 16;
 // Central lists: cells with fewer than kHeavy centrals and at most this many candidates in

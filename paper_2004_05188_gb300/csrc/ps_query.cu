@@ -18,8 +18,8 @@
 //                  (sparser cells) are taken 32 at a time and each of their
 //                  centrals gets one thread that walks its own stencil.
 //   k_rdf_sym      the RDF, and the in-range counts, over unordered pairs of
-//                  neighbour records: where every central is one and the cloud
-//                  is dense (sweep_pays), or in passes.
+//                  neighbour records: where every central is one, the cloud is
+//                  dense and the centrals are many (sweep_pays), or in passes.
 //   k_query_cta    for cells with >= dense_min centrals (an option): one CTA per
 //                  cell; the runs are staged into shared memory with bulk
 //                  asynchronous copies (cp.async.bulk, completion on an mbarrier)
@@ -41,15 +41,6 @@
 #include "ps_sweep.cuh"
 
 namespace ps {
-
-// One-pass queries whose centrals are neighbour records: in dense clouds the RDF is left to the sweep
-// over unordered pairs (half the tests, no kNN beside them), in sparse ones the blocks of the
-// sweep are nearly empty and the query's own pass over each central is the better one.  The cloud's
-// density is known on the device only, where both kernels apply this rule.  Measured (query and sweep,
-// one box): 8e6-ion needle, Sc-Sc + Si-Si (1 to 2 records per cell) 0.165 ms in one pass, 0.348 ms with
-// the sweep; 1e5-ion cylinder, all-all (223 per cell, RDF and k = 1, 4, 10) 0.73 -> 0.37 ms; 2e4-ion cylinder
-// (68 per cell) 0.140 -> 0.106 ms.
-__device__ __forceinline__ bool sweep_pays(const Geo& g) { return (uint64_t)g.n_sel >= 8ull * g.n_cells; }
 
 struct QueryArgs {
   const float4* nrec;
@@ -428,7 +419,7 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : (KMAX <= 16 ? 3 : 2)) k_
   __shared__ float4 s_buf[8][kRing];            // per warp: ring of kept candidates, as interleaved pairs
   __shared__ float s_kq[8][32 * kHalf + 32];    // per warp: kNN insertion queue, [slot][lane] + a spare row
   constexpr int KK = KMAX > 0 ? KMAX : 1;
-  if (KMAX == 0 && a.sweep && sweep_pays(*a.ngeo)) return;  // nothing is left to do here
+  if (KMAX == 0 && a.sweep && sweep_pays(*a.ngeo, *a.cgeo)) return;  // nothing is left to do here
   Hist<RDF> H{};
   H.init(a, smem, 0, true);
   FastBins fb;
@@ -441,7 +432,7 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : (KMAX <= 16 ? 3 : 2)) k_
   const uint32_t n_hi = a.cgeo->work_n4, n_front = n_hi + a.cgeo->work_n2, n_light = a.cgeo->work_n3;
   const Search S = search_of(a);
   const float u_slack = item_slack(ng);
-  const bool swept = a.sweep && sweep_pays(ng);  // RDF and in-range counts are the sweep's
+  const bool swept = a.sweep && sweep_pays(ng, *a.cgeo);  // RDF and in-range counts are the sweep's
   const bool rdf_here = RDF && !swept;
   uint32_t* const nwithin = swept ? nullptr : a.nwithin;
   const float erange = a.emax_near > 0.f ? a.emax_near : H.Emax;  // squared search range of this pass
@@ -854,7 +845,7 @@ __global__ void __launch_bounds__(256, WITHIN ? 3 : 4) k_rdf_sym(const QueryArgs
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ SweepBuf s_sweep[8];
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (a.sweep && !sweep_pays(*a.ngeo)) return;
+  if (a.sweep && !sweep_pays(*a.ngeo, *a.cgeo)) return;
   SweepBuf& buf = s_sweep[w];
   uint64_t wcount = 0;  // bound on the increments of this warp's rows since their last flush (uniform)
   if constexpr (FAST) {
@@ -1298,7 +1289,7 @@ __global__ void __launch_bounds__(256) k_query_epilogue(const Geo* __restrict__ 
                                                         const uint32_t* __restrict__ wacc, uint32_t* __restrict__ nwithin) {
   griddep_wait();
   griddep_launch();
-  if (wacc != nullptr && sweep_pays(*ngeo)) {
+  if (wacc != nullptr && sweep_pays(*ngeo, *cgeo)) {
     const uint32_t n = ngeo->n_sel;
     for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
       if (pfx[j + 1] == pfx[j]) continue;
