@@ -154,6 +154,7 @@ int ps_grid_create(int64_t n_max, const ps_grid_opts* opts, ps_grid** out) {
   const size_t o_sT = take(kSoftFineMax * 16), o_sgs = take(8);
   const size_t o_part = take((size_t)g->scan_tiles_cap * 8), o_sctr = take(8);
   const size_t o_ngeo = take(sizeof(Geo)), o_cgeo = take(sizeof(Geo));
+  const size_t o_heavy = take(heavy_capacity(nm) * 8), o_hmap = take((cc / 32 + 1) * 4);
   void* base = nullptr;
   cudaError_t e = dev_malloc(&base, off);
   if (e != cudaSuccess) {
@@ -187,6 +188,8 @@ int ps_grid_create(int64_t n_max, const ps_grid_opts* opts, ps_grid** out) {
   g->soft_T = reinterpret_cast<float*>(b + o_sT);
   g->soft_gs = reinterpret_cast<double*>(b + o_sgs);
   g->ctr.geo = reinterpret_cast<Geo*>(b + o_cgeo);
+  g->heavy = reinterpret_cast<uint2*>(b + o_heavy);
+  g->heavy_map = reinterpret_cast<uint32_t*>(b + o_hmap);
   g->scan_state = reinterpret_cast<unsigned long long*>(b + o_part);
   g->scan_ctr = reinterpret_cast<uint32_t*>(b + o_sctr);
   e = cudaMemset(g->nbr.geo, 0, sizeof(Geo));

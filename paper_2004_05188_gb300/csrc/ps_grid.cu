@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kThreads) k_geometry_zero(Geo* geo, float r_cu
       geo->status = g.acc_status;
       geo->work_n = geo->work_n2 = geo->work_n3 = geo->work_n4 = 0;
       geo->work_next = geo->work_next2 = geo->work_next3 = 0;
-      geo->work_next2b = geo->work_next3b = geo->sym_next = geo->list_n = 0;
+      geo->work_next2b = geo->work_next3b = geo->sym_next = geo->list_n = geo->n_heavy = geo->heavy_listed = 0;
       for (int a = 0; a < 3; ++a) geo->origin[a] = g.origin[a], geo->dims[a] = g.dims[a];
       geo->h = g.h;
       geo->inv_h = g.inv_h;
@@ -476,12 +476,13 @@ __device__ uint32_t tile_lookback(uint32_t t, uint32_t total, unsigned long long
 
 // End of a single-pass scan (thread 0 of every CTA): the last CTA to finish clears
 // the look-back words and the tile counter for the next scan.
-__device__ void scan_finish(unsigned long long* state, uint32_t* ctr, uint32_t tiles) {
+__device__ void scan_finish(unsigned long long* state, uint32_t* ctr, uint32_t tiles, uint32_t* done = nullptr) {
   if (threadIdx.x == 0) {
     __threadfence();
     if (atomicAdd(&ctr[1], 1u) == gridDim.x - 1) {
       for (uint32_t i = 0; i < tiles; ++i) state[i] = 0ull;
       ctr[0] = 0;
+      if (done) *done = 1u;  // (every CTA is past reading it)
       __threadfence();
       ctr[1] = 0;
     }
@@ -614,6 +615,45 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(uint32_t* __restrict__ co
   scan_finish(state, ctr, tiles);
 }
 
+// The heavy blocks' groups and the map of those blocks (all threads of the grid).  From the last thread block
+// backwards: in small clouds that one has no other work.
+__device__ __forceinline__ void list_heavy(const uint32_t* __restrict__ start, Geo* geo, uint2* __restrict__ heavy,
+                                           uint32_t* __restrict__ map, uint32_t n_warps, int stencil) {
+  const uint32_t ns = geo->n_sel, nc = geo->n_cells, d0 = geo->dims[0], d1 = geo->dims[1], d2 = geo->dims[2];
+  const uint32_t B = sweep_block(nc, ns), nbx = (d0 + B - 1) / B, n_blocks = nbx * d1 * d2;
+  const uint32_t S = sweep_parts(n_blocks, n_warps);
+  const bool ok = geo->status == 0;  // no blocks are listed after a scan that gave up
+  // (a warp writes whole words of the map)
+  for (uint32_t base = (gridDim.x - 1 - blockIdx.x) * blockDim.x; base < n_blocks; base += gridDim.x * blockDim.x) {
+    const uint32_t blk = base + threadIdx.x;
+    bool is = false;
+    if (ok && blk < n_blocks) {
+      const uint32_t row = blk / nbx, ux = (blk - row * nbx) * B;
+      const uint32_t a0 = start[row * d0 + ux], a1 = start[row * d0 + min(ux + B, d0)], n = a1 - a0;
+      if (heavy_block(n, ns, ns, nc, S, n_warps, stencil)) {  // (it could be, if it met every record)
+        const int st = min(stencil, 2), y = (int)(row % d1), z = (int)(row / d1);
+        const uint32_t x0 = ux > (uint32_t)st ? ux - st : 0u, x1 = min(ux + B + st, d0);
+        uint32_t n_cand = 0;
+#pragma unroll 1
+        for (int q = max(z - st, 0); q <= min(z + st, (int)d2 - 1); ++q)
+#pragma unroll 1
+          for (int r = max(y - st, 0); r <= min(y + st, (int)d1 - 1); ++r) {
+            const uint32_t* s = start + ((uint32_t)q * d1 + (uint32_t)r) * d0;
+            n_cand += s[x1] - s[x0];
+          }
+        is = heavy_block(n, n_cand, ns, nc, S, n_warps, stencil);
+      }
+      if (is) {
+        const uint32_t m = (n + kHeavyGroup - 1) / kHeavyGroup, at = atomicAdd(&geo->n_heavy, m);
+#pragma unroll 1
+        for (uint32_t i = 0; i < m; ++i) heavy[at + i] = make_uint2(a0 + i * kHeavyGroup, blk);
+      }
+    }
+    const uint32_t word = __ballot_sync(0xffffffffu, is);  // (thread blocks of whole warps)
+    if (lane_id() == 0 && blk < n_blocks) map[blk >> 5] = word;
+  }
+}
+
 // Central list of a central type set contained in the neighbour set, step 1 of 2.
 // The centrals are then a subset of the neighbour records, which are already
 // sorted by cell: an order-preserving compaction of those records (single-pass
@@ -621,14 +661,23 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(uint32_t* __restrict__ co
 // directly, with no second pass over the whole cloud and no counting sort.  pfx[j]
 // = number of centrals among records 0..j-1 (pfx[n_records] = all), from which
 // k_central_items reads the cell starts.  Also resets the central list's geometry
-// and counters and zeroes the query's outputs.
-__global__ void __launch_bounds__(kScanThreads) k_central_subset(const float4* __restrict__ nrec,
-                                                                 const Geo* __restrict__ ngeo, Geo* cgeo,
+// and counters and zeroes the query's outputs.  With `hv.list` given a sweep over the neighbour records follows:
+// lists their heavy blocks, once per build.
+struct HeavyOut {
+  uint2* list = nullptr;
+  uint32_t* map = nullptr;
+  const uint32_t* nstart = nullptr;
+  uint32_t n_warps = 0;
+  int stencil = 0;
+  bool if_dense = false;  // the sweep runs in dense clouds only (sweep_pays)
+};
+__global__ void __launch_bounds__(kScanThreads) k_central_subset(const float4* __restrict__ nrec, Geo* ngeo, Geo* cgeo,
                                                                  const uint8_t* __restrict__ type,
                                                                  const float* __restrict__ dsrf, Mask mask,
                                                                  float dsrf_min, float4* __restrict__ crec,
                                                                  uint32_t* __restrict__ pfx, unsigned long long* state,
-                                                                 uint32_t* ctr, ZeroOut z, uint32_t* __restrict__ vcount) {
+                                                                 uint32_t* ctr, ZeroOut z, uint32_t* __restrict__ vcount,
+                                                                 HeavyOut hv) {
   griddep_wait();
   griddep_launch();
   __shared__ uint32_t s_warp[32];
@@ -660,6 +709,8 @@ __global__ void __launch_bounds__(kScanThreads) k_central_subset(const float4* _
     if (vcount)
       for (uint32_t i = tid; i < nvc; i += stride) vcount[i] = 0u;
   }
+  const bool list = hv.list != nullptr && ngeo->heavy_listed == 0 && (!hv.if_dense || sweep_pays(nr, ngeo->n_cells, nr));
+  if (list) list_heavy(hv.nstart, ngeo, hv.list, hv.map, hv.n_warps, hv.stencil);
   const uint32_t tiles = (nr + kScanTile - 1) / kScanTile;
   for (;;) {
     if (threadIdx.x == 0) s_tile = atomicAdd(&ctr[0], 1u);
@@ -700,7 +751,7 @@ __global__ void __launch_bounds__(kScanThreads) k_central_subset(const float4* _
     }
     __syncthreads();  // s_tile and s_prefix are rewritten next
   }
-  scan_finish(state, ctr, tiles);
+  scan_finish(state, ctr, tiles, list ? &ngeo->heavy_listed : nullptr);
 }
 
 // Work lists of the central list.  Central type set contained in the neighbour set (`pfx` given),
@@ -870,10 +921,13 @@ int build_neighbour_grid(ps_grid* g, const uint64_t nbr_mask[4], float r_cut, cu
 }
 
 int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsrf_min, cudaStream_t s,
-                       ZeroOut z, bool split, bool vertex, bool items) {
+                       ZeroOut z, bool split, bool vertex, bool items, Sweep sweep) {
   Mask m;
   for (int w = 0; w < 4; ++w) m.w[w] = ctr_mask[w];
   const bool subset = centrals_in_neighbours(g, ctr_mask);
+  HeavyOut hv;
+  if (sweep != kNoSweep)
+    hv = HeavyOut{g->heavy, g->heavy_map, g->nbr.start, (uint32_t)g->num_sms * 32u, g->stencil, sweep == kSweepIfDense};
   if (subset && vertex) {
     // the central prefix over the neighbour records, then the centrals sorted by the
     // vertex-centred grid (ranks in the dense-cell list, unused without dense cells)
@@ -881,7 +935,7 @@ int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4]
     PS_LAUNCH(PS_KID_CENTRAL, s,
               PS_CUDA(launch_pdl(k_central_subset, grid_blocks(g, 1), kScanThreads, 0, s, g->nbr.rec, g->nbr.geo,
                                  g->ctr.geo, g->type, dsrf, m, dsrf_min, (float4*)nullptr, pfx, g->scan_state,
-                                 g->scan_ctr, z, g->ctr.count)));
+                                 g->scan_ctr, z, g->ctr.count, hv)));
     PS_LAUNCH(PS_KID_CENTRAL, s,
               PS_CUDA(launch_pdl(k_vertex_count, grid_blocks(g, 8), kThreads, 0, s, g->nbr.rec, g->nbr.geo, g->ctr.geo,
                                  pfx, g->ctr.count, g->ctr.work)));
@@ -901,7 +955,7 @@ int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4]
     PS_LAUNCH(PS_KID_CENTRAL, s,
               PS_CUDA(launch_pdl(k_central_subset, grid_blocks(g, 1), kScanThreads, 0, s, g->nbr.rec, g->nbr.geo,
                                  g->ctr.geo, g->type, dsrf, m, dsrf_min, items ? g->ctr.rec : (float4*)nullptr, pfx, g->scan_state,
-                                 g->scan_ctr, z, (uint32_t*)nullptr)));
+                                 g->scan_ctr, z, (uint32_t*)nullptr, hv)));
     if (items)
       PS_LAUNCH(PS_KID_SCAN, s,
               PS_CUDA(launch_pdl(k_central_items, grid_blocks(g, 4), kThreads, 0, s, g->nbr.start, (const uint32_t*)pfx, g->ctr.geo,

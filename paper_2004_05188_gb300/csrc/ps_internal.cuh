@@ -88,7 +88,9 @@ struct Geo {
   uint32_t work_n4;    // very heavy warp items (exact query), listed apart and taken before the others
   uint32_t work_next2b;  // second pass over the same items (the exact query's full-radius kNN fallback)
   uint32_t work_next3b;
-  uint32_t sym_next;     // cells taken by the symmetric RDF pass (32 at a time)
+  uint32_t sym_next;     // units taken by the sweep over unordered pairs
+  uint32_t n_heavy;      // groups of the heavy blocks listed for the sweep (neighbour grid)
+  uint32_t heavy_listed; // they have been listed since the build
   uint32_t list_n;       // centrals listed by the near kNN pass for the full-radius search
   uint32_t sub;          // the records of a cell are ordered by its 2^sub x 2^sub x 2^sub sub-cells
 };
@@ -125,6 +127,36 @@ __host__ __device__ __forceinline__ bool sweep_pays(uint64_t n_nbr, uint64_t n_c
 __device__ __forceinline__ bool sweep_pays(const Geo& nbr, const Geo& ctr) {
   return sweep_pays(nbr.n_sel, nbr.n_cells, ctr.n_sel);
 }
+
+// Blocks of the sweep over unordered pairs: x-consecutive cells of one row.  A block costs a run table and
+// the staging whatever it holds, and a wider one more tests per record: blocks of 12 records on average
+// over the bounding box (2e5-ion cylinder, 9 records per cell: 0.272 ms with one cell, 0.236 ms with two; the
+// 8e6-ion needle's 28 records per filled cell need no company).
+__host__ __device__ __forceinline__ uint32_t sweep_block(uint32_t n_cells, uint32_t n_sel) {
+  const float w = 12.f * (float)n_cells / (float)(n_sel ? n_sel : 1u);
+  return w > 7.f ? 8u : (w <= 1.f ? 1u : (uint32_t)ceilf(w));
+}
+// Candidate parts per block of the sweep: at least 4 units per warp of the launch.
+__host__ __device__ __forceinline__ uint32_t sweep_parts(uint64_t n_blocks, uint32_t n_warps) {
+  const uint64_t S = n_blocks >= 4ull * n_warps ? 1u : (4ull * n_warps + n_blocks - 1) / n_blocks;
+  return S < 16u ? (uint32_t)S : 16u;
+}
+// Heavy blocks.  A block of a very dense spot (a cluster far above the mean density, a cloud of a few cells) can hold
+// more work than a warp's share of the whole sweep.  The central list's first kernel lists the records of such
+// blocks in groups of at most 64, which the sweep takes one by one before the blocks.  Heavy: n records against n_cand
+// candidates, n n_cand / 2 above twice a warp's share (by the mean density, an underestimate) and 2^17 tests
+// (40 us) in each of the S parts; even clouds have none.  Whole calls, half-size cells, r = 2 nm (ms): 2e5 ions and
+// 5e4 more in one spot (0.3 nm wide), RDF and k = 1, 5, 10 251 -> 6.1, map 1871 -> 27; 2e6 ions and 5e4 in a spot of
+// 0.5 nm, adjoint of the smoothed RDF 2531 -> 15 (a warp per central's batch, before the sweep: 10.7, 57 and 28).
+constexpr uint32_t kHeavyGroup = 64;
+__host__ __device__ __forceinline__ bool heavy_block(uint32_t n, uint32_t n_cand, uint32_t n_sel, uint32_t n_cells,
+                                                     uint32_t S, uint32_t n_warps, int stencil) {
+  const float w = (float)(2 * stencil + 1), mean = (float)n_sel / (float)n_cells;
+  const float share = (float)n_sel * mean * w * w * w / (float)n_warps;  // twice n_sel w^3 mean / 2
+  return n > kHeavyGroup && 0.5f * (float)n * (float)n_cand > (float)S * (share > 131072.f ? share : 131072.f);
+}
+// (slots for the groups: a block of n > 64 records has at most n / 32.5 of them)
+constexpr uint64_t heavy_capacity(uint64_t n) { return n / 32 + 1; }
 
 // Warp items with at least this many centrals per cell are listed first (largest work first).
 constexpr uint32_t kHeavy = 16;
@@ -231,6 +263,8 @@ struct ps_grid {
   double* soft_m2 = nullptr;
   float* soft_T = nullptr;
   double* soft_gs = nullptr;
+  uint2* heavy = nullptr;         // [heavy_capacity(n_max)] the heavy blocks' groups: first record, block
+  uint32_t* heavy_map = nullptr;  // [cell_cap / 32 + 1] bit per block of the sweep: heavy
   uint2* nbr_witem = nullptr;  // [item_cap] warp items over the neighbour list (adjoint pass B)
   ps::CellList nbr;  // neighbour grid (geometry owner)
   ps::CellList ctr;  // central list, same geometry
@@ -272,10 +306,13 @@ struct ZeroOut {
 // split: size the warp items of dense cells for lanes_per_central (the exact query's staged path);
 // vertex: centrals among the neighbour records sorted by the vertex-centred grid (the query in
 // passes on cells smaller than r_cut), the central prefix in g->cr
+// sweep: a sweep over the neighbour records follows (in dense clouds only)
+enum Sweep { kNoSweep, kSweep, kSweepIfDense };
 // items: false leaves out the central list's cell starts and work items where the centrals are
 // neighbour records (the sweep over unordered pairs needs the records' prefix only)
 int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsrf_min, cudaStream_t s,
-                       ZeroOut z = ZeroOut(), bool split = false, bool vertex = false, bool items = true);
+                       ZeroOut z = ZeroOut(), bool split = false, bool vertex = false, bool items = true,
+                       Sweep sweep = kNoSweep);
 // the centrals are neighbour records of the last build
 inline bool centrals_in_neighbours(const ps_grid* g, const uint64_t ctr_mask[4]) {
   bool subset = !g->pack_type;

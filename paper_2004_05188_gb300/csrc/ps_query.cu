@@ -419,7 +419,8 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : (KMAX <= 16 ? 3 : 2)) k_
   __shared__ float4 s_buf[8][kRing];            // per warp: ring of kept candidates, as interleaved pairs
   __shared__ float s_kq[8][32 * kHalf + 32];    // per warp: kNN insertion queue, [slot][lane] + a spare row
   constexpr int KK = KMAX > 0 ? KMAX : 1;
-  if (KMAX == 0 && a.sweep && sweep_pays(*a.ngeo, *a.cgeo)) return;  // nothing is left to do here
+  const bool swept = a.sweep && sweep_pays(*a.ngeo, *a.cgeo);  // RDF and in-range counts are the sweep's
+  if (KMAX == 0 && swept) return;                              // nothing is left to do here
   Hist<RDF> H{};
   H.init(a, smem, 0, true);
   FastBins fb;
@@ -432,7 +433,6 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : (KMAX <= 16 ? 3 : 2)) k_
   const uint32_t n_hi = a.cgeo->work_n4, n_front = n_hi + a.cgeo->work_n2, n_light = a.cgeo->work_n3;
   const Search S = search_of(a);
   const float u_slack = item_slack(ng);
-  const bool swept = a.sweep && sweep_pays(ng, *a.cgeo);  // RDF and in-range counts are the sweep's
   const bool rdf_here = RDF && !swept;
   uint32_t* const nwithin = swept ? nullptr : a.nwithin;
   const float erange = a.emax_near > 0.f ? a.emax_near : H.Emax;  // squared search range of this pass
@@ -1436,7 +1436,8 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
   // stencils; the ranks of that counting sort take one word per central of the cell arrays)
   const bool split = in_passes;
   const bool vertex = split && n_k > 0 && g->stencil == 2 && (uint64_t)g->n <= (uint64_t)g->cell_cap;
-  int rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, true, vertex, !split || n_k > 0);
+  int rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, true, vertex, !split || n_k > 0,
+                              split ? kSweep : (sweep ? kSweepIfDense : kNoSweep));
   if (rc) return rc;
 
   // staging budget of the CTA kernel: two CTAs per SM

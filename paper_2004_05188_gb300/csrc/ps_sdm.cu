@@ -327,7 +327,7 @@ int run_sdm(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsr
   // (a radius or voxel near the limits of float32 keeps the general kernel)
   const bool sym = centrals_in_neighbours(g, ctr_mask) && spec.r_max > 1e-15 && spec.r_max < 1e15 && spec.w > 1e-15 &&
                    spec.w < 1e15;
-  int rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, false, false, !sym);
+  int rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, false, false, !sym, sym ? kSweep : kNoSweep);
   if (rc) return rc;
   const float ER = (float)(spec.r_max * spec.r_max);
   if (sym) {

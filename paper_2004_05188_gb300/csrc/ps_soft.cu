@@ -798,7 +798,7 @@ int soft_forward(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], floa
   z.p[2] = reinterpret_cast<uint64_t*>(g->soft_m2);
   z.n[0] = z.n[1] = z.n[2] = sa.n_fine;
   const bool sym = centrals_in_neighbours(g, ctr_mask);
-  rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, false, false, !sym);
+  rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, false, false, !sym, sym ? kSweep : kNoSweep);
   if (rc) return rc;
   sa.nrec = g->nbr.rec;
   sa.nstart = g->nbr.start;
@@ -842,7 +842,7 @@ int soft_backward(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], flo
   int rc = soft_setup(g, sigma, scale, bins, sa, w);
   if (rc) return rc;
   const bool sym = centrals_in_neighbours(g, ctr_mask);
-  rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, ZeroOut(), false, false, !sym);
+  rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, ZeroOut(), false, false, !sym, sym ? kSweep : kNoSweep);
   if (rc) return rc;
   PS_CUDA(cudaMemsetAsync(d_grad, 0, (size_t)g->n * 3 * sizeof(float), s));
   PS_CUDA(cudaMemsetAsync(g->soft_gs, 0, sizeof(double), s));

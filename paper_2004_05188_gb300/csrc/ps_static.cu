@@ -45,7 +45,9 @@ constexpr size_t o_part = o_nwitem + align256(kItems * 8);
 constexpr size_t o_sctr = o_part + align256(kTiles * 8);
 constexpr size_t o_ngeo = o_sctr + align256(8);
 constexpr size_t o_cgeo = o_ngeo + align256(sizeof(Geo));
-constexpr size_t kBytes = o_cgeo + align256(sizeof(Geo));
+constexpr size_t o_heavy = o_cgeo + align256(sizeof(Geo));
+constexpr size_t o_hmap = o_heavy + align256(heavy_capacity(kN) * 8);
+constexpr size_t kBytes = o_hmap + align256((kCells / 32 + 1) * 4);
 
 constexpr int kMaxDevices = 64;
 
@@ -124,6 +126,8 @@ extern "C" int ps_spatstat_static(const float* xyz, const uint8_t* type, const f
   g.ctr.witem = reinterpret_cast<uint2*>(b + o_witem);
   g.nbr_witem = reinterpret_cast<uint2*>(b + o_nwitem);
   g.ctr.geo = reinterpret_cast<Geo*>(b + o_cgeo);
+  g.heavy = reinterpret_cast<uint2*>(b + o_heavy);
+  g.heavy_map = reinterpret_cast<uint32_t*>(b + o_hmap);
   g.scan_state = reinterpret_cast<unsigned long long*>(b + o_part);  // zero at load; each scan clears it again
   g.scan_ctr = reinterpret_cast<uint32_t*>(b + o_sctr);
   // Nothing of the previous call leaks into this one: the build's kernels set or clear the counters and the

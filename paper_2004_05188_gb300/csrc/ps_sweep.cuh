@@ -17,6 +17,8 @@
 //   * the kept ones are compacted into tiles of 64, two per lane in registers, and tested against
 //     the records (read two at a time by every lane at once).
 //
+// Blocks that hold more than a warp's share of the work (heavy_block) are listed beforehand in groups of at most
+// 64 records, which are units of their own.
 // The pairs inside the block are met in both orders, with weight 1 for each central end.
 #pragma once
 
@@ -27,7 +29,7 @@ namespace ps {
 constexpr float kMagic = 12582912.0f;           // 1.5 * 2^23: x + kMagic holds floor(x) in its low bits
 constexpr uint32_t kMagicBits = 0x4B400000u;
 
-constexpr uint32_t kSweepRec = 64;        // records staged at a time
+constexpr uint32_t kSweepRec = kHeavyGroup;  // records staged at a time
 constexpr uint32_t kSweepGroup = 64;     // of whole sub-cells
 constexpr uint32_t kSweepTile = 64;       // candidates per tile, two per lane
 constexpr uint32_t kCandSingle = 0u, kCandBoth = 1u, kCandOwn = 2u, kCandSelf = 3u;
@@ -57,6 +59,8 @@ struct SweepArgs {
   const uint32_t* nsub; // sub-cell starts (where the cells have sub-cells)
   const uint32_t* pfx;  // central prefix over the neighbour records
   const Geo* ngeo;
+  const uint2* heavy;         // groups of the heavy blocks: first record, block (ngeo->n_heavy)
+  const uint32_t* heavy_map;  // bit per block: its groups are listed
   uint32_t* next;       // work counter (units taken)
   int stencil;
   float range;          // pairs with d2 < range are in range
@@ -93,6 +97,8 @@ inline SweepArgs sweep_args(const ps_grid* g, uint32_t* next) {
   a.nsub = g->nbr.count;
   a.pfx = reinterpret_cast<const uint32_t*>(g->cr);  // written by the central-list compaction
   a.ngeo = g->nbr.geo;
+  a.heavy = g->heavy;
+  a.heavy_map = g->heavy_map;
   a.next = next;
   a.stencil = g->stencil;
   a.one = 1.0f;
@@ -120,17 +126,6 @@ __device__ __forceinline__ unsigned long long dist2_x2_fma(unsigned long long px
   return f2_fma(f2_fma(f2_mul(dx, dx), one, f2_mul(dy, dy)), one, f2_mul(dz, dz));
 }
 
-// Cells of the grid that one block spans, and the parts that the candidates of a block are split
-// into.  A block costs a run table and the staging whatever it holds, and a wider one more tests
-// per record: blocks of 12 records on average over the bounding box (2e5-ion cylinder, 9 records
-// per cell: 0.272 ms with one cell, 0.236 ms with two; the 8e6-ion needle's 28 records per filled
-// cell need no company), and at least 4 units per warp of the launch.
-__device__ __forceinline__ void sweep_shape(const Geo& g, uint32_t n_warps, uint32_t& B, uint32_t& S) {
-  B = (uint32_t)fminf(8.f, fmaxf(1.f, ceilf(12.f * (float)g.n_cells / (float)max(g.n_sel, 1u))));
-  const uint32_t units = ((g.dims[0] + B - 1) / B) * g.dims[1] * g.dims[2];
-  S = units >= 4 * n_warps ? 1u : min(16u, (4 * n_warps + units - 1) / units);
-}
-
 // Runs every unit.  tile(n_pr, m, nc, central): the staged records (m of them, n_pr pairs, n_pr even,
 // padded with far records), all central or all not, against nc <= 64 candidates in buf.cand.
 // INDEX: fill buf.cidx / buf.ridx.  done(m, central) follows the last tile of the staged records.
@@ -140,9 +135,10 @@ __device__ __forceinline__ void sweep_pairs(const SweepArgs& a, SweepBuf& buf, T
   const Geo g = *a.ngeo;
   const int s = a.stencil, W = 2 * s + 1, inv_w = 65536 / W + 1;
   const uint32_t n_warps = gridDim.x * (blockDim.x >> 5);
-  uint32_t B, S;
-  sweep_shape(g, n_warps, B, S);
-  const uint32_t nbx = (g.dims[0] + B - 1) / B, n_units = nbx * g.dims[1] * g.dims[2] * S;
+  // units: S parts of the candidates each for the groups of the heavy blocks and for the blocks
+  const uint32_t B = sweep_block(g.n_cells, g.n_sel), nbx = (g.dims[0] + B - 1) / B;
+  const uint32_t n_blocks = nbx * g.dims[1] * g.dims[2], S = sweep_parts(n_blocks, n_warps);
+  const uint32_t n_heavy = g.n_heavy, n_units = (n_heavy + n_blocks) * S;
   // a record further than this from the box of the staged ones is out of range of each of them
   // (the slack covers the rounding of both float32 distances)
   const float lim = a.range * 1.00001f;
@@ -152,7 +148,7 @@ __device__ __forceinline__ void sweep_pairs(const SweepArgs& a, SweepBuf& buf, T
     if (lane == 0) {
       const uint32_t cur = *reinterpret_cast<volatile uint32_t*>(a.next);
       const uint32_t left = cur < n_units ? n_units - cur : 0u;
-      take = min(32u, max(1u, left / (8 * n_warps)));
+      take = cur < n_heavy * S ? 1u : min(32u, max(1u, left / (8 * n_warps)));
       base = atomicAdd(a.next, take);
     }
     base = __shfl_sync(0xffffffffu, base, 0);
@@ -161,11 +157,20 @@ __device__ __forceinline__ void sweep_pairs(const SweepArgs& a, SweepBuf& buf, T
     // lane i: block (first cell, row) and records of unit base + i
     uint32_t s0 = 0, s1 = 0, ux = 0, uy = 0, uz = 0, upart = 0;
     if (lane < take && base + lane < n_units) {
-      const uint32_t blk = (base + lane) / S, row = blk / nbx;
+      const uint32_t u = (base + lane) / S;
       upart = (base + lane) % S;
+      uint32_t blk = u - n_heavy;
+      if (u < n_heavy) {
+        const uint2 e = a.heavy[u];
+        s0 = e.x, blk = e.y;
+      }
+      const uint32_t row = blk / nbx;
       ux = (blk % nbx) * B, uy = row % g.dims[1], uz = row / g.dims[1];
-      s0 = a.nstart[row * g.dims[0] + ux];
       s1 = a.nstart[row * g.dims[0] + min(ux + B, g.dims[0])];
+      if (u < n_heavy)
+        s1 = min(s1, s0 + kHeavyGroup);
+      else
+        s0 = n_heavy && ((a.heavy_map[blk >> 5] >> (blk & 31u)) & 1u) ? s1 : a.nstart[row * g.dims[0] + ux];
     }
     uint32_t todo = __ballot_sync(0xffffffffu, s1 > s0);
     while (todo) {
@@ -209,7 +214,8 @@ __device__ __forceinline__ void sweep_pairs(const SweepArgs& a, SweepBuf& buf, T
       // 9e5 ions on 1.5 nm cells 1.36 and 1.15 against 1.12 ms.
       const uint32_t f0 = ((__shfl_sync(0xffffffffu, uz, src_lane) * g.dims[1] + __shfl_sync(0xffffffffu, uy, src_lane)) *
                                g.dims[0] + __shfl_sync(0xffffffffu, ux, src_lane)) << (3 * g.sub);
-      uint32_t q = 0, qe = g.sub ? a0 : a1, g1;
+      // (a group of a heavy block is staged as it is)
+      uint32_t q = 0, qe = g.sub && a1 - a0 > kSweepGroup ? a0 : a1, g1;
       for (uint32_t g0 = a0; g0 < a1; g0 = g1) {
         while (qe == g0) {  // the next sub-cells: lane l proposes 2^l of them
           const uint32_t w = 1u << min(lane, 6u), q1 = q + w, nq = 1u << (3 * g.sub);
