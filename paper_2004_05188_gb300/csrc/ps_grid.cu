@@ -921,7 +921,7 @@ int build_neighbour_grid(ps_grid* g, const uint64_t nbr_mask[4], float r_cut, cu
 }
 
 int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsrf_min, cudaStream_t s,
-                       ZeroOut z, bool split, bool vertex, bool items, Sweep sweep) {
+                       ZeroOut z, bool split, bool vertex, bool items, Sweep sweep, bool records) {
   Mask m;
   for (int w = 0; w < 4; ++w) m.w[w] = ctr_mask[w];
   const bool subset = centrals_in_neighbours(g, ctr_mask);
@@ -954,7 +954,7 @@ int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4]
     uint32_t* pfx = reinterpret_cast<uint32_t*>(g->cr);  // 2 n_max words, n_records + 1 needed
     PS_LAUNCH(PS_KID_CENTRAL, s,
               PS_CUDA(launch_pdl(k_central_subset, grid_blocks(g, 1), kScanThreads, 0, s, g->nbr.rec, g->nbr.geo,
-                                 g->ctr.geo, g->type, dsrf, m, dsrf_min, items ? g->ctr.rec : (float4*)nullptr, pfx, g->scan_state,
+                                 g->ctr.geo, g->type, dsrf, m, dsrf_min, items || records ? g->ctr.rec : (float4*)nullptr, pfx, g->scan_state,
                                  g->scan_ctr, z, (uint32_t*)nullptr, hv)));
     if (items)
       PS_LAUNCH(PS_KID_SCAN, s,

@@ -309,10 +309,11 @@ struct ZeroOut {
 // sweep: a sweep over the neighbour records follows (in dense clouds only)
 enum Sweep { kNoSweep, kSweep, kSweepIfDense };
 // items: false leaves out the central list's cell starts and work items where the centrals are
-// neighbour records (the sweep over unordered pairs needs the records' prefix only)
+// neighbour records (the sweep over unordered pairs needs the records' prefix only), and their records
+// unless those are asked for
 int build_central_list(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsrf_min, cudaStream_t s,
                        ZeroOut z = ZeroOut(), bool split = false, bool vertex = false, bool items = true,
-                       Sweep sweep = kNoSweep);
+                       Sweep sweep = kNoSweep, bool records = false);
 // the centrals are neighbour records of the last build
 inline bool centrals_in_neighbours(const ps_grid* g, const uint64_t ctr_mask[4]) {
   bool subset = !g->pack_type;

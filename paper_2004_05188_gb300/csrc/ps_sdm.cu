@@ -5,8 +5,9 @@
 // the float32 displacement x_j - x_i is binned into cubic voxels of edge w;
 // the paper's setting is w = 0.025 nm with R = 2 nm (Results, strong scaling).
 //
-// Where the centrals are neighbour records every unordered pair is met once
-// (sweep_pairs) and the pairs with two central ends are mirrored afterwards.
+// Where the centrals are neighbour records and not few every unordered pair is met once
+// (sweep_pairs) and the pairs with two central ends are mirrored afterwards; where they
+// are few each gets a warp.
 // Otherwise the enumeration is over the exact query's cell grid and central list:
 // each central gets one thread; the centrals of a dense cell's item share the
 // candidate walk, so their loads of a record broadcast from L1 (cells with at
@@ -39,6 +40,7 @@ struct SdmArgs {
   uint32_t n_vox;
   unsigned long long* H;
   uint64_t* meta;
+  int covers;  // the voxel cube holds every displacement below the ROI radius
 };
 
 constexpr uint32_t kSdmMaxVox = 1024;
@@ -54,40 +56,81 @@ __device__ __forceinline__ int sdm_vox(float d, const float* sV, uint32_t n, flo
   return m;
 }
 
+// one candidate q of central p (index word pidx)
+__device__ __forceinline__ void sdm_pair(const SdmArgs& a, const float* sV, float inv_w, const float4& p, const float4& q,
+                                         uint64_t& in_map, uint64_t& outside) {
+  // the same float32 operations as the squared distance: dx = x_j - x_i
+  const float dx = __fsub_rn(q.x, p.x), dy = __fsub_rn(q.y, p.y), dz = __fsub_rn(q.z, p.z);
+  const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+  if (d2 < a.ER && __float_as_uint(q.w) != __float_as_uint(p.w)) {
+    const uint32_t nv = a.n_vox;
+    const int mx = sdm_vox(dx, sV, nv, inv_w), my = sdm_vox(dy, sV, nv, inv_w), mz = sdm_vox(dz, sV, nv, inv_w);
+    if ((mx | my | mz) < 0) {
+      ++outside;
+    } else {
+      atomicAdd(&a.H[((uint64_t)mz * nv + (uint64_t)my) * nv + (uint64_t)mx], 1ull);
+      ++in_map;
+    }
+  }
+}
+
 // The pairs of one central (record index rec, cell ce of the neighbour grid) with the
 // candidates j0 + off, j0 + off + step, ... of every stencil row.
 __device__ __forceinline__ void sdm_central(const SdmArgs& a, const Geo& ng, const float* sV, float inv_w,
                                             uint32_t rec, uint32_t ce, uint32_t off, uint32_t step, uint64_t& in_map,
                                             uint64_t& outside) {
   const float4 p = __ldg(a.crec + rec);
-  const uint32_t pidx = __float_as_uint(p.w);
   const int st = a.stencil;
   const uint32_t cx = ce % ng.dims[0], cy = (ce / ng.dims[0]) % ng.dims[1], cz = ce / (ng.dims[0] * ng.dims[1]);
   const uint32_t xlo = cx >= (uint32_t)st ? cx - st : 0;
   const uint32_t xhi = cx + st < ng.dims[0] ? cx + st : ng.dims[0] - 1;
   const int ylo = max((int)cy - st, 0), yhi = min((int)cy + st, (int)ng.dims[1] - 1);
   const int zlo = max((int)cz - st, 0), zhi = min((int)cz + st, (int)ng.dims[2] - 1);
-  const uint32_t nv = a.n_vox;
   for (int z = zlo; z <= zhi; ++z)
     for (int y = ylo; y <= yhi; ++y) {
       const uint32_t row = ((uint32_t)z * ng.dims[1] + (uint32_t)y) * ng.dims[0];
       const uint32_t j1 = a.nstart[row + xhi + 1];
-      for (uint32_t j = a.nstart[row + xlo] + off; j < j1; j += step) {
-        const float4 q = __ldg(a.nrec + j);
-        // the same float32 operations as the squared distance: dx = x_j - x_i
-        const float dx = __fsub_rn(q.x, p.x), dy = __fsub_rn(q.y, p.y), dz = __fsub_rn(q.z, p.z);
-        const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-        if (d2 < a.ER && __float_as_uint(q.w) != pidx) {
-          const int mx = sdm_vox(dx, sV, nv, inv_w), my = sdm_vox(dy, sV, nv, inv_w), mz = sdm_vox(dz, sV, nv, inv_w);
-          if ((mx | my | mz) < 0) {
-            ++outside;
-          } else {
-            atomicAdd(&a.H[((uint64_t)mz * nv + (uint64_t)my) * nv + (uint64_t)mx], 1ull);
-            ++in_map;
-          }
-        }
-      }
+      for (uint32_t j = a.nstart[row + xlo] + off; j < j1; j += step)
+        sdm_pair(a, sV, inv_w, p, __ldg(a.nrec + j), in_map, outside);
     }
+}
+
+// The pairs of one central by a warp: lane r holds stencil row r (32 rows at a time), and the rows' records are
+// walked as one list (rows of thin clouds hold a few records each), a position's row found by
+// bisection over the lanes.
+__device__ __forceinline__ void sdm_central_list(const SdmArgs& a, const Geo& ng, const float* sV, float inv_w,
+                                                 const float4& p, uint64_t& in_map, uint64_t& outside) {
+  const uint32_t lane = threadIdx.x & 31, ce = cell_of(ng, p.x, p.y, p.z);
+  const int st = a.stencil, W = 2 * st + 1, n_rows = W * W;
+  const uint32_t cx = ce % ng.dims[0], cy = (ce / ng.dims[0]) % ng.dims[1], cz = ce / (ng.dims[0] * ng.dims[1]);
+  const uint32_t xlo = cx >= (uint32_t)st ? cx - st : 0, xhi = min(cx + st, ng.dims[0] - 1);
+  for (int r0 = 0; r0 < n_rows; r0 += 32) {
+    const int r = r0 + (int)lane, y = (int)cy + r % W - st, z = (int)cz + r / W - st;
+    uint32_t src = 0, pre = 0;
+    if (r < n_rows && y >= 0 && z >= 0 && y < (int)ng.dims[1] && z < (int)ng.dims[2]) {
+      const uint32_t row = ((uint32_t)z * ng.dims[1] + (uint32_t)y) * ng.dims[0];
+      src = a.nstart[row + xlo];
+      pre = a.nstart[row + xhi + 1] - src;
+    }
+    const uint32_t len = pre;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, pre, o);
+      if (lane >= (uint32_t)o) pre += v;
+    }
+    const uint32_t n_list = __shfl_sync(0xffffffffu, pre, 31);
+    pre -= len;
+    const uint32_t first = src - pre;
+    for (uint32_t b = 0; b < n_list; b += 32) {
+      const uint32_t pos = b + lane;
+      uint32_t k = 0;
+#pragma unroll
+      for (uint32_t h = 16; h > 0; h >>= 1)
+        if (__shfl_sync(0xffffffffu, pre, k + h) <= pos) k += h;
+      const uint32_t j = __shfl_sync(0xffffffffu, first, k) + pos;
+      if (pos < n_list) sdm_pair(a, sV, inv_w, p, __ldg(a.nrec + j), in_map, outside);
+    }
+  }
 }
 
 __global__ void __launch_bounds__(256) k_sdm(const SdmArgs a) {
@@ -186,13 +229,19 @@ __global__ void __launch_bounds__(256) k_sdm(const SdmArgs a) {
 // Measured on the 8e6-ion needle (all-all, 160^3 voxels, full-size cells): 131 -> 26.8 ms (31.7 with cells
 // whose records are not ordered by sub-cells).
 // ---------------------------------------------------------------------------
-struct SdmSymArgs {
-  unsigned long long* H;
-  uint64_t* meta;
-  double w;
-  uint32_t n_vox;
-  int covers;  // the voxel cube holds every displacement below the ROI radius
-};
+// Few centrals among the records: the sweep stages and culls every record, a warp per central reads the central's
+// stencil only, row by row, or in thin clouds (rows of fewer than 24 records) the rows as one list.  Measured, whole
+// call, a share of the ions at random (central by central / sweep, ms; before the sweep):
+//   8e6-ion needle, 2 nm, half-size cells (13 per cell)  0.05 6.7 / 6.4 (10.9), 0.02 2.9 / 4.4 (4.1), 0.002 0.65 / 1.8 (0.78)
+//   the same, full-size cells (104)                      0.05 7.9 / 7.0 (19.6), 0.02 3.4 / 5.0 (13.0)
+//   1 nm, half-size cells (1.7), as one list             0.2 5.3 / 5.3 (7.0), 0.1 2.9 / 4.0 (3.8; row by row 4.0)
+//   1 nm, full-size cells (13)                           0.1 3.4 / 2.8 (7.0), 0.05 1.9 / 2.4 (2.6)
+__host__ __device__ __forceinline__ bool sdm_sweep_pays(uint64_t n_nbr, uint64_t n_cells, uint64_t n_ctr) {
+  return 32 * n_ctr >= n_nbr + 8 * n_cells;
+}
+__host__ __device__ __forceinline__ bool sdm_thin(uint64_t n_nbr, uint64_t n_cells, int stencil) {
+  return (2 * stencil + 1) * n_nbr < 24 * n_cells;
+}
 
 __device__ __forceinline__ unsigned long long f2_add_down(unsigned long long a, unsigned long long b) {
   unsigned long long r;
@@ -200,7 +249,7 @@ __device__ __forceinline__ unsigned long long f2_add_down(unsigned long long a, 
   return r;
 }
 
-__global__ void __launch_bounds__(256, 4) k_sdm_sym(const SdmSymArgs a, const __grid_constant__ SweepArgs sw) {
+__global__ void __launch_bounds__(256, 4) k_sdm_sym(const __grid_constant__ SdmArgs a, const __grid_constant__ SweepArgs sw) {
   griddep_wait();
   griddep_launch();
   __shared__ float sV[kSdmMaxVox + 1];
@@ -216,6 +265,35 @@ __global__ void __launch_bounds__(256, 4) k_sdm_sym(const SdmSymArgs a, const __
                            lo2 = f2_pack(mid - eps, mid - eps), magic2 = f2_pack(kMagic, kMagic),
                            one2 = f2_pack(sw.one, sw.one);
   uint64_t in_map = 0, outside = 0;
+  auto totals = [&]() __attribute__((always_inline)) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      in_map += __shfl_xor_sync(0xffffffffu, in_map, o);
+      outside += __shfl_xor_sync(0xffffffffu, outside, o);
+    }
+    if (lane == 0) {
+      if (in_map) atomicAdd((unsigned long long*)&a.meta[1], (unsigned long long)in_map);
+      if (outside) atomicAdd((unsigned long long*)&a.meta[2], (unsigned long long)outside);
+    }
+  };
+  const uint32_t n_ctr = a.cgeo->n_sel;
+  if (!sdm_sweep_pays(a.ngeo->n_sel, a.ngeo->n_cells, n_ctr)) {
+    const Geo ng = *a.ngeo;
+    const bool thin = sdm_thin(ng.n_sel, ng.n_cells, a.stencil);
+    for (;;) {
+      uint32_t i = 0;
+      if (lane == 0) i = atomicAdd(sw.next, 1u);
+      i = __shfl_sync(0xffffffffu, i, 0);
+      if (i >= n_ctr) break;
+      const float4 p = __ldg(a.crec + i);
+      if (thin)
+        sdm_central_list(a, ng, sV, inv_w, p, in_map, outside);
+      else
+        sdm_central(a, ng, sV, inv_w, i, cell_of(ng, p.x, p.y, p.z), lane, 32, in_map, outside);
+    }
+    totals();
+    return;
+  }
   // one displacement of weight v (1, or -1 modulo 2^64) in voxel lin
   auto alone = [&](uint32_t lin, unsigned long long v) {
     atomicAdd(&a.H[lin], v);
@@ -285,21 +363,15 @@ __global__ void __launch_bounds__(256, 4) k_sdm_sym(const SdmSymArgs a, const __
       in_map -= self;
     }
   });
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    in_map += __shfl_xor_sync(0xffffffffu, in_map, o);
-    outside += __shfl_xor_sync(0xffffffffu, outside, o);
-  }
-  if (lane == 0) {
-    if (in_map) atomicAdd((unsigned long long*)&a.meta[1], (unsigned long long)in_map);
-    if (outside) atomicAdd((unsigned long long*)&a.meta[2], (unsigned long long)outside);
-  }
+  totals();
 }
 
 // lower half of the map: its own counts and those of the mirrored upper half
-__global__ void __launch_bounds__(256) k_sdm_mirror(unsigned long long* __restrict__ H, uint32_t N) {
+__global__ void __launch_bounds__(256) k_sdm_mirror(unsigned long long* __restrict__ H, uint32_t N,
+                                                    const Geo* __restrict__ ngeo, const Geo* __restrict__ cgeo) {
   griddep_wait();
   griddep_launch();
+  if (!sdm_sweep_pays(ngeo->n_sel, ngeo->n_cells, cgeo->n_sel)) return;  // (every displacement was counted where it lies)
   const uint32_t half = N / 2;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < half; i += gridDim.x * blockDim.x) H[i] += H[N - 1 - i];
 }
@@ -327,29 +399,9 @@ int run_sdm(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsr
   // (a radius or voxel near the limits of float32 keeps the general kernel)
   const bool sym = centrals_in_neighbours(g, ctr_mask) && spec.r_max > 1e-15 && spec.r_max < 1e15 && spec.w > 1e-15 &&
                    spec.w < 1e15;
-  int rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, false, false, !sym, sym ? kSweep : kNoSweep);
+  int rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, false, false, !sym, sym ? kSweep : kNoSweep, true);
   if (rc) return rc;
   const float ER = (float)(spec.r_max * spec.r_max);
-  if (sym) {
-    SdmSymArgs a = {};
-    a.H = reinterpret_cast<unsigned long long*>(d_hist);
-    a.meta = d_meta;
-    a.w = spec.w;
-    a.n_vox = spec.n_vox;
-    // |dx| >= V[n] would give dx^2 >= ER
-    const double top = (double)(float)((double)spec.n_vox * 0.5 * spec.w);
-    a.covers = top * top >= (double)ER;
-    SweepArgs sw = sweep_args(g, &g->ctr.geo->sym_next);
-    sw.range = ER;
-    int per_sm = 0;
-    PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sdm_sym, 256, 0));
-    if (per_sm < 1) return fail(PS_ERR_UNSUPPORTED, "SDM kernel does not fit on an SM");
-    PS_LAUNCH(PS_KID_SDM, s, PS_CUDA(launch_pdl(k_sdm_sym, g->num_sms * per_sm, 256, 0, s, a, sw)));
-    PS_LAUNCH(PS_KID_SDM, s, PS_CUDA(launch_pdl(k_sdm_mirror, g->num_sms * 8, 256, 0, s, a.H, (uint32_t)nh)));
-    PS_LAUNCH(PS_KID_EPILOGUE, s, PS_CUDA(launch_pdl(k_sdm_epilogue, 1, 32, 0, s, g->nbr.geo, g->ctr.geo, d_meta)));
-    PS_CUDA(cudaGetLastError());
-    return PS_OK;
-  }
   SdmArgs a;
   memset(&a, 0, sizeof(a));
   a.nrec = g->nbr.rec;
@@ -367,6 +419,21 @@ int run_sdm(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float dsr
   a.n_vox = spec.n_vox;
   a.H = reinterpret_cast<unsigned long long*>(d_hist);
   a.meta = d_meta;
+  if (sym) {
+    // |dx| >= V[n] would give dx^2 >= ER
+    const double top = (double)(float)((double)spec.n_vox * 0.5 * spec.w);
+    a.covers = top * top >= (double)ER;
+    SweepArgs sw = sweep_args(g, &g->ctr.geo->sym_next);
+    sw.range = ER;
+    int per_sm = 0;
+    PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sdm_sym, 256, 0));
+    if (per_sm < 1) return fail(PS_ERR_UNSUPPORTED, "SDM kernel does not fit on an SM");
+    PS_LAUNCH(PS_KID_SDM, s, PS_CUDA(launch_pdl(k_sdm_sym, g->num_sms * per_sm, 256, 0, s, a, sw)));
+    PS_LAUNCH(PS_KID_SDM, s, PS_CUDA(launch_pdl(k_sdm_mirror, g->num_sms * 8, 256, 0, s, a.H, (uint32_t)nh, g->nbr.geo, g->ctr.geo)));
+    PS_LAUNCH(PS_KID_EPILOGUE, s, PS_CUDA(launch_pdl(k_sdm_epilogue, 1, 32, 0, s, g->nbr.geo, g->ctr.geo, d_meta)));
+    PS_CUDA(cudaGetLastError());
+    return PS_OK;
+  }
   int per_sm = 0;
   PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sdm, 256, 0));
   if (per_sm < 1) return fail(PS_ERR_UNSUPPORTED, "SDM kernel does not fit on an SM");
