@@ -997,6 +997,7 @@ static int launch_rdf_sym(const ps_grid* g, const QueryArgs& qa, const SweepArgs
 // near kNN pass on the vertex-centred central list
 // ---------------------------------------------------------------------------
 constexpr uint32_t kQueue = 40;  // queue rows per lane; inserted when fewer than 16 are free
+constexpr uint32_t kVertexSmem = 8 * (16 * 16 + 16 * 8 + (kQueue + 1) * 32 * 4);  // the kernel's static shared memory
 
 // One warp per item (up to 32 centrals of a vertex cell, one to eight lanes each), its candidates the
 // records of the 2 x 2 x 2 cells around the vertex, staged 32 at a time as interleaved pairs.  A sorted
@@ -1017,6 +1018,7 @@ __global__ void __launch_bounds__(256, KMAX <= 13 ? 4 : 2) k_knn_vertex(const __
   __shared__ float4 s_xy[8][16];
   __shared__ float2 s_z[8][16];
   __shared__ float s_kq[8][(kQueue + 1) * 32];
+  static_assert(sizeof(s_xy) + sizeof(s_z) + sizeof(s_kq) == kVertexSmem, "run_query asks whether this fits");
   Hist<false> H{};
   H.init(a, smem, 0, true);
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1432,17 +1434,20 @@ int run_query(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], float d
   qa.type = g->type;
   for (int w = 0; w < 4; ++w) qa.nbr.w[w] = g->nbr_mask[w];
   qa.one = 1.0f;
+  int dev_smem = 0;
+  PS_CUDA(cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
   // the query in passes, and its near kNN pass on the vertex-centred central list (two-cell
-  // stencils; the ranks of that counting sort take one word per central of the cell arrays)
+  // stencils; the ranks of that counting sort take one word per central of the cell arrays; its queues
+  // take 3 KB more than k_query_warp's may, which does the pass where the kNN histograms nearly fill an SM,
+  // such as 32 k values of 1,419 to 1,440 bins)
   const bool split = in_passes;
-  const bool vertex = split && n_k > 0 && g->stencil == 2 && (uint64_t)g->n <= (uint64_t)g->cell_cap;
+  const bool vertex = split && n_k > 0 && g->stencil == 2 && (uint64_t)g->n <= (uint64_t)g->cell_cap &&
+                      smem_layout(bins.n_bins, n_k, false, 0, true).total + kVertexSmem <= (uint32_t)dev_smem;
   int rc = build_central_list(g, dsrf, ctr_mask, dsrf_min, s, z, true, vertex, !split || n_k > 0,
                               split ? kSweep : (sweep ? kSweepIfDense : kNoSweep));
   if (rc) return rc;
 
   // staging budget of the CTA kernel: two CTAs per SM
-  int dev_smem = 0;
-  PS_CUDA(cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
   const SmemLayout base = smem_layout(bins.n_bins, n_k, rdf, 0, false, qa.lut_n);
   const uint32_t budget = (uint32_t)dev_smem / 2 - 2048;
   if (base.total + 16 * 1024 > (uint32_t)dev_smem - 1024)
