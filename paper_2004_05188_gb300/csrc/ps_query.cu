@@ -557,8 +557,9 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : (KMAX <= 16 ? 3 : 2)) k_
 
     item_scan(S, ng, c, box, ring, nb, all, emax, near_max, batch, [](float) { return true; });
     if (all) {
-      // the centrals met themselves once each, at d2 = 0 (a non-finite one did not)
-      bool self = valid && sub == 0 && dist2(p.x, p.y, p.z, p.x, p.y, p.z) == 0.f;
+      // the centrals met themselves once each, at d2 = 0 (a non-finite one did not, nor any where the range
+      // squared is 0 in float32)
+      bool self = valid && sub == 0 && emax > 0.f && dist2(p.x, p.y, p.z, p.x, p.y, p.z) == 0.f;
       if (self && !a.self_all) self = in_mask(a.nbr, a.type[pidx]);
       within -= (uint32_t)self;
       if (MODE == kRdfDirect && rdf_here) {
