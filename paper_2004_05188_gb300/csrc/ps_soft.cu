@@ -308,15 +308,22 @@ __device__ __forceinline__ unsigned long long soft_d2(unsigned long long dx, uns
   return f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
 }
 
-// The forward's moments of a fine bin in integers: the weights, the remainders in units of w / 2^13
-// (half of float32's step of u at 2 nm and sigma = 0.05 nm) and their squares in units of w^2 / 2^13.
-// Integer shared-memory atomics run at the rate of the plain count (measured, 2 of 5 lanes active
-// at random places, cycles per warp and SM: one count 4.5, three integers 5.4, a count and two
-// floats 12.1), and the sums do not round.  A bin's sums stay inside 32 bits while its weight is
-// below 2^19: a warp looks the counts over after every 2^14 that it may have added, and drains the
-// rows to the global moments when one has reached 2^18 (8 warps: below 2^18 + 8 (2^14 + 2^13)).
-constexpr float kSoftQ = 8192.0f;
-constexpr uint32_t kSoftLook = 1u << 14, kSoftDrain = 1u << 18;
+// The forward's moments of a fine bin in integers: the weights, the remainders in units of w / 2^18 and their
+// squares in units of w^2 / 2^18.  The sums do not round, and a unit of the remainders is at most float32's step
+// of u from the 32nd bin on (u = 0.8 sigma), so that they hold what the distance does; where nearer pairs
+// are not rare (LOW, fewer than 512 fine bins: sigma above a sixth of the range) the remainders take units of
+// w / 2^22 in two words, the low kSoftLow bits apart.  (Units of w / 2^13 showed wherever the sums have few or
+// equal pairs: a lattice of 343 ions, a = 0.286 and sigma = 0.2 nm, 1.6e-7 of h against FP64, float32 sums 1.0e-7,
+// now 4e-8; 50 ions, sigma = 0.5 nm, 3.7e-8, 2.0e-8 and 7e-9.)
+// Integer shared-memory atomics run at the rate of the plain count (measured, 2 of 5 lanes active at random
+// places, cycles per warp and SM: one count 4.5, three integers 5.4, a count and two floats 12.1).  A bin's sums
+// stay inside 32 bits while its weight is below 2^14: the addition of the weight returns the bin's weight
+// before it, and a warp that meets one of 2^12 in its turn of 4 records drains all bins to the global
+// moments.  A turn adds at most 512 to a bin, and a warp that has not met the limit in one turn meets it in the
+// next: below 2^12 + 8 * 2 * 512.
+constexpr float kSoftQ = 262144.0f, kSoftQLow = 4194304.0f;
+constexpr uint32_t kSoftLow = 11, kSoftLowFine = 512;
+constexpr uint32_t kSoftDrain = 1u << 12;
 
 // Forward where the centrals are neighbour records: every unordered pair once (sweep_pairs), its
 // moments straight from the testing lane into the CTA's shared fine grid.  Bound by the shared-
@@ -324,7 +331,10 @@ constexpr uint32_t kSoftLook = 1u << 14, kSoftDrain = 1u << 18;
 // half-size cells / 2e5 cylinder on full-size cells (ms): 36.8 -> 17.7 / 14.5 -> 0.79 (before: a warp
 // list of the hits of every candidate of the half stencil, a float sum per moment, cells not split;
 // 27.4 / 1.25 with the sweep and float sums; 19.4 / 0.92 with a row of bins per moment, which takes
-// two more additions per pair than the three moments of a bin side by side).
+// two more additions per pair than the three moments of a bin side by side); 17.7 -> 18.6 / 0.79 -> 0.82 with
+// the finer units (the returned weights; with every turn of 2 records checked 20.2, with the low bits in a
+// fourth word 22.6).
+template <bool LOW>
 __global__ void __launch_bounds__(256, 4) k_soft_fwd_sym(const SoftArgs a, const __grid_constant__ SweepArgs sw,
                                                          double unit1, double unit2) {
   griddep_wait();
@@ -333,19 +343,20 @@ __global__ void __launch_bounds__(256, 4) k_soft_fwd_sym(const SoftArgs a, const
   __shared__ SweepBuf s_sweep[8];
   const uint32_t nf = a.n_fine, nf4 = (nf + 3u) & ~3u, lane = threadIdx.x & 31;
   uint32_t* sM = reinterpret_cast<uint32_t*>(smem);  // [nf4][3]: the three moments of a bin side by side
-  for (uint32_t m = threadIdx.x; m < 3 * nf4; m += blockDim.x) sM[m] = 0;
+  uint32_t* sL = sM + 3 * nf4;                       // LOW [nf4]: the remainders' low bits
+  for (uint32_t m = threadIdx.x; m < (LOW ? 4 : 3) * nf4; m += blockDim.x) sM[m] = 0;
   __syncthreads();
   SweepBuf& buf = s_sweep[threadIdx.x >> 5];
   const SoftFine fine(a);
-  const float rc = a.rc, q1 = kSoftQ * a.inv_w, q2 = kSoftQ * a.inv_w * a.inv_w;
+  const float rc = a.rc, q1 = (LOW ? kSoftQLow : kSoftQ) * a.inv_w, q2 = kSoftQ * a.inv_w * a.inv_w;
   const unsigned long long q1_2 = f2_pack(q1, q1), q2_2 = f2_pack(q2, q2);
-  const uint32_t base = smem_u32(sM) - 12u * kMagicBits;
-  uint32_t added = 0;  // bound on the weights this warp has added since it last looked (uniform)
+  const uint32_t base = smem_u32(sM) - 12u * kMagicBits, base_l = smem_u32(sL) - 4u * kMagicBits;
   // the rows' bins i, i + step, ... to the global moments
   auto drain = [&](uint32_t i, uint32_t step) {
     for (; i < nf; i += step) {
-      const int32_t v0 = (int32_t)atomicExch(&sM[3 * i], 0u), v1 = (int32_t)atomicExch(&sM[3 * i + 1], 0u),
+      const int32_t v0 = (int32_t)atomicExch(&sM[3 * i], 0u), vh = (int32_t)atomicExch(&sM[3 * i + 1], 0u),
                     v2 = (int32_t)atomicExch(&sM[3 * i + 2], 0u);
+      const int64_t v1 = LOW ? (int64_t)vh * (1 << kSoftLow) + (int32_t)atomicExch(&sL[i], 0u) : (int64_t)vh;
       // (a count may stand below zero when its self pairs were drained before they were taken out)
       if (v0) atomicAdd(&a.M0[i], (unsigned long long)(long long)v0);
       if (v1) atomicAdd(&a.M1[i], (double)v1 * unit1);
@@ -359,8 +370,9 @@ __global__ void __launch_bounds__(256, 4) k_soft_fwd_sym(const SoftArgs a, const
     const uint32_t w0 = k0 == kCandBoth ? 2u : 1u, w1 = k1 == kCandBoth ? 2u : 1u;
     const unsigned long long x0 = f2_pack(c0.x, c0.x), y0 = f2_pack(c0.y, c0.y), z0 = f2_pack(c0.z, c0.z);
     const unsigned long long x1 = f2_pack(c1.x, c1.x), y1 = f2_pack(c1.y, c1.y), z1 = f2_pack(c1.z, c1.z);
-    auto deposit = [&](unsigned long long d2, uint32_t wt) __attribute__((always_inline)) {
+    auto deposit = [&](unsigned long long d2, uint32_t wt, uint32_t& hot) __attribute__((always_inline)) {
       const uint32_t off = 0u - kMagicBits * wt;
+      const uint32_t off_h = 0u - (kMagicBits >> kSoftLow) * wt;  // (kMagicBits is a multiple of 2^kSoftLow)
       float da, db, u[2], mm[2], r1[2], r2[2];
       f2_unpack(d2, da, db);
       const unsigned long long u2 = f2_mul(f2_pack(sqrt_fast(da), sqrt_fast(db)), fine.scale2);
@@ -373,8 +385,17 @@ __global__ void __launch_bounds__(256, 4) k_soft_fwd_sym(const SoftArgs a, const
       for (int e = 0; e < 2; ++e) {
         if (u[e] < rc) {
           const uint32_t at = __float_as_uint(mm[e]) * 12u + base;
-          asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at), "r"(wt));
-          asm volatile("red.shared.add.u32 [%0+4], %1;" ::"r"(at), "r"(__float_as_uint(r1[e]) * wt + off));
+          uint32_t old;
+          asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(at), "r"(wt));
+          hot |= old;
+          const uint32_t q = __float_as_uint(r1[e]);
+          if (LOW) {
+            const uint32_t at_l = __float_as_uint(mm[e]) * 4u + base_l;
+            asm volatile("red.shared.add.u32 [%0+4], %1;" ::"r"(at), "r"((q >> kSoftLow) * wt + off_h));
+            asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at_l), "r"((q & ((1u << kSoftLow) - 1u)) * wt));
+          } else {
+            asm volatile("red.shared.add.u32 [%0+4], %1;" ::"r"(at), "r"(q * wt + off));
+          }
           asm volatile("red.shared.add.u32 [%0+8], %1;" ::"r"(at), "r"(__float_as_uint(r2[e]) * wt + off));
         }
       }
@@ -382,26 +403,24 @@ __global__ void __launch_bounds__(256, 4) k_soft_fwd_sym(const SoftArgs a, const
     const ulonglong2* rxy = reinterpret_cast<const ulonglong2*>(buf.rxy);
     const unsigned long long* rz = reinterpret_cast<const unsigned long long*>(buf.rz);
 #pragma unroll 1
-    for (uint32_t k = 0; k < n_pr; ++k) {
-      const ulonglong2 xy = rxy[k];
-      const unsigned long long zz = rz[k];
-      deposit(soft_d2(f2_sub(x0, xy.x), f2_sub(y0, xy.y), f2_sub(z0, zz)), w0);
-      deposit(soft_d2(f2_sub(x1, xy.x), f2_sub(y1, xy.y), f2_sub(z1, zz)), w1);
+    for (uint32_t k = 0; k < n_pr; k += 2) {
+      uint32_t hot = 0;
+#pragma unroll
+      for (uint32_t i = 0; i < 2; ++i) {
+        const ulonglong2 xy = rxy[k + i];
+        const unsigned long long zz = rz[k + i];
+        deposit(soft_d2(f2_sub(x0, xy.x), f2_sub(y0, xy.y), f2_sub(z0, zz)), w0, hot);
+        deposit(soft_d2(f2_sub(x1, xy.x), f2_sub(y1, xy.y), f2_sub(z1, zz)), w1, hot);
+      }
+      if (__any_sync(0xffffffffu, hot >= kSoftDrain)) drain(lane, 32);
     }
     // the staged records met themselves once each, at u = 0: taken out of bin 0 (remainder -w / 2)
     const uint32_t self = __popc(__ballot_sync(0xffffffffu, k0 == kCandSelf)) +
                           __popc(__ballot_sync(0xffffffffu, k1 == kCandSelf));
     if (self && lane == 0) {
       atomicAdd(&sM[0], 0u - self);
-      atomicAdd(&sM[1], self * (uint32_t)(kSoftQ / 2));
+      atomicAdd(&sM[1], self * (LOW ? (uint32_t)(kSoftQLow / 2) >> kSoftLow : (uint32_t)(kSoftQ / 2)));
       atomicAdd(&sM[2], 0u - self * (uint32_t)(kSoftQ / 4));
-    }
-    added += 2u * kSweepTile * m;
-    if (added >= kSoftLook) {
-      added = 0;
-      uint32_t top = 0;
-      for (uint32_t i = lane; i < nf4; i += 32) top = max(top, reinterpret_cast<const volatile uint32_t*>(sM)[3 * i]);
-      if (__any_sync(0xffffffffu, top >= kSoftDrain)) drain(lane, 32);
     }
   });
   __syncthreads();
@@ -808,13 +827,15 @@ int soft_forward(ps_grid* g, const float* dsrf, const uint64_t ctr_mask[4], floa
   sa.M2 = g->soft_m2;
   int blocks = 0;
   if (sym) {
-    const uint32_t smem = ((sa.n_fine + 3u) & ~3u) * 12;
-    rc = launch_grid_for(g, (const void*)k_soft_fwd_sym, smem, &blocks);
+    const bool low = sa.n_fine < kSoftLowFine;
+    const uint32_t smem = ((sa.n_fine + 3u) & ~3u) * (low ? 16 : 12);
+    auto kern = low ? k_soft_fwd_sym<true> : k_soft_fwd_sym<false>;
+    rc = launch_grid_for(g, (const void*)kern, smem, &blocks);
     if (rc) return rc;
     SweepArgs sw = sweep_args(g, &g->ctr.geo->sym_next);
     sw.range = sa.rc2u;
     PS_LAUNCH(PS_KID_SOFT_FWD, s,
-              PS_CUDA(launch_pdl(k_soft_fwd_sym, blocks, 256, smem, s, sa, sw, w / (double)kSoftQ,
+              PS_CUDA(launch_pdl(kern, blocks, 256, smem, s, sa, sw, w / (double)(low ? kSoftQLow : kSoftQ),
                                  w * w / (double)kSoftQ)));
   } else {
     const uint32_t smem = sa.n_fine * 12;
