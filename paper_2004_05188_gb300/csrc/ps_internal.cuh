@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
 #include <string>
 
 #include "../../include/ps.h"
@@ -11,6 +12,20 @@
 namespace ps {
 
 constexpr uint32_t kSoftFineMax = 8192;  // fine-grid bins of the smoothed RDF
+// Width of the fine bins for the range rc: at most sigma / 40, wider where that takes more than kSoftFineMax bins
+// (one of them spare, for the rounding of floor(rc / w)).  With 10 significant bits (rounded down, or up
+// where it is the number of bins that sets it) every centre (m + 1/2) w has at most 14 + 10 of them, which float32
+// holds; 11 bits leave half of the centres from bin 4,096 on between two of its values.
+inline double soft_width(float sigma, double rc) {
+  auto bits10 = [](double x, bool up) {
+    int e;
+    const double f = std::frexp(x, &e) * 1024.0;
+    return std::ldexp(up ? std::ceil(f) : std::floor(f), e - 10);
+  };
+  const double w = bits10((double)sigma / 40.0, false);
+  return rc / w > (double)(kSoftFineMax - 2) ? bits10(rc / (double)(kSoftFineMax - 2), true) : w;
+}
+inline uint32_t soft_bins(double w, double rc) { return (uint32_t)std::ceil(rc / w) + 1; }
 constexpr float kMinCellScale = 1.0f / 3.0f;  // cell edge / r_cut: stencils of at most 3 cells
 
 // ---------------------------------------------------------------------------

@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(256) k_soft_fwd(const SoftArgs a) {
 }
 
 // Pairs of the sweep as packed distances: the range test is u < rc (u = scale * distance), the fine
-// bin floor(u / w).  w has 11 significant bits and n_fine < 2^13, so that the bin centres (m + 1/2) w
-// are exact in float32 and the remainder u - (m + 1/2) w carries only the rounding of u.
+// bin floor(u / w).  The bin centres (m + 1/2) w are exact in float32 (see soft_width), so that the remainder
+// u - (m + 1/2) w carries only the rounding of u.
 struct SoftFine {
   unsigned long long scale2, inv_w2, w2, half_w2, magic2;
   __device__ explicit SoftFine(const SoftArgs& a) {
@@ -761,16 +761,8 @@ static int soft_setup(ps_grid* g, float sigma, float scale, ps_bins bins, SoftAr
   const double rc = stop + 6.0 * (double)sigma;
   if ((double)g->r_cut * (double)scale < rc * (1.0 + 1e-6))
     return fail(PS_ERR_INVALID_ARG, "smoothed RDF: grid r_cut * scale must cover stop + 6 sigma");
-  // fine width: at most sigma / 40, 11 significant bits (rounded down), and one spare bin for the
-  // rounding of floor(rc / w); wider (rounded up) where that takes more than kSoftFineMax bins
-  auto bits11 = [](double x, bool up) {
-    int e;
-    const double f = std::frexp(x, &e) * 2048.0;
-    return std::ldexp(up ? std::ceil(f) : std::floor(f), e - 11);
-  };
-  double w = bits11((double)sigma / 40.0, false);
-  if (rc / w > (double)(kSoftFineMax - 2)) w = bits11(rc / (double)(kSoftFineMax - 2), true);
-  sa.n_fine = (uint32_t)std::ceil(rc / w) + 1;
+  const double w = soft_width(sigma, rc);
+  sa.n_fine = soft_bins(w, rc);
   sa.w = (float)w;
   sa.inv_w = (float)(1.0 / w);
   sa.scale = scale;
