@@ -846,9 +846,10 @@ def rooflines(prof, st, steps, peaks, hbm_peak, hbm_src, traffic):
         "algorithmic_bytes_per_launch": (algorithmic_bytes("query", st, next(c for c in st["combos"]
                                                                             if c["name"] == traffic["combination"]))
                                          if traffic and d.get("traffic") else None),
-        "per_unit": f"{FLOPS_PER_CANDIDATE} FP32 operations per candidate test (3 sub, 3 mul, 2 add, 1 compare) of "
-                    "the cells' stencils; the kernels leave out the candidates beyond reach of a block's bounding box "
-                    "(about a third on half-size cells), which are counted here all the same",
+        "per_unit": f"{FLOPS_PER_CANDIDATE} FP32 operations per distance test (3 sub, 3 mul, 2 add, 1 compare) that the "
+                    "statistic cannot do without: RDF over unordered pairs, each pair in range once; one pass, each "
+                    "neighbour in range of a central; near kNN, each record of a central's block.  The tests that find "
+                    "a pair out of range are not counted",
         "flops_per_launch": d.get("flops_per_launch"), "launches": d.get("launches"),
         "avg_launch_ms": d.get("avg_launch_ms"),
         "by_kernel": by_kernel,
@@ -878,11 +879,13 @@ def rooflines(prof, st, steps, peaks, hbm_peak, hbm_src, traffic):
 
 def combo_stats(ps, g, o, name, ctr, nbr, X, T, D, t_host, wl, stencil, split=False):
     """Counts of one combination after its build + query (reporting only, untimed).  candidates:
-    the distance tests of the query -- one pass: every central against its stencil; in passes
-    (split): every central against its near kNN block (its own 2 x 2 x 2 cells on half-size
-    cells, the 27 cells around its cell on third-size cells) plus every unordered pair of records
-    in each other's stencil once (symmetric RDF), the few full-radius fallback searches not
-    counted; one pass over a dense cloud with many centrals leaves the RDF to that pass as well."""
+    the distance tests that the query cannot do without -- one pass: every neighbour in range of a
+    central; in passes (split): every central against its near kNN block (its own 2 x 2 x 2 cells on
+    half-size cells, the 27 cells around its cell on third-size cells) plus every unordered pair in
+    range once (symmetric RDF; half the binned pairs, exact where both ends are central), the few
+    full-radius fallback searches not counted; one pass over a dense cloud with many centrals leaves
+    the RDF to that pass as well.  The kernels make more tests, of pairs that turn out to be out of range
+    (stencil_pairs bounds them, less what lies beyond reach of a block's bounding box)."""
     meta = o["meta"].cpu().numpy()
     if meta[3] != 0:
         raise RuntimeError(f"device status {meta[3]} for {name}")
@@ -892,6 +895,7 @@ def combo_stats(ps, g, o, name, ctr, nbr, X, T, D, t_host, wl, stencil, split=Fa
     n_typed = sum(int(np.count_nonzero(lut[t_host[a:a + (1 << 26)]])) for a in range(0, t_host.shape[0], 1 << 26))
     subset = bool(np.all((mc & ~mn) == 0))
     cs = g.cell_scale
+    n_pairs = int(meta[1]) + int(meta[2])
     if split and subset and stencil >= 2:
         if not wl["ks"]:
             near = 0
@@ -900,7 +904,8 @@ def combo_stats(ps, g, o, name, ctr, nbr, X, T, D, t_host, wl, stencil, split=Fa
         else:  # the 27 cells around the central's cell
             near = candidate_tests(X, T, D, ctr, nbr, wl["dsrf_min"], info, 1)
         full = candidate_tests(X, T, D, nbr, nbr, wl["dsrf_min"], info, stencil, all_records=True, cell_scale=cs)
-        sym = (full - info["n_nbr"]) // 2
+        stencil_pairs = near + (full - info["n_nbr"]) // 2
+        sym = (n_pairs + 1) // 2
         by_pass = {"query": near, "rdf_sym": sym}
         cands = near + sym
         swept = False
@@ -908,16 +913,18 @@ def combo_stats(ps, g, o, name, ctr, nbr, X, T, D, t_host, wl, stencil, split=Fa
           and 8 * int(meta[0]) >= info["n_nbr"] + 8 * info["n_cells"]):  # (as sweep_pays in ps_internal.cuh)
         # the RDF over unordered pairs, the kNN's tests not counted
         full = candidate_tests(X, T, D, nbr, nbr, wl["dsrf_min"], info, stencil, all_records=True, cell_scale=cs)
-        cands = (full - info["n_nbr"]) // 2
+        stencil_pairs = (full - info["n_nbr"]) // 2
+        cands = (n_pairs + 1) // 2
         by_pass = {"rdf_sym": cands}
         swept = True
     else:
-        cands = candidate_tests(X, T, D, ctr, nbr, wl["dsrf_min"], info, stencil, cell_scale=cs)
+        stencil_pairs = candidate_tests(X, T, D, ctr, nbr, wl["dsrf_min"], info, stencil, cell_scale=cs)
+        cands = n_pairs
         by_pass = {"query": cands}
         swept = False
     return dict(name=name, n_nbr=info["n_nbr"], n_cells=info["n_cells"], n_central=int(meta[0]),
                 n_ctr_typed=n_typed, n_pairs_local=int(meta[1]), subset=subset, candidates=cands,
-                candidates_by_pass=by_pass, split=bool(split and subset and stencil >= 2), swept=swept)
+                stencil_pairs=int(stencil_pairs), candidates_by_pass=by_pass, split=bool(split and subset and stencil >= 2), swept=swept)
 
 
 def e2e_runner(dev, stream, sets, hosts, step, outs, res_h):
