@@ -406,9 +406,9 @@ constexpr int kNoRdf = 0, kRdfGeneral = 1, kRdfDirect = 2;
 // 75 instructions per 32 tests, of which the bins take 16, the near tests 18, the insertions 17.
 // Near candidates are tested a second time for the queue: one loop for both spills at 64 registers
 // (0.347 ms there, but 0.174 -> 0.193 ms where the kNN is alone).  In-range counts without the RDF are
-// taken beside the kNN (5e5-ion needle, k = 16, r = 1 nm: 0.511 -> 0.456 ms).  Lists of more than 12 stop
-// at the tighter bound over a central's lanes (5e4 ions, k = 32: 0.126 -> 0.117 ms; with shorter lists it costs what
-// it saves); those of up to 16 run 3 CTAs per SM (3e6-ion needle, Al about Sc, k = 16: 0.447 -> 0.406 ms),
+// taken beside the kNN (5e5-ion needle, k = 16, r = 1 nm: 0.511 -> 0.456 ms).  Lists of more than 12, and the
+// lists of 8 and more lanes, stop at the tighter bound over a central's lanes (5e4 ions, k = 32: 0.126 -> 0.117 ms;
+// shorter lists of few lanes: it costs what it saves); those of up to 16 run 3 CTAs per SM (3e6-ion needle, Al about Sc, k = 16: 0.447 -> 0.406 ms),
 // longer ones 2 (5e5-ion needle, k = 32: 0.757 against 0.783 ms with 3).
 template <int KMAX, int MODE>
 __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : (KMAX <= 16 ? 3 : 2)) k_query_warp(const __grid_constant__ QueryArgs a) {
@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : (KMAX <= 16 ? 3 : 2)) k_
           for (uint32_t q = 0; q < m; ++q)
             if (q < qn) topk_insert(top, queue_at(q0, q));
           float kth = top[KK - 1];  // an upper bound of the central's k-th distance in each of its lanes
-          if constexpr (KK > 12)
+          if (KK > 12 || L >= 8u)
             kth = topk_bound(top, L);
           else
             for (uint32_t o = 1; o < L; o <<= 1) kth = fminf(kth, __shfl_xor_sync(0xffffffffu, kth, o));
@@ -567,48 +567,49 @@ __global__ void __launch_bounds__(256, KMAX <= 12 ? 4 : (KMAX <= 16 ? 3 : 2)) k_
         if (lane == 0 && n_self) red_shared(row_base + 4u * kMagicBits, 0u - n_self);
       }
     }
-    // merge the partial lists of the L lanes of each central (disjoint candidate subsets); the
-    // partner's sorted list is read from the warp's queue buffer in a rolled loop, which keeps
-    // the kernel's code small (its speed depends on the instruction cache)
-    for (uint32_t o = 1; o < L; o <<= 1) {
-      within += __shfl_xor_sync(0xffffffffu, within, o);
-      if constexpr (KMAX > 0 && KK * 32 <= 32 * kHalf) {
+    // merge the sorted lists of the L lanes of each central (disjoint candidate subsets): the smallest head
+    // is taken k_need times, rank by rank into the queue buffer, a column per central.  (Merging pairs of
+    // lists by insertion takes lg L rounds of up to KK insertions: ~1000 instructions at 16 lanes and KK =
+    // 10, ~8000 at 32, against ~250 and ~1400.  Thin clouds, where most items hold one to three centrals: 5e4-ion
+    // cylinder, third-size cells, r = 1 nm, k = 32, whole call 0.61 -> 0.42 ms, k = 10 with per-ion counts
+    // 0.253 -> 0.238; 1e6 ions, half-size cells, r = 1.5 nm, 5 % of them central 0.578 -> 0.553 ms.)
+    const uint32_t n_col = 32u >> lg;
+    if (L > 1u) {
+      for (uint32_t o = 1; o < L; o <<= 1) within += __shfl_xor_sync(0xffffffffu, within, o);
+      if constexpr (KMAX > 0) {
+        const uint32_t group = ((1u << L) - 1u) << (lane & ~(L - 1u));
         __syncwarp();
-#pragma unroll
-        for (int t = 0; t < KK; ++t) kq[t * 32 + lane] = top[t];
-        __syncwarp();
-        const float* ot = kq + (lane ^ o);
 #pragma unroll 1
-        for (int t = 0; t < KK; ++t) {
-          const float v = ot[t * 32];
-          if (!(v < top[KK - 1])) break;  // the partner's list is sorted
-          topk_insert(top, v);
-        }
-      } else if constexpr (KMAX > 0) {
-        float other[KK];
+        for (uint32_t rank = 0; rank < a.k_need; ++rank) {
+          float m = top[0];
+          for (uint32_t o = 1; o < L; o <<= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+          const uint32_t heads = __ballot_sync(0xffffffffu, top[0] == m) & group;
+          if ((int)lane == __ffs(heads) - 1) {
 #pragma unroll
-        for (int t = 0; t < KK; ++t) other[t] = __shfl_xor_sync(0xffffffffu, top[t], o);
-#pragma unroll
-        for (int t = 0; t < KK; ++t) {
-          if (!(other[t] < top[KK - 1])) break;  // the partner's list is sorted
-          topk_insert(top, other[t]);
+            for (int t = 0; t + 1 < KK; ++t) top[t] = top[t + 1];
+            top[KK - 1] = INFINITY;
+          }
+          if (sub == 0) kq[rank * n_col + ci] = m;
         }
+        __syncwarp();
       }
     }
+    auto ranked = [&](uint32_t i) -> float { return L > 1u ? kq[i * n_col + ci] : topk_get(top, i); };
     if (valid && sub == 0) {
       if (nwithin) nwithin[pidx] = within;
       if (KMAX > 0) {
-        const float kd = topk_get(top, a.k_need - 1);
+        const float kd = ranked(a.k_need - 1);
         const bool found = !(a.emax_near > 0.f) || kd < a.emax_near;
         if (a.emax_near > 0.f) a.need[c0 + ci] = found ? 0u : 1u;
         if (found)
-          for (uint32_t q = 0; q < a.n_k; ++q) H.kth(a, q, topk_get(top, a.ks[q] - 1), pidx);
+          for (uint32_t q = 0; q < a.n_k; ++q) H.kth(a, q, ranked(a.ks[q] - 1), pidx);
       }
     }
   }
 
   // ---- items from the back: sparse cells, one thread per central ----
   // central record and cell of the taken items' centrals (<= 32 * 15, kHeavy - 1 per item)
+  static_assert(PS_K_MAX * 16 <= 32 * kHalf + 32, "ranks of two lanes per central in the queue buffer");
   static_assert(32 * (kHeavy - 1) <= 4 * kRing && 32 * (kHeavy - 1) <= 32 * kHalf + 32, "light items taken at once");
   uint32_t* cl_rec = reinterpret_cast<uint32_t*>(s_buf[w]);
   uint32_t* cl_cell = reinterpret_cast<uint32_t*>(s_kq[w]);
