@@ -682,19 +682,21 @@ __global__ void __launch_bounds__(kScanThreads) k_central_subset(const float4* _
   griddep_launch();
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_tile, s_prefix;
-  const uint32_t nr = ngeo->n_sel;
+  // (the loads that every thread needs stand together: the stores below may alias the geometry)
+  const uint32_t nr = ngeo->n_sel, nbr_cells = ngeo->n_cells, listed = ngeo->heavy_listed;
   // vcount given: the central list is the grid of cells centred on the vertices (origin half a
   // cell lower, one more cell per axis), filled by k_vertex_count / k_vertex_scatter; its counts
   // are zeroed here and no records are written
-  const uint32_t nvc = (ngeo->dims[0] + 1) * (ngeo->dims[1] + 1) * (ngeo->dims[2] + 1);
+  const uint32_t nvc = vcount ? (ngeo->dims[0] + 1) * (ngeo->dims[1] + 1) * (ngeo->dims[2] + 1) : 0u;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     // every field but n_sel, which the thread that scans the last tile writes
-    const float half = vcount ? __fmul_rn(0.5f, ngeo->h) : 0.0f;
+    const Geo n = *ngeo;
+    const float half = vcount ? __fmul_rn(0.5f, n.h) : 0.0f;
     for (int a = 0; a < 3; ++a)
-      cgeo->origin[a] = __fsub_rn(ngeo->origin[a], half), cgeo->dims[a] = ngeo->dims[a] + (vcount ? 1u : 0u);
-    cgeo->inv_h = ngeo->inv_h;
-    cgeo->h = ngeo->h;
-    cgeo->n_cells = vcount ? nvc : ngeo->n_cells;
+      cgeo->origin[a] = __fsub_rn(n.origin[a], half), cgeo->dims[a] = n.dims[a] + (vcount ? 1u : 0u);
+    cgeo->inv_h = n.inv_h;
+    cgeo->h = n.h;
+    cgeo->n_cells = vcount ? nvc : nbr_cells;
     cgeo->status = 0;
     cgeo->work_n = cgeo->work_n2 = cgeo->work_n3 = cgeo->work_n4 = 0;
     cgeo->work_next = cgeo->work_next2 = cgeo->work_next3 = 0;
@@ -709,7 +711,7 @@ __global__ void __launch_bounds__(kScanThreads) k_central_subset(const float4* _
     if (vcount)
       for (uint32_t i = tid; i < nvc; i += stride) vcount[i] = 0u;
   }
-  const bool list = hv.list != nullptr && ngeo->heavy_listed == 0 && (!hv.if_dense || sweep_pays(nr, ngeo->n_cells, nr));
+  const bool list = hv.list != nullptr && listed == 0 && (!hv.if_dense || sweep_pays(nr, nbr_cells, nr));
   if (list) list_heavy(hv.nstart, ngeo, hv.list, hv.map, hv.n_warps, hv.stencil);
   const uint32_t tiles = (nr + kScanTile - 1) / kScanTile;
   for (;;) {

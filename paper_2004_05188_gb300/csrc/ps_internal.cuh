@@ -137,7 +137,7 @@ __host__ __device__ __forceinline__ uint32_t sub_cells(uint64_t n_rec, uint64_t 
 //   0.91; 8e6-ion needle, Si about all (0.002) 0.36.  The thinner the cloud the larger the share has to be: 4e6-ion
 //   needle, r = 1 nm (13 per cell) 0.92 and 1.19 at 0.35, 0.78 and 1.05 at 0.2, 0.67 and 0.89 at 0.1.
 __host__ __device__ __forceinline__ bool sweep_pays(uint64_t n_nbr, uint64_t n_cells, uint64_t n_ctr) {
-  return n_nbr >= 8 * n_cells && 8 * n_ctr >= n_nbr + 8 * n_cells;
+  return (n_nbr >= 8 * n_cells) & (8 * n_ctr >= n_nbr + 8 * n_cells);  // (both at once: their loads wait together)
 }
 __device__ __forceinline__ bool sweep_pays(const Geo& nbr, const Geo& ctr) {
   return sweep_pays(nbr.n_sel, nbr.n_cells, ctr.n_sel);
