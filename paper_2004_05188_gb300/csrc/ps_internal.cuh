@@ -194,7 +194,8 @@ __host__ __device__ __forceinline__ uint32_t lanes_per_central(uint32_t n_cand, 
 
 // Small clouds: enough lanes per central that the query has as many items as the chip takes warps
 // (about 3,600 on 152 SMs): an item tests its thousands of candidates one after the other, and too few
-// items leave the chip idle for the length of that chain.  2e4-ion cylinder, one pass: 0.317 -> 0.140 ms;
+// items leave the chip idle for the length of that chain.  A fixed number, so that the items of a cloud, and the arrays
+// for them, do not depend on the device.  2e4-ion cylinder, one pass: 0.317 -> 0.140 ms;
 // 3e4 ions, per-ion outputs: 0.64 ms for 912 items, 0.40 for 1824, 0.28 for 3648 and 0.27 for 7296 (which
 // costs the 1e5-ion cloud 10 %: more lanes per central share less of a candidate's load).
 constexpr uint32_t kFillItems = 3648;

@@ -73,6 +73,11 @@ __device__ __forceinline__ uint32_t bin_index(float d2, const float* sE, uint32_
   return (uint32_t)b;
 }
 
+// The inline assembly below writes shared memory without telling the compiler so (no "memory" clobber, which
+// would make it reload what the pair loops hold in registers).  That is sound because C++ code reads or
+// writes those words only behind a barrier: volatile statements keep their order among themselves and
+// around __syncwarp / __syncthreads / the votes, which the compiler takes as barriers for memory.
+//
 // Insertion queue of a lane: a column of a [row][32 lanes] array, `at` the shared address of its next
 // slot.  Every value is stored and the slot taken only if it is below thr: no branch, and one
 // predicated add per value.

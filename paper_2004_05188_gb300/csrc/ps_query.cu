@@ -385,14 +385,14 @@ __device__ __forceinline__ float4 far_record() { return make_float4(INFINITY, IN
 
 // ---------------------------------------------------------------------------
 // warp kernel
-//   heavy items (cells with >= kHeavy centrals, batches of 4..32 centrals): one to eight lanes per
-//     central (item_lanes).  The candidates are read 32 at a time, the stencil's rows nearest
-//     first, and kept only within range of the bounding box of the item's centrals (the
+//   heavy items (cells with at least kHeavy centrals or more than kSparseCand candidates, batches of up
+//     to 32 centrals): one to sixteen lanes per central (item_lanes).  The candidates are read 64 at
+//     a time, the stencil's rows nearest first, and kept only within range of the bounding box of the item's centrals (the
 //     histogram's range, or for kNN alone the largest k-th distance so far); the kept ones are
 //     compacted into a ring of 128 in shared memory as interleaved pairs and tested 32 or 64 at a
 //     time, two per packed test.  Candidates further from the box than every current k-th distance skip
 //     the kNN part of the test.
-//   light items (cells with < kHeavy centrals): the warp takes 32 items at a
+//   light items (the other cells with centrals): the warp takes 32 items at a
 //     time and gives each of their centrals a thread of its own that walks its
 //     own stencil (the records of neighbouring centrals' cells hit in L1).
 // ---------------------------------------------------------------------------
@@ -1001,7 +1001,7 @@ static int launch_rdf_sym(const ps_grid* g, const QueryArgs& qa, const SweepArgs
 constexpr uint32_t kQueue = 40;  // queue rows per lane; inserted when fewer than 16 are free
 constexpr uint32_t kVertexSmem = 8 * (16 * 16 + 16 * 8 + (kQueue + 1) * 32 * 4);  // the kernel's static shared memory
 
-// One warp per item (up to 32 centrals of a vertex cell, one to eight lanes each), its candidates the
+// One warp per item (up to 32 centrals of a vertex cell, one to sixteen lanes each), its candidates the
 // records of the 2 x 2 x 2 cells around the vertex, staged 32 at a time as interleaved pairs.  A sorted
 // insertion costs ~25 instructions for the whole warp whichever lanes need it, so the candidates
 // are filtered first: by the central's reach and by the radius that holds k + 3 sqrt(k) records

@@ -385,6 +385,7 @@ __global__ void __launch_bounds__(256, 4) k_soft_fwd_sym(const SoftArgs a, const
       for (int e = 0; e < 2; ++e) {
         if (u[e] < rc) {
           const uint32_t at = __float_as_uint(mm[e]) * 12u + base;
+          // (without "memory" clobbers: C++ code touches these words only behind barriers and votes, see ps_items.cuh)
           uint32_t old;
           asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(at), "r"(wt));
           hot |= old;
