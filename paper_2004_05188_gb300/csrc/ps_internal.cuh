@@ -148,8 +148,8 @@ __device__ __forceinline__ bool sweep_pays(const Geo& nbr, const Geo& ctr) {
 // over the bounding box (2e5-ion cylinder, 9 records per cell: 0.272 ms with one cell, 0.236 ms with two; the
 // 8e6-ion needle's 28 records per filled cell need no company).
 __host__ __device__ __forceinline__ uint32_t sweep_block(uint32_t n_cells, uint32_t n_sel) {
-  const float w = 12.f * (float)n_cells / (float)(n_sel ? n_sel : 1u);
-  return w > 7.f ? 8u : (w <= 1.f ? 1u : (uint32_t)ceilf(w));
+  const uint64_t n = n_sel ? n_sel : 1u, w = (12ull * n_cells + n - 1) / n;  // (integers: two translation units agree on it)
+  return w > 8 ? 8u : (uint32_t)w;
 }
 // Candidate parts per block of the sweep: at least 4 units per warp of the launch.
 __host__ __device__ __forceinline__ uint32_t sweep_parts(uint64_t n_blocks, uint32_t n_warps) {
