@@ -854,7 +854,8 @@ def rooflines(prof, st, steps, peaks, hbm_peak, hbm_src, traffic):
         "avg_launch_ms": d.get("avg_launch_ms"),
         "by_kernel": by_kernel,
         "all_query_passes": {"achieved": alu, "frac": alu / alu_peak if alu_peak > 0 else None, "launches": q_n,
-                             "avg_launch_ms": q_ms / max(1, q_n), "candidate_tests_per_step": cands // max(1, steps)},
+                             "avg_launch_ms": q_ms / max(1, q_n), "candidate_tests_per_step": cands // max(1, steps),
+                             "stencil_pairs_per_step": sum(c.get("stencil_pairs", 0) for c in st["combos"])},
         "pass_ms_per_step": {f: prof[f][1] / max(1, steps) for f in QUERY_FAMS},
         "timing": "CUDA events around every launch on the launching stream, inside the timed region",
         "time_share": q_ms / tot_ms if tot_ms > 0 else None,
