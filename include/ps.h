@@ -113,7 +113,7 @@ typedef struct {
                          have fewer than k neighbours there, and the RDF over unordered pairs (each
                          pair tested once, counted once per central end).  Same results; 0
                          (default): one combined pass, which leaves the RDF and the in-range
-                         counts of dense clouds to the pass over unordered pairs as well */
+                         counts of dense clouds with many centrals to the pass over unordered pairs as well */
 } ps_grid_opts;
 
 typedef struct ps_grid ps_grid; /* opaque; owns its device scratch */
